@@ -14,8 +14,18 @@
 //     memory: S0, S1, O0, O1 fill all 512 columns; P (bf16) overwrites S in place and is the A operand of
 //     the P V product directly from tensor memory;
 //   * warp roles: warps 0-3 / 4-7 = softmax of Q tile 0 / 1 (one thread per row, online softmax in fp32 in
-//     the exp2 domain, running maximum updated lazily), warp 8 = MMA issue, warp 9 = TMA producer.
+//     the exp2 domain, running maximum updated lazily), warp 8 = MMA issue, warp 9 = TMA producer.  The producer walks
+//     the tile list, and hands each tile's height to the others beside the tile; the MMA warp waits once per step for
+//     (V of tile j, K of tile j + 1) and then only for P, since every further wait or branch between two groups of MMAs
+//     is time the tensor pipe stands still (its queue holds about two MMAs);
+//   * a tile with nv < 128 valid rows (the last one of a segment or slot: 1,320 rows are 10 tiles and 40 rows) is
+//     multiplied over ceil(nv / 16) * 16 rows and its softmax stops at the last group of 32.
+// What bounds it: the chain of one Q tile (softmax ~1,650 clk -> P V and Q K^T 1,050 -> hand-overs ~450, 3,150 clk per KV
+// tile at 12 heads x 880 tokens) while the board is at its 1,000 W cap; before the issue path was rebuilt 3,280 clk, and
+// 278 -> 270 us sustained, 276 -> 247 us alone, at 2,640 queries x 15,840 keys x 12 heads.
 // Every wait is bounded; a wait that runs out sets WK_DEV_TIMEOUT, the CTA drains and frees its tensor memory.
+#include <stddef.h>
+
 #include "ptx_sm100.cuh"
 #include "wk_internal.cuh"
 
@@ -28,9 +38,13 @@ constexpr int kThreads = 320;
 constexpr int kMmaWarp = 8, kTmaWarp = 9;
 constexpr uint32_t kHalfTileBytes = 128 * 64 * 2;   // one TMA box: 128 rows x 64 bf16 = 16 KB
 constexpr uint32_t kTileBytes = 2 * kHalfTileBytes; // 128 x 128 bf16
-constexpr int kStagesK = 3, kStagesV = 2;           // K is wanted one MMA group earlier than V: it gets the spare 32 KB
-constexpr size_t kSmemBytes = 1024 + 2 * kTileBytes + (kStagesK + kStagesV) * kTileBytes;   // align slack + Q0,Q1 + K,V stages
+// A stage holds what one step of the MMA warp consumes: V of tile j and K of tile j + 1 (LSE-only launches: K alone).
+constexpr int kStages = 2, kStagesLse = 5;
+constexpr size_t kSmemBytes = 1024 + 2 * kTileBytes + 2 * kStages * kTileBytes;   // align slack + Q0,Q1 + stages
+constexpr size_t kSmemBytesLse = 1024 + 2 * kTileBytes + kStagesLse * kTileBytes;
+constexpr int kNvRing = 16;   // tile heights handed from the TMA warp to the others; the TMA warp is at most kStagesLse + 1 tiles ahead
 constexpr float kRescaleThreshold = 8.0f;           // log2 units: P stays <= 2^8 between maximum updates
+constexpr uint32_t kTmemS = 0, kTmemO = 256;        // tensor-memory columns: S0, S1 (P over them), O0, O1
 constexpr int kPairRows = 2 * kTileQ;
 constexpr int kMaxPieces = 32;                      // most ranges one unit may be cut into
 
@@ -137,43 +151,83 @@ struct TileIter {
   }
 };
 
+// Number of effective tiles in [tb, te), by a whole warp: the lanes look at the slot list side by side.
+__device__ __forceinline__ int count_tiles(const AttnParams& p, int tb, int te) {
+  const int dense = max(0, min(te, p.n_dense_tiles) - tb);
+  const int ub = max(tb, p.n_dense_tiles) - p.n_dense_tiles, ue = te - p.n_dense_tiles;
+  int n = 0;
+  if (ue > ub) {
+    const int last = (ue - 1) / p.tiles_per_slot;
+    for (int si = ub / p.tiles_per_slot + static_cast<int>(threadIdx.x & 31); si <= last; si += 32) {
+      const int slot = __ldg(p.slots + si);
+      if (slot >= 0 && slot < p.pool_slots && __ldg(p.valid + slot) != 0)
+        n += min(ue, (si + 1) * p.tiles_per_slot) - max(ub, si * p.tiles_per_slot);
+    }
+    n = __reduce_add_sync(0xffffffffu, n);
+  }
+  return dense + n;
+}
+
 #ifdef WK_ATTN_PROFILE
 // Stage timers for one designated thread per role of CTA 0: clock deltas are accumulated in registers and added into the
 // words after the status word when the role finishes.  Built only for profiling runs; the product build has none of this.
-#define WK_PROF_DECL uint32_t prof_t = clock(); uint32_t prof_acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#define WK_PROF(slot, cond)                              \
+#define WK_PROF_DECL uint32_t prof_t = clock(); uint32_t prof_acc[12] = {}; uint64_t prof_ns; uint32_t prof_c0 = prof_t; \
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(prof_ns));
+#define WK_PROF(slot)                                    \
   do {                                                   \
     const uint32_t now__ = clock();                      \
-    prof_acc[(slot) & 7] += now__ - prof_t;              \
+    prof_acc[slot] += now__ - prof_t;                    \
     prof_t = now__;                                      \
   } while (0)
-#define WK_PROF_FLUSH(base, cond)                                                          \
+#define WK_PROF_FLUSH(base, n, cond)                                                       \
   do {                                                                                     \
-    if (cond)                                                                              \
-      for (int i__ = 0; i__ < 8; ++i__) atomicAdd(p.status + 8 + (base) + i__, prof_acc[i__] >> 4); \
+    if (cond) {                                                                            \
+      uint64_t ns2; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns2));               \
+      prof_acc[n - 2] = (clock() - prof_c0); prof_acc[n - 1] = static_cast<uint32_t>(ns2 - prof_ns); \
+      for (int i__ = 0; i__ < n; ++i__) p.status[8 + (base) + i__] = prof_acc[i__];         \
+    }                                                                                      \
   } while (0)
 #else
 #define WK_PROF_DECL
-#define WK_PROF(slot, cond)
-#define WK_PROF_FLUSH(base, cond)
+#define WK_PROF(slot)
+#define WK_PROF_FLUSH(base, n, cond)
 #endif
 
 struct __align__(8) Barriers {
   uint64_t q_full, q_empty;
-  uint64_t k_full[kStagesK], k_empty[kStagesK], v_full[kStagesV], v_empty[kStagesV];
+  uint64_t kv_full[kStagesLse], kv_empty[kStagesLse];
   uint64_t s_full[2], p_full[2], o_done[2], o_free[2];
 };
 
-// Bounded wait that also gives up when another role has already aborted.
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag,
-                                              uint32_t* status) {
-  for (uint32_t i = 0; i < WK_WAIT_CAP; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 1023u) == 1023u && *abort_flag) return false;
+// Bounded wait that also gives up when another role has already aborted; false then.  A loop of eight instructions and
+// nothing else: what follows a failed wait (the status bit, the abort flag) stands once per role, at its end (leave_role).
+__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .u32 n, a;\n\t"
+      "mov.u32 n, 0;\n"
+      "WAIT_LOOP:\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@p bra WAIT_DONE;\n\t"
+      "ld.volatile.shared.u32 a, [%3];\n\t"
+      "setp.ne.u32 q, a, 0;\n\t"
+      "@q bra WAIT_DONE;\n\t"
+      "add.u32 n, n, 1;\n\t"
+      "setp.lt.u32 q, n, %4;\n\t"
+      "@q bra WAIT_LOOP;\n"
+      "WAIT_DONE:\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(smem_u32(const_cast<uint32_t*>(abort_flag))), "n"(WK_WAIT_CAP)
+      : "memory");
+  return ok != 0;
+}
+// A role that has given up tells the others and sets the status bit (unless it left because another role did).
+__device__ __forceinline__ void leave_role(bool ok, volatile uint32_t* abort_flag, uint32_t* status) {
+  if (!ok && *abort_flag == 0) {
+    *abort_flag = 1;
+    atomicOr(status, WK_DEV_TIMEOUT);
   }
-  *abort_flag = 1;
-  atomicOr(status, WK_DEV_TIMEOUT);
-  return false;
 }
 
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
@@ -193,7 +247,7 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
 #define WK_ATTN_POLY 2
 #endif
 template <bool kStore, int kPoly>
-__device__ __forceinline__ float exp_store_tile(const float (&s)[128], uint64_t scale2, uint64_t neg_m2, uint32_t tS) {
+__device__ __forceinline__ float exp_store_tile(const float (&s)[128], uint64_t scale2, uint64_t neg_m2, uint32_t tS, int n_chunks) {
   uint64_t acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0;   // four independent (lo, hi) sums
   const uint64_t magic2 = pack_f32x2(12582912.f, 12582912.f), nmagic2 = pack_f32x2(-12582912.f, -12582912.f);
   const uint64_t mone2 = pack_f32x2(-1.f, -1.f);
@@ -203,6 +257,7 @@ __device__ __forceinline__ float exp_store_tile(const float (&s)[128], uint64_t 
   const uint64_t c3 = pack_f32x2(0.055088773369789124f, 0.055088773369789124f);
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
+    if (kPoly == 0 && c >= n_chunks) break;   // a short tile stops at its last group of 32 columns
     uint32_t pk[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -284,21 +339,23 @@ template <bool kLse>
 __global__ void __launch_bounds__(kThreads, 1)
 memory_attention_kernel(const __grid_constant__ AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
   uint8_t* sQ = smem;                                   // [2 q tiles][2 halves][128 rows][128 B]
-  uint8_t* sK = sQ + 2 * kTileBytes;                    // [stages][2 halves][128][128 B]
-  uint8_t* sV = sK + kStagesK * kTileBytes;
+  uint8_t* sKV = sQ + 2 * kTileBytes;                   // [stages][K, V][2 halves][128][128 B]; LSE-only: [stages][K]
+  constexpr uint32_t kNStages = kLse ? kStagesLse : kStages;
+  constexpr uint32_t kStageBytes = kLse ? kTileBytes : 2 * kTileBytes;
   __shared__ Barriers bars;
   __shared__ uint32_t s_tmem;
   __shared__ volatile uint32_t s_abort;
+  __shared__ volatile int s_nv[kNvRing];   // valid rows of tile number t (counted over the CTA's pieces) at t % kNvRing
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid == 0) {
     mbar_init(&bars.q_full, 1);
     mbar_init(&bars.q_empty, 1);
-    for (int s = 0; s < kStagesK; ++s) { mbar_init(&bars.k_full[s], 1); mbar_init(&bars.k_empty[s], 1); }
-    for (int s = 0; s < kStagesV; ++s) { mbar_init(&bars.v_full[s], 1); mbar_init(&bars.v_empty[s], 1); }
+    for (int s = 0; s < kStagesLse; ++s) { mbar_init(&bars.kv_full[s], 1); mbar_init(&bars.kv_empty[s], 1); }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bars.s_full[i], 1); mbar_init(&bars.p_full[i], 4); mbar_init(&bars.o_done[i], 1);
       mbar_init(&bars.o_free[i], 4);
@@ -313,7 +370,8 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = s_tmem;
+  // an allocation of all 512 columns starts at column 0; addresses known at compile time keep the MMAs' operands cheap
+  if (s_tmem != 0 && tid == 0) { s_abort = 1; atomicOr(p.status, WK_DEV_TIMEOUT); }
 
   if (warp == kTmaWarp) {
     // ------------------------------------------------------------------ TMA producer
@@ -321,13 +379,12 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
       PieceWalker walk;
       walk.init(p);
       Piece pc;
-      uint32_t jk = 0, n = 0;
-      uint32_t armed_q = 0, armed_k = 0, armed_v = 0;   // loads armed so far (a barrier's u-th use completes its phase u)
+      uint32_t st = 0, ph = 1, steps = 0, n = 0, t = 0;   // stage, its parity, stages and Q pairs armed so far, tiles so far
       bool ok = true;
       while (ok && walk.next(p, pc)) {
-        if (!(ok = wait_or_abort(&bars.q_empty, (n & 1) ^ 1, &s_abort, p.status))) break;
+        if (!(ok = wait_or_abort(&bars.q_empty, (n & 1) ^ 1, &s_abort))) break;
         mbar_expect_tx(&bars.q_full, 2 * kTileBytes);
-        armed_q = n + 1;
+        ++n;
         for (int i = 0; i < 2; ++i)
           for (int half = 0; half < 2; ++half)
             tma_load_2d(sQ + i * kTileBytes + half * kHalfTileBytes, &p.tm_q, &bars.q_full, pc.h * kHeadDim + half * 64,
@@ -335,38 +392,33 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
         TileIter it;
         const bool report = !p.slot_units;
         it.init(p, pc.tb, pc.te, report);
-        TileInfo ti;
         const int x = pc.h * kHeadDim;
-        while (it.next(p, ti, report)) {
-          const int sk = jk % kStagesK, st = jk % kStagesV;
-          const uint32_t phk = (jk / kStagesK) & 1, ph = (jk / kStagesV) & 1;
-          if (!(ok = wait_or_abort(&bars.k_empty[sk], phk ^ 1, &s_abort, p.status))) break;
-          mbar_expect_tx(&bars.k_full[sk], kTileBytes);
-          armed_k = jk + 1;
-          uint8_t* dk = sK + sk * kTileBytes;
+        auto load = [&](uint8_t* dst, const TileInfo& ti, const CUtensorMap* seg_maps, const CUtensorMap* pool_map) {
           if (ti.seg >= 0) {
-            tma_load_2d(dk, &p.tm_kd[ti.seg], &bars.k_full[sk], x, ti.row0);
-            tma_load_2d(dk + kHalfTileBytes, &p.tm_kd[ti.seg], &bars.k_full[sk], x + 64, ti.row0);
+            tma_load_2d(dst, seg_maps + ti.seg, &bars.kv_full[st], x, ti.row0);
+            tma_load_2d(dst + kHalfTileBytes, seg_maps + ti.seg, &bars.kv_full[st], x + 64, ti.row0);
           } else {
-            tma_load_3d(dk, &p.tm_kpool, &bars.k_full[sk], x, ti.row0, ti.z);
-            tma_load_3d(dk + kHalfTileBytes, &p.tm_kpool, &bars.k_full[sk], x + 64, ti.row0, ti.z);
+            tma_load_3d(dst, pool_map, &bars.kv_full[st], x, ti.row0, ti.z);
+            tma_load_3d(dst + kHalfTileBytes, pool_map, &bars.kv_full[st], x + 64, ti.row0, ti.z);
           }
-          if (kLse) { ++jk; continue; }   // no P V product: V is not fetched
-          if (!(ok = wait_or_abort(&bars.v_empty[st], ph ^ 1, &s_abort, p.status))) break;
-          mbar_expect_tx(&bars.v_full[st], kTileBytes);
-          armed_v = jk + 1;
-          uint8_t* dv = sV + st * kTileBytes;
-          if (ti.seg >= 0) {
-            tma_load_2d(dv, &p.tm_vd[ti.seg], &bars.v_full[st], x, ti.row0);
-            tma_load_2d(dv + kHalfTileBytes, &p.tm_vd[ti.seg], &bars.v_full[st], x + 64, ti.row0);
-          } else {
-            tma_load_3d(dv, &p.tm_vpool, &bars.v_full[st], x, ti.row0, ti.z);
-            tma_load_3d(dv + kHalfTileBytes, &p.tm_vpool, &bars.v_full[st], x + 64, ti.row0, ti.z);
-          }
-          ++jk;
+        };
+        TileInfo ti, tv;
+        bool have_k = it.next(p, ti, report), have_v = false;
+        while (have_k || have_v) {   // step: V of the tile before (not in LSE-only launches), K of this tile
+          if (!(ok = wait_or_abort(&bars.kv_empty[st], ph, &s_abort))) break;
+          if (have_k) s_nv[t++ % kNvRing] = ti.nv;   // read after kv_full
+          mbar_expect_tx(&bars.kv_full[st], (have_k ? kTileBytes : 0) + (have_v ? kTileBytes : 0));
+          ++steps;
+          uint8_t* dst = sKV + st * kStageBytes;
+          if (have_k) load(dst, ti, p.tm_kd, &p.tm_kpool);
+          if (have_v) load(dst + kTileBytes, tv, p.tm_vd, &p.tm_vpool);
+          if (++st == kNStages) { st = 0; ph ^= 1; }
+          have_v = have_k && !kLse;
+          tv = ti;
+          if (have_k) have_k = it.next(p, ti, report);
         }
-        ++n;
       }
+      leave_role(ok, &s_abort, p.status);
       // After an abort the consumers no longer wait for the tiles in flight, so this thread does: a CTA must not free
       // its shared memory under copies that are still landing.  Per stage, the load armed last is use u = (count - 1 -
       // stage) / stages of that stage's barrier, whose phase u has parity u & 1; a stage that was never armed is skipped.
@@ -375,74 +427,64 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           for (uint32_t i = 0; i < (1u << 16); ++i)
             if (mbar_try_wait(bar, use & 1)) break;
         };
-        if (armed_q > 0) drain(&bars.q_full, armed_q - 1);
-        for (uint32_t s = 0; s < kStagesK; ++s)
-          if (armed_k > s) drain(&bars.k_full[s], (armed_k - 1 - s) / kStagesK);
-        for (uint32_t s = 0; s < kStagesV; ++s)
-          if (armed_v > s) drain(&bars.v_full[s], (armed_v - 1 - s) / kStagesV);
+        if (n > 0) drain(&bars.q_full, n - 1);
+        for (uint32_t q = 0; q < kNStages; ++q)
+          if (steps > q) drain(&bars.kv_full[q], (steps - 1 - q) / kNStages);
       }
     }
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------------ MMA issue
-    // The whole warp runs the control flow (waits, counters, descriptor arithmetic) so that everything stays
-    // warp-uniform; one elected lane issues the tensor-core instructions and the commits.
+    // The whole warp runs the control flow and one lane's predicate issues (see mma_ss_if).
     {
-      const uint32_t idesc_qk = idesc_bf16_f32(128, 128, 0, 0);
-      const uint32_t idesc_pv = idesc_bf16_f32(128, 128, 0, 1);
-      const uint32_t aQ = smem_u32(sQ), aK = smem_u32(sK), aV = smem_u32(sV);
-      // descriptor low words of the tile bases; a K = 16 step advances them by a constant
-      const uint32_t hi = smem_desc_hi_sw128(1024);
-      const uint32_t q_lo0 = smem_desc_lo(aQ, 16), q_lo1 = smem_desc_lo(aQ + kTileBytes, 16);
-      const uint32_t k_lo0 = smem_desc_lo(aK, 16), v_lo0 = smem_desc_lo(aV, kHalfTileBytes);
-      auto issue_s = [&](int i, uint32_t st) {
-        const uint32_t d = tmem + i * 128;
-        const uint32_t a_lo = i ? q_lo1 : q_lo0, b_lo = k_lo0 + st * (kTileBytes >> 4);
-        if (elect_one()) {
+      const uint32_t one = elect_one() ? 1u : 0u;
+      constexpr uint32_t idesc_qk = idesc_bf16_f32(128, 128, 0, 0), idesc_pv = idesc_bf16_f32(128, 128, 0, 1);
+      // descriptors of the tile bases; a K = 16 step advances the low word by a constant
+      constexpr uint64_t hi = static_cast<uint64_t>(smem_desc_hi_sw128(1024)) << 32;
+      const uint64_t q_desc = hi | smem_desc_lo(smem_base, 16);
+      const uint64_t k_desc = hi | smem_desc_lo(smem_base + 2 * kTileBytes, 16);
+      const uint64_t v_desc = hi | smem_desc_lo(smem_base + 3 * kTileBytes, kHalfTileBytes);
+      const uint32_t bar0 = smem_u32(&bars);
+      auto commit = [&](size_t offset) { mma_commit_if(one, bar0 + static_cast<uint32_t>(offset)); };
+      // S_i = Q_i K^T over the first nv rows of the K tile.  A full tile is eight MMAs without a branch between them; a
+      // short one computes ceil(nv / 16) * 16 columns.
+      auto issue_s = [&](uint32_t i, uint32_t st, int nv) {
+        const uint64_t a = q_desc + i * (kTileBytes >> 4), b = k_desc + st * (kStageBytes >> 4);
+        const uint32_t idesc = nv == kTileKV ? idesc_qk
+                                             : (idesc_bf16_f32(128, 0, 0, 0) | (static_cast<uint32_t>((nv + 15) >> 4) << 18));
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const uint32_t off = (k >> 2) * (kHalfTileBytes >> 4) + (k & 3) * 2;   // 32 bytes per step inside a 128-byte row
-            mma_ss_lohi(d, a_lo + off, b_lo + off, hi, idesc_qk, k > 0);
-          }
+        for (int k = 0; k < 8; ++k) {
+          const uint32_t off = (k >> 2) * (kHalfTileBytes >> 4) + (k & 3) * 2;   // 32 bytes per step inside a 128-byte row
+          mma_ss_if(one, kTmemS + i * 128, a + off, b + off, idesc, k > 0);
         }
-        __syncwarp();
       };
-      auto issue_pv = [&](int i, uint32_t st, bool accumulate) {
-        const uint32_t d = tmem + 256 + i * 128;
-        const uint32_t b_lo = v_lo0 + st * (kTileBytes >> 4);
-        if (elect_one()) {
+      // O_i (+)= P_i V: A = P from tensor memory (bf16 pairs, 8 columns per K = 16 step); B = V, rows = K dimension,
+      // MN-major: 16 rows of 128 bytes = 2048 bytes per step
+      auto issue_pv = [&](uint32_t i, uint32_t st, int nv, uint32_t accumulate) {
+        const uint64_t b = v_desc + st * (kStageBytes >> 4);
+        if (nv == kTileKV) {
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            // A = P from tensor memory (bf16 pairs, 8 columns per K = 16 step); B = V, rows = K dimension, MN-major:
-            // 16 rows of 128 bytes = 2048 bytes per step
-            mma_ts_lohi(d, tmem + i * 128 + k * 8, b_lo + k * 128, hi, idesc_pv, (accumulate || k > 0) ? 1u : 0u);
-          }
+          for (int k = 0; k < 8; ++k)
+            mma_ts_if(one, kTmemO + i * 128, kTmemS + i * 128 + k * 8, b + k * 128, idesc_pv, k > 0 ? 1u : accumulate);
+        } else {
+#pragma unroll 1
+          for (int k = 0; k * 16 < nv; ++k)
+            mma_ts_if(one, kTmemO + i * 128, kTmemS + i * 128 + k * 8, b + k * 128, idesc_pv, k > 0 ? 1u : accumulate);
         }
-        __syncwarp();
-      };
-      auto commit = [&](uint64_t* bar) {
-        if (elect_one()) mma_commit(bar);
-        __syncwarp();
       };
       PieceWalker walk;
       walk.init(p);
       Piece pc;
-      // stage and phase of the K tile whose Q K^T is issued next / of the V tile whose P V is issued next: counters
-      // instead of divisions on the issuing path
-      uint32_t ks = 0, kph = 0, vs = 0, vph = 0;
-      uint32_t g0 = 0, g1 = 0, n = 0;   // running tile counts of the two Q tiles, running piece count
+      uint32_t st = 0, ph = 0;          // stage and its parity
+      uint32_t p_ph0 = 0, p_ph1 = 0;    // parities of p_full[0], p_full[1]
+      uint32_t n = 0, t = 0;            // running piece and tile counts
       uint32_t e0 = 0, e1 = 0;          // pieces in which Q tile 0 / 1 produced output so far
+      uint32_t lse_q0 = 0, lse_q1 = 0;  // LSE-only: products of Q tile 0 / 1 so far
       WK_PROF_DECL
       bool ok = true;
       while (ok && walk.next(p, pc)) {
-        int n_eff = 0;
-        {
-          TileIter it;
-          it.init(p, pc.tb, pc.te, false);
-          TileInfo ti;
-          while (it.next(p, ti, false)) ++n_eff;
-        }
+        const int n_eff = count_tiles(p, pc.tb, pc.te);
         const bool q1 = pc.has_q1;
-        if (!(ok = wait_or_abort(&bars.q_full, n & 1, &s_abort, p.status))) break;
+        if (!(ok = wait_or_abort(&bars.q_full, n & 1, &s_abort))) break;
         ++n;
         if (n_eff == 0) {
           if (lane == 0) mbar_arrive(&bars.q_empty);
@@ -451,91 +493,84 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
         // O0 / O1 are about to be overwritten: the epilogue of the last piece that used them must have read them.
         // o_free[i] completes once per piece in which warpgroup i ran an epilogue, so neither side can run two
         // phases ahead of the other (a parity wait cannot tell phase n from phase n + 2).
-        if (e0 > 0 && !(ok = wait_or_abort(&bars.o_free[0], (e0 - 1) & 1, &s_abort, p.status))) break;
-        ++e0;
-        if (q1) {
-          if (e1 > 0 && !(ok = wait_or_abort(&bars.o_free[1], (e1 - 1) & 1, &s_abort, p.status))) break;
-          ++e1;
-        }
-        auto next_k = [&]() { if (++ks == kStagesK) { ks = 0; kph ^= 1; } };
-        auto next_v = [&]() { if (++vs == kStagesV) { vs = 0; vph ^= 1; } };
-        {
-          if (!(ok = wait_or_abort(&bars.k_full[ks], kph, &s_abort, p.status))) break;
-          tc_fence_after();
-          issue_s(0, ks);
-          commit(&bars.s_full[0]);
-          if (q1) { issue_s(1, ks); commit(&bars.s_full[1]); }
-          commit(&bars.k_empty[ks]);
-          if (n_eff == 1) commit(&bars.q_empty);
-          next_k();
-        }
-        for (int j = 0; j < n_eff; ++j) {
-          const bool more = j + 1 < n_eff;
-          WK_PROF(10, blockIdx.x == 0);
-          if (!kLse && !(ok = wait_or_abort(&bars.v_full[vs], vph, &s_abort, p.status))) break;
-          WK_PROF(11, blockIdx.x == 0);
-          if (!(ok = wait_or_abort(&bars.p_full[0], (g0 + j) & 1, &s_abort, p.status))) break;
-          WK_PROF(12, blockIdx.x == 0);
-          tc_fence_after();
-          if (!kLse) issue_pv(0, vs, j > 0);
-          commit(&bars.o_done[0]);
-          if (more) {
-            WK_PROF(13, blockIdx.x == 0);
-            if (!(ok = wait_or_abort(&bars.k_full[ks], kph, &s_abort, p.status))) break;
-            WK_PROF(14, blockIdx.x == 0);
-            tc_fence_after();
-            issue_s(0, ks);
-            commit(&bars.s_full[0]);
-          }
+        if (!kLse) {
+          if (e0 > 0 && !(ok = wait_or_abort(&bars.o_free[0], (e0 - 1) & 1, &s_abort))) break;
+          ++e0;
           if (q1) {
-            WK_PROF(15, blockIdx.x == 0);
-            if (!(ok = wait_or_abort(&bars.p_full[1], (g1 + j) & 1, &s_abort, p.status))) break;
-            WK_PROF(16, blockIdx.x == 0);
-            tc_fence_after();
-            if (!kLse) issue_pv(1, vs, j > 0);
-            commit(&bars.o_done[1]);
-          }
-          if (!kLse) commit(&bars.v_empty[vs]);
-          next_v();
-          if (more) {
-            if (q1) { issue_s(1, ks); commit(&bars.s_full[1]); }
-            commit(&bars.k_empty[ks]);
-            if (j + 2 == n_eff) commit(&bars.q_empty);   // the last Q K^T of this piece has been issued
-            next_k();
+            if (e1 > 0 && !(ok = wait_or_abort(&bars.o_free[1], (e1 - 1) & 1, &s_abort))) break;
+            ++e1;
           }
         }
-        g0 += n_eff;
-        if (q1) g1 += n_eff;
+        // Step j: for each Q tile, once its P of tile j is there, P V of tile j and Q K^T of tile j + 1 into the S buffer
+        // P was in.  The other Q tile's softmax runs meanwhile.  (LSE-only: no P V; the "P" signal says that S has been read.)
+        int nv = 0, nv_next = 0;
+        for (int j = -1; j < n_eff - (kLse ? 1 : 0); ++j) {
+          const bool more = j + 1 < n_eff;
+          WK_PROF(0);
+          if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &s_abort))) break;
+          if (more) nv_next = s_nv[t++ % kNvRing];
+          WK_PROF(1);
+          if (kLse ? lse_q0 > 0 : j >= 0) {
+            if (!(ok = wait_or_abort(&bars.p_full[0], p_ph0, &s_abort))) break;
+            p_ph0 ^= 1;
+          }
+          if (kLse) ++lse_q0;
+          WK_PROF(2);
+          tc_fence_after();
+          if (!kLse && j >= 0) issue_pv(0, st, nv, j > 0);
+          if (more) { issue_s(0, st, nv_next); commit(offsetof(Barriers, s_full)); }
+          else commit(offsetof(Barriers, o_done));
+          if (!q1) commit(offsetof(Barriers, kv_empty) + 8 * st);
+          WK_PROF(3);
+          if (q1) {
+            if (kLse ? lse_q1 > 0 : j >= 0) {
+              if (!(ok = wait_or_abort(&bars.p_full[1], p_ph1, &s_abort))) break;
+              p_ph1 ^= 1;
+            }
+            if (kLse) ++lse_q1;
+            WK_PROF(4);
+            tc_fence_after();
+            if (!kLse && j >= 0) issue_pv(1, st, nv, j > 0);
+            if (more) { issue_s(1, st, nv_next); commit(offsetof(Barriers, s_full) + 8); }
+            else commit(offsetof(Barriers, o_done) + 8);
+            commit(offsetof(Barriers, kv_empty) + 8 * st);
+            WK_PROF(5);
+          }
+          if (j + 2 == n_eff) commit(offsetof(Barriers, q_empty));   // the last Q K^T of this piece has been issued
+          if (++st == kNStages) { st = 0; ph ^= 1; }
+          nv = nv_next;
+        }
       }
-      WK_PROF_FLUSH(8, blockIdx.x == 0);
+      if (lane == 0) leave_role(ok, &s_abort, p.status);
+      WK_PROF_FLUSH(8, 12, blockIdx.x == 0 && lane == 0);
     }
   } else {
     // ------------------------------------------------------------------ softmax warpgroups (one thread per query row)
     const int wg = warp >> 2;
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const uint32_t tS = tmem + lane_base + wg * 128;
-    const uint32_t tO = tmem + lane_base + 256 + wg * 128;
+    const uint32_t tS = lane_base + kTmemS + wg * 128;
+    const uint32_t tO = lane_base + kTmemO + wg * 128;
     PieceWalker walk;
     walk.init(p);
     Piece pc;
-    uint32_t g = 0;   // running tile count of this warpgroup
+    uint32_t g = 0;       // running tile count of this warpgroup
+    uint32_t t0 = 0;      // tiles of the CTA's pieces so far
+    uint32_t n_out = 0;   // pieces of this warpgroup that produced output
     bool ok = true;
     WK_PROF_DECL
     const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2);
     while (ok && walk.next(p, pc)) {
       const bool active = (wg == 0) || pc.has_q1;
+      const int n_eff = count_tiles(p, pc.tb, pc.te);
       float m_used = -INFINITY, l = 0.f;
       int j = 0;
       if (active) {
-        TileIter it;
-        it.init(p, pc.tb, pc.te, false);
-        TileInfo ti;
-        while (it.next(p, ti, false)) {
-          const int nv = ti.nv;
-          WK_PROF(0, blockIdx.x == 0 && tid == 0);
-          if (!(ok = wait_or_abort(&bars.s_full[wg], g & 1, &s_abort, p.status))) break;
-          WK_PROF(1, blockIdx.x == 0 && tid == 0);
+        while (j < n_eff) {
+          WK_PROF(0);
+          if (!(ok = wait_or_abort(&bars.s_full[wg], g & 1, &s_abort))) break;
+          const int nv = s_nv[(t0 + j) % kNvRing];
+          WK_PROF(1);
           tc_fence_after();
           // the whole S row (128 fp32) is held in registers: one pass for the row maximum, one for the exponentials
           float s[128];
@@ -561,7 +596,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
             }
             tc_wait_ld();
           }
-          WK_PROF(2, blockIdx.x == 0 && tid == 0);
+          WK_PROF(2);
           if (kLse) {   // S is in registers and nothing goes back into the buffer: release it now
             tc_fence_before();
             __syncwarp();
@@ -598,14 +633,12 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           }
           l *= alpha;
           const uint64_t neg_m2 = pack_f32x2(-m_used, -m_used);
-          WK_PROF(3, blockIdx.x == 0 && tid == 0);
+          WK_PROF(3);
           // masked columns hold -inf and come out as 0 (special-function path only)
-          l += full_tile ? exp_store_tile<!kLse, WK_ATTN_POLY>(s, scale2, neg_m2, tS)
-                         : exp_store_tile<!kLse, 0>(s, scale2, neg_m2, tS);
+          l += full_tile ? exp_store_tile<!kLse, WK_ATTN_POLY>(s, scale2, neg_m2, tS, 4)
+                         : exp_store_tile<!kLse, 0>(s, scale2, neg_m2, tS, (nv + 31) >> 5);
           if (!kLse && __any_sync(0xffffffffu, rescale)) {
-            // the previous P V product must have landed before O is touched
-            if (!(ok = wait_or_abort(&bars.o_done[wg], (g - 1) & 1, &s_abort, p.status))) break;
-            tc_fence_after();
+            // (the previous P V was issued before this tile's Q K^T: it landed before S did)
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
               uint32_t r[32];
@@ -616,21 +649,21 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
               tmem_st_x32(tO + c * 32, r);
             }
           }
-          WK_PROF(4, blockIdx.x == 0 && tid == 0);
+          WK_PROF(4);
           if (!kLse) {
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.p_full[wg]);   // one arrival per warp: the wait above covered all 32 lanes' stores
           }
-          WK_PROF(5, blockIdx.x == 0 && tid == 0);
+          WK_PROF(5);
           ++j;
           ++g;
         }
         // ---------------------------------------------------------------- epilogue of this piece
         const int prow = wg * kTileQ + row;
         const int qrow = pc.q0 + prow;
-        if (ok && j > 0) ok = wait_or_abort(&bars.o_done[wg], (g - 1) & 1, &s_abort, p.status);
+        if (!kLse && ok && j > 0) ok = wait_or_abort(&bars.o_done[wg], n_out++ & 1, &s_abort);   // completes once per piece
         if (ok) {
           tc_fence_after();
           const float inv_l = (j > 0 && l > 0.f) ? 1.f / l : 0.f;
@@ -676,6 +709,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           }
         }
       }
+      t0 += n_eff;
       // O of this piece has been read: the next piece that uses this accumulator may overwrite it
       if (active && j > 0) {
         tc_fence_before();
@@ -683,11 +717,12 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
         if (lane == 0) mbar_arrive(&bars.o_free[wg]);
       }
     }
-    WK_PROF_FLUSH(0, blockIdx.x == 0 && tid == 0);
+    if (!ok) leave_role(false, &s_abort, p.status);
+    WK_PROF_FLUSH(0, 8, blockIdx.x == 0 && tid == 0);
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, 512);
+  if (warp == 0) tmem_dealloc(s_tmem, 512);
 }
 
 // Merge the pieces of every unit that was cut: O = sum_s w_s O_s / sum_s w_s with w_s = exp(lse_s - max lse).
@@ -751,7 +786,7 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
     WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           static_cast<int>(kSmemBytes)));
     WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          static_cast<int>(kSmemBytes)));
+                                          static_cast<int>(kSmemBytesLse)));
     ctx->attn_attr_set = true;
   }
   AttnParams p;
@@ -835,7 +870,7 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   if (G > W) G = W;
   const int max_slots = attention_partial_slots(p.H, ctx->max_lq, ctx->max_splits);
   if (!lse_only && 2 * G > max_slots) return WK_ERR_SHAPE;
-  if (lse_only) memory_attention_kernel<true><<<static_cast<unsigned>(G), kThreads, kSmemBytes, s>>>(p);
+  if (lse_only) memory_attention_kernel<true><<<static_cast<unsigned>(G), kThreads, kSmemBytesLse, s>>>(p);
   else memory_attention_kernel<false><<<static_cast<unsigned>(G), kThreads, kSmemBytes, s>>>(p);
   if ((st = after_launch(ctx)) != WK_OK) return st;
   if (!lse_only && G != p.n_units) {   // some unit was cut
