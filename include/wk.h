@@ -241,8 +241,8 @@ typedef struct {
  *   slots_dev [n_slots] int32 in device memory (e.g. wk_retrieve's output); an entry that is -1 is
  *             skipped silently, any other out-of-range or invalid entry is skipped and sets
  *             WK_DEV_BAD_SLOT; a slot listed twice is attended twice
- *   kv_splits 0 = default: one CTA per (head, 256-row query block) when those fill at least three quarters of the SMs
- *             (nothing is merged afterwards), else the (block x KV-tile) space cut into one equal range per SM;
+ *   kv_splits 0 = default: whole (head, 256-row query block) units in full waves over the SMs; the units of the last,
+ *             partial wave cut into equal KV ranges over all SMs and merged where that is faster;
  *             s in 1 .. max_splits = cut every block's KV range into s parts; -g = cut the whole space into g
  *             equal ranges (g CTAs; needs 2 g partial slots, see wk_scratch_bytes)
  * Errors: WK_ERR_SHAPE (lq > max_lq, n_slots > max_k, n_segs > max_dense_segments, kv_splits > max_splits),

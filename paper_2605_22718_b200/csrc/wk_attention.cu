@@ -2,10 +2,10 @@
 // [dense segments ..., retrieved pool slots ...] of one layer.  O = softmax(scale Q K^T) V per head.
 //
 // Flash-style kernel on the 5th-generation tensor cores:
-//   * a work unit is (head, 256 query rows = two 128-row Q tiles); the flat space unit x KV tile is cut into equal
-//     contiguous ranges, one per CTA (one CTA per SM by default), so every SM gets the same amount of work.  A range
-//     that covers a whole unit writes bf16 output directly; otherwise it writes a normalised fp32 partial plus its
-//     log-sum-exp and combine_kernel merges the (at most three) pieces of that unit;
+//   * a work unit is (head, 256 query rows = two 128-row Q tiles).  CTAs (one per SM) take whole units, which go straight to
+//     bf16 output and share a head's K/V tiles through L2 because they walk the keys in step; the units of a last, partial
+//     wave are cut into ranges over all SMs where that pays (split_default): a range writes a normalised fp32 partial plus
+//     its log-sum-exp per piece, and combine_kernel merges them;
 //   * K/V tiles (128 rows x 128 columns of one head, bf16) are fetched by TMA straight from where they lie:
 //     a dense segment (2-D tensor map per segment) or a pool slot (3-D tensor map [layer*slot][row][col]; the
 //     slot id is read from device memory, so the retrieval result never visits the host).  Rows past the end
@@ -59,6 +59,7 @@ struct AttnParams {
   const int32_t* valid;
   int n_slots, pool_slots, layer, C, tiles_per_slot;
   int n_tiles, n_qpairs, n_units;
+  int n_full, n_ranges;
   int lq, H;
   int lse_only;     // 1: only the log-sum-exp is wanted (query-based retrieval): no V loads, no P V product, no O
   int slot_units;   // 1: every listed slot is a problem of its own: unit = (slot ordinal, head, q-pair), n_tiles =
@@ -66,13 +67,15 @@ struct AttnParams {
   float scale_log2;
   __nv_bfloat16* O;
   float* lse;
-  float* opart;     // [2 * gridDim.x][256][128] fp32
-  float* lsepart;   // [2 * gridDim.x][256]
+  float4* opart;    // [2 * n_ranges][32 groups of 4 columns][256 rows] fp32: a warp's 32 rows are one contiguous store
+  float* lsepart;   // [2 * n_ranges][256]
   uint32_t* status;
 };
 
-__device__ __forceinline__ int64_t range_start(const AttnParams& p, int c, int G) {
-  return static_cast<int64_t>(c) * p.n_units * p.n_tiles / G;
+// Work distribution.  Units 0 .. n_full - 1 are done whole, unit u by CTA u % gridDim.x; the tiles of the remaining units
+// are numbered through and cut into n_ranges equal ranges, range c done by CTA c.
+__host__ __device__ __forceinline__ int64_t range_start(int64_t tail_tiles, int n_ranges, int c) {
+  return static_cast<int64_t>(c) * tail_tiles / n_ranges;
 }
 
 struct TileInfo {
@@ -301,35 +304,71 @@ struct Piece {
   bool has_q1;
 };
 struct PieceWalker {
-  int64_t pos, end, start;
-  int cta;
+  int full;            // next whole unit
+  int u, tb;           // next unit of this CTA's range and the first tile in it
+  int u_last, tb_last; // a range that starts inside a unit does that unit's piece last: by then the other CTAs are about
+  int len_last;        // as far into the keys, so that CTAs of a head go on sharing its tiles through L2
+  int64_t left;        // tiles of the range not handed out yet (the postponed piece not counted)
   __device__ __forceinline__ void init(const AttnParams& p) {
-    cta = blockIdx.x;
-    start = range_start(p, cta, gridDim.x);
-    end = range_start(p, cta + 1, gridDim.x);
-    pos = start;
+    full = blockIdx.x;
+    left = 0;
+    len_last = 0;
+    if (p.n_full == p.n_units || blockIdx.x >= p.n_ranges) return;
+    const int64_t tail = static_cast<int64_t>(p.n_units - p.n_full) * p.n_tiles;
+    const int64_t start = range_start(tail, p.n_ranges, blockIdx.x);
+    left = range_start(tail, p.n_ranges, blockIdx.x + 1) - start;
+    const int ur = static_cast<int>(start / p.n_tiles);
+    u = p.n_full + ur;
+    tb = static_cast<int>(start - static_cast<int64_t>(ur) * p.n_tiles);
+    if (tb > 0) {
+      u_last = u++;
+      tb_last = tb;
+      len_last = static_cast<int>(min(left, static_cast<int64_t>(p.n_tiles - tb)));
+      left -= len_last;
+      tb = 0;
+    }
   }
   __device__ __forceinline__ bool next(const AttnParams& p, Piece& pc) {
-    if (pos >= end) return false;
-    int u = static_cast<int>(pos / p.n_tiles);
-    pc.tb = static_cast<int>(pos - static_cast<int64_t>(u) * p.n_tiles);
-    const int64_t room = end - pos;
-    pc.te = static_cast<int>(min(static_cast<int64_t>(p.n_tiles), pc.tb + room));
-    const bool full = pc.tb == 0 && pc.te == p.n_tiles;
-    pc.slot = full ? -1 : 2 * cta + (pos == start ? 0 : 1);
-    pos += pc.te - pc.tb;
+    int v;
+    if (full < p.n_full) {
+      v = full;
+      full += gridDim.x;
+      pc.tb = 0;
+      pc.te = p.n_tiles;
+      pc.slot = -1;
+    } else if (left > 0) {
+      v = u++;
+      pc.tb = 0;
+      pc.te = static_cast<int>(min(left, static_cast<int64_t>(p.n_tiles)));
+      left -= pc.te;
+      // partial results: slot 2 c for the piece that range c starts with, 2 c + 1 for the one it ends with
+      pc.slot = pc.te == p.n_tiles ? -1 : 2 * static_cast<int>(blockIdx.x) + (tb_first(p, v) ? 0 : 1);
+    } else if (len_last > 0) {
+      v = u_last;
+      pc.tb = tb_last;
+      pc.te = tb_last + len_last;
+      len_last = 0;
+      pc.slot = 2 * static_cast<int>(blockIdx.x);
+    } else {
+      return false;
+    }
     pc.ord = 0;
     if (p.slot_units) {   // the unit's tiles are those of one slot: shift the range into that slot's part of the tile space
       const int base = p.H * p.n_qpairs;
-      pc.ord = u / base;
-      u -= pc.ord * base;
+      pc.ord = v / base;
+      v -= pc.ord * base;
       pc.tb += pc.ord * p.tiles_per_slot;
       pc.te += pc.ord * p.tiles_per_slot;
     }
-    pc.h = u / p.n_qpairs;
-    pc.q0 = (u - pc.h * p.n_qpairs) * kPairRows;
+    pc.h = v / p.n_qpairs;
+    pc.q0 = (v - pc.h * p.n_qpairs) * kPairRows;
     pc.has_q1 = pc.q0 + kTileQ < p.lq;
     return true;
+  }
+  // is unit v, entered at its first tile, the start of this CTA's range?
+  __device__ __forceinline__ bool tb_first(const AttnParams& p, int v) const {
+    const int64_t tail = static_cast<int64_t>(p.n_units - p.n_full) * p.n_tiles;
+    return range_start(tail, p.n_ranges, blockIdx.x) == static_cast<int64_t>(v - p.n_full) * p.n_tiles;
   }
 };
 
@@ -370,6 +409,9 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // everything above runs under the end of the kernel before this one; nothing is read or written before this wait
+  dep_wait();
+  dep_release();
   // an allocation of all 512 columns starts at column 0; addresses known at compile time keep the MMAs' operands cheap
   if (s_tmem != 0 && tid == 0) { s_abort = 1; atomicOr(p.status, WK_DEV_TIMEOUT); }
 
@@ -490,17 +532,6 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           if (lane == 0) mbar_arrive(&bars.q_empty);
           continue;
         }
-        // O0 / O1 are about to be overwritten: the epilogue of the last piece that used them must have read them.
-        // o_free[i] completes once per piece in which warpgroup i ran an epilogue, so neither side can run two
-        // phases ahead of the other (a parity wait cannot tell phase n from phase n + 2).
-        if (!kLse) {
-          if (e0 > 0 && !(ok = wait_or_abort(&bars.o_free[0], (e0 - 1) & 1, &s_abort))) break;
-          ++e0;
-          if (q1) {
-            if (e1 > 0 && !(ok = wait_or_abort(&bars.o_free[1], (e1 - 1) & 1, &s_abort))) break;
-            ++e1;
-          }
-        }
         // Step j: for each Q tile, once its P of tile j is there, P V of tile j and Q K^T of tile j + 1 into the S buffer
         // P was in.  The other Q tile's softmax runs meanwhile.  (LSE-only: no P V; the "P" signal says that S has been read.)
         int nv = 0, nv_next = 0;
@@ -516,6 +547,10 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           }
           if (kLse) ++lse_q0;
           WK_PROF(2);
+          // A piece's first P V overwrites O: the epilogue of the last piece that used it must have read it.  o_free[i]
+          // completes once per piece in which warpgroup i ran an epilogue, so neither side can run two phases ahead of the
+          // other (a parity wait cannot tell phase n from phase n + 2).
+          if (!kLse && j == 0 && e0++ > 0 && !(ok = wait_or_abort(&bars.o_free[0], e0 & 1, &s_abort))) break;
           tc_fence_after();
           if (!kLse && j >= 0) issue_pv(0, st, nv, j > 0);
           if (more) { issue_s(0, st, nv_next); commit(offsetof(Barriers, s_full)); }
@@ -529,6 +564,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
             }
             if (kLse) ++lse_q1;
             WK_PROF(4);
+            if (!kLse && j == 0 && e1++ > 0 && !(ok = wait_or_abort(&bars.o_free[1], e1 & 1, &s_abort))) break;
             tc_fence_after();
             if (!kLse && j >= 0) issue_pv(1, st, nv, j > 0);
             if (more) { issue_s(1, st, nv_next); commit(offsetof(Barriers, s_full) + 8); }
@@ -691,11 +727,10 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
                   dst[v] = o;
                 }
               } else {
-                float4* dst = reinterpret_cast<float4*>(
-                    p.opart + (static_cast<int64_t>(pc.slot) * kPairRows + prow) * kHeadDim + c * 32);
+                float4* dst = p.opart + (static_cast<int64_t>(pc.slot) * 32 + c * 8) * kPairRows + prow;
 #pragma unroll
                 for (int v = 0; v < 8; ++v)
-                  dst[v] = make_float4(__uint_as_float(r[4 * v]) * inv_l, __uint_as_float(r[4 * v + 1]) * inv_l,
+                  dst[v * kPairRows] = make_float4(__uint_as_float(r[4 * v]) * inv_l, __uint_as_float(r[4 * v + 1]) * inv_l,
                                        __uint_as_float(r[4 * v + 2]) * inv_l, __uint_as_float(r[4 * v + 3]) * inv_l);
               }
             }
@@ -725,50 +760,73 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
   if (warp == 0) tmem_dealloc(s_tmem, 512);
 }
 
-// Merge the pieces of every unit that was cut: O = sum_s w_s O_s / sum_s w_s with w_s = exp(lse_s - max lse).
-// One warp per (unit, row of the 256-row pair); units written directly by a single CTA are left alone.
-__global__ void __launch_bounds__(256)
-combine_kernel(const float* __restrict__ opart, const float* __restrict__ lsepart, int G, int n_units, int n_tiles,
+// Merge the pieces of every unit that was cut: O = sum_s w_s O_s / sum_s w_s with w_s = exp(lse_s - max lse).  Bound by
+// reading the fp32 partials (they come from L2).  A block merges 32 rows x 32 columns of one unit: warp w holds column
+// group w of the 32 rows, so that every load is one contiguous 512-byte line, and the bf16 result leaves through shared
+// memory as 64 contiguous bytes per row.  Units written directly by a single CTA are left alone.
+constexpr int kCombineThreads = 256;
+__global__ void __launch_bounds__(kCombineThreads)
+combine_kernel(const float4* __restrict__ opart, const float* __restrict__ lsepart, int G, int n_full, int n_units, int n_tiles,
                int n_qpairs, int H, int lq, __nv_bfloat16* __restrict__ O, float* __restrict__ lse_out) {
-  const int warp_global = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp_global >= n_units * kPairRows) return;
-  const int u = warp_global / kPairRows, prow = warp_global - u * kPairRows;
-  const int h = u / n_qpairs, qrow = (u - h * n_qpairs) * kPairRows + prow;
-  if (qrow >= lq) return;
-  const int64_t W = static_cast<int64_t>(n_units) * n_tiles;
-  const int64_t ustart = static_cast<int64_t>(u) * n_tiles, uend = ustart + n_tiles;
-  auto start_of = [&](int c) { return static_cast<int64_t>(c) * W / G; };
-  int c = static_cast<int>(ustart * G / W);
-  if (c >= G) c = G - 1;
-  while (c > 0 && start_of(c) > ustart) --c;
-  while (c + 1 < G && start_of(c + 1) <= ustart) ++c;
-  if (start_of(c) <= ustart && start_of(c + 1) >= uend) return;   // one CTA covered the whole unit
-  int slot[kMaxPieces];
-  int np = 0;
-  for (int cc = c; cc < G && start_of(cc) < uend && np < kMaxPieces; ++cc) {
-    const int64_t sc = start_of(cc), ec = start_of(cc + 1);
-    if (ec <= ustart || ec == sc) continue;
-    const int64_t ps = sc > ustart ? sc : ustart;
-    slot[np++] = 2 * cc + (ps == sc ? 0 : 1);
-  }
+  __shared__ int s_slot[kMaxPieces];
+  __shared__ float s_lse[kMaxPieces][32], s_w[kMaxPieces][32];
+  __shared__ __align__(16) uint2 s_out[32][8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ut = blockIdx.x >> 5, u = n_full + ut, rg = (blockIdx.x >> 2) & 7, cg = blockIdx.x & 3;   // unit, row group, column group
+  const int h = u / n_qpairs, qrow0 = (u - h * n_qpairs) * kPairRows + rg * 32;
+  dep_wait();
+  if (qrow0 >= lq) return;
+  // the CTAs whose ranges touch the unit: lane i looks at the i-th one (every range holds at least one tile)
+  const int64_t W = static_cast<int64_t>(n_units - n_full) * n_tiles;
+  const int64_t ustart = static_cast<int64_t>(ut) * n_tiles, uend = ustart + n_tiles;
+  auto start_of = [&](int c) { return range_start(W, G, c); };
+  int c0 = static_cast<int>(ustart * G / W);
+  while (c0 > 0 && start_of(c0) > ustart) --c0;
+  while (c0 + 1 < G && start_of(c0 + 1) <= ustart) ++c0;
+  const int cc = c0 + lane;
+  const int64_t sc = start_of(cc);
+  const bool mine = cc < G && sc < uend;
+  const int np = __popc(__ballot_sync(0xffffffffu, mine));
+  if (np == 1 && start_of(c0) <= ustart && start_of(c0 + 1) >= uend) return;   // one CTA covered the whole unit
+  if (warp == 0 && mine) s_slot[lane] = 2 * cc + (sc >= ustart ? 0 : 1);
+  __syncthreads();
+  for (int s = warp; s < np; s += kCombineThreads / 32)
+    s_lse[s][lane] = __ldcg(lsepart + static_cast<int64_t>(s_slot[s]) * kPairRows + rg * 32 + lane);
+  __syncthreads();
   float mx = -INFINITY;
-  for (int s = 0; s < np; ++s) mx = fmaxf(mx, lsepart[static_cast<int64_t>(slot[s]) * kPairRows + prow]);
+  for (int s = 0; s < np; ++s) mx = fmaxf(mx, s_lse[s][lane]);
+  for (int s = warp; s < np; s += kCombineThreads / 32)
+    s_w[s][lane] = s_lse[s][lane] == -INFINITY ? 0.f : expf(s_lse[s][lane] - mx);
+  __syncthreads();
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   float wsum = 0.f;
-  for (int s = 0; s < np; ++s) {
-    const int64_t idx = static_cast<int64_t>(slot[s]) * kPairRows + prow;
-    const float ls = lsepart[idx];
-    const float w = (ls == -INFINITY) ? 0.f : expf(ls - mx);
-    const float4 o = reinterpret_cast<const float4*>(opart + idx * kHeadDim)[lane];
-    acc.x = fmaf(w, o.x, acc.x); acc.y = fmaf(w, o.y, acc.y); acc.z = fmaf(w, o.z, acc.z); acc.w = fmaf(w, o.w, acc.w);
-    wsum += w;
+  const int64_t at = static_cast<int64_t>(cg * 8 + warp) * kPairRows + rg * 32 + lane;
+  for (int s0 = 0; s0 < np; s0 += 8) {   // eight pieces' loads in flight
+    float4 o[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      o[i] = s0 + i < np ? __ldcg(opart + static_cast<int64_t>(s_slot[s0 + i]) * 32 * kPairRows + at) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (s0 + i < np) {
+        const float w = s_w[s0 + i][lane];
+        acc.x = fmaf(w, o[i].x, acc.x); acc.y = fmaf(w, o[i].y, acc.y);
+        acc.z = fmaf(w, o[i].z, acc.z); acc.w = fmaf(w, o[i].w, acc.w);
+        wsum += w;
+      }
+    }
   }
   const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
-  uint2 out;
-  out.x = ptx::pack_bf16x2(acc.x * inv, acc.y * inv);
-  out.y = ptx::pack_bf16x2(acc.z * inv, acc.w * inv);
-  reinterpret_cast<uint2*>(O + (static_cast<int64_t>(qrow) * H + h) * kHeadDim)[lane] = out;
-  if (lse_out && lane == 0) lse_out[static_cast<int64_t>(h) * lq + qrow] = wsum > 0.f ? mx + logf(wsum) : -INFINITY;
+  s_out[lane][warp] = make_uint2(ptx::pack_bf16x2(acc.x * inv, acc.y * inv), ptx::pack_bf16x2(acc.z * inv, acc.w * inv));
+  __syncthreads();
+  if (tid < 128) {
+    const int r = tid >> 2, v = tid & 3;
+    if (qrow0 + r < lq)
+      reinterpret_cast<uint4*>(O + (static_cast<int64_t>(qrow0 + r) * H + h) * kHeadDim + cg * 32)[v] =
+          reinterpret_cast<const uint4*>(&s_out[r][0])[v];
+  }
+  if (lse_out && cg == 0 && warp == 0 && qrow0 + lane < lq)
+    lse_out[static_cast<int64_t>(h) * lq + qrow0 + lane] = wsum > 0.f ? mx + logf(wsum) : -INFINITY;
 }
 
 }  // namespace
@@ -777,6 +835,36 @@ int attention_partial_slots(int n_heads, int max_lq, int max_splits) {
   const int units = n_heads * ((max_lq + kPairRows - 1) / kPairRows);
   const int by_split = units * (max_splits > 1 ? max_splits : 1);
   return 2 * (by_split > 256 ? by_split : 256);
+}
+
+// Default distribution over the SMs: whole units in full waves, then, where it pays, the units of the last, partial wave
+// cut into equal ranges over all SMs and merged.  The cut saves (sms - rest) / sms of a unit's tiles; it costs about 4
+// tile times (the combine launch, a second prologue) and 13 more when every CTA writes partials.  Measured on 148 SMs,
+// whole -> cut, back to back: 40 heads x 4,680 queries x 32,760 keys (rest 20 of 148) 3,136 -> 2,897 us; 12 heads x 880
+// tokens, 167,640 keys (rest 132) 2,782 -> 2,716; 8 heads x 7,920 keys (rest 88) 122 -> 101; 2 heads x 3,960 keys (rest 8)
+// 61 -> 24; and the other way round for 12 heads x 15,840 keys (rest 132) 266 -> 269, 16 heads x 7,200 keys (rest 128)
+// 125 -> 136, 24 heads x 9,000 keys (rest 140) 322 -> 336.
+static void split_default(int64_t units, int64_t tiles, int64_t sms, int64_t* G, int64_t* n_full, int64_t* ranges) {
+  const int64_t waves = units / sms, rest = units - waves * sms;
+  *G = units < sms ? units : sms;
+  *n_full = units;
+  *ranges = 0;
+  if (rest == 0 || (sms - rest) * tiles < 4 * sms + 13 * rest) return;
+  *n_full = waves * sms;
+  // Where whole cuts of every unit use nearly all SMs, no CTA gets two pieces; pieces of fewer than 4 tiles cost more in
+  // prologues and partials than they save (2 heads x 3,960 keys: 144 unaligned ranges 23.3 us, 128 aligned 21.2, 64
+  // aligned 20.1, 40 unaligned 24.9).
+  int64_t cuts = sms / rest;
+  if (cuts > kMaxPieces - 2) cuts = kMaxPieces - 2;
+  int64_t r = sms;
+  if (cuts >= 2 && ((sms - cuts * rest) * 8 <= sms || cuts == kMaxPieces - 2)) {
+    int64_t per = (tiles + cuts - 1) / cuts;
+    if (per < 4) per = 4;
+    r = rest * ((tiles + per - 1) / per);
+  }
+  if (r > rest * tiles) r = rest * tiles;
+  *ranges = r;
+  *G = waves > 0 ? sms : r;
 }
 
 wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int lq, const wk_dense_seg* segs, int n_segs,
@@ -831,7 +919,7 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   p.scale_log2 = ctx->scale * 1.4426950408889634f;
   p.O = O;
   p.lse = lse;
-  p.opart = reinterpret_cast<float*>(ctx->scratch_base + ctx->sl.opart_off);
+  p.opart = reinterpret_cast<float4*>(ctx->scratch_base + ctx->sl.opart_off);
   p.lsepart = reinterpret_cast<float*>(ctx->scratch_base + ctx->sl.lsepart_off);
   p.status = ctx->status_dev;
   if (lse_only) {
@@ -840,43 +928,40 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
     p.n_tiles = p.tiles_per_slot;
     p.n_units *= n_slots;
   }
-  const int64_t W = static_cast<int64_t>(p.n_units) * p.n_tiles;
-  int64_t G;
+  const int64_t sms = ctx->sm_count;
+  int64_t G, n_full = 0, ranges = 0;   // CTAs, units done whole, ranges the rest is cut into
   if (lse_only) {
     // whole units per CTA (nothing to merge): the largest divisor of the unit count that fits the SMs, unless that
     // would leave more than a quarter of them idle -- then one CTA per unit
     G = 1;
-    for (int g = ctx->sm_count < p.n_units ? ctx->sm_count : p.n_units; g >= 1; --g)
+    for (int64_t g = sms < p.n_units ? sms : p.n_units; g >= 1; --g)
       if (p.n_units % g == 0) { G = g; break; }
-    if (G * 4 < static_cast<int64_t>(ctx->sm_count) * 3 && p.n_units > G) G = p.n_units;
+    if (G * 4 < sms * 3 && p.n_units > G) G = p.n_units;
+    ranges = G;
   } else if (kv_splits == 0) {
-    // One CTA per (head, q-pair) whenever that keeps most SMs busy: under the board's power cap the extra fp32
-    // partials and the combine pass of a finer cut cost more than the idle SMs (measured at the Matrix-Game shape:
-    // 132 CTAs beat 148 equal ranges by 12 %).  Small problems are cut into one equal range per SM instead.
-    if (p.n_units * 4 >= ctx->sm_count * 3) {
-      G = p.n_units;
-    } else {
-      G = ctx->sm_count;
-      if (G > static_cast<int64_t>(p.n_units) * (kMaxPieces - 2)) G = static_cast<int64_t>(p.n_units) * (kMaxPieces - 2);
-    }
+    split_default(p.n_units, p.n_tiles, sms, &G, &n_full, &ranges);
   } else if (kv_splits > 0) {
     int sp = kv_splits < p.n_tiles ? kv_splits : p.n_tiles;
     if (sp > kMaxPieces) sp = kMaxPieces;
-    G = static_cast<int64_t>(p.n_units) * sp;  // every unit cut into exactly sp ranges
+    if (sp == 1) n_full = G = p.n_units;
+    else ranges = G = static_cast<int64_t>(p.n_units) * sp;   // every unit cut into exactly sp ranges
   } else {
-    G = -static_cast<int64_t>(kv_splits);      // caller-chosen number of equal ranges
+    ranges = G = -static_cast<int64_t>(kv_splits);      // caller-chosen number of equal ranges
+    const int64_t W = static_cast<int64_t>(p.n_units) * p.n_tiles;
     if (G * p.n_tiles > W * (kMaxPieces - 2)) return WK_ERR_SHAPE;   // a unit would be cut into too many pieces
+    if (G > W) ranges = G = W;
   }
-  if (G > W) G = W;
   const int max_slots = attention_partial_slots(p.H, ctx->max_lq, ctx->max_splits);
-  if (!lse_only && 2 * G > max_slots) return WK_ERR_SHAPE;
-  if (lse_only) memory_attention_kernel<true><<<static_cast<unsigned>(G), kThreads, kSmemBytesLse, s>>>(p);
-  else memory_attention_kernel<false><<<static_cast<unsigned>(G), kThreads, kSmemBytes, s>>>(p);
+  if (!lse_only && 2 * ranges > max_slots) return WK_ERR_SHAPE;
+  p.n_full = static_cast<int>(n_full);
+  p.n_ranges = static_cast<int>(ranges);
+  const dim3 grid(static_cast<unsigned>(G)), block(kThreads);
+  if (lse_only) launch_chained(memory_attention_kernel<true>, grid, block, kSmemBytesLse, s, p);
+  else launch_chained(memory_attention_kernel<false>, grid, block, kSmemBytes, s, p);
   if ((st = after_launch(ctx)) != WK_OK) return st;
-  if (!lse_only && G != p.n_units) {   // some unit was cut
-    const int64_t warps = static_cast<int64_t>(p.n_units) * kPairRows;
-    combine_kernel<<<static_cast<unsigned>((warps * 32 + 255) / 256), 256, 0, s>>>(
-        p.opart, p.lsepart, static_cast<int>(G), p.n_units, p.n_tiles, p.n_qpairs, p.H, lq, O, lse);
+  if (!lse_only && n_full != p.n_units) {   // some unit was cut
+    launch_chained(combine_kernel, dim3(static_cast<unsigned>(p.n_units - n_full) * 32), dim3(kCombineThreads), 0, s, p.opart,
+                   p.lsepart, p.n_ranges, p.n_full, p.n_units, p.n_tiles, p.n_qpairs, p.H, lq, O, lse);
     if ((st = after_launch(ctx)) != WK_OK) return st;
   }
   return WK_OK;

@@ -59,3 +59,35 @@ def test_short_tiles_of_pool_slots(T, n_keep):
         assert kv.poll_status() == (0, 0)
         assert_attention_close(O, O_ref, f"C={T + n_keep} splits={splits}")
         np.testing.assert_allclose(lse.cpu().numpy(), L_ref, atol=2e-3)
+
+
+@pytest.mark.parametrize("H,lq,rows", [
+    (1, 100, 4500),      # one unit cut into as many pieces as a unit may have
+    (7, 256, 2000),      # 7 units, every one cut into equal parts, one piece per CTA
+    (9, 2000, 900),      # 72 units: ranges that end inside units, two pieces per CTA
+    (20, 2100, 640),     # 180 units: one whole wave, the rest cut (or not) by the rule
+    (29, 1300, 2600),    # 174 units: whole units and a cut piece on the same CTA
+])
+def test_work_distributions(H, lq, rows):
+    """The default distribution over the SMs (whole units, aligned cuts, ranges across units) against one CTA per unit,
+    and one head against the oracle."""
+    from paper_2605_22718_b200 import WorldKV
+    kv = WorldKV(n_layers=1, n_heads=H, tokens_per_frame=8, n_keep=4, pool_slots=1, max_k=1, max_lq=lq)
+    D = H * 128
+    K = wi.query_bf16(61, 0, 0, 1, rows, D).reshape(rows, H, 128)
+    V = wi.query_bf16(62, 0, 0, 2, rows, D).reshape(rows, H, 128)
+    Qb = wi.query_bf16(63, 0, 0, 0, lq, D).reshape(lq, H, 128)
+    Q, seg = wd.to_device_bf16(Qb), (wd.to_device_bf16(K), wd.to_device_bf16(V))
+    out = {}
+    for splits in (0, 1):
+        lse = torch.empty((H, lq), dtype=torch.float32, device="cuda")
+        out[splits] = kv.memory_attention(0, Q, [seg], None, 0, lse_out=lse, kv_splits=splits).clone(), lse
+        assert kv.poll_status() == (0, 0)
+    # the two differ by one bf16 rounding of the output and the fp32 merge
+    a, b = out[0][0].float(), out[1][0].float()
+    assert float((a - b).norm() / b.norm()) < 4e-3
+    assert float((out[0][1] - out[1][1]).abs().max()) < 1e-3
+    h = H - 1
+    O_ref, L_ref = o.memory_attention(Qb[:, h:h + 1], [(K[:, h:h + 1], V[:, h:h + 1])], o.PoolModel(n_slots=1, n_layers=1), 0, [])
+    assert_attention_close(out[0][0][:, h:h + 1], O_ref, f"H={H}")
+    np.testing.assert_allclose(out[0][1][h:h + 1].cpu().numpy(), L_ref, atol=2e-3)
