@@ -34,17 +34,18 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kThreads = 320;
-constexpr int kMmaWarp = 8, kTmaWarp = 9;
+// softmax warps, then the MMA warp, then the TMA warp.  LSE-only launches have a softmax warpgroup per S buffer.
+template <bool kLse> constexpr int kSoftWarps = kLse ? 16 : 8;
+template <bool kLse> constexpr int kThreads = 32 * (kSoftWarps<kLse> + 2);
 constexpr uint32_t kHalfTileBytes = 128 * 64 * 2;   // one TMA box: 128 rows x 64 bf16 = 16 KB
 constexpr uint32_t kTileBytes = 2 * kHalfTileBytes; // 128 x 128 bf16
 // A stage holds what one step of the MMA warp consumes: V of tile j and K of tile j + 1 (LSE-only launches: K alone).
-constexpr int kStages = 2, kStagesLse = 5;
+constexpr int kStages = 2, kStagesLse = 4;
 constexpr size_t kSmemBytes = 1024 + 2 * kTileBytes + 2 * kStages * kTileBytes;   // align slack + Q0,Q1 + stages
 constexpr size_t kSmemBytesLse = 1024 + 2 * kTileBytes + kStagesLse * kTileBytes;
 constexpr int kNvRing = 16;   // tile heights handed from the TMA warp to the others; the TMA warp is at most kStagesLse + 1 tiles ahead
 constexpr float kRescaleThreshold = 8.0f;           // log2 units: P stays <= 2^8 between maximum updates
-constexpr uint32_t kTmemS = 0, kTmemO = 256;        // tensor-memory columns: S0, S1 (P over them), O0, O1
+constexpr uint32_t kTmemS = 0, kTmemO = 256;        // tensor-memory columns: S0, S1 (P over them), O0, O1; LSE-only: S0, S1 twice
 constexpr int kPairRows = 2 * kTileQ;
 constexpr int kMaxPieces = 32;                      // most ranges one unit may be cut into
 
@@ -199,7 +200,7 @@ __device__ __forceinline__ int count_tiles(const AttnParams& p, int tb, int te) 
 struct __align__(8) Barriers {
   uint64_t q_full, q_empty;
   uint64_t kv_full[kStagesLse], kv_empty[kStagesLse];
-  uint64_t s_full[2], p_full[2], o_done[2], o_free[2];
+  uint64_t s_full[4], p_full[4], o_done[2], o_free[2], m_full[2], m_empty[2];   // index of s_full, p_full: Q tile + 2 x S buffer (LSE-only)
 };
 
 // Bounded wait that also gives up when another role has already aborted; false then.  A loop of eight instructions and
@@ -238,26 +239,53 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
-// P = 2^(s * scale - m) for one row of a tile: rounds to bf16, stores into tensor memory over S (64 columns), returns
-// the fp32 row sum.  The exponentials are the kernel's second bound (16 per clock and SM on the special-function unit,
-// as many clocks per tile as its tensor-core work), so kPoly of every 8 column pairs take 2^x from the FMA pipe instead:
-// x = n + f with n = round(x) by the add-a-large-constant trick, 2^f on [-1/2, 1/2] by a cubic (relative error 7.7e-5,
-// far inside the bf16 rounding P gets anyway: 2e-3), 2^n by adding n to the exponent field; all in packed fp32 pairs.
-// That path needs x >= -126 (it clamps at -120; such a weight is 1e-36 of the row's largest) and finite x, so tiles with
-// masked columns (-inf) take kPoly = 0.
-// kStore = false (LSE-only launches): only the row sum is wanted, nothing is written.
+// 2^x of a pair.  The exponentials are the kernel's second bound (16 per clock and SM on the special-function unit, as many
+// clocks per tile as its tensor-core work), so a share of the pairs takes 2^x from the FMA pipe instead: x = n + f with
+// n = round(x) by the add-a-large-constant trick, 2^f on [-1/2, 1/2] by a cubic (relative error 7.7e-5, far inside the bf16
+// rounding P gets anyway: 2e-3), 2^n by adding n to the exponent field; all in packed fp32 pairs.  That path clamps at
+// x = -120 (a weight of 1e-36) and needs x < 127.
+template <bool kPoly>
+__device__ __forceinline__ void exp2_pair(uint64_t e, float& p0, float& p1) {
+  float e0, e1;
+  unpack_f32x2(e, e0, e1);
+  if (kPoly) {
+    const uint64_t magic2 = pack_f32x2(12582912.f, 12582912.f), nmagic2 = pack_f32x2(-12582912.f, -12582912.f);
+    const uint64_t mone2 = pack_f32x2(-1.f, -1.f);
+    const uint64_t c0 = pack_f32x2(0.9999289512634277f, 0.9999289512634277f);
+    const uint64_t c1 = pack_f32x2(0.6932762265205383f, 0.6932762265205383f);
+    const uint64_t c2 = pack_f32x2(0.242604061961174f, 0.242604061961174f);
+    const uint64_t c3 = pack_f32x2(0.055088773369789124f, 0.055088773369789124f);
+    const uint64_t x = pack_f32x2(fmaxf(e0, -120.f), fmaxf(e1, -120.f));
+    const uint64_t t = add_f32x2(x, magic2);                  // low mantissa bits = round(x)
+    const uint64_t f = fma_f32x2(add_f32x2(t, nmagic2), mone2, x);   // x - round(x), in [-1/2, 1/2]
+    uint64_t y = fma_f32x2(c3, f, c2);
+    y = fma_f32x2(y, f, c1);
+    y = fma_f32x2(y, f, c0);
+    float t0, t1, y0, y1;
+    unpack_f32x2(t, t0, t1);
+    unpack_f32x2(y, y0, y1);
+    p0 = __uint_as_float(__float_as_uint(y0) + (__float_as_uint(t0) << 23));
+    p1 = __uint_as_float(__float_as_uint(y1) + (__float_as_uint(t1) << 23));
+  } else {
+    p0 = ex2_approx(e0);
+    p1 = ex2_approx(e1);
+  }
+}
+__device__ __forceinline__ float sum4_f32x2(const uint64_t (&acc)[4]) {
+  float a, b;
+  unpack_f32x2(add_f32x2(add_f32x2(acc[0], acc[1]), add_f32x2(acc[2], acc[3])), a, b);
+  return a + b;
+}
+
+// P = 2^(s * scale - m) for one row of a tile: rounds to bf16, stores into tensor memory over S (64 columns), returns the
+// fp32 row sum.  kPoly of every 8 column pairs take the FMA pipe (sustained, 12 heads x 15,840 keys: 276 / 277 / 270 / 291 us
+// at 0 / 1 / 2 / 3); tiles with masked columns (-inf) take kPoly = 0 and stop after n_chunks groups of 32 columns.
 #ifndef WK_ATTN_POLY
 #define WK_ATTN_POLY 2
 #endif
-template <bool kStore, int kPoly>
+template <int kPoly>
 __device__ __forceinline__ float exp_store_tile(const float (&s)[128], uint64_t scale2, uint64_t neg_m2, uint32_t tS, int n_chunks) {
-  uint64_t acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0;   // four independent (lo, hi) sums
-  const uint64_t magic2 = pack_f32x2(12582912.f, 12582912.f), nmagic2 = pack_f32x2(-12582912.f, -12582912.f);
-  const uint64_t mone2 = pack_f32x2(-1.f, -1.f);
-  const uint64_t c0 = pack_f32x2(0.9999289512634277f, 0.9999289512634277f);
-  const uint64_t c1 = pack_f32x2(0.6932762265205383f, 0.6932762265205383f);
-  const uint64_t c2 = pack_f32x2(0.242604061961174f, 0.242604061961174f);
-  const uint64_t c3 = pack_f32x2(0.055088773369789124f, 0.055088773369789124f);
+  uint64_t acc[4] = {0, 0, 0, 0};   // four independent (lo, hi) sums
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     if (kPoly == 0 && c >= n_chunks) break;   // a short tile stops at its last group of 32 columns
@@ -265,36 +293,40 @@ __device__ __forceinline__ float exp_store_tile(const float (&s)[128], uint64_t 
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       const uint64_t e = fma_f32x2(pack_f32x2(s[c * 32 + 2 * i], s[c * 32 + 2 * i + 1]), scale2, neg_m2);
-      float e0, e1, p0, p1;
-      unpack_f32x2(e, e0, e1);
-      if ((i & 7) < kPoly) {
-        const uint64_t x = pack_f32x2(fmaxf(e0, -120.f), fmaxf(e1, -120.f));
-        const uint64_t t = add_f32x2(x, magic2);                  // low mantissa bits = round(x)
-        const uint64_t f = fma_f32x2(add_f32x2(t, nmagic2), mone2, x);   // x - round(x), in [-1/2, 1/2]
-        uint64_t y = fma_f32x2(c3, f, c2);
-        y = fma_f32x2(y, f, c1);
-        y = fma_f32x2(y, f, c0);
-        float t0, t1, y0, y1;
-        unpack_f32x2(t, t0, t1);
-        unpack_f32x2(y, y0, y1);
-        p0 = __uint_as_float(__float_as_uint(y0) + (__float_as_uint(t0) << 23));
-        p1 = __uint_as_float(__float_as_uint(y1) + (__float_as_uint(t1) << 23));
-      } else {
-        p0 = ex2_approx(e0);
-        p1 = ex2_approx(e1);
-      }
-      const uint64_t pp = pack_f32x2(p0, p1);
-      if ((i & 3) == 0) acc0 = add_f32x2(acc0, pp);
-      else if ((i & 3) == 1) acc1 = add_f32x2(acc1, pp);
-      else if ((i & 3) == 2) acc2 = add_f32x2(acc2, pp);
-      else acc3 = add_f32x2(acc3, pp);
-      if (kStore) pk[i] = pack_bf16x2(p0, p1);
+      float p0, p1;
+      if ((i & 7) < kPoly) exp2_pair<true>(e, p0, p1);
+      else exp2_pair<false>(e, p0, p1);
+      acc[i & 3] = add_f32x2(acc[i & 3], pack_f32x2(p0, p1));
+      pk[i] = pack_bf16x2(p0, p1);
     }
-    if (kStore) tmem_st_x16(tS + c * 16, pk);
+    tmem_st_x16(tS + c * 16, pk);
   }
-  float a, b;
-  unpack_f32x2(add_f32x2(add_f32x2(acc0, acc1), add_f32x2(acc2, acc3)), a, b);
-  return a + b;
+  return sum4_f32x2(acc);
+}
+
+// LSE-only launches: sum of 2^(s * scale - m) over 32 columns of a row held in registers.  kLsePoly of every 8 pairs take
+// the FMA pipe; big = the largest of their raw values (the caller checks that they stay below the path's limit).
+#ifndef WK_LSE_POLY
+#define WK_LSE_POLY 2
+#endif
+__device__ __forceinline__ void lse_chunk(uint32_t (&r)[32], int rem, uint64_t scale2, uint64_t neg_m2, uint64_t (&acc)[4], float& big) {
+  if (rem < 32) {   // columns past the end of the slot
+#pragma unroll
+    for (int i = 0; i < 32; ++i) r[i] = i < rem ? r[i] : 0xff800000u;
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const float s0 = __uint_as_float(r[2 * i]), s1 = __uint_as_float(r[2 * i + 1]);
+    const uint64_t e = fma_f32x2(pack_f32x2(s0, s1), scale2, neg_m2);
+    float p0, p1;
+    if ((i & 7) < WK_LSE_POLY) {
+      exp2_pair<true>(e, p0, p1);
+      big = fmax3(big, s0, s1);
+    } else {
+      exp2_pair<false>(e, p0, p1);
+    }
+    acc[i & 3] = add_f32x2(acc[i & 3], pack_f32x2(p0, p1));
+  }
 }
 
 // One piece of work: unit u, KV tiles [tb, te), and where its result goes.
@@ -372,10 +404,12 @@ struct PieceWalker {
   }
 };
 
-// kLse = true is the LSE-only instantiation (query-based retrieval): no V, no P, no O; a softmax thread hands its S
-// buffer back as soon as the row is in registers, so the next Q K^T runs under the exponentials.
+// kLse = true is the LSE-only instantiation (query-based retrieval): no V, no P, no O.  S has two buffers per Q tile and a
+// softmax warpgroup per buffer, so the tensor pipe works ahead of the softmax, which bounds it (issue and special-function
+// unit) until the board's power cap does.  2,640 queries x 12 heads x 250 slots of 1,320 rows: two warpgroups and one buffer
+// per Q tile on 132 SMs 4,070 us; all SMs, two buffers, streamed sums 3,540; four warpgroups 3,070 (2,136 clk per KV tile).
 template <bool kLse>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads<kLse>, 1)
 memory_attention_kernel(const __grid_constant__ AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -387,6 +421,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
   __shared__ Barriers bars;
   __shared__ uint32_t s_tmem;
   __shared__ volatile uint32_t s_abort;
+  __shared__ float2 s_merge[kLse ? 2 : 1][kLse ? 128 : 1];   // (reference, sum) of a Q tile's odd KV tiles
   __shared__ volatile int s_nv[kNvRing];   // valid rows of tile number t (counted over the CTA's pieces) at t % kNvRing
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -395,10 +430,8 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
     mbar_init(&bars.q_full, 1);
     mbar_init(&bars.q_empty, 1);
     for (int s = 0; s < kStagesLse; ++s) { mbar_init(&bars.kv_full[s], 1); mbar_init(&bars.kv_empty[s], 1); }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&bars.s_full[i], 1); mbar_init(&bars.p_full[i], 4); mbar_init(&bars.o_done[i], 1);
-      mbar_init(&bars.o_free[i], 4);
-    }
+    for (int i = 0; i < 4; ++i) { mbar_init(&bars.s_full[i], 1); mbar_init(&bars.p_full[i], 4); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&bars.o_done[i], 1); mbar_init(&bars.o_free[i], 4); mbar_init(&bars.m_full[i], 4); mbar_init(&bars.m_empty[i], 4); }
     s_abort = 0;
     fence_mbar_init();
   }
@@ -415,7 +448,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
   // an allocation of all 512 columns starts at column 0; addresses known at compile time keep the MMAs' operands cheap
   if (s_tmem != 0 && tid == 0) { s_abort = 1; atomicOr(p.status, WK_DEV_TIMEOUT); }
 
-  if (warp == kTmaWarp) {
+  if (warp == kSoftWarps<kLse> + 1) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       PieceWalker walk;
@@ -429,8 +462,8 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
         ++n;
         for (int i = 0; i < 2; ++i)
           for (int half = 0; half < 2; ++half)
-            tma_load_2d(sQ + i * kTileBytes + half * kHalfTileBytes, &p.tm_q, &bars.q_full, pc.h * kHeadDim + half * 64,
-                        pc.q0 + i * kTileQ);
+            tma_load_2d(sQ + i * kTileBytes + half * kHalfTileBytes, &p.tm_q, &bars.q_full,
+                        pc.h * kHeadDim + half * 64, pc.q0 + i * kTileQ);
         TileIter it;
         const bool report = !p.slot_units;
         it.init(p, pc.tb, pc.te, report);
@@ -474,7 +507,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           if (steps > q) drain(&bars.kv_full[q], (steps - 1 - q) / kNStages);
       }
     }
-  } else if (warp == kMmaWarp) {
+  } else if (warp == kSoftWarps<kLse>) {
     // ------------------------------------------------------------------ MMA issue
     // The whole warp runs the control flow and one lane's predicate issues (see mma_ss_if).
     {
@@ -489,14 +522,14 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
       auto commit = [&](size_t offset) { mma_commit_if(one, bar0 + static_cast<uint32_t>(offset)); };
       // S_i = Q_i K^T over the first nv rows of the K tile.  A full tile is eight MMAs without a branch between them; a
       // short one computes ceil(nv / 16) * 16 columns.
-      auto issue_s = [&](uint32_t i, uint32_t st, int nv) {
-        const uint64_t a = q_desc + i * (kTileBytes >> 4), b = k_desc + st * (kStageBytes >> 4);
+      auto issue_s = [&](uint32_t qt, uint32_t d, uint32_t st, int nv) {   // qt: Q tile in shared memory, d: S columns
+        const uint64_t a = q_desc + qt * (kTileBytes >> 4), b = k_desc + st * (kStageBytes >> 4);
         const uint32_t idesc = nv == kTileKV ? idesc_qk
                                              : (idesc_bf16_f32(128, 0, 0, 0) | (static_cast<uint32_t>((nv + 15) >> 4) << 18));
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const uint32_t off = (k >> 2) * (kHalfTileBytes >> 4) + (k & 3) * 2;   // 32 bytes per step inside a 128-byte row
-          mma_ss_if(one, kTmemS + i * 128, a + off, b + off, idesc, k > 0);
+          mma_ss_if(one, d, a + off, b + off, idesc, k > 0);
         }
       };
       // O_i (+)= P_i V: A = P from tensor memory (bf16 pairs, 8 columns per K = 16 step); B = V, rows = K dimension,
@@ -532,42 +565,70 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           if (lane == 0) mbar_arrive(&bars.q_empty);
           continue;
         }
+        if (kLse) {
+          // LSE-only: two S buffers per Q tile, no P V; p_full says that a buffer has been read
+          for (int j = 0; j < n_eff; ++j) {
+            WK_PROF(0);
+            if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &s_abort))) break;
+            const int nv = s_nv[t++ % kNvRing];
+            const uint32_t b0 = lse_q0 & 1, b1 = lse_q1 & 1;
+            WK_PROF(1);
+            if (lse_q0 >= 2 && !(ok = wait_or_abort(&bars.p_full[2 * b0], ((lse_q0 >> 1) & 1) ^ 1, &s_abort))) break;
+            ++lse_q0;
+            WK_PROF(2);
+            tc_fence_after();
+            issue_s(0, b0 * 256, st, nv);
+            commit(offsetof(Barriers, s_full) + 16 * b0);
+            WK_PROF(3);
+            if (q1) {
+              if (lse_q1 >= 2 && !(ok = wait_or_abort(&bars.p_full[2 * b1 + 1], ((lse_q1 >> 1) & 1) ^ 1, &s_abort))) break;
+              ++lse_q1;
+              WK_PROF(4);
+              tc_fence_after();
+              issue_s(1, b1 * 256 + 128, st, nv);
+              commit(offsetof(Barriers, s_full) + 16 * b1 + 8);
+            }
+            commit(offsetof(Barriers, kv_empty) + 8 * st);
+            if (j + 1 == n_eff) commit(offsetof(Barriers, q_empty));
+            WK_PROF(5);
+            if (++st == kNStages) { st = 0; ph ^= 1; }
+          }
+          continue;
+        }
         // Step j: for each Q tile, once its P of tile j is there, P V of tile j and Q K^T of tile j + 1 into the S buffer
-        // P was in.  The other Q tile's softmax runs meanwhile.  (LSE-only: no P V; the "P" signal says that S has been read.)
+        // P was in.  The other Q tile's softmax runs meanwhile.
         int nv = 0, nv_next = 0;
-        for (int j = -1; j < n_eff - (kLse ? 1 : 0); ++j) {
+        for (int j = -1; j < n_eff; ++j) {
           const bool more = j + 1 < n_eff;
           WK_PROF(0);
           if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &s_abort))) break;
           if (more) nv_next = s_nv[t++ % kNvRing];
           WK_PROF(1);
-          if (kLse ? lse_q0 > 0 : j >= 0) {
+          if (j >= 0) {
             if (!(ok = wait_or_abort(&bars.p_full[0], p_ph0, &s_abort))) break;
             p_ph0 ^= 1;
           }
-          if (kLse) ++lse_q0;
           WK_PROF(2);
           // A piece's first P V overwrites O: the epilogue of the last piece that used it must have read it.  o_free[i]
           // completes once per piece in which warpgroup i ran an epilogue, so neither side can run two phases ahead of the
           // other (a parity wait cannot tell phase n from phase n + 2).
-          if (!kLse && j == 0 && e0++ > 0 && !(ok = wait_or_abort(&bars.o_free[0], e0 & 1, &s_abort))) break;
+          if (j == 0 && e0++ > 0 && !(ok = wait_or_abort(&bars.o_free[0], e0 & 1, &s_abort))) break;
           tc_fence_after();
-          if (!kLse && j >= 0) issue_pv(0, st, nv, j > 0);
-          if (more) { issue_s(0, st, nv_next); commit(offsetof(Barriers, s_full)); }
+          if (j >= 0) issue_pv(0, st, nv, j > 0);
+          if (more) { issue_s(0, kTmemS, st, nv_next); commit(offsetof(Barriers, s_full)); }
           else commit(offsetof(Barriers, o_done));
           if (!q1) commit(offsetof(Barriers, kv_empty) + 8 * st);
           WK_PROF(3);
           if (q1) {
-            if (kLse ? lse_q1 > 0 : j >= 0) {
+            if (j >= 0) {
               if (!(ok = wait_or_abort(&bars.p_full[1], p_ph1, &s_abort))) break;
               p_ph1 ^= 1;
             }
-            if (kLse) ++lse_q1;
             WK_PROF(4);
-            if (!kLse && j == 0 && e1++ > 0 && !(ok = wait_or_abort(&bars.o_free[1], e1 & 1, &s_abort))) break;
+            if (j == 0 && e1++ > 0 && !(ok = wait_or_abort(&bars.o_free[1], e1 & 1, &s_abort))) break;
             tc_fence_after();
-            if (!kLse && j >= 0) issue_pv(1, st, nv, j > 0);
-            if (more) { issue_s(1, st, nv_next); commit(offsetof(Barriers, s_full) + 8); }
+            if (j >= 0) issue_pv(1, st, nv, j > 0);
+            if (more) { issue_s(1, kTmemS + 128, st, nv_next); commit(offsetof(Barriers, s_full) + 8); }
             else commit(offsetof(Barriers, o_done) + 8);
             commit(offsetof(Barriers, kv_empty) + 8 * st);
             WK_PROF(5);
@@ -580,6 +641,101 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
       if (lane == 0) leave_role(ok, &s_abort, p.status);
       WK_PROF_FLUSH(8, 12, blockIdx.x == 0 && lane == 0);
     }
+  } else if (kLse) {
+    // ------------------------------------------------------------------ LSE-only softmax warpgroups (one thread per row)
+    // Warpgroup qt + 2 b works on S buffer b of Q tile qt, i.e. on every other KV tile of these rows: four warps per
+    // scheduler instead of two, which is what hides the latencies of this issue-bound loop.  At the end of a unit the two
+    // warpgroups of a Q tile merge (reference, sum) through shared memory.
+    const int wg = warp >> 2, qt = wg & 1, buf = wg >> 1;
+    const int row = (warp & 3) * 32 + lane;
+    const uint32_t tS = (static_cast<uint32_t>((warp & 3) * 32) << 16) + buf * 256 + qt * 128;
+    const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2);
+    PieceWalker walk;
+    walk.init(p);
+    Piece pc;
+    uint32_t g = 0;     // KV tiles of this Q tile so far: tile number g is in buffer g & 1
+    uint32_t t0 = 0;    // tiles of the CTA's pieces so far
+    uint32_t n = 0;     // units of this Q tile so far
+    bool ok = true;
+    WK_PROF_DECL
+    while (ok && walk.next(p, pc)) {
+      const int n_eff = count_tiles(p, pc.tb, pc.te);
+      if (qt == 1 && !pc.has_q1) { t0 += n_eff; continue; }
+      float m = 0.f, l = 0.f;
+      bool first = true;
+      for (int j = (g ^ buf) & 1; j < n_eff; j += 2) {
+        WK_PROF(0);
+        if (!(ok = wait_or_abort(&bars.s_full[wg], ((g + j) >> 1) & 1, &s_abort))) break;
+        WK_PROF(1);
+        const int nv = s_nv[(t0 + j) % kNvRing], n_ch = (nv + 31) >> 5;
+        tc_fence_after();
+        // The row is streamed from tensor memory 32 columns at a time, without a maximum: the sum is taken against a fixed
+        // reference, 0 at first (logits of a few log2 units lose nothing there).  A warp in which a row's tile sum leaves
+        // [2^-12 (first tile only), 2^15] reads S again and takes the row's maximum as its reference from there on.
+        float sum = 0.f;
+#pragma unroll 1
+        for (int attempt = 0; attempt < 2; ++attempt) {
+          const uint64_t neg_m2 = pack_f32x2(-m, -m);
+          uint64_t acc[4] = {0, 0, 0, 0};
+          float big = -INFINITY;
+#pragma unroll 1
+          for (int c = 0; c < n_ch; ++c) {
+            uint32_t r[32];
+            tmem_ld_x32(tS + c * 32, r);
+            tc_wait_ld();
+            lse_chunk(r, nv - c * 32, scale2, neg_m2, acc, big);
+          }
+          sum = sum4_f32x2(acc);
+          const bool off = !(sum <= 32768.f) || big * p.scale_log2 - m > 100.f || (first && sum < 2.44140625e-4f);
+          if (attempt > 0 || !__any_sync(0xffffffffu, off)) break;
+          float mx = -INFINITY;
+#pragma unroll 1
+          for (int c = 0; c < n_ch; ++c) {
+            uint32_t r[32];
+            tmem_ld_x32(tS + c * 32, r);
+            tc_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 32; ++i) mx = fmaxf(mx, i < nv - c * 32 ? __uint_as_float(r[i]) : -INFINITY);
+          }
+          if (off) {
+            const float m_new = first ? mx * p.scale_log2 : fmaxf(m, mx * p.scale_log2);
+            l *= ex2_approx(m - m_new);
+            m = m_new;
+          }
+        }
+        WK_PROF(4);
+        l += sum;
+        first = false;
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars.p_full[wg]);   // the buffer has been read
+      }
+      if (!ok) break;
+      g += n_eff;
+      t0 += n_eff;
+      if (buf == 1) {
+        if (!(ok = wait_or_abort(&bars.m_empty[qt], (n & 1) ^ 1, &s_abort))) break;
+        s_merge[qt][row] = make_float2(m, l);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars.m_full[qt]);
+      } else {
+        if (!(ok = wait_or_abort(&bars.m_full[qt], n & 1, &s_abort))) break;
+        const float2 o = s_merge[qt][row];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars.m_empty[qt]);
+        const int qrow = pc.q0 + qt * kTileQ + row;
+        if (qrow < p.lq) {
+          // (a warpgroup without tiles leaves a sum of 0, a stale slot two of them)
+          const float mm = l > 0.f ? (o.y > 0.f ? fmaxf(m, o.x) : m) : o.x;
+          const float sum = (l > 0.f ? l * ex2_approx(m - mm) : 0.f) + (o.y > 0.f ? o.y * ex2_approx(o.x - mm) : 0.f);
+          p.lse[(static_cast<int64_t>(pc.ord) * p.H + pc.h) * p.lq + qrow] =
+              sum > 0.f ? (mm + log2f(sum)) * 0.6931471805599453f : -INFINITY;
+        }
+      }
+      ++n;
+    }
+    if (!ok) leave_role(false, &s_abort, p.status);
+    WK_PROF_FLUSH(0, 8, blockIdx.x == 0 && tid == 0);
   } else {
     // ------------------------------------------------------------------ softmax warpgroups (one thread per query row)
     const int wg = warp >> 2;
@@ -633,11 +789,6 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
             tc_wait_ld();
           }
           WK_PROF(2);
-          if (kLse) {   // S is in registers and nothing goes back into the buffer: release it now
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&bars.p_full[wg]);
-          }
           const bool full_tile = nv == kTileKV;
           if (!full_tile) {   // rows past the end of the segment were zero-filled by TMA: mask them out
             c0 = c1 = c2 = c3 = -INFINITY;
@@ -671,9 +822,9 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           const uint64_t neg_m2 = pack_f32x2(-m_used, -m_used);
           WK_PROF(3);
           // masked columns hold -inf and come out as 0 (special-function path only)
-          l += full_tile ? exp_store_tile<!kLse, WK_ATTN_POLY>(s, scale2, neg_m2, tS, 4)
-                         : exp_store_tile<!kLse, 0>(s, scale2, neg_m2, tS, (nv + 31) >> 5);
-          if (!kLse && __any_sync(0xffffffffu, rescale)) {
+          l += full_tile ? exp_store_tile<WK_ATTN_POLY>(s, scale2, neg_m2, tS, 4)
+                         : exp_store_tile<0>(s, scale2, neg_m2, tS, (nv + 31) >> 5);
+          if (__any_sync(0xffffffffu, rescale)) {
             // (the previous P V was issued before this tile's Q K^T: it landed before S did)
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
@@ -686,12 +837,10 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
             }
           }
           WK_PROF(4);
-          if (!kLse) {
-            tc_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&bars.p_full[wg]);   // one arrival per warp: the wait above covered all 32 lanes' stores
-          }
+          tc_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bars.p_full[wg]);   // one arrival per warp: the wait above covered all 32 lanes' stores
           WK_PROF(5);
           ++j;
           ++g;
@@ -699,7 +848,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
         // ---------------------------------------------------------------- epilogue of this piece
         const int prow = wg * kTileQ + row;
         const int qrow = pc.q0 + prow;
-        if (!kLse && ok && j > 0) ok = wait_or_abort(&bars.o_done[wg], n_out++ & 1, &s_abort);   // completes once per piece
+        if (ok && j > 0) ok = wait_or_abort(&bars.o_done[wg], n_out++ & 1, &s_abort);   // completes once per piece
         if (ok) {
           tc_fence_after();
           const float inv_l = (j > 0 && l > 0.f) ? 1.f / l : 0.f;
@@ -707,14 +856,14 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             uint32_t r[32];
-            if (!kLse && j > 0) {
+            if (j > 0) {
               tmem_ld_x32(tO + c * 32, r);
               tc_wait_ld();
             } else {
 #pragma unroll
               for (int i = 0; i < 32; ++i) r[i] = 0u;
             }
-            if (!kLse && qrow < p.lq) {
+            if (qrow < p.lq) {
               if (pc.slot < 0) {
                 uint4* dst = reinterpret_cast<uint4*>(p.O + (static_cast<int64_t>(qrow) * p.H + pc.h) * kHeadDim + c * 32);
 #pragma unroll
@@ -737,7 +886,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           }
           if (qrow < p.lq) {
             if (pc.slot < 0) {
-              if (p.lse) p.lse[(static_cast<int64_t>(pc.ord) * p.H + pc.h) * p.lq + qrow] = lse;
+              if (p.lse) p.lse[static_cast<int64_t>(pc.h) * p.lq + qrow] = lse;
             } else {
               p.lsepart[static_cast<int64_t>(pc.slot) * kPairRows + prow] = lse;
             }
@@ -931,13 +1080,9 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   const int64_t sms = ctx->sm_count;
   int64_t G, n_full = 0, ranges = 0;   // CTAs, units done whole, ranges the rest is cut into
   if (lse_only) {
-    // whole units per CTA (nothing to merge): the largest divisor of the unit count that fits the SMs, unless that
-    // would leave more than a quarter of them idle -- then one CTA per unit
-    G = 1;
-    for (int64_t g = sms < p.n_units ? sms : p.n_units; g >= 1; --g)
-      if (p.n_units % g == 0) { G = g; break; }
-    if (G * 4 < sms * 3 && p.n_units > G) G = p.n_units;
-    ranges = G;
+    // whole units, dealt out one by one: the CTAs of one (slot, head) run side by side and share its tiles through L2
+    n_full = p.n_units;
+    G = sms < n_full ? sms : n_full;
   } else if (kv_splits == 0) {
     split_default(p.n_units, p.n_tiles, sms, &G, &n_full, &ranges);
   } else if (kv_splits > 0) {
@@ -955,9 +1100,9 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   if (!lse_only && 2 * ranges > max_slots) return WK_ERR_SHAPE;
   p.n_full = static_cast<int>(n_full);
   p.n_ranges = static_cast<int>(ranges);
-  const dim3 grid(static_cast<unsigned>(G)), block(kThreads);
-  if (lse_only) launch_chained(memory_attention_kernel<true>, grid, block, kSmemBytesLse, s, p);
-  else launch_chained(memory_attention_kernel<false>, grid, block, kSmemBytes, s, p);
+  const dim3 grid(static_cast<unsigned>(G));
+  if (lse_only) launch_chained(memory_attention_kernel<true>, grid, dim3(kThreads<true>), kSmemBytesLse, s, p);
+  else launch_chained(memory_attention_kernel<false>, grid, dim3(kThreads<false>), kSmemBytes, s, p);
   if ((st = after_launch(ctx)) != WK_OK) return st;
   if (!lse_only && n_full != p.n_units) {   // some unit was cut
     launch_chained(combine_kernel, dim3(static_cast<unsigned>(p.n_units - n_full) * 32), dim3(kCombineThreads), 0, s, p.opart,

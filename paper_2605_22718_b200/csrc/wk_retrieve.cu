@@ -87,68 +87,125 @@ retrieve_kernel(const float* __restrict__ poses, const int32_t* __restrict__ val
 // ---- query-based retrieval (Appendix C) --------------------------------------------------------------------------
 // lse[slot][h][r] holds, for every valid slot, the log-sum-exp of query row r of head h over that slot's stored keys.
 // The softmax mass of a slot for (h, r) is exp(lse[slot] - logsumexp over slots); a slot's score is the mean mass.
-// query_mass: one thread per (h, r); the masses are added over the warp by shuffles, over the block in a fixed order,
-// and every block leaves one partial per slot -- no floating-point atomics, so the ranking is reproducible.
-constexpr int kMassThreads = 256;
+// query_mass: a block takes 256 (h, r) columns, eight warps side by side; four warps share a column group's slots.  Each
+// warp first takes the running maximum and sum of its slots, eight loads in flight, the four shares meet in shared memory,
+// and a second walk (the values come from L2 now) turns them into masses, added over the warp's columns by shuffles and over
+// the block in a fixed order: one partial per (block, slot), no floating-point atomics, so the ranking is reproducible.
+// Bound by reading the LSEs twice; 250 slots x 31,680 columns: one thread per column with three serial walks 116 us.
+constexpr int kMassCols = 256, kMassThreads = 1024, kMassShares = 4;
 
 __global__ void __launch_bounds__(kMassThreads)
 query_mass(const float* __restrict__ lse, const int32_t* __restrict__ valid, int n_slots, int n_hr,
            double* __restrict__ block_part /*[gridDim.x][n_slots]*/) {
-  extern __shared__ float warp_part[];   // [8 warps][n_slots]
+  extern __shared__ float s_dyn[];                       // [8 column groups][n_slots] masses, then n_slots validity words
+  __shared__ float s_mx[kMassShares][kMassCols], s_den[kMassShares][kMassCols];
+  float* s_mass = s_dyn;
+  int32_t* s_valid = reinterpret_cast<int32_t*>(s_dyn + 8 * n_slots);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int i = blockIdx.x * kMassThreads + tid;
+  const int cg = warp & 7, share = warp >> 3, col = cg * 32 + lane;
+  const int i = blockIdx.x * kMassCols + col;
   const bool live = i < n_hr;
-  float mx = -INFINITY;
-  for (int s = 0; s < n_slots; ++s)
-    if (valid[s] && live) mx = fmaxf(mx, lse[static_cast<int64_t>(s) * n_hr + i]);
-  float den = 0.f;
-  for (int s = 0; s < n_slots; ++s)
-    if (valid[s] && live) den += expf(lse[static_cast<int64_t>(s) * n_hr + i] - mx);
-  const float inv = (live && den > 0.f) ? 1.f / den : 0.f;
-  for (int s = 0; s < n_slots; ++s) {
-    float m = 0.f;
-    if (valid[s] && live) m = expf(lse[static_cast<int64_t>(s) * n_hr + i] - mx) * inv;
+  const float* mine = lse + (live ? i : 0);
+  dep_wait();
+  dep_release();
+  for (int s = tid; s < n_slots; s += kMassThreads) s_valid[s] = valid[s];
+  __syncthreads();
+  float mx = -INFINITY, den = 0.f;
+  for (int s0 = share; s0 < n_slots; s0 += 8 * kMassShares) {
+    float v[8];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-    if (lane == 0) warp_part[warp * n_slots + s] = m;
+    for (int k = 0; k < 8; ++k) {
+      const int s = s0 + k * kMassShares;
+      v[k] = s < n_slots && s_valid[s] ? __ldcg(mine + static_cast<int64_t>(s) * n_hr) : -INFINITY;
+    }
+    float m8 = mx;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) m8 = fmaxf(m8, v[k]);
+    if (m8 > -INFINITY) {
+      float add = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) add += expf(v[k] - m8);
+      den = den * expf(mx - m8) + add;
+      mx = m8;
+    }
+  }
+  s_mx[share][col] = mx;
+  s_den[share][col] = den;
+  __syncthreads();
+  mx = fmaxf(fmaxf(s_mx[0][col], s_mx[1][col]), fmaxf(s_mx[2][col], s_mx[3][col]));
+  den = 0.f;
+  if (mx > -INFINITY) {
+#pragma unroll
+    for (int k = 0; k < kMassShares; ++k) den += s_den[k][col] * expf(s_mx[k][col] - mx);
+  }
+  const float inv = (live && den > 0.f) ? 1.f / den : 0.f;
+  for (int s0 = share; s0 < n_slots; s0 += 8 * kMassShares) {
+    float v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int s = s0 + k * kMassShares;
+      v[k] = s < n_slots && s_valid[s] ? __ldcg(mine + static_cast<int64_t>(s) * n_hr) : -INFINITY;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int s = s0 + k * kMassShares;
+      float m = inv > 0.f ? expf(v[k] - mx) * inv : 0.f;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+      if (lane == 0 && s < n_slots) s_mass[cg * n_slots + s] = m;
+    }
   }
   __syncthreads();
   for (int s = tid; s < n_slots; s += kMassThreads) {
     double t = 0.0;
-    for (int w = 0; w < kMassThreads / 32; ++w) t += static_cast<double>(warp_part[w * n_slots + s]);
+    for (int w = 0; w < 8; ++w) t += static_cast<double>(s_mass[w * n_slots + s]);
     block_part[static_cast<int64_t>(blockIdx.x) * n_slots + s] = t;
   }
 }
 
-// One CTA: adds the blocks' partials in order, ranks the valid slots by (score descending, slot ascending).
+// One CTA: adds the blocks' partials in a fixed order, ranks the valid slots by (score descending, slot ascending).  1024
+// threads share the slots: P of them per slot, each with every P-th block and every P-th comparison.
 __global__ void __launch_bounds__(1024)
 query_topk(const double* __restrict__ block_part, int n_blocks, const int32_t* __restrict__ valid, int n_slots, int n_hr,
            int k, int max_k, int32_t* __restrict__ slots_out, float* __restrict__ score_out) {
-  __shared__ double score[1024];
+  __shared__ double score[1024], part[1024];
+  __shared__ int s_rank[1024];
   const int tid = threadIdx.x;
-  for (int s = tid; s < n_slots; s += 1024) {
-    double t = 0.0;
-    for (int b = 0; b < n_blocks; ++b) t += block_part[static_cast<int64_t>(b) * n_slots + s];
-    score[s] = valid[s] ? t / static_cast<double>(n_hr) : -1.0;   // negative marks "not a candidate"
-  }
+  int P = 1;
+  while (P < 8 && n_slots * P * 2 <= 1024) P <<= 1;
+  const int s = tid % n_slots, q = tid / n_slots;   // slot and share (threads with q >= P idle)
+  s_rank[tid] = 0;
+  dep_wait();
   for (int i = tid; i < max_k; i += 1024) {
     slots_out[i] = -1;
     if (score_out) score_out[i] = 0.f;
   }
+  double t = 0.0;
+  if (q < P) {
+#pragma unroll 8
+    for (int b = q; b < n_blocks; b += P) t += __ldcg(block_part + static_cast<int64_t>(b) * n_slots + s);
+  }
+  part[tid] = t;
   __syncthreads();
-  for (int s = tid; s < n_slots; s += 1024) {
-    const double v = score[s];
-    if (v < 0.0) continue;
+  if (q == 0) {
+    for (int w = 1; w < P; ++w) t += part[w * n_slots + s];
+    score[s] = valid[s] ? t / static_cast<double>(n_hr) : -1.0;   // negative marks "not a candidate"
+  }
+  __syncthreads();
+  const double v = score[s];
+  if (q < P && v >= 0.0) {
     int rank = 0;
-    for (int u = 0; u < n_slots; ++u) {
+#pragma unroll 4
+    for (int u = q; u < n_slots; u += P) {
       const double w = score[u];
-      if (w < 0.0) continue;
-      rank += (w > v) || (w == v && u < s);
+      rank += w >= 0.0 && (w > v || (w == v && u < s));
     }
-    if (rank < k) {
-      slots_out[rank] = s;
-      if (score_out) score_out[rank] = static_cast<float>(v);
-    }
+    if (rank) atomicAdd(&s_rank[s], rank);
+  }
+  __syncthreads();
+  if (q == 0 && v >= 0.0 && s_rank[s] < k) {
+    slots_out[s_rank[s]] = s;
+    if (score_out) score_out[s_rank[s]] = static_cast<float>(v);
   }
 }
 
@@ -178,11 +235,11 @@ wk_status launch_retrieve_query(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, 
   // problem of its own in one launch (slots that hold nothing come back as -inf and are masked by the valid flags)
   wk_status st = launch_attention(ctx, layer, Q, lq, nullptr, 0, ids, S, nullptr, lse, 1, s, true);
   if (st != WK_OK) return st;
-  const int blocks = (n_hr + kMassThreads - 1) / kMassThreads;
-  query_mass<<<blocks, kMassThreads, static_cast<size_t>(kMassThreads / 32) * S * sizeof(float), s>>>(lse, ctx->valid_dev, S,
-                                                                                                     n_hr, part);
+  const int blocks = (n_hr + kMassCols - 1) / kMassCols;
+  launch_chained(query_mass, dim3(blocks), dim3(kMassThreads), static_cast<size_t>(9) * S * sizeof(float), s, lse, ctx->valid_dev, S,
+                 n_hr, part);
   if ((st = after_launch(ctx)) != WK_OK) return st;
-  query_topk<<<1, 1024, 0, s>>>(part, blocks, ctx->valid_dev, S, n_hr, k, ctx->cfg.max_k, slots_out, score_out);
+  launch_chained(query_topk, dim3(1), dim3(1024), 0, s, part, blocks, ctx->valid_dev, S, n_hr, k, ctx->cfg.max_k, slots_out, score_out);
   return after_launch(ctx);
 }
 

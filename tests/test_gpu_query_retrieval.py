@@ -122,3 +122,29 @@ def test_query_retrieval_many_slots_matrix_game_heads():
     assert Qb.shape[0] == 300
     for k in (1, 2, 8):
         _check(kv, sc, 0, Qb, k)
+
+
+@pytest.mark.parametrize("T,n_keep,n_chunks,pool_slots,lq,gain", [
+    (40, 24, 9, 9, 129, 1.0),       # C = 64: one short tile per slot, the second Q tile has one row
+    (90, 38, 7, 7, 128, 1.0),       # C = 128: exactly one tile, no second Q tile
+    (90, 39, 5, 600, 256, 1.0),     # C = 129: a tile and one row; most slots of the pool empty
+    (150, 150, 6, 8, 300, 1.0),     # C = 300: three tiles, odd and even tiles on different warpgroups
+    (150, 150, 6, 8, 300, 12.0),    # logits far outside the fixed reference's range, up and down, in most rows
+    (60, 20, 3, 3, 40, 40.0),
+])
+def test_query_scores_at_tile_edges(T, n_keep, n_chunks, pool_slots, lq, gain):
+    """Scores of every stored chunk against the oracle at the sizes where the LSE-only kernel's tiles, units and reference
+    change."""
+    kv, sc = _scene(T=T, H=2, n_keep=n_keep, n_chunks=n_chunks, pool_slots=pool_slots, max_lq=lq, n_layers=1, seed=17)
+    Qb = wi.query_bf16(17, 0, 0, 0, lq, 256)
+    f = (Qb.astype(np.uint32) << 16).view(np.float32) * np.float32(gain)
+    Qb = wi.f32_to_bf16_bits(f) if hasattr(wi, "f32_to_bf16_bits") else wi.gen.f32_to_bf16_bits(f)
+    Q = wd.to_device_bf16(Qb).view(lq, 2, 128)
+    score = torch.empty((kv.max_k,), dtype=torch.float32, device="cuda")
+    slots, n = kv.retrieve_query(0, Q, kv.max_k, score_out=score)
+    assert kv.poll_status() == (0, 0) and n == n_chunks
+    ref_slots, ref = o.query_scores(Qb.reshape(lq, 2, 128), sc.pool, 0)
+    got = dict(zip(slots.cpu().numpy()[:n].tolist(), score.cpu().numpy()[:n].tolist()))
+    assert sorted(got) == sorted(ref_slots)
+    np.testing.assert_allclose([got[s] for s in ref_slots], ref, rtol=SCORE_RTOL, atol=1e-7)
+    assert (slots.cpu().numpy()[n:] == -1).all()
