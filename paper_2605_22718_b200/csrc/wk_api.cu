@@ -284,6 +284,7 @@ static wk_status append_checked(wk_ctx* ctx, int32_t layer0, int32_t n, const vo
     st = launch_slot_mark(ctx, slot, 1, si.pose, s);
     if (st != WK_OK) return st;
     si.state = SLOT_VALID;
+    ++ctx->n_valid;
     si.seq = ctx->next_seq++;
   }
   *slot_io_host = slot;
@@ -405,6 +406,7 @@ wk_status wk_pool_load_host(wk_ctx* ctx, int32_t layer0, int32_t n, const void* 
     wk_status st = launch_slot_mark(ctx, slot, 1, si.pose, s);
     if (st != WK_OK) return st;
     si.state = SLOT_VALID;
+    ++ctx->n_valid;
     si.seq = ctx->next_seq++;
   }
   *slot_io_host = slot;
@@ -419,6 +421,7 @@ wk_status wk_pool_evict(wk_ctx* ctx, int32_t slot, void* stream) {
   wk_status st = launch_slot_mark(ctx, slot, 0, ctx->slots[slot].pose, static_cast<cudaStream_t>(stream));
   if (st != WK_OK) return st;
   ctx->slots[slot].state = SLOT_FREE;
+  --ctx->n_valid;
   ctx->slots[slot].tag = -1;
   return WK_OK;
 }
@@ -434,9 +437,7 @@ int32_t wk_pool_oldest(const wk_ctx* ctx) {
 
 int32_t wk_pool_count(const wk_ctx* ctx) {
   if (!ctx) return 0;
-  int n = 0;
-  for (const auto& s : ctx->slots) n += (s.state == SLOT_VALID);
-  return n;
+  return ctx->n_valid;
 }
 
 int64_t wk_pool_tag(const wk_ctx* ctx, int32_t slot) {

@@ -72,6 +72,7 @@ struct wk_ctx {
   // host bookkeeping of the pool
   std::vector<wk::SlotInfo> slots;
   int64_t next_seq = 0;
+  int32_t n_valid = 0;   // slots in state SLOT_VALID
   // tensor maps
   CUtensorMap tm_kpool, tm_vpool;
   std::vector<wk::TmapKey> tmap_cache;
