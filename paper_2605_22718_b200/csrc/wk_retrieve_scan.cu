@@ -8,6 +8,8 @@
 //       r_j > R* + (pi / mt_lo) * max(0, T* - t_j)
 // (a pivot with the larger translation term loses at most (T* - t_j) / mt_lo there and gains at least (r_j - R*) / pi).
 //
+// Arrays of up to 2^17 poses with k <= 16 take two kernels: scan_max (the exact maxima) and scan_select on all poses.  Longer
+// ones, or longer lists, take three:
 //   scan_sample  a strided sample of the candidates (one in 128, 2^15 .. 2^18 of them): per block the largest t,
 //                and for each of k disjoint sample classes the candidate with the smallest r + pi t / (roughly max t),
 //                in fp32 -- pivots only have to be real candidates, not the best ones
@@ -37,6 +39,7 @@ constexpr int kScanWarm = 256;       // candidates of the first, list-seeding ro
 constexpr int kPendLow = 256;        // survivors of the cheap bound are decided once this many have gathered
 constexpr int kScanCap = kScanLow + kSelThreads + 64;   // between two checks at most one entry per thread is added
 constexpr int kScanMaxBlocks = 1024;
+constexpr int64_t kScanTwice = 1 << 17;   // longest array that is walked twice instead of sampled and filtered
 
 constexpr int kSampleBlocks = 128;          // scan_sample's grid
 constexpr int kSampleThreads = 256;
@@ -56,6 +59,10 @@ struct SampleRecord {
   double t_max;                              // largest squared translation distance among the block's samples (fp32 value)
   double dot_min;                            // smallest |quaternion dot| among them (fp32 value; 2 = none)
   unsigned long long best[kScanMaxK];        // per class: (fp32 key bits << 32) | candidate index; ~0 = none
+};
+// one record per scan_max block (candidate arrays that are walked twice)
+struct MaxRecord {
+  double t_max, dot_min;
 };
 struct ScanEntry {
   double d;
@@ -95,11 +102,71 @@ __device__ __forceinline__ float rot_lower_bound(float adot32) {
   return 2.f * sqrtf(om + om) * (1.f - 3e-6f);
 }
 
+// Exact maxima of a candidate array that is small enough to be walked twice (the second time from L2): one record per
+// block.  Bound by reading the poses.
+constexpr int kMaxThreads = 512, kMaxUnroll = 4;
+__global__ void __launch_bounds__(kMaxThreads)
+scan_max(const float4* __restrict__ poses, const int32_t* __restrict__ valid, int64_t n, Cur8 cur, ScanHeader* __restrict__ h,
+         MaxRecord* __restrict__ rec, uint32_t* __restrict__ status) {
+  __shared__ double s_t[kMaxThreads / 32], s_d[kMaxThreads / 32];
+  dep_wait();
+  dep_release();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (blockIdx.x == 0 && tid == 0) h->ticket = 0u;
+  double mt = 0.0, md = 2.0;
+  bool bad = false;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * kMaxThreads;
+  for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * kMaxThreads + tid; i0 < n; i0 += kMaxUnroll * stride) {
+    float4 a[kMaxUnroll], b[kMaxUnroll];
+    bool live[kMaxUnroll];
+#pragma unroll
+    for (int u = 0; u < kMaxUnroll; ++u) {
+      const int64_t i = i0 + u * stride;
+      live[u] = i < n;
+      if (live[u]) {
+        a[u] = __ldg(poses + 2 * i);
+        b[u] = __ldg(poses + 2 * i + 1);
+        if (valid) live[u] = __ldg(valid + i) != 0;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kMaxUnroll; ++u) {
+      if (!live[u]) continue;
+      const Cand c = candidate(a[u], b[u], cur.v);
+      if (isfinite(c.t) && isfinite(c.adot)) {
+        mt = fmax(mt, c.t);
+        md = fmin(md, c.adot);
+      } else {
+        bad = true;
+      }
+    }
+  }
+  if (bad) atomicOr(status, WK_DEV_NONFINITE);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    mt = fmax(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+    md = fmin(md, __shfl_xor_sync(0xffffffffu, md, o));
+  }
+  if (lane == 0) { s_t[warp] = mt; s_d[warp] = md; }
+  __syncthreads();
+  if (warp == 0) {
+    mt = lane < kMaxThreads / 32 ? s_t[lane] : 0.0;
+    md = lane < kMaxThreads / 32 ? s_d[lane] : 2.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mt = fmax(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+      md = fmin(md, __shfl_xor_sync(0xffffffffu, md, o));
+    }
+    if (lane == 0) rec[blockIdx.x] = MaxRecord{mt, md};
+  }
+}
+
 __global__ void __launch_bounds__(kSampleThreads)
 scan_sample(const float4* __restrict__ poses, const int32_t* __restrict__ valid, int64_t n, int64_t n_samples, Cur8 cur,
             int k, ScanHeader* __restrict__ h, SampleRecord* __restrict__ rec) {
   __shared__ float s_tmax[kSampleThreads / 32], s_dmin[kSampleThreads / 32];
   __shared__ unsigned long long s_best[kScanMaxK];
+  dep_wait();
   dep_release();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (blockIdx.x == 0 && tid == 0) {   // the header fields scan_filter accumulates into
@@ -196,23 +263,48 @@ scan_filter(const float4* __restrict__ poses, const int32_t* __restrict__ valid,
   dep_wait();
   dep_release();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // ---- pivots: per class the best record over the sample blocks (four threads per class, a quarter of the records
-  // each), then the exact terms of those k candidates
-  __shared__ unsigned long long s_best[kScanMaxK];
-  if (tid < kScanMaxK) s_best[tid] = ~0ull;
-  __syncthreads();
+  // ---- pivots: per class the best record over the sample blocks, then the exact terms of those k candidates.  Neighbouring
+  // lanes read neighbouring classes of one record (every block reads all of them at once: scattered reads cost 3 us more
+  // per call); a thread's records are all in flight together, and the shares of a class meet in shared memory.
+  __shared__ unsigned long long s_share[kScanThreads];
   {
-    const int g = tid & (kScanMaxK - 1), part = tid >> 6;   // 256 threads = 64 classes x 4 parts
+    int lg = 3;
+    while ((1 << lg) < k) ++lg;                               // classes padded to a power of two, 8 .. 64
+    const int g = tid & ((1 << lg) - 1), part = tid >> lg, parts = kScanThreads >> lg;
+    unsigned long long best = ~0ull;
     if (g < k) {
-      unsigned long long best = ~0ull;
-      for (int b = part; b < n_rec; b += kScanThreads / kScanMaxK) {
-        const unsigned long long v = __ldcg(&rec[b].best[g]);
-        best = v < best ? v : best;
+      for (int b0 = part; b0 < n_rec; b0 += 8 * parts) {
+        unsigned long long v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = b0 + u * parts < n_rec ? __ldcg(&rec[b0 + u * parts].best[g]) : ~0ull;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) best = v[u] < best ? v[u] : best;
       }
-      if (best != ~0ull) atomicMin(&s_best[g], best);
     }
+    s_share[tid] = best;
     double tm = tid < n_rec ? __ldcg(&rec[tid].t_max) : 0.0;   // n_rec <= 128 < 256 threads
     double dm = tid < n_rec ? __ldcg(&rec[tid].dot_min) : 2.0;
+    __syncthreads();
+    if (part == 0 && g < k) {
+#pragma unroll 4
+      for (int q = 1; q < parts; ++q) {
+        const unsigned long long v = s_share[(q << lg) + g];
+        best = v < best ? v : best;
+      }
+    }
+    if (part == 0 && g < k) {
+      double t = -1.0, r = -1.0;   // negative: no pivot in this class
+      if (best != ~0ull) {
+        const int64_t i = static_cast<int64_t>(best & 0xFFFFFFFFull);
+        const Cand c = candidate(__ldg(poses + 2 * i), __ldg(poses + 2 * i + 1), cur.v);
+        if (isfinite(c.t) && isfinite(c.adot)) {
+          t = c.t;
+          r = 2.0 * acos(fmin(1.0, c.adot));
+        }
+      }
+      s_t[g] = t;
+      s_r[g] = r;
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       tm = fmax(tm, __shfl_xor_sync(0xffffffffu, tm, o));
@@ -221,42 +313,37 @@ scan_filter(const float4* __restrict__ poses, const int32_t* __restrict__ valid,
     if (lane == 0) { s_mt[warp] = tm; s_md[warp] = dm; }
   }
   __syncthreads();
-  if (tid < kScanMaxK) {
-    double t = -1.0, r = -1.0;   // negative: no pivot in this class
-    if (tid < k && s_best[tid] != ~0ull) {
-      const int64_t i = static_cast<int64_t>(s_best[tid] & 0xFFFFFFFFull);
-      const Cand c = candidate(__ldg(poses + 2 * i), __ldg(poses + 2 * i + 1), cur.v);
-      if (isfinite(c.t) && isfinite(c.adot)) {
-        t = c.t;
-        r = 2.0 * acos(fmin(1.0, c.adot));
-      }
-    }
-    s_t[tid] = t;
-    s_r[tid] = r;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    double mt_lo = 0.0, md_hi = 2.0;
-    for (int w = 0; w < kScanThreads / 32; ++w) { mt_lo = fmax(mt_lo, s_mt[w]); md_hi = fmin(md_hi, s_md[w]); }
-    // the sample's records seed every thread's: a candidate below them (by more than fp32 rounding) cannot hold a maximum
-    s_rec_t = static_cast<float>(mt_lo);
-    s_rec_d = static_cast<float>(md_hi);
-    mt_lo *= 1.0 - 2e-6;   // the records hold fp32 values: below the true maximum after this
+  if (warp == 0) {
+    double mt_lo = lane < kScanThreads / 32 ? s_mt[lane] : 0.0, md_hi = lane < kScanThreads / 32 ? s_md[lane] : 2.0;
     double Ts = 0.0, Rs = 0.0;
     bool all = k > 0;
-    for (int g = 0; g < k; ++g) {
+    for (int g = lane; g < k; g += 32) {
       all = all && s_t[g] >= 0.0;
       Ts = fmax(Ts, s_t[g]);
       Rs = fmax(Rs, s_r[g]);
     }
-    if (!all) {             // fewer than k pivots: nothing can be ruled out
-      s_Tstar = INFINITY;
-      s_Rstar = INFINITY;
-      s_slope = 0.f;
-    } else {                // every quantity rounded to the side that keeps more candidates
-      s_Tstar = Ts < 3.0e38 ? __double2float_ru(Ts * (1.0 + 1e-6)) : INFINITY;
-      s_Rstar = __double2float_ru(Rs * (1.0 + 1e-6));
-      s_slope = (Ts > 0.0 && mt_lo > 0.0) ? __double2float_ru(3.1415927 / mt_lo * (1.0 + 1e-6)) : (Ts > 0.0 ? INFINITY : 0.f);
+    all = __all_sync(0xffffffffu, all) != 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mt_lo = fmax(mt_lo, __shfl_xor_sync(0xffffffffu, mt_lo, o));
+      md_hi = fmin(md_hi, __shfl_xor_sync(0xffffffffu, md_hi, o));
+      Ts = fmax(Ts, __shfl_xor_sync(0xffffffffu, Ts, o));
+      Rs = fmax(Rs, __shfl_xor_sync(0xffffffffu, Rs, o));
+    }
+    if (lane == 0) {
+      // the sample's records seed every thread's: a candidate below them (by more than fp32 rounding) cannot hold a maximum
+      s_rec_t = static_cast<float>(mt_lo);
+      s_rec_d = static_cast<float>(md_hi);
+      mt_lo *= 1.0 - 2e-6;   // the records hold fp32 values: below the true maximum after this
+      if (!all) {             // fewer than k pivots: nothing can be ruled out
+        s_Tstar = INFINITY;
+        s_Rstar = INFINITY;
+        s_slope = 0.f;
+      } else {                // every quantity rounded to the side that keeps more candidates
+        s_Tstar = Ts < 3.0e38 ? __double2float_ru(Ts * (1.0 + 1e-6)) : INFINITY;
+        s_Rstar = __double2float_ru(Rs * (1.0 + 1e-6));
+        s_slope = (Ts > 0.0 && mt_lo > 0.0) ? __double2float_ru(3.1415927 / mt_lo * (1.0 + 1e-6)) : (Ts > 0.0 ? INFINITY : 0.f);
+      }
     }
   }
   __syncthreads();
@@ -380,10 +467,12 @@ __device__ __forceinline__ void block_rank(const unsigned long long* key, const 
     const unsigned long long ke = key[e];
     const int32_t ie = idx[e];
     int r = 0;
-#pragma unroll 4
+    // no branch in the loop: a condition around the index load costs more than the load
+#pragma unroll 8
     for (int u = p; u < n; u += P) {
       const unsigned long long ku = key[u];
-      r += (ku < ke) || (ku == ke && idx[u] < ie);
+      const int32_t iu = idx[u];
+      r += static_cast<int>(ku < ke) | (static_cast<int>(ku == ke) & static_cast<int>(iu < ie));
     }
     if (r) atomicAdd(&rank[e], r);
   }
@@ -475,7 +564,8 @@ struct TopK {
 
 __global__ void __launch_bounds__(kSelThreads, 2)
 scan_select(const float4* __restrict__ poses, const int32_t* __restrict__ valid_all, int64_t n_all, Cur8 cur,
-            ScanHeader* __restrict__ h, const uint32_t* __restrict__ surv, int k,
+            ScanHeader* __restrict__ h, const MaxRecord* __restrict__ max_rec /*null: a filter has run*/, int n_rec,
+            const uint32_t* __restrict__ surv, int k,
             ScanEntry* __restrict__ block_out /*[gridDim.x][k]*/, int out_capacity, int32_t* __restrict__ ids_out,
             double* __restrict__ dist_out) {
   __shared__ unsigned long long s_key[2 * kScanCap];
@@ -492,12 +582,29 @@ scan_select(const float4* __restrict__ poses, const int32_t* __restrict__ valid_
   TopK top;
   top.init(s_key, s_i, s_rank, &s_cnt, &s_tau, k);
   // what is walked: the survivor list, or -- if it overflowed -- every pose (entry e is then candidate e)
-  const bool listed = h->overflow == 0u;
+  const bool listed = max_rec == nullptr && h->overflow == 0u;
   const int64_t n = listed ? static_cast<int64_t>(h->n_surv) : n_all;
   const int32_t* valid = listed ? nullptr : valid_all;      // listed candidates have been checked already
   auto cand_of = [&](int64_t e) -> int32_t { return listed ? static_cast<int32_t>(__ldg(surv + e)) : static_cast<int32_t>(e); };
-  const double mt = __longlong_as_double(static_cast<long long>(h->t_max_bits));
-  const double mr = 2.0 * acos(fmin(1.0, __longlong_as_double(static_cast<long long>(h->dot_min_bits))));
+  double mt, md;
+  if (max_rec) {   // the records of scan_max, one per lane of every warp at a time
+    mt = 0.0;
+    md = 2.0;
+    for (int r = threadIdx.x & 31; r < n_rec; r += 32) {
+      const double2 v = __ldcg(reinterpret_cast<const double2*>(max_rec + r));
+      mt = fmax(mt, v.x);
+      md = fmin(md, v.y);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mt = fmax(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+      md = fmin(md, __shfl_xor_sync(0xffffffffu, md, o));
+    }
+  } else {
+    mt = __longlong_as_double(static_cast<long long>(h->t_max_bits));
+    md = __longlong_as_double(static_cast<long long>(h->dot_min_bits));
+  }
+  const double mr = 2.0 * acos(fmin(1.0, md));
   // Cheap lower bound of the distance, in fp32 from the fp32 inputs: acos(x) >= sqrt(2 (1 - x)) on [0, 1], so
   //   d >= t / mt + 2 sqrt(2 (1 - |dot|)) / mr.
   // Its rounding error is below 1e-6 relative once 4e-7 is taken off 1 - |dot| (the absolute error of the fp32 dot);
@@ -646,28 +753,38 @@ scan_select(const float4* __restrict__ poses, const int32_t* __restrict__ valid_
   if (k == 0) return;
   // A list that holds k entries proves that k candidates lie within its last distance: nothing beyond the smallest such
   // distance can be among the k best.  Every list is sorted, so what remains of it is a prefix.
-  // Likewise the k-th smallest of the lists' first entries: k candidates lie within it.  With candidates dealt to the
-  // blocks at random this is the sharper cut by far (it leaves little more than k entries).
+  // Likewise, at any depth d, the ceil(k / (d + 1))-th smallest of the lists' entries number d: that many lists have d + 1
+  // entries within it, k in all.  With candidates dealt to the blocks at random this is the sharper cut by far (it leaves
+  // little more than k entries); the depth is the smallest at which half of the lists are enough.
   unsigned long long* heads = reinterpret_cast<unsigned long long*>(s_pend);   // [n_lists] <= 1024 (s_pend is free by now)
+  // (any lists give a valid cut; the first 128 keep the counting short and still leave only a few k entries)
+  const int n_heads = n_lists < 128 ? n_lists : 128;
+  const int depth = 2 * k <= n_heads ? 0 : (2 * k + n_heads - 1) / n_heads - 1;
+  const int want = (k + depth) / (depth + 1);
   for (int l = tid; l < n_lists; l += blockDim.x) {
     const ScanEntry x = entry(l, k - 1);
+    const ScanEntry f = entry(l, depth < k ? depth : k - 1);
     if (x.i >= 0) atomicMin(&s_min, static_cast<unsigned long long>(__double_as_longlong(x.d)));
-    const ScanEntry f = entry(l, 0);
-    heads[l] = f.i >= 0 ? static_cast<unsigned long long>(__double_as_longlong(f.d)) : kInf;
+    if (l < n_heads) {
+      heads[l] = f.i >= 0 ? static_cast<unsigned long long>(__double_as_longlong(f.d)) : kInf;
+      s_rank[l] = 0;
+    }
   }
   __syncthreads();
-  // (any k lists give a valid cut; the first 128 keep the counting short and still leave only a few k entries)
-  const int n_heads = n_lists < 128 ? n_lists : 128;
-  if (n_heads >= k) {
-    for (int l = tid; l < n_heads; l += blockDim.x) {
+  if (n_heads >= want && depth < k) {
+    const int l = tid & 127, part = tid >> 7;   // four threads share a list's comparisons
+    if (l < n_heads) {
       const unsigned long long hl = heads[l];
       int rank = 0;
-      for (int u = 0; u < n_heads; ++u) {
+#pragma unroll 4
+      for (int u = part; u < n_heads; u += kSelThreads / 128) {
         const unsigned long long hu = heads[u];
-        rank += (hu < hl) || (hu == hl && u < l);
+        rank += static_cast<int>(hu < hl) | (static_cast<int>(hu == hl) & static_cast<int>(u < l));
       }
-      if (rank == k - 1 && hl != kInf) atomicMin(&s_min, hl);
+      if (rank) atomicAdd(&s_rank[l], rank);
     }
+    __syncthreads();
+    if (tid < n_heads && s_rank[tid] == want - 1 && heads[tid] != kInf) atomicMin(&s_min, heads[tid]);
   }
   __syncthreads();
   const unsigned long long cut = s_min;
@@ -784,13 +901,27 @@ wk_status launch_retrieve_scan(wk_ctx* ctx, const float* poses, const int32_t* v
   if (sel_blocks < 1) sel_blocks = 1;
   wk_status st;
   const float4* p4 = reinterpret_cast<const float4*>(poses);
-  scan_sample<<<sample_blocks, kSampleThreads, 0, s>>>(p4, valid, n, n_samples, cur, k, sc.h, sc.rec);
+  // Small arrays and short lists are walked twice (the second time from L2): two launches instead of three, and no sample
+  // whose latency the filter would have to wait for.  Two walks against three kernels, k = 16: 2^14 17.5 / 19.7 us, 2^16 20.1
+  // / 22.2, 2^17 22.8 / 23.9, 2^18 25.2 / 24.6; k = 64: 2^14 40 / 24 (every block has to find 64 of few candidates).
+  if (n <= kScanTwice && k <= 16) {
+    int64_t mb = (n + kMaxThreads * 2 - 1) / (kMaxThreads * 2);
+    if (mb > 2 * ctx->sm_count) mb = 2 * ctx->sm_count;
+    if (mb < 1) mb = 1;
+    MaxRecord* mrec = reinterpret_cast<MaxRecord*>(sc.rec);
+    launch_chained(scan_max, dim3(static_cast<unsigned>(mb)), dim3(kMaxThreads), 0, s, p4, valid, n, cur, sc.h, mrec, ctx->status_dev);
+    if ((st = after_launch(ctx)) != WK_OK) return st;
+    launch_chained(scan_select, dim3(static_cast<unsigned>(sel_blocks)), dim3(kSelThreads), 0, s, p4, valid, n, cur, sc.h, mrec,
+                   static_cast<int>(mb), sc.surv, k, sc.block_out, out_capacity, ids_out, dist_out);
+    return after_launch(ctx);
+  }
+  launch_chained(scan_sample, dim3(sample_blocks), dim3(kSampleThreads), 0, s, p4, valid, n, n_samples, cur, k, sc.h, sc.rec);
   if ((st = after_launch(ctx)) != WK_OK) return st;
   launch_chained(scan_filter, dim3(static_cast<unsigned>(blocks)), dim3(kScanThreads), 0, s, p4, valid, n, cur, k, sc.rec,
                  sample_blocks, sc.h, sc.surv, ctx->status_dev);
   if ((st = after_launch(ctx)) != WK_OK) return st;
-  launch_chained(scan_select, dim3(static_cast<unsigned>(sel_blocks)), dim3(kSelThreads), 0, s, p4, valid, n, cur, sc.h,
-                 sc.surv, k, sc.block_out, out_capacity, ids_out, dist_out);
+  launch_chained(scan_select, dim3(static_cast<unsigned>(sel_blocks)), dim3(kSelThreads), 0, s, p4, valid, n, cur, sc.h, nullptr,
+                 0, sc.surv, k, sc.block_out, out_capacity, ids_out, dist_out);
   return after_launch(ctx);
 }
 

@@ -148,3 +148,28 @@ def test_scan_many_equal_distances(kv):
     assert got.tolist() == list(range(first, first + 16))
     same = np.repeat(poses[0][None], 300000, axis=0)
     assert _check(kv, same, poses[0], 64, need_margin=False).tolist() == list(range(64))
+
+
+@pytest.mark.parametrize("n", [2047, 2048, 2049, 16384, (1 << 17) - 1, 1 << 17, (1 << 17) + 1])
+@pytest.mark.parametrize("k", [1, 16, 17, 64])
+def test_scan_on_both_sides_of_the_two_walk_rule(n, k):
+    """Arrays of up to 2^17 poses with k <= 16 are walked twice, others sampled and filtered; few lists with many wanted
+    entries make the merge look deeper into them.  Holes and repeated poses (ties by index) in all of them."""
+    from paper_2605_22718_b200 import WorldKV
+    kv = WorldKV(n_layers=1, n_heads=1, tokens_per_frame=8, n_keep=4, pool_slots=1, max_k=1)
+    poses = wi.random_poses(n % 1000 + k, n + 1)
+    cur = poses[n]
+    poses = poses[:n].copy()
+    poses[n // 2:n // 2 + 40] = poses[11]
+    valid = np.ones(n, dtype=np.int32)
+    valid[::5] = 0
+    for v in (None, valid):
+        dist = torch.empty(k, dtype=torch.float64, device="cuda")
+        ids = kv.retrieve_scan(torch.from_numpy(poses).cuda(), cur, k, valid=None if v is None else torch.from_numpy(v).cuda(),
+                               dist_out=dist)
+        assert kv.poll_status() == (0, 0)
+        ok = np.arange(n) if v is None else np.flatnonzero(v)
+        d = o.retrieval_distances(cur, poses[ok])
+        order = np.lexsort((ok, d))[:k]
+        np.testing.assert_array_equal(ids.cpu().numpy(), ok[order])
+        np.testing.assert_allclose(dist.cpu().numpy(), d[order], rtol=1e-12, atol=1e-14)
