@@ -249,10 +249,17 @@ wk_status wk_compress_chunk(wk_ctx* ctx, const void* K_chunks, int64_t batch_str
                          scores_out, static_cast<cudaStream_t>(stream));
 }
 
+static wk_status free_slot(wk_ctx* ctx, int slot) {
+  ctx->slots[slot].state = SLOT_FREE;
+  --ctx->n_valid;
+  ctx->slots[slot].tag = -1;
+  return WK_OK;
+}
+
 // Shared by wk_pool_append and wk_pool_compress_append: slot choice and bookkeeping around the gather kernel.
 static wk_status append_checked(wk_ctx* ctx, int32_t layer0, int32_t n, const void* K_chunks, const void* V_chunks,
                                 int64_t batch_stride_elems, const int32_t* keep_idx_dev, const float* pose_host,
-                                int64_t chunk_tag, int32_t* slot_io_host, cudaStream_t s, bool after_selection) {
+                                int64_t chunk_tag, int32_t* slot_io_host, cudaStream_t s, const AnchorStore* stored) {
   int slot = *slot_io_host;
   if (slot < 0) {
     if (slot != -1) return WK_ERR_BAD_SLOT;
@@ -267,9 +274,10 @@ static wk_status append_checked(wk_ctx* ctx, int32_t layer0, int32_t n, const vo
   for (int l = layer0; l < layer0 + n; ++l) {
     if (si.state == SLOT_OPEN && si.layer_mask[l]) return WK_ERR_BAD_SLOT;  // layer stored twice
   }
+  const bool last = (si.state == SLOT_FREE ? 0 : si.layers_done) + n == ctx->cfg.n_layers;   // the slot becomes visible
   wk_status st = launch_append(ctx, layer0, n, slot, static_cast<const __nv_bfloat16*>(K_chunks),
-                               static_cast<const __nv_bfloat16*>(V_chunks), batch_stride_elems, keep_idx_dev, s,
-                               after_selection);
+                               static_cast<const __nv_bfloat16*>(V_chunks), batch_stride_elems, keep_idx_dev, s, stored,
+                               last ? (si.state == SLOT_FREE ? pose_host : si.pose) : nullptr);
   if (st != WK_OK) return st;
   if (si.state == SLOT_FREE) {
     si.state = SLOT_OPEN;
@@ -280,9 +288,7 @@ static wk_status append_checked(wk_ctx* ctx, int32_t layer0, int32_t n, const vo
   }
   for (int l = layer0; l < layer0 + n; ++l) si.layer_mask[l] = 1;
   si.layers_done += n;
-  if (si.layers_done == ctx->cfg.n_layers) {
-    st = launch_slot_mark(ctx, slot, 1, si.pose, s);
-    if (st != WK_OK) return st;
+  if (last) {
     si.state = SLOT_VALID;
     ++ctx->n_valid;
     si.seq = ctx->next_seq++;
@@ -301,7 +307,7 @@ wk_status wk_pool_append(wk_ctx* ctx, int32_t layer0, int32_t n, const void* K_c
   if (layer0 < 0 || n < 1 || layer0 + n > ctx->cfg.n_layers) return WK_ERR_SHAPE;
   if (n > 1 && batch_stride_elems < static_cast<int64_t>(ctx->FT) * ctx->D) return WK_ERR_ARG;
   return append_checked(ctx, layer0, n, K_chunks, V_chunks, batch_stride_elems, keep_idx_dev, pose_host, chunk_tag,
-                        slot_io_host, static_cast<cudaStream_t>(stream), false);
+                        slot_io_host, static_cast<cudaStream_t>(stream), nullptr);
 }
 
 wk_status wk_pool_compress_append(wk_ctx* ctx, int32_t layer0, int32_t n, const void* K_chunks, const void* V_chunks,
@@ -329,16 +335,24 @@ wk_status wk_pool_compress_append(wk_ctx* ctx, int32_t layer0, int32_t n, const 
     if (!have_free) {
       const int victim = wk_pool_oldest(ctx);
       if (!evict_oldest_if_full || victim < 0) return WK_ERR_POOL_FULL;
-      wk_status st = wk_pool_evict(ctx, victim, stream);
+      // the chunk goes into the slot just freed; if this call stores all of its layers, the slot's own mark comes with them
+      wk_status st = n == ctx->cfg.n_layers ? free_slot(ctx, victim) : wk_pool_evict(ctx, victim, stream);
       if (st != WK_OK) return st;
       if (evicted_slot_host) *evicted_slot_host = victim;
     }
+    for (slot = 0; ctx->slots[slot].state != SLOT_FREE; ++slot) {}   // the slot append_checked will pick
   }
+  AnchorStore store{pool_rows(ctx, ctx->Kpool, layer0, slot), static_cast<const __nv_bfloat16*>(V_chunks),
+                    pool_rows(ctx, ctx->Vpool, layer0, slot),
+                    static_cast<int64_t>(ctx->C) * ctx->D * ctx->cfg.pool_slots, false, false};
   wk_status st = launch_compress(ctx, static_cast<const __nv_bfloat16*>(K_chunks), batch_stride_elems, n, keep_idx_dev,
-                                 nullptr, s);
-  if (st != WK_OK) return st;
+                                 nullptr, s, &store);
+  if (st != WK_OK) {   // the freed slot's mark is still up
+    if (*slot_io_host < 0) launch_slot_mark(ctx, slot, 0, ctx->slots[slot].pose, s);
+    return st;
+  }
   return append_checked(ctx, layer0, n, K_chunks, V_chunks, batch_stride_elems, keep_idx_dev, pose_host, chunk_tag,
-                        slot_io_host, s, true);
+                        slot_io_host, s, &store);
 }
 
 size_t wk_host_chunk_bytes(const wk_ctx* ctx) {
@@ -420,10 +434,7 @@ wk_status wk_pool_evict(wk_ctx* ctx, int32_t slot, void* stream) {
   if (slot < 0 || slot >= ctx->cfg.pool_slots || ctx->slots[slot].state != SLOT_VALID) return WK_ERR_BAD_SLOT;
   wk_status st = launch_slot_mark(ctx, slot, 0, ctx->slots[slot].pose, static_cast<cudaStream_t>(stream));
   if (st != WK_OK) return st;
-  ctx->slots[slot].state = SLOT_FREE;
-  --ctx->n_valid;
-  ctx->slots[slot].tag = -1;
-  return WK_OK;
+  return free_slot(ctx, slot);
 }
 
 int32_t wk_pool_oldest(const wk_ctx* ctx) {

@@ -30,6 +30,11 @@ namespace {
 
 constexpr int kMaxNormParts = 32;     // pitch of the per-problem |m|^2 record in scratch (one share is used)
 constexpr int kScoreThreads = 256;
+constexpr int kCopyRows = 16;         // rows per piece of the V copy that rides along with the scoring
+struct FusedQueue {
+  uint32_t a_next, s_next, exited;   // compress_fused
+  uint32_t copy_next;                // pieces of V's anchor frames handed out by score_select; reset by anchor_rows
+};
 
 __device__ __forceinline__ double bf16_to_f64(uint32_t bits16) {
   return static_cast<double>(__uint_as_float(bits16 << 16));
@@ -272,7 +277,8 @@ __device__ __forceinline__ void anchor_role(uint8_t* smem, int b, int part, int 
                                             double* __restrict__ partial, int max_parts, uint32_t* __restrict__ tickets,
                                             double* __restrict__ m64, float* __restrict__ m32, double* __restrict__ mnorm2,
                                             uint32_t* __restrict__ status, uint32_t* ready, uint32_t epoch,
-                                            uint64_t* bar, uint32_t& gbase) {
+                                            uint64_t* bar, uint32_t& gbase, __nv_bfloat16* __restrict__ kdst) {
+  // kdst (may be null): where the chunk's anchor rows are to be stored; they go there from the staging buffer
   // bar[2]: the caller's two mbarriers (initialised once per CTA, count 1); gbase: bulk copies this CTA has waited for so
   // far -- copy number n lands in buffer n & 1 and completes phase n >> 1 of barrier n & 1
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -304,7 +310,10 @@ __device__ __forceinline__ void anchor_role(uint8_t* smem, int b, int part, int 
   int g = 0;
   for (; g < n_groups; ++g) {
     if (g + 1 < n_groups) {
-      if (tid == 0) issue(g + 1);     // its buffer was released by the barrier that ended group g - 1
+      if (tid == 0) {
+        if (kdst) ptx::bulk_store_wait_read();   // group g - 1 has left the buffer for the pool
+        issue(g + 1);     // its buffer was released by the barrier that ended group g - 1
+      }
       armed = g + 2;
     }
     const uint32_t n_cur = gbase + g;
@@ -315,6 +324,8 @@ __device__ __forceinline__ void anchor_role(uint8_t* smem, int b, int part, int 
     }
     const int rows = min(G, r1 - (r0 + g * G));
     const uint8_t* buf = rows_s + (n_cur & 1) * G * row_bytes;
+    if (kdst && tid == 0)
+      ptx::bulk_store_1d(kdst + static_cast<int64_t>(r0 + g * G) * D, buf, static_cast<uint32_t>(rows * row_bytes));
     // ---- phase 1: norms (integer-pipe conversions; redone exactly when a norm falls outside the safe range)
     group_norms<false>(buf, row_bytes, rows, nseg, seg_vecs, vecs, n2_s);
     bool redo = false;
@@ -357,6 +368,7 @@ __device__ __forceinline__ void anchor_role(uint8_t* smem, int b, int part, int 
       for (uint32_t i = 0; i < (1u << 16); ++i)
         if (ptx::mbar_try_wait(&bar[(gbase + gg) & 1], ((gbase + gg) >> 1) & 1)) break;
   }
+  if (kdst && tid == 0) ptx::bulk_store_wait_done();   // also before the buffers serve other work
   gbase += static_cast<uint32_t>(armed);   // every issued copy has been waited for (or given up on) by now
   __syncthreads();
   // ---- this CTA's slice
@@ -476,16 +488,20 @@ __device__ __forceinline__ void row_inverse_norms(const double (&p)[VPL], int hs
   }
 }
 
-template <int VPL, int NW>
+template <int VPL, int NW, bool kStore>
 __global__ void __launch_bounds__(NW * 32, 1)
 anchor_rows(const __nv_bfloat16* __restrict__ K, int64_t stride, int chunks, int T, int D, int hs, int wpr, int R,
             double* __restrict__ partial, int max_parts, uint32_t* __restrict__ tickets, double* __restrict__ m64,
-            float* __restrict__ m32, double* __restrict__ mnorm2) {
+            float* __restrict__ m32, double* __restrict__ mnorm2, __nv_bfloat16* __restrict__ kdst, int64_t kdst_stride,
+            uint32_t* __restrict__ copy_queue) {
+  // kStore: chunk b's row r is also stored at kdst + b * kdst_stride + r * D, from the registers it is in; the
+  // kernel is bound by the conversions, so the writes ride along
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(16) double n2x[2 * NW];
   double* sacc = reinterpret_cast<double*>(smem);   // [n_sets][D]
   dep_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (kStore && blockIdx.x == 0 && tid == 0) *copy_queue = 0u;
   const int n_sets = NW / wpr, set = warp / wpr, wr = warp - set * wpr;
   const int vecs = D >> 3, vstep = 32 * wpr, v0 = wr * 32 + lane;
   uint32_t active = 0;
@@ -522,6 +538,12 @@ anchor_rows(const __nv_bfloat16* __restrict__ K, int64_t stride, int chunks, int
     load_row(r, q);
     for (; r < r1; r += n_sets) {
       double x[8 * VPL], p[VPL], inv[VPL];
+      if (kStore) {
+        uint4* drow = reinterpret_cast<uint4*>(kdst + static_cast<int64_t>(b) * kdst_stride) + static_cast<int64_t>(r) * vecs;
+#pragma unroll
+        for (int i = 0; i < VPL; ++i)
+          if ((active >> i) & 1u) __stcs(drow + voff[i], q[i]);
+      }
       row_convert<VPL>(q, active, x, p);
       load_row(r + n_sets, q);   // the next row's loads fly while this one is finished
       row_inverse_norms<VPL, NW>(p, hs, wpr, set, wr, n2x, xc, inv);
@@ -934,16 +956,46 @@ __device__ __forceinline__ bool score_role(uint8_t* smem, int b, int blk, const 
   return false;
 }
 
-__global__ void __launch_bounds__(kScoreThreads)
+__global__ void __launch_bounds__(kScoreThreads, 4)   // 64 registers: the grid is sized for four CTAs per SM
 score_select(const __nv_bfloat16* __restrict__ K, int64_t stride, int T, int NA, int D, int n_keep, int nblk,
              const float* __restrict__ m32, const double* __restrict__ m64, const double* __restrict__ mnorm,
              float* __restrict__ s32, float* __restrict__ scores_out, uint32_t* __restrict__ tickets,
-             int32_t* __restrict__ keep_idx, uint32_t* __restrict__ status) {
+             int32_t* __restrict__ keep_idx, uint32_t* __restrict__ status, const __nv_bfloat16* __restrict__ vsrc,
+             __nv_bfloat16* __restrict__ vdst, int64_t dst_stride, uint32_t* __restrict__ copy_queue) {
   extern __shared__ __align__(16) uint8_t smem[];
   dep_wait();
   dep_release();
-  score_role(smem, blockIdx.x / nblk, blockIdx.x % nblk, K, stride, T, NA, D, n_keep, nblk, m32, m64, mnorm, s32, scores_out,
-             tickets, keep_idx, status);
+  const int b = blockIdx.x / nblk, blk = blockIdx.x % nblk;
+  score_role(smem, b, blk, K, stride, T, NA, D, n_keep, nblk, m32, m64, mnorm, s32, scores_out, tickets, keep_idx, status);
+  if (vsrc == nullptr) return;
+  // The call also stores the chunk: V's anchor frame needs no selection, so the CTAs copy it, kCopyRows rows at a time from
+  // a common queue, once their own rows are scored; the selections (one CTA per chunk, ~10 us in which the memory would
+  // idle) run under the copies of the others.  (Copied by the next kernel's first blocks instead, as soon as CTAs left, the
+  // copies starved the scoring CTAs that were still streaming: 55 us to the last of them instead of 30; with equal shares
+  // instead of a queue the selecting CTAs came last: 139 instead of 131 us for the whole call of 30 problems.)
+  __shared__ uint32_t s_piece;
+  const int vecs = D >> 3;
+  const uint32_t per = static_cast<uint32_t>((T + kCopyRows - 1) / kCopyRows), pieces = per * (gridDim.x / nblk);
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_piece = atomicAdd(copy_queue, 1u);
+    __syncthreads();
+    const uint32_t piece = s_piece;
+    if (piece >= pieces) break;
+    const uint32_t c = piece / per;
+    const int r0 = static_cast<int>(piece - c * per) * kCopyRows, total = min(kCopyRows, T - r0) * vecs;
+    const uint4* src = reinterpret_cast<const uint4*>(vsrc + static_cast<int64_t>(c) * stride) + static_cast<int64_t>(r0) * vecs;
+    uint4* dst = reinterpret_cast<uint4*>(vdst + static_cast<int64_t>(c) * dst_stride) + static_cast<int64_t>(r0) * vecs;
+    for (int v0 = threadIdx.x; v0 < total; v0 += 4 * kScoreThreads) {
+      uint4 q[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (v0 + u * kScoreThreads < total) q[u] = __ldcs(src + v0 + u * kScoreThreads);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (v0 + u * kScoreThreads < total) __stcs(dst + v0 + u * kScoreThreads, q[u]);
+    }
+  }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -957,9 +1009,6 @@ score_select(const __nv_bfloat16* __restrict__ K, int64_t stride, int T, int NA,
 // run on every SM; nobody waits while there is work of either kind.  The only wait left: a CTA that has taken a score item
 // of a chunk that is not ready yet (the head moved on between its look and its take) -- bounded, status WK_DEV_TIMEOUT.
 // ------------------------------------------------------------------------------------------------
-struct FusedQueue {
-  uint32_t a_next, s_next, exited, pad;
-};
 
 template <int VPT>
 __global__ void __launch_bounds__(kAnchorThreads, VPT == 1 ? 4 : (VPT == 2 ? 3 : 2))
@@ -968,7 +1017,7 @@ compress_fused(const __nv_bfloat16* __restrict__ K, int64_t stride, int chunks, 
                uint32_t* __restrict__ tickets_a, uint32_t* __restrict__ tickets_s, uint32_t* ready, FusedQueue* q,
                uint32_t epoch, double* __restrict__ m64, float* __restrict__ m32, double* __restrict__ mnorm,
                float* __restrict__ s32, float* __restrict__ scores_out, int32_t* __restrict__ keep_idx,
-               uint32_t* __restrict__ status) {
+               uint32_t* __restrict__ status, __nv_bfloat16* __restrict__ kdst, int64_t kdst_stride) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) uint64_t bar[2];
   __shared__ int s_kind, s_item;
@@ -1026,7 +1075,8 @@ compress_fused(const __nv_bfloat16* __restrict__ K, int64_t stride, int chunks, 
     if (kind == 0) {
       staged_chunk = -1;
       anchor_role<VPT>(smem, item / parts, item % parts, parts, K, stride, T, D, G, rpp, partial, max_parts, tickets_a,
-                       m64, m32, mnorm, status, ready, epoch, bar, gbase);
+                       m64, m32, mnorm, status, ready, epoch, bar, gbase,
+                       kdst ? kdst + (item / parts) * kdst_stride : nullptr);
     } else if (kind == 1) {
       const int c = item / nblk;
       const bool kept = score_role(smem, c, item % nblk, K, stride, T, NA, D, n_keep, nblk, m32, m64, mnorm, s32,
@@ -1152,29 +1202,32 @@ namespace {
 template <int VPL, int NW>
 void launch_rows(dim3 grid, size_t smem, cudaStream_t s, const __nv_bfloat16* K, int64_t stride, int chunks, int T, int D,
                  int hs, int wpr, int R, double* partial, int max_parts, uint32_t* tickets, double* m64, float* m32,
-                 double* mnorm) {
+                 double* mnorm, const AnchorStore* store, uint32_t* copy_queue) {
+  auto* kernel = store ? anchor_rows<VPL, NW, true> : anchor_rows<VPL, NW, false>;
   if (smem > 40 * 1024)   // the kernel's static shared memory comes on top
-    cudaFuncSetAttribute(anchor_rows<VPL, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  anchor_rows<VPL, NW><<<grid, NW * 32, smem, s>>>(K, stride, chunks, T, D, hs, wpr, R, partial, max_parts, tickets, m64, m32,
-                                                   mnorm);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  kernel<<<grid, NW * 32, smem, s>>>(K, stride, chunks, T, D, hs, wpr, R, partial, max_parts, tickets, m64, m32, mnorm,
+                                     store ? store->Kdst : nullptr, store ? store->dst_stride : 0, copy_queue);
 }
 
 template <int VPT>
 void launch_fused(unsigned grid, size_t smem, cudaStream_t s, const __nv_bfloat16* K, int64_t stride, int chunks, int T, int NA,
                   int D, int n_keep, int G, int rpp, int parts, int nblk, int layer_ctas, double* partial, int max_parts,
                   uint32_t* tickets_a, uint32_t* tickets_s, uint32_t* ready, FusedQueue* q, uint32_t epoch, double* m64,
-                  float* m32, double* mnorm, float* s32, float* scores_out, int32_t* keep_idx, uint32_t* status) {
+                  float* m32, double* mnorm, float* s32, float* scores_out, int32_t* keep_idx, uint32_t* status,
+                  const AnchorStore* store) {
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(compress_fused<VPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   compress_fused<VPT><<<grid, kAnchorThreads, smem, s>>>(K, stride, chunks, T, NA, D, n_keep, G, rpp, parts, nblk, layer_ctas,
                                                          partial, max_parts, tickets_a, tickets_s, ready, q, epoch, m64, m32,
-                                                         mnorm, s32, scores_out, keep_idx, status);
+                                                         mnorm, s32, scores_out, keep_idx, status, store ? store->Kdst : nullptr,
+                                                         store ? store->dst_stride : 0);
 }
 
 }  // namespace
 
 wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, int chunks, int32_t* keep_idx,
-                          float* scores_out, cudaStream_t s) {
+                          float* scores_out, cudaStream_t s, AnchorStore* store) {
   const int T = ctx->cfg.tokens_per_frame, NA = ctx->NA, n_keep = ctx->cfg.n_keep;
   // whole-token keys: one problem per chunk, D columns; per-head keys: n_heads problems per chunk, 128 columns each.
   // The streaming kernels walk whole rows either way (DF columns); only the selection sees (chunk, head) problems.
@@ -1229,7 +1282,8 @@ wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, i
       uint32_t* ready = tickets + 2 * ctx->max_batch;
       FusedQueue* q = reinterpret_cast<FusedQueue*>(tickets + 3 * ctx->max_batch);
       const uint32_t epoch = ++ctx->compress_epoch;
-#define WK_FUSED(V) launch_fused<V>(grid_f, smem_f, s, K, stride, chunks, T, NA, DF, n_keep, G, rpp, parts, nblk, ctx->sm_count, partial, max_parts, tickets, tickets + ctx->max_batch, ready, q, epoch, m64, m32, mnorm, s32, scores_out, keep_idx, ctx->status_dev)
+#define WK_FUSED(V) launch_fused<V>(grid_f, smem_f, s, K, stride, chunks, T, NA, DF, n_keep, G, rpp, parts, nblk, ctx->sm_count, partial, max_parts, tickets, tickets + ctx->max_batch, ready, q, epoch, m64, m32, mnorm, s32, scores_out, keep_idx, ctx->status_dev, store)
+      if (store) store->k_done = true;
       if (vpt <= 1) WK_FUSED(1);
       else if (vpt == 2) WK_FUSED(2);
       else if (vpt == 3) WK_FUSED(3);
@@ -1254,7 +1308,8 @@ wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, i
       const int64_t r_min = (T + max_parts - 2) / (max_parts - 1);
       if (R < r_min) R = r_min;
       const dim3 grid(static_cast<unsigned>((total + R - 1) / R));
-#define WK_ROWS(V, W) launch_rows<V, W>(grid, smem_r, s, K, stride, chunks, T, DF, hs, wpr, static_cast<int>(R), partial, max_parts, tickets, m64, m32, mnorm)
+#define WK_ROWS(V, W) launch_rows<V, W>(grid, smem_r, s, K, stride, chunks, T, DF, hs, wpr, static_cast<int>(R), partial, max_parts, tickets, m64, m32, mnorm, store, &reinterpret_cast<FusedQueue*>(tickets + 3 * ctx->max_batch)->copy_next)
+      if (store) store->k_done = true;
       if (per_head) {
         switch (vpl) {
           case 1: WK_ROWS(1, kRowWarpsHead); break;
@@ -1306,7 +1361,10 @@ wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, i
         WK_CUDA_TRY(ctx, cudaFuncSetAttribute(score_select, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_s)));
       launch_chained(score_select, dim3(static_cast<unsigned>(nblk) * chunks), dim3(kScoreThreads), smem_s, s, K, stride, T, NA,
                      DF, n_keep, nblk, m32, m64, mnorm, s32, scores_out, tickets + ctx->max_batch,
-                     select_here ? keep_idx : static_cast<int32_t*>(nullptr), ctx->status_dev);
+                     select_here ? keep_idx : static_cast<int32_t*>(nullptr), ctx->status_dev,
+                     store ? store->Vsrc : nullptr, store ? store->Vdst : nullptr, store ? store->dst_stride : 0,
+                     &reinterpret_cast<FusedQueue*>(tickets + 3 * ctx->max_batch)->copy_next);
+      if (store) store->v_done = true;
       if ((st = after_launch(ctx)) != WK_OK) return st;
       if (select_here) return WK_OK;
     }

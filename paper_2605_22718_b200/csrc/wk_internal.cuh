@@ -116,12 +116,25 @@ const CUtensorMap* cached_rows_map(wk_ctx* ctx, const void* base, int32_t rows, 
 int attention_partial_slots(int n_heads, int max_lq, int max_splits);
 
 // Kernel launchers (one per translation unit).
+// Where the scoring kernels may store the anchor frame on their way: chunk b's row i of K (V) goes to Kdst (Vdst) +
+// b * dst_stride + i * D; V's chunks are as far apart as K's.  k_done / v_done tell what they did (calls that need no
+// scores have no such kernels).
+struct AnchorStore {
+  __nv_bfloat16* Kdst;
+  const __nv_bfloat16* Vsrc;
+  __nv_bfloat16* Vdst;
+  int64_t dst_stride;
+  bool k_done, v_done;
+};
 wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, int batch, int32_t* keep_idx,
-                          float* scores_out, cudaStream_t s);
-// after_selection: the launch is chained to the selection kernel that writes keep_idx (same stream, issued just before)
-// and walks the layers last to first.
+                          float* scores_out, cudaStream_t s, AnchorStore* store = nullptr);
+// stored: null for any index list; else what launch_compress, issued just before on the same stream, has stored already.  The
+// launch is then chained to the selection that writes keep_idx, whose first T rows are the anchor frame, and walks the
+// layers last to first.
+// mark_pose: non-null marks the slot valid with that pose (its last layers are in this call).
 wk_status launch_append(wk_ctx* ctx, int layer0, int n, int slot, const __nv_bfloat16* K, const __nv_bfloat16* V,
-                        int64_t stride, const int32_t* keep_idx, cudaStream_t s, bool after_selection = false);
+                        int64_t stride, const int32_t* keep_idx, cudaStream_t s, const AnchorStore* stored, const float* mark_pose);
+__nv_bfloat16* pool_rows(wk_ctx* ctx, __nv_bfloat16* base, int layer, int slot);   // first stored row of (layer, slot)
 wk_status launch_slot_mark(wk_ctx* ctx, int slot, int valid, const float* pose, cudaStream_t s);
 wk_status launch_retrieve(wk_ctx* ctx, const float* cur_pose, int k, int32_t* slots_out, double* dist_out, cudaStream_t s);
 // Kernels of one call that depend on each other in a chain are launched so that a kernel may be scheduled while its

@@ -7,26 +7,78 @@ namespace {
 
 constexpr int kAppendThreads = 256;
 
-// grid = (ceil(C / rows_per_cta), n_layers_in_call, 2 [K|V]); one warp per kept row, 16-byte vectors.  With per-head
-// keep-sets (hs = n_heads index lists per layer) every 128-column block of a stored row has its own source token.
+constexpr int kAppendRows = 32;   // stored rows per block
+
+struct Pose8 { float v[8]; };
+
+struct AppendParams {
+  const __nv_bfloat16 *Ksrc, *Vsrc;
+  int64_t stride;               // elements between layers of the source chunk
+  const int32_t* keep_idx;
+  int hs, T, C, FT, D, n;       // index lists per layer, anchor rows, stored rows, chunk rows, row width, layers
+  __nv_bfloat16 *Kdst, *Vdst;
+  int64_t dst_layer_stride;
+  int k_row0, v_row0;           // first row of K / V that the index list is needed for (0 or T)
+  int v_anchor_blocks;          // blocks that copy V's anchor frame: they come first and do not wait for the selection
+  int reverse;
+  int mark_slot;                // >= 0: mark this slot valid
+  int32_t* valid;
+  float* poses;
+  Pose8 pose;
+  uint32_t* status;
+};
+
+// Bound by memory (5.6-6.5 TB/s of reads and writes).  One warp per stored row, 16-byte vectors, four loads in flight per
+// lane before the first store.  With per-head keep-sets (hs = n_heads index lists per layer) every 128-column block of a
+// stored row has its own source token.  Behind a selection, the anchor frame needs no index list: the scoring kernels have
+// stored its K rows and, at widths up to 2,048 columns, its V rows; where they have not, V's are copied by the first blocks,
+// which do not wait for the selection.
 __global__ void __launch_bounds__(kAppendThreads)
-append_rows(const __nv_bfloat16* __restrict__ Ksrc, const __nv_bfloat16* __restrict__ Vsrc, int64_t stride,
-            const int32_t* __restrict__ keep_idx, int hs, int C, int FT, int D, __nv_bfloat16* __restrict__ Kdst,
-            __nv_bfloat16* __restrict__ Vdst, int64_t dst_layer_stride, int rows_per_cta, int reverse,
-            uint32_t* __restrict__ status) {
+append_rows(const __grid_constant__ AppendParams p) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int vecs = p.D >> 3;
+  int id = blockIdx.x;
+  // Marking here is safe: a kernel behind this one on the stream sees the slot only once all of this one's rows are stored.
+  if (id == 0 && p.mark_slot >= 0) {
+    if (threadIdx.x < 8) p.poses[p.mark_slot * 8 + threadIdx.x] = p.pose.v[threadIdx.x];
+    if (threadIdx.x == 0) p.valid[p.mark_slot] = 1;
+  }
+  if (id < p.v_anchor_blocks) {
+    // (every earlier kernel on the stream but the selection has finished: the scoring kernel lets this one start only
+    // after it has waited for them itself)
+    const int per = (p.T + kAppendRows - 1) / kAppendRows;
+    const int l = id / per, r0 = (id - l * per) * kAppendRows, rows = min(kAppendRows, p.T - r0);
+    const uint4* src = reinterpret_cast<const uint4*>(p.Vsrc + static_cast<int64_t>(l) * p.stride) + static_cast<int64_t>(r0) * vecs;
+    uint4* dst = reinterpret_cast<uint4*>(p.Vdst + static_cast<int64_t>(l) * p.dst_layer_stride) + static_cast<int64_t>(r0) * vecs;
+    const int total = rows * vecs;   // the rows are contiguous on both sides
+    for (int v0 = threadIdx.x; v0 < total; v0 += 4 * kAppendThreads) {
+      uint4 q[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (v0 + u * kAppendThreads < total) q[u] = __ldcs(src + v0 + u * kAppendThreads);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (v0 + u * kAppendThreads < total) dst[v0 + u * kAppendThreads] = q[u];
+    }
+    return;
+  }
   dep_wait();   // returns at once unless the launch was chained to the selection that writes keep_idx
+  id -= p.v_anchor_blocks;
+  const int per_k = (p.C - p.k_row0 + kAppendRows - 1) / kAppendRows, per_v = (p.C - p.v_row0 + kAppendRows - 1) / kAppendRows;
   // reverse: walk the layers last to first, so that the layers whose keys the scoring pass touched last (and L2 still
   // holds) are gathered first
-  const int l = reverse ? static_cast<int>(gridDim.y) - 1 - static_cast<int>(blockIdx.y) : static_cast<int>(blockIdx.y);
-  const int which = blockIdx.z, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const __nv_bfloat16* src = (which ? Vsrc : Ksrc) + static_cast<int64_t>(l) * stride;
-  __nv_bfloat16* dst = (which ? Vdst : Kdst) + static_cast<int64_t>(l) * dst_layer_stride;
-  const int32_t* idx = keep_idx + static_cast<int64_t>(l) * hs * C;
-  const int vecs = D >> 3, vecs_per_list = vecs / hs;
-  const int r0 = blockIdx.x * rows_per_cta, r1 = min(C, r0 + rows_per_cta);
+  const int lb = id / (per_k + per_v);
+  const int l = p.reverse ? p.n - 1 - lb : lb;
+  int blk = id - lb * (per_k + per_v);
+  const bool is_v = blk >= per_k;
+  if (is_v) blk -= per_k;
+  const __nv_bfloat16* src = (is_v ? p.Vsrc : p.Ksrc) + static_cast<int64_t>(l) * p.stride;
+  __nv_bfloat16* dst = (is_v ? p.Vdst : p.Kdst) + static_cast<int64_t>(l) * p.dst_layer_stride;
+  const int32_t* idx = p.keep_idx + static_cast<int64_t>(l) * p.hs * p.C;
+  const int vecs_per_list = vecs / p.hs;
+  const int r0 = (is_v ? p.v_row0 : p.k_row0) + blk * kAppendRows, r1 = min(p.C, r0 + kAppendRows);
   for (int r = r0 + warp; r < r1; r += kAppendThreads / 32) {
-    uint4* d = reinterpret_cast<uint4*>(dst + static_cast<int64_t>(r) * D);
-    // four 16-byte loads of the row in flight per lane before the first store
+    uint4* d = reinterpret_cast<uint4*>(dst + static_cast<int64_t>(r) * p.D);
     for (int v0 = lane; v0 < vecs; v0 += 128) {
       uint4 q[4];
       bool ok[4];
@@ -35,12 +87,12 @@ append_rows(const __nv_bfloat16* __restrict__ Ksrc, const __nv_bfloat16* __restr
         const int v = v0 + 32 * u;
         ok[u] = v < vecs;
         if (ok[u]) {
-          const int j = idx[(v / vecs_per_list) * C + r];
-          if (j < 0 || j >= FT) {                   // never dereference a bad index
-            atomicOr(status, WK_DEV_BAD_SLOT);
+          const int j = idx[(v / vecs_per_list) * p.C + r];
+          if (j < 0 || j >= p.FT) {                   // never dereference a bad index
+            atomicOr(p.status, WK_DEV_BAD_SLOT);
             ok[u] = false;
           } else {
-            q[u] = __ldg(reinterpret_cast<const uint4*>(src + static_cast<int64_t>(j) * D) + v);
+            q[u] = __ldg(reinterpret_cast<const uint4*>(src + static_cast<int64_t>(j) * p.D) + v);
           }
         }
       }
@@ -51,8 +103,6 @@ append_rows(const __nv_bfloat16* __restrict__ Ksrc, const __nv_bfloat16* __restr
   }
 }
 
-struct Pose8 { float v[8]; };
-
 __global__ void slot_mark(int32_t* __restrict__ valid, float* __restrict__ poses, int slot, int is_valid, Pose8 pose) {
   if (threadIdx.x < 8) poses[slot * 8 + threadIdx.x] = pose.v[threadIdx.x];
   if (threadIdx.x == 0) valid[slot] = is_valid;
@@ -60,22 +110,40 @@ __global__ void slot_mark(int32_t* __restrict__ valid, float* __restrict__ poses
 
 }  // namespace
 
+__nv_bfloat16* pool_rows(wk_ctx* ctx, __nv_bfloat16* base, int layer, int slot) {
+  return base + (static_cast<int64_t>(layer) * ctx->cfg.pool_slots + slot) * ctx->C * ctx->D;
+}
+
 wk_status launch_append(wk_ctx* ctx, int layer0, int n, int slot, const __nv_bfloat16* K, const __nv_bfloat16* V,
-                        int64_t stride, const int32_t* keep_idx, cudaStream_t s, bool after_selection) {
-  const int C = ctx->C, D = ctx->D;
-  const int64_t slot_elems = static_cast<int64_t>(C) * D;
-  const int64_t layer_stride = slot_elems * ctx->cfg.pool_slots;
-  __nv_bfloat16* Kdst = ctx->Kpool + layer0 * layer_stride + slot * slot_elems;
-  __nv_bfloat16* Vdst = ctx->Vpool + layer0 * layer_stride + slot * slot_elems;
-  const int rows_per_cta = 32;
-  const dim3 grid((C + rows_per_cta - 1) / rows_per_cta, n, 2);
-  const int hs = ctx->cfg.score_mode == WK_SCORE_PER_HEAD ? ctx->cfg.n_heads : 1;
-  if (after_selection)
-    launch_chained(append_rows, grid, dim3(kAppendThreads), 0, s, K, V, stride, keep_idx, hs, C, ctx->FT, D, Kdst, Vdst,
-                   layer_stride, rows_per_cta, 1, ctx->status_dev);
-  else
-    append_rows<<<grid, kAppendThreads, 0, s>>>(K, V, stride, keep_idx, hs, C, ctx->FT, D, Kdst, Vdst, layer_stride,
-                                                rows_per_cta, 0, ctx->status_dev);
+                        int64_t stride, const int32_t* keep_idx, cudaStream_t s, const AnchorStore* stored, const float* mark_pose) {
+  const int T = ctx->cfg.tokens_per_frame, C = ctx->C;
+  AppendParams p;
+  p.Ksrc = K;
+  p.Vsrc = V;
+  p.stride = stride;
+  p.keep_idx = keep_idx;
+  p.hs = ctx->cfg.score_mode == WK_SCORE_PER_HEAD ? ctx->cfg.n_heads : 1;
+  p.T = T;
+  p.C = C;
+  p.FT = ctx->FT;
+  p.D = ctx->D;
+  p.n = n;
+  p.Kdst = pool_rows(ctx, ctx->Kpool, layer0, slot);
+  p.Vdst = pool_rows(ctx, ctx->Vpool, layer0, slot);
+  p.dst_layer_stride = static_cast<int64_t>(C) * ctx->D * ctx->cfg.pool_slots;
+  p.k_row0 = stored && stored->k_done ? T : 0;
+  p.v_row0 = stored ? T : 0;
+  p.v_anchor_blocks = stored && !stored->v_done ? n * ((T + kAppendRows - 1) / kAppendRows) : 0;
+  p.reverse = stored != nullptr;
+  p.mark_slot = mark_pose ? slot : -1;
+  p.valid = ctx->valid_dev;
+  p.poses = ctx->poses_dev;
+  for (int i = 0; i < 8; ++i) p.pose.v[i] = mark_pose ? mark_pose[i] : 0.f;
+  p.status = ctx->status_dev;
+  const int per_k = (C - p.k_row0 + kAppendRows - 1) / kAppendRows, per_v = (C - p.v_row0 + kAppendRows - 1) / kAppendRows;
+  const dim3 grid(static_cast<unsigned>(p.v_anchor_blocks + n * (per_k + per_v)));
+  if (stored) launch_chained(append_rows, grid, dim3(kAppendThreads), 0, s, p);
+  else append_rows<<<grid, kAppendThreads, 0, s>>>(p);
   return after_launch(ctx);
 }
 
