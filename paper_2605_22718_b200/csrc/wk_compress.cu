@@ -29,6 +29,8 @@ namespace wk {
 namespace {
 
 constexpr int kMaxNormParts = 32;     // pitch of the per-problem |m|^2 record in scratch (one share is used)
+// Dynamic shared memory from which a kernel asks for more than the default 48 KB: its static arrays come on top.
+constexpr size_t kSmemOptIn = 40 * 1024;
 constexpr int kScoreThreads = 256;
 constexpr int kCopyRows = 16;         // rows per piece of the V copy that rides along with the scoring
 struct FusedQueue {
@@ -1204,7 +1206,7 @@ void launch_rows(dim3 grid, size_t smem, cudaStream_t s, const __nv_bfloat16* K,
                  int hs, int wpr, int R, double* partial, int max_parts, uint32_t* tickets, double* m64, float* m32,
                  double* mnorm, const AnchorStore* store, uint32_t* copy_queue) {
   auto* kernel = store ? anchor_rows<VPL, NW, true> : anchor_rows<VPL, NW, false>;
-  if (smem > 40 * 1024)   // the kernel's static shared memory comes on top
+  if (smem > kSmemOptIn)
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   kernel<<<grid, NW * 32, smem, s>>>(K, stride, chunks, T, D, hs, wpr, R, partial, max_parts, tickets, m64, m32, mnorm,
                                      store ? store->Kdst : nullptr, store ? store->dst_stride : 0, copy_queue);
@@ -1216,7 +1218,7 @@ void launch_fused(unsigned grid, size_t smem, cudaStream_t s, const __nv_bfloat1
                   uint32_t* tickets_a, uint32_t* tickets_s, uint32_t* ready, FusedQueue* q, uint32_t epoch, double* m64,
                   float* m32, double* mnorm, float* s32, float* scores_out, int32_t* keep_idx, uint32_t* status,
                   const AnchorStore* store) {
-  if (smem > 48 * 1024)
+  if (smem > kSmemOptIn)
     cudaFuncSetAttribute(compress_fused<VPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   compress_fused<VPT><<<grid, kAnchorThreads, smem, s>>>(K, stride, chunks, T, NA, D, n_keep, G, rpp, parts, nblk, layer_ctas,
                                                          partial, max_parts, tickets_a, tickets_s, ready, q, epoch, m64, m32,
@@ -1349,7 +1351,7 @@ wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, i
     }
     const int nblk = (NA + srows - 1) / srows;
     if (per_head) {
-      if (smem_m > 48 * 1024)
+      if (smem_m > kSmemOptIn)
         WK_CUDA_TRY(ctx, cudaFuncSetAttribute(head_score, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_m)));
       launch_chained(head_score, dim3(nblk, chunks), dim3(kScoreThreads), smem_m, s, K, stride, T, NA, DF, H, m32, s32,
                      scores_out, ctx->status_dev);
@@ -1357,7 +1359,7 @@ wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, i
     } else {
       const bool select_here = n_keep > 0 && n_keep < NA;
       const size_t smem_s = select_here && smem_sel > smem_m ? smem_sel : smem_m;
-      if (smem_s > 48 * 1024)
+      if (smem_s > kSmemOptIn)
         WK_CUDA_TRY(ctx, cudaFuncSetAttribute(score_select, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_s)));
       launch_chained(score_select, dim3(static_cast<unsigned>(nblk) * chunks), dim3(kScoreThreads), smem_s, s, K, stride, T, NA,
                      DF, n_keep, nblk, m32, m64, mnorm, s32, scores_out, tickets + ctx->max_batch,
@@ -1370,7 +1372,7 @@ wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, i
     }
   }
   // per-head keys, and the cases that need no scores (n_keep = 0 or everything kept): a selection launch of its own
-  if (smem_sel > 48 * 1024) {
+  if (smem_sel > kSmemOptIn) {
     WK_CUDA_TRY(ctx, cudaFuncSetAttribute(select_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           static_cast<int>(smem_sel)));
     WK_CUDA_TRY(ctx, cudaFuncSetAttribute(select_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,

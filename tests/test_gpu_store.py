@@ -48,3 +48,22 @@ def test_one_call_equals_two(T, H, n_keep, L, per_head):
     assert a.poll_status() == (0, 0) and b.poll_status() == (0, 0)
     # the whole pool buffer: slot poses and validity flags as well
     assert torch.equal(a.pool, b.pool)
+
+
+@pytest.mark.parametrize("T", [1385, 1400, 1414, 1445, 1446])
+@pytest.mark.parametrize("H,per_head", [(1, False), (17, False), (1, True)])
+def test_selection_space_around_48_kilobytes(T, H, per_head):
+    """2 T scores take 17 bytes each in the selection's shared memory: just below 48 KB the kernel's static arrays push a
+    launch over the default limit."""
+    from paper_2605_22718_b200 import WorldKV, SCORE_PER_HEAD
+    from oracle import worldkv_oracle as o
+    D, n_keep = H * 128, T // 2
+    kv = WorldKV(n_layers=1, n_heads=H, tokens_per_frame=T, n_keep=n_keep, pool_slots=1, max_k=1,
+                 score_mode=SCORE_PER_HEAD if per_head else 0)
+    bits = wi.key_chunk_bf16(4, 0, 1, T, D, 0.1)
+    keep = kv.compress_chunk(wd.to_device_bf16(bits)[None]).cpu().numpy()[0]
+    assert kv.poll_status() == (0, 0)
+    if per_head:
+        np.testing.assert_array_equal(keep, o.compress_chunk_per_head(bits, T, n_keep, H)[0])
+    else:
+        np.testing.assert_array_equal(keep, o.compress_chunk(bits, T, n_keep)[0])
