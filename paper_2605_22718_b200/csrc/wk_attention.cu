@@ -9,20 +9,23 @@
 //   * K/V tiles (128 rows x 128 columns of one head, bf16) are fetched by TMA straight from where they lie:
 //     a dense segment (2-D tensor map per segment) or a pool slot (3-D tensor map [layer*slot][row][col]; the
 //     slot id is read from device memory, so the retrieval result never visits the host).  Rows past the end
-//     of a segment/slot are zero-filled by TMA and masked to -inf before the row maximum;
+//     of a segment/slot are zero-filled by TMA and masked to -inf before the exponentials;
 //   * S = Q K^T and O += P V are tcgen05.mma (M = 128, N = 128, K = 16 steps) with fp32 accumulators in tensor
 //     memory: S0, S1, O0, O1 fill all 512 columns; P (bf16) overwrites S in place and is the A operand of
 //     the P V product directly from tensor memory;
-//   * warp roles: warps 0-3 / 4-7 = softmax of Q tile 0 / 1 (one thread per row, online softmax in fp32 in
-//     the exp2 domain, running maximum updated lazily), warp 8 = MMA issue, warp 9 = TMA producer.  The producer walks
-//     the tile list, and hands each tile's height to the others beside the tile; the MMA warp waits once per step for
+//   * warp roles: warps 0-3 / 4-7 = softmax of Q tile 0 / 1 (one thread per row, fp32 in the exp2
+//     domain, against a reference taken at the start of a piece: see kStreamMax), warp 8 = MMA issue, warp 9 = TMA producer.  The
+//     producer walks the tile list, and hands each tile's height to the others beside the tile; the MMA warp waits once per step for
 //     (V of tile j, K of tile j + 1) and then only for P, since every further wait or branch between two groups of MMAs
 //     is time the tensor pipe stands still (its queue holds about two MMAs);
 //   * a tile with nv < 128 valid rows (the last one of a segment or slot: 1,320 rows are 10 tiles and 40 rows) is
 //     multiplied over ceil(nv / 16) * 16 rows and its softmax stops at the last group of 32.
-// What bounds it: the chain of one Q tile (softmax ~1,650 clk -> P V and Q K^T 1,050 -> hand-overs ~450, 3,150 clk per KV
-// tile at 12 heads x 880 tokens) while the board is at its 1,000 W cap; before the issue path was rebuilt 3,280 clk, and
-// 278 -> 270 us sustained, 276 -> 247 us alone, at 2,640 queries x 15,840 keys x 12 heads.
+//   * every commit after a step's first makes the MMA warp wait until the queue of the tensor pipe has drained, so it commits
+//     only S and O; stages and Q are given back by the softmax warpgroup that sees the last S of a step.
+// What bounds it: the board's 1,000 W cap (1.46-1.65 GHz when run back to back), and at that clock the chain of one Q tile
+// (softmax ~1,130 clk -> P V, Q K^T and hand-overs ~1,350; the tensor pipe works 2,050 of 2,550 clk per KV tile at
+// 167,640 keys x 12 heads, 2,840 before the softmax was streamed).  2,640 queries x 15,840 keys x 12 heads, back
+// to back: 278 us, 273 with the issue path rebuilt, 255 streamed; 4,680 x 32,760 x 40: 3,209 -> 2,960 -> 2,760.
 // Every wait is bounded; a wait that runs out sets WK_DEV_TIMEOUT, the CTA drains and frees its tensor memory.
 #include <stddef.h>
 
@@ -44,6 +47,13 @@ constexpr int kStages = 2, kStagesLse = 4;
 constexpr size_t kSmemBytes = 1024 + 2 * kTileBytes + 2 * kStages * kTileBytes;   // align slack + Q0,Q1 + stages
 constexpr size_t kSmemBytesLse = 1024 + 2 * kTileBytes + kStagesLse * kTileBytes;
 constexpr int kNvRing = 16;   // tile heights handed from the TMA warp to the others; the TMA warp is at most kStagesLse + 1 tiles ahead
+// The softmax has two forms.  Streamed: P = 2^(s * scale - m) with m = the largest of the row's first 32 logits of the
+// piece, so that S is read once and the exponentials of a tile's first columns do not wait for a maximum over its last.
+// bf16 and fp32 share one exponent range: nothing is lost while the sum (at least 1) stays within kStreamMax and O is
+// finite, which each row checks at the end of a piece.  Safe: against a running maximum, for a CTA in which a row failed
+// the check (a logit some 69 natural units above the first 32); it does its work again.  12 heads x 2,640 queries x 15,840
+// keys, back to back: 255 us streamed, 273 with a running maximum for all, 535 when every CTA does both.
+constexpr float kStreamMax = 0x1p100f;
 constexpr float kRescaleThreshold = 8.0f;           // log2 units: P stays <= 2^8 between maximum updates
 constexpr uint32_t kTmemS = 0, kTmemO = 256;        // tensor-memory columns: S0, S1 (P over them), O0, O1; LSE-only: S0, S1 twice
 constexpr int kPairRows = 2 * kTileQ;
@@ -240,7 +250,8 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return d;
 }
 // 2^x of a pair.  The exponentials are the kernel's second bound (16 per clock and SM on the special-function unit, as many
-// clocks per tile as its tensor-core work), so a share of the pairs takes 2^x from the FMA pipe instead: x = n + f with
+// clocks per tile as its tensor-core work; 254 us at a share of 1/8 against 258 at 0 and 256 at 2/8 for 12 heads x 15,840
+// keys), so a share of the pairs takes 2^x from the FMA pipe instead: x = n + f with
 // n = round(x) by the add-a-large-constant trick, 2^f on [-1/2, 1/2] by a cubic (relative error 7.7e-5, far inside the bf16
 // rounding P gets anyway: 2e-3), 2^n by adding n to the exponent field; all in packed fp32 pairs.  That path clamps at
 // x = -120 (a weight of 1e-36) and needs x < 127.
@@ -277,40 +288,13 @@ __device__ __forceinline__ float sum4_f32x2(const uint64_t (&acc)[4]) {
   return a + b;
 }
 
-// P = 2^(s * scale - m) for one row of a tile: rounds to bf16, stores into tensor memory over S (64 columns), returns the
-// fp32 row sum.  kPoly of every 8 column pairs take the FMA pipe (sustained, 12 heads x 15,840 keys: 276 / 277 / 270 / 291 us
-// at 0 / 1 / 2 / 3); tiles with masked columns (-inf) take kPoly = 0 and stop after n_chunks groups of 32 columns.
-#ifndef WK_ATTN_POLY
-#define WK_ATTN_POLY 2
-#endif
-template <int kPoly>
-__device__ __forceinline__ float exp_store_tile(const float (&s)[128], uint64_t scale2, uint64_t neg_m2, uint32_t tS, int n_chunks) {
-  uint64_t acc[4] = {0, 0, 0, 0};   // four independent (lo, hi) sums
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    if (kPoly == 0 && c >= n_chunks) break;   // a short tile stops at its last group of 32 columns
-    uint32_t pk[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const uint64_t e = fma_f32x2(pack_f32x2(s[c * 32 + 2 * i], s[c * 32 + 2 * i + 1]), scale2, neg_m2);
-      float p0, p1;
-      if ((i & 7) < kPoly) exp2_pair<true>(e, p0, p1);
-      else exp2_pair<false>(e, p0, p1);
-      acc[i & 3] = add_f32x2(acc[i & 3], pack_f32x2(p0, p1));
-      pk[i] = pack_bf16x2(p0, p1);
-    }
-    tmem_st_x16(tS + c * 16, pk);
-  }
-  return sum4_f32x2(acc);
-}
-
-// LSE-only launches: sum of 2^(s * scale - m) over 32 columns of a row held in registers.  kLsePoly of every 8 pairs take
-// the FMA pipe; big = the largest of their raw values (the caller checks that they stay below the path's limit).
-#ifndef WK_LSE_POLY
-#define WK_LSE_POLY 2
-#endif
-__device__ __forceinline__ void lse_chunk(uint32_t (&r)[32], int rem, uint64_t scale2, uint64_t neg_m2, uint64_t (&acc)[4], float& big) {
-  if (rem < 32) {   // columns past the end of the slot
+// P = 2^(s * scale - m) of 32 columns of a row: sums go to four independent (lo, hi) accumulators.  kPoly of every 8 pairs
+// take the FMA pipe; big = the largest of their raw values (the caller checks that they stay below that path's limit).
+template <int kPoly, bool kStore>
+__device__ __forceinline__ void exp_chunk(uint32_t (&r)[32], int rem, uint64_t scale2, uint64_t neg_m2, uint64_t (&acc)[4],
+                                          float& big, uint32_t tP) {
+  uint32_t pk[16];
+  if (rem < 32) {   // columns past the end of the segment or slot
 #pragma unroll
     for (int i = 0; i < 32; ++i) r[i] = i < rem ? r[i] : 0xff800000u;
   }
@@ -319,15 +303,23 @@ __device__ __forceinline__ void lse_chunk(uint32_t (&r)[32], int rem, uint64_t s
     const float s0 = __uint_as_float(r[2 * i]), s1 = __uint_as_float(r[2 * i + 1]);
     const uint64_t e = fma_f32x2(pack_f32x2(s0, s1), scale2, neg_m2);
     float p0, p1;
-    if ((i & 7) < WK_LSE_POLY) {
+    if ((i & 7) < kPoly) {
       exp2_pair<true>(e, p0, p1);
       big = fmax3(big, s0, s1);
     } else {
       exp2_pair<false>(e, p0, p1);
     }
     acc[i & 3] = add_f32x2(acc[i & 3], pack_f32x2(p0, p1));
+    if (kStore) pk[i] = pack_bf16x2(p0, p1);
   }
+  if (kStore) tmem_st_x16(tP, pk);   // bf16, over S columns that have been read
 }
+#ifndef WK_ATTN_POLY
+#define WK_ATTN_POLY 1
+#endif
+#ifndef WK_LSE_POLY
+#define WK_LSE_POLY 2
+#endif
 
 // One piece of work: unit u, KV tiles [tb, te), and where its result goes.
 struct Piece {
@@ -408,46 +400,26 @@ struct PieceWalker {
 // softmax warpgroup per buffer, so the tensor pipe works ahead of the softmax, which bounds it (issue and special-function
 // unit) until the board's power cap does.  2,640 queries x 12 heads x 250 slots of 1,320 rows: two warpgroups and one buffer
 // per Q tile on 132 SMs 4,070 us; all SMs, two buffers, streamed sums 3,540; four warpgroups 3,070 (2,136 clk per KV tile).
+// What the roles of a CTA share besides the tiles.
 template <bool kLse>
-__global__ void __launch_bounds__(kThreads<kLse>, 1)
-memory_attention_kernel(const __grid_constant__ AttnParams p) {
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
+struct CtaShared {
+  Barriers bars;
+  uint32_t tmem;
+  volatile uint32_t abort, again;   // again: a row failed the streamed softmax's check
+  float2 merge[kLse ? 2 : 1][kLse ? 128 : 1];   // (reference, sum) of a Q tile's odd KV tiles
+  volatile int nv[kNvRing];   // valid rows of tile number t (counted over the CTA's pieces) at t % kNvRing
+};
+
+// All of a CTA's work, with the streamed softmax or with a running maximum (safe).
+template <bool kLse, bool safe>
+__device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<kLse>& sh, uint8_t* smem) {
+  const uint32_t smem_base = smem_u32(smem);
   uint8_t* sQ = smem;                                   // [2 q tiles][2 halves][128 rows][128 B]
   uint8_t* sKV = sQ + 2 * kTileBytes;                   // [stages][K, V][2 halves][128][128 B]; LSE-only: [stages][K]
   constexpr uint32_t kNStages = kLse ? kStagesLse : kStages;
   constexpr uint32_t kStageBytes = kLse ? kTileBytes : 2 * kTileBytes;
-  __shared__ Barriers bars;
-  __shared__ uint32_t s_tmem;
-  __shared__ volatile uint32_t s_abort;
-  __shared__ float2 s_merge[kLse ? 2 : 1][kLse ? 128 : 1];   // (reference, sum) of a Q tile's odd KV tiles
-  __shared__ volatile int s_nv[kNvRing];   // valid rows of tile number t (counted over the CTA's pieces) at t % kNvRing
-
+  Barriers& bars = sh.bars;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-
-  if (tid == 0) {
-    mbar_init(&bars.q_full, 1);
-    mbar_init(&bars.q_empty, 1);
-    for (int s = 0; s < kStagesLse; ++s) { mbar_init(&bars.kv_full[s], 1); mbar_init(&bars.kv_empty[s], 1); }
-    for (int i = 0; i < 4; ++i) { mbar_init(&bars.s_full[i], 1); mbar_init(&bars.p_full[i], 4); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&bars.o_done[i], 1); mbar_init(&bars.o_free[i], 4); mbar_init(&bars.m_full[i], 4); mbar_init(&bars.m_empty[i], 4); }
-    s_abort = 0;
-    fence_mbar_init();
-  }
-  if (warp == 0) {
-    tmem_alloc(&s_tmem, 512);
-    tmem_relinquish();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  // everything above runs under the end of the kernel before this one; nothing is read or written before this wait
-  dep_wait();
-  dep_release();
-  // an allocation of all 512 columns starts at column 0; addresses known at compile time keep the MMAs' operands cheap
-  if (s_tmem != 0 && tid == 0) { s_abort = 1; atomicOr(p.status, WK_DEV_TIMEOUT); }
-
   if (warp == kSoftWarps<kLse> + 1) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
@@ -457,7 +429,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
       uint32_t st = 0, ph = 1, steps = 0, n = 0, t = 0;   // stage, its parity, stages and Q pairs armed so far, tiles so far
       bool ok = true;
       while (ok && walk.next(p, pc)) {
-        if (!(ok = wait_or_abort(&bars.q_empty, (n & 1) ^ 1, &s_abort))) break;
+        if (!(ok = wait_or_abort(&bars.q_empty, (n & 1) ^ 1, &sh.abort))) break;
         mbar_expect_tx(&bars.q_full, 2 * kTileBytes);
         ++n;
         for (int i = 0; i < 2; ++i)
@@ -480,8 +452,8 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
         TileInfo ti, tv;
         bool have_k = it.next(p, ti, report), have_v = false;
         while (have_k || have_v) {   // step: V of the tile before (not in LSE-only launches), K of this tile
-          if (!(ok = wait_or_abort(&bars.kv_empty[st], ph, &s_abort))) break;
-          if (have_k) s_nv[t++ % kNvRing] = ti.nv;   // read after kv_full
+          if (!(ok = wait_or_abort(&bars.kv_empty[st], ph, &sh.abort))) break;
+          if (have_k) sh.nv[t++ % kNvRing] = ti.nv;   // read after kv_full
           mbar_expect_tx(&bars.kv_full[st], (have_k ? kTileBytes : 0) + (have_v ? kTileBytes : 0));
           ++steps;
           uint8_t* dst = sKV + st * kStageBytes;
@@ -493,11 +465,11 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           if (have_k) have_k = it.next(p, ti, report);
         }
       }
-      leave_role(ok, &s_abort, p.status);
+      leave_role(ok, &sh.abort, p.status);
       // After an abort the consumers no longer wait for the tiles in flight, so this thread does: a CTA must not free
       // its shared memory under copies that are still landing.  Per stage, the load armed last is use u = (count - 1 -
       // stage) / stages of that stage's barrier, whose phase u has parity u & 1; a stage that was never armed is skipped.
-      if (s_abort) {
+      if (sh.abort) {
         auto drain = [](uint64_t* bar, uint32_t use) {
           for (uint32_t i = 0; i < (1u << 16); ++i)
             if (mbar_try_wait(bar, use & 1)) break;
@@ -559,7 +531,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
       while (ok && walk.next(p, pc)) {
         const int n_eff = count_tiles(p, pc.tb, pc.te);
         const bool q1 = pc.has_q1;
-        if (!(ok = wait_or_abort(&bars.q_full, n & 1, &s_abort))) break;
+        if (!(ok = wait_or_abort(&bars.q_full, n & 1, &sh.abort))) break;
         ++n;
         if (n_eff == 0) {
           if (lane == 0) mbar_arrive(&bars.q_empty);
@@ -569,11 +541,11 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           // LSE-only: two S buffers per Q tile, no P V; p_full says that a buffer has been read
           for (int j = 0; j < n_eff; ++j) {
             WK_PROF(0);
-            if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &s_abort))) break;
-            const int nv = s_nv[t++ % kNvRing];
+            if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &sh.abort))) break;
+            const int nv = sh.nv[t++ % kNvRing];
             const uint32_t b0 = lse_q0 & 1, b1 = lse_q1 & 1;
             WK_PROF(1);
-            if (lse_q0 >= 2 && !(ok = wait_or_abort(&bars.p_full[2 * b0], ((lse_q0 >> 1) & 1) ^ 1, &s_abort))) break;
+            if (lse_q0 >= 2 && !(ok = wait_or_abort(&bars.p_full[2 * b0], ((lse_q0 >> 1) & 1) ^ 1, &sh.abort))) break;
             ++lse_q0;
             WK_PROF(2);
             tc_fence_after();
@@ -581,15 +553,13 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
             commit(offsetof(Barriers, s_full) + 16 * b0);
             WK_PROF(3);
             if (q1) {
-              if (lse_q1 >= 2 && !(ok = wait_or_abort(&bars.p_full[2 * b1 + 1], ((lse_q1 >> 1) & 1) ^ 1, &s_abort))) break;
+              if (lse_q1 >= 2 && !(ok = wait_or_abort(&bars.p_full[2 * b1 + 1], ((lse_q1 >> 1) & 1) ^ 1, &sh.abort))) break;
               ++lse_q1;
               WK_PROF(4);
               tc_fence_after();
               issue_s(1, b1 * 256 + 128, st, nv);
               commit(offsetof(Barriers, s_full) + 16 * b1 + 8);
             }
-            commit(offsetof(Barriers, kv_empty) + 8 * st);
-            if (j + 1 == n_eff) commit(offsetof(Barriers, q_empty));
             WK_PROF(5);
             if (++st == kNStages) { st = 0; ph ^= 1; }
           }
@@ -601,44 +571,41 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
         for (int j = -1; j < n_eff; ++j) {
           const bool more = j + 1 < n_eff;
           WK_PROF(0);
-          if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &s_abort))) break;
-          if (more) nv_next = s_nv[t++ % kNvRing];
+          if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &sh.abort))) break;   // later steps: behind p_full[0]
           WK_PROF(1);
           if (j >= 0) {
-            if (!(ok = wait_or_abort(&bars.p_full[0], p_ph0, &s_abort))) break;
+            if (!(ok = wait_or_abort(&bars.p_full[0], p_ph0, &sh.abort))) break;
             p_ph0 ^= 1;
           }
           WK_PROF(2);
+          if (more) nv_next = sh.nv[t++ % kNvRing];
           // A piece's first P V overwrites O: the epilogue of the last piece that used it must have read it.  o_free[i]
           // completes once per piece in which warpgroup i ran an epilogue, so neither side can run two phases ahead of the
           // other (a parity wait cannot tell phase n from phase n + 2).
-          if (j == 0 && e0++ > 0 && !(ok = wait_or_abort(&bars.o_free[0], e0 & 1, &s_abort))) break;
+          if (j == 0 && e0++ > 0 && !(ok = wait_or_abort(&bars.o_free[0], e0 & 1, &sh.abort))) break;
           tc_fence_after();
           if (j >= 0) issue_pv(0, st, nv, j > 0);
           if (more) { issue_s(0, kTmemS, st, nv_next); commit(offsetof(Barriers, s_full)); }
           else commit(offsetof(Barriers, o_done));
-          if (!q1) commit(offsetof(Barriers, kv_empty) + 8 * st);
           WK_PROF(3);
           if (q1) {
             if (j >= 0) {
-              if (!(ok = wait_or_abort(&bars.p_full[1], p_ph1, &s_abort))) break;
+              if (!(ok = wait_or_abort(&bars.p_full[1], p_ph1, &sh.abort))) break;
               p_ph1 ^= 1;
             }
             WK_PROF(4);
-            if (j == 0 && e1++ > 0 && !(ok = wait_or_abort(&bars.o_free[1], e1 & 1, &s_abort))) break;
+            if (j == 0 && e1++ > 0 && !(ok = wait_or_abort(&bars.o_free[1], e1 & 1, &sh.abort))) break;
             tc_fence_after();
             if (j >= 0) issue_pv(1, st, nv, j > 0);
             if (more) { issue_s(1, kTmemS + 128, st, nv_next); commit(offsetof(Barriers, s_full) + 8); }
             else commit(offsetof(Barriers, o_done) + 8);
-            commit(offsetof(Barriers, kv_empty) + 8 * st);
             WK_PROF(5);
           }
-          if (j + 2 == n_eff) commit(offsetof(Barriers, q_empty));   // the last Q K^T of this piece has been issued
           if (++st == kNStages) { st = 0; ph ^= 1; }
           nv = nv_next;
         }
       }
-      if (lane == 0) leave_role(ok, &s_abort, p.status);
+      if (lane == 0) leave_role(ok, &sh.abort, p.status);
       WK_PROF_FLUSH(8, 12, blockIdx.x == 0 && lane == 0);
     }
   } else if (kLse) {
@@ -661,13 +628,18 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
     while (ok && walk.next(p, pc)) {
       const int n_eff = count_tiles(p, pc.tb, pc.te);
       if (qt == 1 && !pc.has_q1) { t0 += n_eff; continue; }
+      const bool releases = qt == (pc.has_q1 ? 1 : 0);   // the Q tile whose product comes last
       float m = 0.f, l = 0.f;
       bool first = true;
       for (int j = (g ^ buf) & 1; j < n_eff; j += 2) {
         WK_PROF(0);
-        if (!(ok = wait_or_abort(&bars.s_full[wg], ((g + j) >> 1) & 1, &s_abort))) break;
+        if (!(ok = wait_or_abort(&bars.s_full[wg], ((g + j) >> 1) & 1, &sh.abort))) break;
         WK_PROF(1);
-        const int nv = s_nv[(t0 + j) % kNvRing], n_ch = (nv + 31) >> 5;
+        const int nv = sh.nv[(t0 + j) % kNvRing], n_ch = (nv + 31) >> 5;
+        if (releases && row == 0) {   // the products that read this tile's stage (and, with the last tile, Q) are done
+          mbar_arrive(&bars.kv_empty[(t0 + j) % kNStages]);
+          if (j + 1 == n_eff) mbar_arrive(&bars.q_empty);
+        }
         tc_fence_after();
         // The row is streamed from tensor memory 32 columns at a time, without a maximum: the sum is taken against a fixed
         // reference, 0 at first (logits of a few log2 units lose nothing there).  A warp in which a row's tile sum leaves
@@ -682,8 +654,8 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           for (int c = 0; c < n_ch; ++c) {
             uint32_t r[32];
             tmem_ld_x32(tS + c * 32, r);
-            tc_wait_ld();
-            lse_chunk(r, nv - c * 32, scale2, neg_m2, acc, big);
+            tc_wait_ld(r);
+            exp_chunk<WK_LSE_POLY, false>(r, nv - c * 32, scale2, neg_m2, acc, big, 0);
           }
           sum = sum4_f32x2(acc);
           const bool off = !(sum <= 32768.f) || big * p.scale_log2 - m > 100.f || (first && sum < 2.44140625e-4f);
@@ -693,7 +665,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
           for (int c = 0; c < n_ch; ++c) {
             uint32_t r[32];
             tmem_ld_x32(tS + c * 32, r);
-            tc_wait_ld();
+            tc_wait_ld(r);
 #pragma unroll
             for (int i = 0; i < 32; ++i) mx = fmaxf(mx, i < nv - c * 32 ? __uint_as_float(r[i]) : -INFINITY);
           }
@@ -714,13 +686,13 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
       g += n_eff;
       t0 += n_eff;
       if (buf == 1) {
-        if (!(ok = wait_or_abort(&bars.m_empty[qt], (n & 1) ^ 1, &s_abort))) break;
-        s_merge[qt][row] = make_float2(m, l);
+        if (!(ok = wait_or_abort(&bars.m_empty[qt], (n & 1) ^ 1, &sh.abort))) break;
+        sh.merge[qt][row] = make_float2(m, l);
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars.m_full[qt]);
       } else {
-        if (!(ok = wait_or_abort(&bars.m_full[qt], n & 1, &s_abort))) break;
-        const float2 o = s_merge[qt][row];
+        if (!(ok = wait_or_abort(&bars.m_full[qt], n & 1, &sh.abort))) break;
+        const float2 o = sh.merge[qt][row];
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars.m_empty[qt]);
         const int qrow = pc.q0 + qt * kTileQ + row;
@@ -734,7 +706,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
       }
       ++n;
     }
-    if (!ok) leave_role(false, &s_abort, p.status);
+    if (!ok) leave_role(false, &sh.abort, p.status);
     WK_PROF_FLUSH(0, 8, blockIdx.x == 0 && tid == 0);
   } else {
     // ------------------------------------------------------------------ softmax warpgroups (one thread per query row)
@@ -749,98 +721,104 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
     uint32_t g = 0;       // running tile count of this warpgroup
     uint32_t t0 = 0;      // tiles of the CTA's pieces so far
     uint32_t n_out = 0;   // pieces of this warpgroup that produced output
+    uint32_t steps = 0;   // stages used by the pieces so far (tiles + 1 each)
     bool ok = true;
     WK_PROF_DECL
     const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2);
     while (ok && walk.next(p, pc)) {
       const bool active = (wg == 0) || pc.has_q1;
+      // S of tile j of the Q tile that comes last in a step is there: the step that filled it is done with its stage (and,
+      // with the last tile, with Q).  The MMA warp could commit to these barriers itself, but every commit after the first
+      // makes it wait until the queue of the tensor pipe has drained.
+      const bool releases = wg == (pc.has_q1 ? 1 : 0);
       const int n_eff = count_tiles(p, pc.tb, pc.te);
-      float m_used = -INFINITY, l = 0.f;
+      float m_used = -INFINITY, l = 0.f, big = -INFINITY;
       int j = 0;
       if (active) {
         while (j < n_eff) {
           WK_PROF(0);
-          if (!(ok = wait_or_abort(&bars.s_full[wg], g & 1, &s_abort))) break;
-          const int nv = s_nv[(t0 + j) % kNvRing];
+          if (!(ok = wait_or_abort(&bars.s_full[wg], g & 1, &sh.abort))) break;
+          const int nv = sh.nv[(t0 + j) % kNvRing];
           WK_PROF(1);
+          if (releases && row == 0) {
+            mbar_arrive(&bars.kv_empty[(steps + j) % kNStages]);
+            if (j + 1 == n_eff) mbar_arrive(&bars.q_empty);
+          }
           tc_fence_after();
-          // the whole S row (128 fp32) is held in registers: one pass for the row maximum, one for the exponentials
-          float s[128];
-          float c0 = -INFINITY, c1 = -INFINITY, c2 = -INFINITY, c3 = -INFINITY;
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
-            // the second 64 columns are in flight while the maximum of the first 64 is taken
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
+          const int n_ch = (nv + 31) >> 5;
+          if (safe) {   // move the reference when the row's maximum has left it by more than the threshold
+            float mx = -INFINITY;
+#pragma unroll 1
+            for (int c = 0; c < n_ch; ++c) {
               uint32_t r[32];
-              tmem_ld_x32(tS + hf * 64 + c * 32, r);
+              tmem_ld_x32(tS + c * 32, r);
+              tc_wait_ld(r);
 #pragma unroll
-              for (int i = 0; i < 32; ++i) s[hf * 64 + c * 32 + i] = __uint_as_float(r[i]);
+              for (int i = 0; i < 32; ++i) mx = fmaxf(mx, i < nv - c * 32 ? __uint_as_float(r[i]) : -INFINITY);
             }
-            if (hf == 1) {
+            const float m_new = fmaxf(m_used, mx * p.scale_log2);
+            const bool move = m_new > m_used + kRescaleThreshold;    // also true on the first tile (m_used = -inf)
+            if (__any_sync(0xffffffffu, move)) {
+              // (the previous P V was issued before this tile's Q K^T: it landed before S did)
+              const float alpha = move ? ex2_approx(m_used - m_new) : 1.f;
+              if (move) m_used = m_new;
+              l *= alpha;
+#pragma unroll 1
+              for (int c = 0; c < 4 && j > 0; ++c) {
+                uint32_t r[32];
+                tmem_ld_x32(tO + c * 32, r);
+                tc_wait_ld(r);
 #pragma unroll
-              for (int i = 0; i < 64; i += 8) {
-                c0 = fmax3(c0, s[i], s[i + 1]);
-                c1 = fmax3(c1, s[i + 2], s[i + 3]);
-                c2 = fmax3(c2, s[i + 4], s[i + 5]);
-                c3 = fmax3(c3, s[i + 6], s[i + 7]);
+                for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
+                tmem_st_x32(tO + c * 32, r);
               }
             }
-            tc_wait_ld();
           }
-          WK_PROF(2);
-          const bool full_tile = nv == kTileKV;
-          if (!full_tile) {   // rows past the end of the segment were zero-filled by TMA: mask them out
-            c0 = c1 = c2 = c3 = -INFINITY;
+          // The row is streamed from tensor memory 32 columns at a time; the next 32 are in flight while these are worked on.
+          {
+            uint64_t acc[4] = {0, 0, 0, 0};
+            uint32_t ra[32], rb[32];
+            tmem_ld_x32(tS, ra);
+            if (!safe && j == 0) {
+              tc_wait_ld(ra);
+              float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-            for (int i = 0; i < 128; ++i) s[i] = i < nv ? s[i] : -INFINITY;
-#pragma unroll
-            for (int i = 0; i < 64; i += 8) {
-              c0 = fmax3(c0, s[i], s[i + 1]);
-              c1 = fmax3(c1, s[i + 2], s[i + 3]);
-              c2 = fmax3(c2, s[i + 4], s[i + 5]);
-              c3 = fmax3(c3, s[i + 6], s[i + 7]);
+              for (int i = 0; i < 32; i += 2)
+                mx[(i >> 1) & 1] = fmax3(mx[(i >> 1) & 1], i < nv ? __uint_as_float(ra[i]) : -INFINITY,
+                                         i + 1 < nv ? __uint_as_float(ra[i + 1]) : -INFINITY);
+              m_used = fmaxf(mx[0], mx[1]) * p.scale_log2;
             }
-          }
+            const uint64_t neg_m2 = pack_f32x2(-m_used, -m_used);
+            WK_PROF(2);
+            if (nv == kTileKV) {
 #pragma unroll
-          for (int i = 64; i < 128; i += 8) {
-            c0 = fmax3(c0, s[i], s[i + 1]);
-            c1 = fmax3(c1, s[i + 2], s[i + 3]);
-            c2 = fmax3(c2, s[i + 4], s[i + 5]);
-            c3 = fmax3(c3, s[i + 6], s[i + 7]);
-          }
-          const float mx = fmaxf(fmax3(c0, c1, c2), c3);
-          const float m_new = fmaxf(m_used, mx * p.scale_log2);
-          float alpha = 1.f;
-          bool rescale = false;
-          if (m_new > m_used + kRescaleThreshold) {    // also true on the first tile (m_used = -inf)
-            alpha = ex2_approx(m_used - m_new);
-            m_used = m_new;
-            rescale = j > 0;
-          }
-          l *= alpha;
-          const uint64_t neg_m2 = pack_f32x2(-m_used, -m_used);
-          WK_PROF(3);
-          // masked columns hold -inf and come out as 0 (special-function path only)
-          l += full_tile ? exp_store_tile<WK_ATTN_POLY>(s, scale2, neg_m2, tS, 4)
-                         : exp_store_tile<0>(s, scale2, neg_m2, tS, (nv + 31) >> 5);
-          if (__any_sync(0xffffffffu, rescale)) {
-            // (the previous P V was issued before this tile's Q K^T: it landed before S did)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              uint32_t r[32];
-              tmem_ld_x32(tO + c * 32, r);
-              tc_wait_ld();
-#pragma unroll
-              for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
-              tmem_st_x32(tO + c * 32, r);
+              for (int c = 0; c < 4; c += 2) {
+                tc_wait_ld(ra);
+                tmem_ld_x32(tS + c * 32 + 32, rb);
+                exp_chunk<WK_ATTN_POLY, true>(ra, 32, scale2, neg_m2, acc, big, tS + c * 16);
+                tc_wait_ld(rb);
+                if (c < 2) tmem_ld_x32(tS + c * 32 + 64, ra);
+                exp_chunk<WK_ATTN_POLY, true>(rb, 32, scale2, neg_m2, acc, big, tS + c * 16 + 16);
+              }
+            } else {
+#pragma unroll 1
+              for (int c = 0; c < n_ch; ++c) {
+                tc_wait_ld(ra);
+                exp_chunk<WK_ATTN_POLY, true>(ra, nv - c * 32, scale2, neg_m2, acc, big, tS + c * 16);
+                if (c + 1 < n_ch) tmem_ld_x32(tS + c * 32 + 32, ra);
+              }
             }
+            l += sum4_f32x2(acc);
+            WK_PROF(4);
           }
-          WK_PROF(4);
           tc_wait_st();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&bars.p_full[wg]);   // one arrival per warp: the wait above covered all 32 lanes' stores
+          if (lane == 0) {
+            // The MMA warp's next step reads this tile's V and the next tile's K as well.  Waiting for them here leaves it
+            // one barrier less to look at between two groups of MMAs (about 200 clocks each).
+            mbar_arrive(&bars.p_full[wg]);   // one arrival per warp: the wait above covered all 32 lanes' stores
+          }
           WK_PROF(5);
           ++j;
           ++g;
@@ -848,9 +826,11 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
         // ---------------------------------------------------------------- epilogue of this piece
         const int prow = wg * kTileQ + row;
         const int qrow = pc.q0 + prow;
-        if (ok && j > 0) ok = wait_or_abort(&bars.o_done[wg], n_out++ & 1, &s_abort);   // completes once per piece
+        if (ok && j > 0) ok = wait_or_abort(&bars.o_done[wg], n_out++ & 1, &sh.abort);   // completes once per piece
+        if (ok && j > 0 && releases && row == 0) mbar_arrive(&bars.kv_empty[(steps + n_eff) % kNStages]);   // the last V
         if (ok) {
           tc_fence_after();
+          uint32_t o_max = 0;   // bits of the largest |O|
           const float inv_l = (j > 0 && l > 0.f) ? 1.f / l : 0.f;
           const float lse = (j > 0 && l > 0.f) ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
 #pragma unroll
@@ -858,7 +838,9 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
             uint32_t r[32];
             if (j > 0) {
               tmem_ld_x32(tO + c * 32, r);
-              tc_wait_ld();
+              tc_wait_ld(r);
+#pragma unroll
+              for (int i = 0; i < 32; ++i) o_max = max(o_max, r[i] & 0x7fffffffu);
             } else {
 #pragma unroll
               for (int i = 0; i < 32; ++i) r[i] = 0u;
@@ -890,10 +872,13 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
             } else {
               p.lsepart[static_cast<int64_t>(pc.slot) * kPairRows + prow] = lse;
             }
+            const bool fine = l <= kStreamMax && big * p.scale_log2 - m_used < 120.f && o_max < 0x7f800000u;   // false for NaN
+            if (j > 0 && !safe && !fine) sh.again = 1;
           }
         }
       }
       t0 += n_eff;
+      if (n_eff > 0) steps += n_eff + 1;
       // O of this piece has been read: the next piece that uses this accumulator may overwrite it
       if (active && j > 0) {
         tc_fence_before();
@@ -901,12 +886,71 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
         if (lane == 0) mbar_arrive(&bars.o_free[wg]);
       }
     }
-    if (!ok) leave_role(false, &s_abort, p.status);
+    if (!ok) leave_role(false, &sh.abort, p.status);
     WK_PROF_FLUSH(0, 8, blockIdx.x == 0 && tid == 0);
+  }
+}
+// The second pass is a call: inlined, it costs the first one registers (12 heads x 15,840 keys: 264 against 256 us).
+__device__ __noinline__ void attention_again(const AttnParams& p, CtaShared<false>& sh, uint8_t* smem) {
+  attention_roles<false, true>(p, sh, smem);
+}
+
+template <bool kLse>
+__global__ void __launch_bounds__(kThreads<kLse>, 1)
+memory_attention_kernel(const __grid_constant__ AttnParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + (((smem_u32(smem_raw) + 1023u) & ~1023u) - smem_u32(smem_raw));
+  __shared__ CtaShared<kLse> sh;
+  const int tid = threadIdx.x;
+  auto init_barriers = [&]() {
+    mbar_init(&sh.bars.q_full, 1);
+    mbar_init(&sh.bars.q_empty, 1);
+    for (int s = 0; s < kStagesLse; ++s) { mbar_init(&sh.bars.kv_full[s], 1); mbar_init(&sh.bars.kv_empty[s], 1); }
+    for (int i = 0; i < 4; ++i) { mbar_init(&sh.bars.s_full[i], 1); mbar_init(&sh.bars.p_full[i], 4); }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&sh.bars.o_done[i], 1);
+      mbar_init(&sh.bars.o_free[i], 4);
+      mbar_init(&sh.bars.m_full[i], 4);
+      mbar_init(&sh.bars.m_empty[i], 4);
+    }
+    fence_mbar_init();
+  };
+  if (tid == 0) {
+    init_barriers();
+    sh.again = 0;
+    sh.abort = 0;
+  }
+  if (tid < 32) {
+    tmem_alloc(&sh.tmem, 512);
+    tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(s_tmem, 512);
+  tc_fence_after();
+  // everything above runs under the end of the kernel before this one; nothing is read or written before this wait
+  dep_wait();
+  dep_release();
+  // an allocation of all 512 columns starts at column 0; addresses known at compile time keep the MMAs' operands cheap
+  if (sh.tmem != 0 && tid == 0) { sh.abort = 1; atomicOr(p.status, WK_DEV_TIMEOUT); }
+
+  attention_roles<kLse, false>(p, sh, smem);
+  tc_fence_before();
+  __syncthreads();
+  if constexpr (!kLse) {
+    if (sh.again && !sh.abort) {   // the same for all threads
+      // All roles have finished and nothing is in flight: the barriers start afresh, and so do the roles.
+      if (tid == 0) {
+        for (uint32_t i = 0; i < sizeof(Barriers) / 8; ++i) mbar_inval(reinterpret_cast<uint64_t*>(&sh.bars) + i);
+        init_barriers();
+      }
+      __syncthreads();
+      tc_fence_after();
+      attention_again(p, sh, smem);
+      tc_fence_before();
+      __syncthreads();
+    }
+  }
+  if (tid < 32) tmem_dealloc(sh.tmem, 512);
 }
 
 // Merge the pieces of every unit that was cut: O = sum_s w_s O_s / sum_s w_s with w_s = exp(lse_s - max lse).  Bound by
