@@ -1033,10 +1033,11 @@ int attention_partial_slots(int n_heads, int max_lq, int max_splits) {
 // Default distribution over the SMs: whole units in full waves, then, where it pays, the units of the last, partial wave
 // cut into equal ranges over all SMs and merged.  The cut saves (sms - rest) / sms of a unit's tiles; it costs about 4
 // tile times (the combine launch, a second prologue) and 13 more when every CTA writes partials.  Measured on 148 SMs,
-// whole -> cut, back to back: 40 heads x 4,680 queries x 32,760 keys (rest 20 of 148) 3,136 -> 2,897 us; 12 heads x 880
-// tokens, 167,640 keys (rest 132) 2,782 -> 2,716; 8 heads x 7,920 keys (rest 88) 122 -> 101; 2 heads x 3,960 keys (rest 8)
-// 61 -> 24; and the other way round for 12 heads x 15,840 keys (rest 132) 266 -> 269, 16 heads x 7,200 keys (rest 128)
-// 125 -> 136, 24 heads x 9,000 keys (rest 140) 322 -> 336.
+// whole -> cut, back to back: 40 heads x 4,680 queries x 32,760 keys (rest 20 of 148) 2,933 -> 2,718 us; 12 heads x 880
+// tokens (rest 132), 167,640 keys 2,559 -> 2,500, 40,000 keys 612 -> 598, 24,000 keys 372 -> 372; 10 heads x 15,840 keys
+// (rest 110) 230 -> 216; 2 heads x 3,960 keys (rest 8) 61 -> 24; and the other way round for 12 heads x 15,840 keys
+// 247 -> 255 and 13,200 keys 209 -> 217.  At 12 heads x 18,480 keys, just beyond the line, 289 -> 292 back to back and
+// 300 -> 296 with pauses between the calls (a cut leaves fewer SMs idle, which the power cap rewards less).
 static void split_default(int64_t units, int64_t tiles, int64_t sms, int64_t* G, int64_t* n_full, int64_t* ranges) {
   const int64_t waves = units / sms, rest = units - waves * sms;
   *G = units < sms ? units : sms;
