@@ -1032,18 +1032,19 @@ int attention_partial_slots(int n_heads, int max_lq, int max_splits) {
 
 // Default distribution over the SMs: whole units in full waves, then, where it pays, the units of the last, partial wave
 // cut into equal ranges over all SMs and merged.  The cut saves (sms - rest) / sms of a unit's tiles; it costs about 4
-// tile times (the combine launch, a second prologue) and 13 more when every CTA writes partials.  Measured on 148 SMs,
+// tile times (the combine launch, a second prologue) and 16 more when every CTA writes partials.  Measured on 148 SMs,
 // whole -> cut, back to back: 40 heads x 4,680 queries x 32,760 keys (rest 20 of 148) 2,933 -> 2,718 us; 12 heads x 880
-// tokens (rest 132), 167,640 keys 2,559 -> 2,500, 40,000 keys 612 -> 598, 24,000 keys 372 -> 372; 10 heads x 15,840 keys
-// (rest 110) 230 -> 216; 2 heads x 3,960 keys (rest 8) 61 -> 24; and the other way round for 12 heads x 15,840 keys
-// 247 -> 255 and 13,200 keys 209 -> 217.  At 12 heads x 18,480 keys, just beyond the line, 289 -> 292 back to back and
-// 300 -> 296 with pauses between the calls (a cut leaves fewer SMs idle, which the power cap rewards less).
+// tokens (rest 132), 167,640 keys 2,559 -> 2,500, 40,000 keys 612 -> 598, 22,500 keys 348 -> 347; 10 heads x 15,840 keys
+// (rest 110) 230 -> 216; 8 heads (rest 88) x 4,500 keys 66 -> 63; 2 heads x 3,960 keys (rest 8) 61 -> 24.  The other way
+// round: 12 heads x 18,480 keys 286 -> 291, 15,840 keys 247 -> 255; 11 heads (rest 121) x 10,000 keys 152 -> 158, x 12,000
+// 182 -> 185; 10 heads x 7,500 keys 108 -> 113; 8 heads x 3,000 keys 48 -> 51.  (With pauses between the calls the cut is
+// worth 1 to 2 % more: it leaves no SM idle, which the power cap does not reward.)
 static void split_default(int64_t units, int64_t tiles, int64_t sms, int64_t* G, int64_t* n_full, int64_t* ranges) {
   const int64_t waves = units / sms, rest = units - waves * sms;
   *G = units < sms ? units : sms;
   *n_full = units;
   *ranges = 0;
-  if (rest == 0 || (sms - rest) * tiles < 4 * sms + 13 * rest) return;
+  if (rest == 0 || (sms - rest) * tiles < 4 * sms + 16 * rest) return;
   *n_full = waves * sms;
   // Where whole cuts of every unit use nearly all SMs, no CTA gets two pieces; pieces of fewer than 4 tiles cost more in
   // prologues and partials than they save (2 heads x 3,960 keys: 144 unaligned ranges 23.3 us, 128 aligned 21.2, 64
