@@ -72,9 +72,8 @@ struct AttnParams {
   int n_tiles, n_qpairs, n_units;
   int n_full, n_ranges;
   int lq, H;
-  int lse_only;     // 1: only the log-sum-exp is wanted (query-based retrieval): no V loads, no P V product, no O
   int slot_units;   // 1: every listed slot is a problem of its own: unit = (slot ordinal, head, q-pair), n_tiles =
-                    //    tiles_per_slot, lse laid out [slot ordinal][H][lq]; stale slots give -inf and are not reported
+                    //    tiles_per_slot, lse laid out [slot ordinal][H][lq]; stale slots give -inf and are not reported (LSE-only launches)
   float scale_log2;
   __nv_bfloat16* O;
   float* lse;
@@ -1106,8 +1105,7 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   p.tiles_per_slot = (ctx->C + kTileKV - 1) / kTileKV;
   p.n_tiles = tiles + n_slots * p.tiles_per_slot;
   p.lq = lq;
-  p.lse_only = lse_only ? 1 : 0;
-  p.slot_units = p.lse_only;
+  p.slot_units = lse_only ? 1 : 0;
   p.H = ctx->cfg.n_heads;
   p.n_qpairs = (lq + kPairRows - 1) / kPairRows;
   p.n_units = p.n_qpairs * p.H;
