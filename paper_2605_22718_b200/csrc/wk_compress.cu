@@ -35,7 +35,7 @@ constexpr int kScoreThreads = 256;
 constexpr int kCopyRows = 16;         // rows per piece of the V copy that rides along with the scoring
 struct FusedQueue {
   uint32_t a_next, s_next, exited;   // compress_fused
-  uint32_t copy_next;                // pieces of V's anchor frames handed out by score_select; reset by anchor_rows
+  uint32_t copy_next;                // pieces of V's anchor frames handed out by score_select; reset by every anchor pass that a store's score_select follows
 };
 
 __device__ __forceinline__ double bf16_to_f64(uint32_t bits16) {
@@ -589,13 +589,14 @@ anchor_rows(const __nv_bfloat16* __restrict__ K, int64_t stride, int chunks, int
 __global__ void __launch_bounds__(kAnchorThreads)
 anchor_pass_wide(const __nv_bfloat16* __restrict__ K, int64_t stride, int T, int D, int parts,
                  double* __restrict__ partial, uint32_t* __restrict__ counters, double* __restrict__ m64,
-                 float* __restrict__ m32, double* __restrict__ mnorm) {
+                 float* __restrict__ m32, double* __restrict__ mnorm, uint32_t* __restrict__ copy_queue) {
   extern __shared__ __align__(16) uint8_t smem[];
   double* acc = reinterpret_cast<double*>(smem);   // [D]
   __shared__ double red[kAnchorThreads / 32];
   __shared__ double inv_s;
   __shared__ uint32_t is_last;
   const int b = blockIdx.y, part = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (b == 0 && part == 0 && tid == 0) *copy_queue = 0u;
   const __nv_bfloat16* Kb = K + static_cast<int64_t>(b) * stride;
   for (int c = tid; c < D; c += kAnchorThreads) acc[c] = 0.0;
   __syncthreads();
@@ -1245,6 +1246,7 @@ wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, i
   double* mnorm = reinterpret_cast<double*>(sc + ctx->sl.mnorm_off);
   double* partial = reinterpret_cast<double*>(sc + ctx->sl.part_off);
   uint32_t* tickets = reinterpret_cast<uint32_t*>(sc + ctx->sl.cnt_off);   // [2][max_batch]: anchor pass, score pass
+  uint32_t* copy_queue = &reinterpret_cast<FusedQueue*>(tickets + 3 * ctx->max_batch)->copy_next;
   const int max_parts = ctx->sl.anchor_parts;
   const bool need_scores = (n_keep > 0 && n_keep < NA) || scores_out != nullptr;
   const size_t smem_sel = static_cast<size_t>(NA) * (4 + 4 + 8 + 1) + 16;
@@ -1310,7 +1312,7 @@ wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, i
       const int64_t r_min = (T + max_parts - 2) / (max_parts - 1);
       if (R < r_min) R = r_min;
       const dim3 grid(static_cast<unsigned>((total + R - 1) / R));
-#define WK_ROWS(V, W) launch_rows<V, W>(grid, smem_r, s, K, stride, chunks, T, DF, hs, wpr, static_cast<int>(R), partial, max_parts, tickets, m64, m32, mnorm, store, &reinterpret_cast<FusedQueue*>(tickets + 3 * ctx->max_batch)->copy_next)
+#define WK_ROWS(V, W) launch_rows<V, W>(grid, smem_r, s, K, stride, chunks, T, DF, hs, wpr, static_cast<int>(R), partial, max_parts, tickets, m64, m32, mnorm, store, copy_queue)
       if (store) store->k_done = true;
       if (per_head) {
         switch (vpl) {
@@ -1337,7 +1339,7 @@ wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, i
       WK_CUDA_TRY(ctx, cudaFuncSetAttribute(anchor_pass_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             static_cast<int>(smem_acc)));
       anchor_pass_wide<<<grid_a, kAnchorThreads, smem_acc, s>>>(K, stride, T, DF, max_parts, partial, tickets, m64, m32,
-                                                                mnorm);
+                                                                mnorm, copy_queue);
     }
     if ((st = after_launch(ctx)) != WK_OK) return st;
     // blocks of rows of score_select / head_score: whole rounds of its 8 warps x 2 rows, and as few full waves of CTAs (four resident
@@ -1365,7 +1367,7 @@ wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, i
                      DF, n_keep, nblk, m32, m64, mnorm, s32, scores_out, tickets + ctx->max_batch,
                      select_here ? keep_idx : static_cast<int32_t*>(nullptr), ctx->status_dev,
                      store ? store->Vsrc : nullptr, store ? store->Vdst : nullptr, store ? store->dst_stride : 0,
-                     &reinterpret_cast<FusedQueue*>(tickets + 3 * ctx->max_batch)->copy_next);
+                     copy_queue);
       if (store) store->v_done = true;
       if ((st = after_launch(ctx)) != WK_OK) return st;
       if (select_here) return WK_OK;

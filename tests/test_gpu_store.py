@@ -18,6 +18,8 @@ pytestmark = pytest.mark.gpu
     (45, 20, 44, 3, False),    # wide rows: both passes in one launch, rows stored from the staging buffer
     (65, 40, 32, 2, False),    # 5,120 columns
     (7, 40, 3, 5, False),      # groups of fewer than four rows
+    (9, 65, 5, 2, False),      # rows of more than 8,192 columns: an anchor pass of their own
+    (20, 72, 7, 3, False),
     (20, 3, 0, 2, False),      # nothing kept but the anchor: no scoring pass
     (20, 24, 40, 2, False),    # everything kept
     (50, 12, 25, 2, True),
