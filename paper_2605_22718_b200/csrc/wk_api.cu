@@ -324,6 +324,7 @@ wk_status wk_pool_compress_append(wk_ctx* ctx, int32_t layer0, int32_t n, const 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // everything that can fail on the host is settled before the first launch
   int slot = *slot_io_host;
+  bool mark_is_up = false;   // the slot is free on the host, and the device's mark still says otherwise
   if (slot < -1 || slot >= ctx->cfg.pool_slots) return WK_ERR_BAD_SLOT;
   if (slot >= 0) {
     if (ctx->slots[slot].state != SLOT_OPEN) return WK_ERR_BAD_SLOT;
@@ -336,7 +337,8 @@ wk_status wk_pool_compress_append(wk_ctx* ctx, int32_t layer0, int32_t n, const 
       const int victim = wk_pool_oldest(ctx);
       if (!evict_oldest_if_full || victim < 0) return WK_ERR_POOL_FULL;
       // the chunk goes into the slot just freed; if this call stores all of its layers, the slot's own mark comes with them
-      wk_status st = n == ctx->cfg.n_layers ? free_slot(ctx, victim) : wk_pool_evict(ctx, victim, stream);
+      mark_is_up = n == ctx->cfg.n_layers;
+      wk_status st = mark_is_up ? free_slot(ctx, victim) : wk_pool_evict(ctx, victim, stream);
       if (st != WK_OK) return st;
       if (evicted_slot_host) *evicted_slot_host = victim;
     }
@@ -347,12 +349,11 @@ wk_status wk_pool_compress_append(wk_ctx* ctx, int32_t layer0, int32_t n, const 
                     static_cast<int64_t>(ctx->C) * ctx->D * ctx->cfg.pool_slots, false, false};
   wk_status st = launch_compress(ctx, static_cast<const __nv_bfloat16*>(K_chunks), batch_stride_elems, n, keep_idx_dev,
                                  nullptr, s, &store);
-  if (st != WK_OK) {   // the freed slot's mark is still up
-    if (*slot_io_host < 0) launch_slot_mark(ctx, slot, 0, ctx->slots[slot].pose, s);
-    return st;
-  }
-  return append_checked(ctx, layer0, n, K_chunks, V_chunks, batch_stride_elems, keep_idx_dev, pose_host, chunk_tag,
+  if (st == WK_OK)
+    st = append_checked(ctx, layer0, n, K_chunks, V_chunks, batch_stride_elems, keep_idx_dev, pose_host, chunk_tag,
                         slot_io_host, s, &store);
+  if (st != WK_OK && mark_is_up) launch_slot_mark(ctx, slot, 0, ctx->slots[slot].pose, s);
+  return st;
 }
 
 size_t wk_host_chunk_bytes(const wk_ctx* ctx) {
