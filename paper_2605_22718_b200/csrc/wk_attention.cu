@@ -11,10 +11,10 @@
 //     slot id is read from device memory, so the retrieval result never visits the host).  Rows past the end
 //     of a segment/slot are zero-filled by TMA and masked to -inf before the exponentials;
 //   * S = Q K^T and O += P V are tcgen05.mma (M = 128, N = 128, K = 16 steps) with fp32 accumulators in tensor
-//     memory: S0, S1, O0, O1 fill all 512 columns; P (bf16) overwrites S in place and is the A operand of
+//     memory: S0, S1, O0, O1 fill all 512 columns; P (bf16) overwrites the second half of S and is the A operand of
 //     the P V product directly from tensor memory;
 //   * warp roles: warps 0-3 / 4-7 = softmax of Q tile 0 / 1 (one thread per row, fp32 in the exp2
-//     domain, against a reference taken at the start of a piece: see kStreamMax), warp 8 = MMA issue, warp 9 = TMA producer.  The
+//     domain, against a reference that follows the row's maximum: see kStreamSum), warp 8 = MMA issue, warp 9 = TMA producer.  The
 //     producer walks the tile list, and hands each tile's height to the others beside the tile; the MMA warp waits once per step for
 //     (V of tile j, K of tile j + 1) and then only for P, since every further wait or branch between two groups of MMAs
 //     is time the tensor pipe stands still (its queue holds about two MMAs);
@@ -22,10 +22,10 @@
 //     multiplied over ceil(nv / 16) * 16 rows and its softmax stops at the last group of 32.
 //   * every commit after a step's first makes the MMA warp wait until the queue of the tensor pipe has drained, so it commits
 //     only S and O; stages and Q are given back by the softmax warpgroup that sees the last S of a step.
-// What bounds it: the board's 1,000 W cap (1.46-1.65 GHz when run back to back), and at that clock the chain of one Q tile
-// (softmax ~1,130 clk -> P V, Q K^T and hand-overs ~1,350; the tensor pipe works 2,050 of 2,550 clk per KV tile at
-// 167,640 keys x 12 heads, 2,840 before the softmax was streamed).  2,640 queries x 15,840 keys x 12 heads, back
-// to back: 278 us, 273 with the issue path rebuilt, 255 streamed; 4,680 x 32,760 x 40: 3,209 -> 2,960 -> 2,760.
+// What bounds it: the chain of one Q tile (S -> softmax -> P V, Q K^T and the hand-overs between them), of which the two Q tiles
+// hide each other's only in part, at the clock that the board's 1,000 W cap leaves.  2,640 queries x 15,840 keys x 12 heads is
+// one unit of 129 KV tiles on each of 132 SMs: 263 us back to back are 2.04 us per tile, prologue and epilogue included, where the
+// tensor pipe needs 2,048 clk (1.24 us at 1.65 GHz).  4,680 x 32,760 x 40: 2,860 us.
 // Every wait is bounded; a wait that runs out sets WK_DEV_TIMEOUT, the CTA drains and frees its tensor memory.
 #include <stddef.h>
 
@@ -47,15 +47,19 @@ constexpr int kStages = 2, kStagesLse = 4;
 constexpr size_t kSmemBytes = 1024 + 2 * kTileBytes + 2 * kStages * kTileBytes;   // align slack + Q0,Q1 + stages
 constexpr size_t kSmemBytesLse = 1024 + 2 * kTileBytes + kStagesLse * kTileBytes;
 constexpr int kNvRing = 16;   // tile heights handed from the TMA warp to the others; the TMA warp is at most kStagesLse + 1 tiles ahead
-// The softmax has two forms.  Streamed: P = 2^(s * scale - m) with m = the largest of the row's first 32 logits of the
-// piece, so that S is read once and the exponentials of a tile's first columns do not wait for a maximum over its last.
-// bf16 and fp32 share one exponent range: nothing is lost while the sum (at least 1) stays within kStreamMax and O is
-// finite, which each row checks at the end of a piece.  Safe: against a running maximum, for a CTA in which a row failed
-// the check (a logit some 69 natural units above the first 32); it does its work again.  12 heads x 2,640 queries x 15,840
-// keys, back to back: 255 us streamed, 273 with a running maximum for all, 535 when every CTA does both.
-constexpr float kStreamMax = 0x1p100f;
+// The softmax weighs a key with P = 2^(s * scale - m), where m is a maximum that the row has reached: rounded to bf16, the
+// weight of the key that set it is exactly 1, so a dominating key returns its V row unchanged.  (Against a reference that is
+// no maximum, say the largest of the first 32 logits, every weight is rounded: relative error of O 2.3e-3 instead of 2.1e-3 ..
+// 1.6e-3 for logits with a standard deviation of 4 to 16.)  m moves when the maximum has left it by more than kRescaleThreshold.
+// Taking the maximum first costs a pass over S before the first exponential.  A piece's first tile and ragged tiles of more than
+// 64 rows pay for it; other tiles are streamed on trust.  Their sum tells whether that was right: no weight above 2^8 hides in a
+// sum of at most kStreamSum.  A warp in which a row's sum is larger still has all of S (columns 0-63 in tensor memory, the others
+// in registers), moves its references to the maximum and streams the tile again; tiles after that are read for the maximum
+// first, twice as many each time.  12 heads x 2,640 queries x 15,840 keys, back to back: 273 us with the maximum first for all,
+// 263 this way, 259 without the check; logits of standard deviation 4 / 16 / 40 (18,480 keys): 316 / 307 / 305, and 229 at 1.
 constexpr float kRescaleThreshold = 8.0f;           // log2 units: P stays <= 2^8 between maximum updates
-constexpr uint32_t kTmemS = 0, kTmemO = 256;        // tensor-memory columns: S0, S1 (P over them), O0, O1; LSE-only: S0, S1 twice
+constexpr float kStreamSum = 256.0f;
+constexpr uint32_t kTmemS = 0, kTmemP = 64, kTmemO = 256;        // tensor-memory columns: S0, S1 (P over their second half), O0, O1; LSE-only: S0, S1 twice
 constexpr int kPairRows = 2 * kTileQ;
 constexpr int kMaxPieces = 32;                      // most ranges one unit may be cut into
 
@@ -249,7 +253,7 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return d;
 }
 // 2^x of a pair.  The exponentials are the kernel's second bound (16 per clock and SM on the special-function unit, as many
-// clocks per tile as its tensor-core work; 254 us at a share of 1/8 against 258 at 0 and 256 at 2/8 for 12 heads x 15,840
+// clocks per tile as its tensor-core work; 266 us at a share of 0 or 1/8, 263 at 2/8 for 12 heads x 15,840
 // keys), so a share of the pairs takes 2^x from the FMA pipe instead: x = n + f with
 // n = round(x) by the add-a-large-constant trick, 2^f on [-1/2, 1/2] by a cubic (relative error 7.7e-5, far inside the bf16
 // rounding P gets anyway: 2e-3), 2^n by adding n to the exponent field; all in packed fp32 pairs.  That path clamps at
@@ -287,12 +291,12 @@ __device__ __forceinline__ float sum4_f32x2(const uint64_t (&acc)[4]) {
   return a + b;
 }
 
-// P = 2^(s * scale - m) of 32 columns of a row: sums go to four independent (lo, hi) accumulators.  kPoly of every 8 pairs
-// take the FMA pipe; big = the largest of their raw values (the caller checks that they stay below that path's limit).
-template <int kPoly, bool kStore>
+// P = 2^(s * scale - m) of 32 columns of a row: sums go to four independent (lo, hi) accumulators, bf16 pairs to pk (kPack).
+// kPoly of every 8 pairs take the FMA pipe; big = the largest of their raw values (the caller checks that they stay below that
+// path's limit).
+template <int kPoly, bool kPack>
 __device__ __forceinline__ void exp_chunk(uint32_t (&r)[32], int rem, uint64_t scale2, uint64_t neg_m2, uint64_t (&acc)[4],
-                                          float& big, uint32_t tP) {
-  uint32_t pk[16];
+                                          float& big, uint32_t (&pk)[16]) {
   if (rem < 32) {   // columns past the end of the segment or slot
 #pragma unroll
     for (int i = 0; i < 32; ++i) r[i] = i < rem ? r[i] : 0xff800000u;
@@ -309,12 +313,54 @@ __device__ __forceinline__ void exp_chunk(uint32_t (&r)[32], int rem, uint64_t s
       exp2_pair<false>(e, p0, p1);
     }
     acc[i & 3] = add_f32x2(acc[i & 3], pack_f32x2(p0, p1));
-    if (kStore) pk[i] = pack_bf16x2(p0, p1);
+    if (kPack) pk[i] = pack_bf16x2(p0, p1);
   }
-  if (kStore) tmem_st_x16(tP, pk);   // bf16, over S columns that have been read
+}
+// The largest of a row's first nv columns of S, 32 kLoads columns in flight at a time.
+template <int kLoads>
+__device__ __forceinline__ float row_max(uint32_t tS, int nv) {
+  float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll 1
+  for (int c = 0; c < nv; c += 32 * kLoads) {
+    uint32_t r[kLoads][32];
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) tmem_ld_x32(tS + c + 32 * k, r[k]);
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) tc_wait_ld(r[k]);
+    if (nv - c < 32 * kLoads) {
+#pragma unroll
+      for (int i = 0; i < 32 * kLoads; ++i)
+        if (c + i >= nv) r[i >> 5][i & 31] = 0xff800000u;
+    }
+#pragma unroll
+    for (int i = 0; i < 32 * kLoads; i += 2)
+      mx[(i >> 1) & 1] = fmax3(mx[(i >> 1) & 1], __uint_as_float(r[i >> 5][i & 31]), __uint_as_float(r[i >> 5][(i & 31) + 1]));
+  }
+  return fmaxf(mx[0], mx[1]);
+}
+// Moves a row's reference m up to its maximum over the tile in S where that is more than `slack` above it, and the sum l and the
+// accumulator O (if it holds anything yet) with it.
+__device__ __forceinline__ void follow_max(uint32_t tS, uint32_t tO, int nv, float scale_log2, float slack, float& m, float& l, bool has_o) {
+  const float m_new = fmaxf(m, row_max<2>(tS, nv) * scale_log2);
+  const bool move = m_new > m + slack;
+  if (__any_sync(0xffffffffu, move)) {
+    // (the previous P V was issued before this tile's Q K^T: it landed before S did)
+    const float alpha = move ? ex2_approx(m - m_new) : 1.f;
+    if (move) m = m_new;
+    l *= alpha;
+#pragma unroll 1
+    for (int c = 0; c < 128 && has_o; c += 32) {
+      uint32_t r[32];
+      tmem_ld_x32(tO + c, r);
+      tc_wait_ld(r);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
+      tmem_st_x32(tO + c, r);
+    }
+  }
 }
 #ifndef WK_ATTN_POLY
-#define WK_ATTN_POLY 1
+#define WK_ATTN_POLY 2
 #endif
 #ifndef WK_LSE_POLY
 #define WK_LSE_POLY 2
@@ -404,13 +450,13 @@ template <bool kLse>
 struct CtaShared {
   Barriers bars;
   uint32_t tmem;
-  volatile uint32_t abort, again;   // again: a row failed the streamed softmax's check
+  volatile uint32_t abort;
   float2 merge[kLse ? 2 : 1][kLse ? 128 : 1];   // (reference, sum) of a Q tile's odd KV tiles
   volatile int nv[kNvRing];   // valid rows of tile number t (counted over the CTA's pieces) at t % kNvRing
 };
 
-// All of a CTA's work, with the streamed softmax or with a running maximum (safe).
-template <bool kLse, bool safe>
+// All of a CTA's work.
+template <bool kLse>
 __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<kLse>& sh, uint8_t* smem) {
   const uint32_t smem_base = smem_u32(smem);
   uint8_t* sQ = smem;                                   // [2 q tiles][2 halves][128 rows][128 B]
@@ -510,11 +556,11 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
         if (nv == kTileKV) {
 #pragma unroll
           for (int k = 0; k < 8; ++k)
-            mma_ts_if(one, kTmemO + i * 128, kTmemS + i * 128 + k * 8, b + k * 128, idesc_pv, k > 0 ? 1u : accumulate);
+            mma_ts_if(one, kTmemO + i * 128, kTmemP + i * 128 + k * 8, b + k * 128, idesc_pv, k > 0 ? 1u : accumulate);
         } else {
 #pragma unroll 1
           for (int k = 0; k * 16 < nv; ++k)
-            mma_ts_if(one, kTmemO + i * 128, kTmemS + i * 128 + k * 8, b + k * 128, idesc_pv, k > 0 ? 1u : accumulate);
+            mma_ts_if(one, kTmemO + i * 128, kTmemP + i * 128 + k * 8, b + k * 128, idesc_pv, k > 0 ? 1u : accumulate);
         }
       };
       PieceWalker walk;
@@ -570,7 +616,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
         for (int j = -1; j < n_eff; ++j) {
           const bool more = j + 1 < n_eff;
           WK_PROF(0);
-          if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &sh.abort))) break;   // later steps: behind p_full[0]
+          if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &sh.abort))) break;
           WK_PROF(1);
           if (j >= 0) {
             if (!(ok = wait_or_abort(&bars.p_full[0], p_ph0, &sh.abort))) break;
@@ -651,23 +697,15 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
           float big = -INFINITY;
 #pragma unroll 1
           for (int c = 0; c < n_ch; ++c) {
-            uint32_t r[32];
+            uint32_t r[32], none[16];
             tmem_ld_x32(tS + c * 32, r);
             tc_wait_ld(r);
-            exp_chunk<WK_LSE_POLY, false>(r, nv - c * 32, scale2, neg_m2, acc, big, 0);
+            exp_chunk<WK_LSE_POLY, false>(r, nv - c * 32, scale2, neg_m2, acc, big, none);
           }
           sum = sum4_f32x2(acc);
           const bool off = !(sum <= 32768.f) || big * p.scale_log2 - m > 100.f || (first && sum < 2.44140625e-4f);
           if (attempt > 0 || !__any_sync(0xffffffffu, off)) break;
-          float mx = -INFINITY;
-#pragma unroll 1
-          for (int c = 0; c < n_ch; ++c) {
-            uint32_t r[32];
-            tmem_ld_x32(tS + c * 32, r);
-            tc_wait_ld(r);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) mx = fmaxf(mx, i < nv - c * 32 ? __uint_as_float(r[i]) : -INFINITY);
-          }
+          const float mx = row_max<1>(tS, nv);
           if (off) {
             const float m_new = first ? mx * p.scale_log2 : fmaxf(m, mx * p.scale_log2);
             l *= ex2_approx(m - m_new);
@@ -713,6 +751,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const uint32_t tS = lane_base + kTmemS + wg * 128;
+    const uint32_t tP = lane_base + kTmemP + wg * 128;
     const uint32_t tO = lane_base + kTmemO + wg * 128;
     PieceWalker walk;
     walk.init(p);
@@ -731,7 +770,8 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       // makes it wait until the queue of the tensor pipe has drained.
       const bool releases = wg == (pc.has_q1 ? 1 : 0);
       const int n_eff = count_tiles(p, pc.tb, pc.te);
-      float m_used = -INFINITY, l = 0.f, big = -INFINITY;
+      float m_used = -INFINITY, l = 0.f;
+      int careful = 0, redos = 0;   // tiles whose maximum is taken first from here on; tiles streamed twice so far
       int j = 0;
       if (active) {
         while (j < n_eff) {
@@ -744,80 +784,84 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
             if (j + 1 == n_eff) mbar_arrive(&bars.q_empty);
           }
           tc_fence_after();
-          const int n_ch = (nv + 31) >> 5;
-          if (safe) {   // move the reference when the row's maximum has left it by more than the threshold
-            float mx = -INFINITY;
-#pragma unroll 1
-            for (int c = 0; c < n_ch; ++c) {
-              uint32_t r[32];
-              tmem_ld_x32(tS + c * 32, r);
-              tc_wait_ld(r);
-#pragma unroll
-              for (int i = 0; i < 32; ++i) mx = fmaxf(mx, i < nv - c * 32 ? __uint_as_float(r[i]) : -INFINITY);
-            }
-            const float m_new = fmaxf(m_used, mx * p.scale_log2);
-            const bool move = m_new > m_used + kRescaleThreshold;    // also true on the first tile (m_used = -inf)
-            if (__any_sync(0xffffffffu, move)) {
-              // (the previous P V was issued before this tile's Q K^T: it landed before S did)
-              const float alpha = move ? ex2_approx(m_used - m_new) : 1.f;
-              if (move) m_used = m_new;
-              l *= alpha;
-#pragma unroll 1
-              for (int c = 0; c < 4 && j > 0; ++c) {
-                uint32_t r[32];
-                tmem_ld_x32(tO + c * 32, r);
-                tc_wait_ld(r);
-#pragma unroll
-                for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
-                tmem_st_x32(tO + c * 32, r);
-              }
-            }
-          }
-          // The row is streamed from tensor memory 32 columns at a time; the next 32 are in flight while these are worked on.
-          {
+          // known: the row's maximum over the tile is taken before the exponentials
+          bool known = j == 0 || (nv > 64 && nv < kTileKV) || careful > 0;
+          float slack = kRescaleThreshold;
+          if (careful > 0) --careful;
+          for (;;) {
+            if (known) follow_max(tS, tO, nv, p.scale_log2, slack, m_used, l, j > 0);
+            // The row is streamed from tensor memory 32 columns at a time; the next 32 are in flight while these are worked on.
             uint64_t acc[4] = {0, 0, 0, 0};
-            uint32_t ra[32], rb[32];
-            tmem_ld_x32(tS, ra);
-            if (!safe && j == 0) {
-              tc_wait_ld(ra);
-              float mx[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-              for (int i = 0; i < 32; i += 2)
-                mx[(i >> 1) & 1] = fmax3(mx[(i >> 1) & 1], i < nv ? __uint_as_float(ra[i]) : -INFINITY,
-                                         i + 1 < nv ? __uint_as_float(ra[i + 1]) : -INFINITY);
-              m_used = fmaxf(mx[0], mx[1]) * p.scale_log2;
-            }
             const uint64_t neg_m2 = pack_f32x2(-m_used, -m_used);
+            float big = -INFINITY;
+            uint32_t ra[32], rb[32];
             WK_PROF(2);
             if (nv == kTileKV) {
-#pragma unroll
-              for (int c = 0; c < 4; c += 2) {
-                tc_wait_ld(ra);
-                tmem_ld_x32(tS + c * 32 + 32, rb);
-                exp_chunk<WK_ATTN_POLY, true>(ra, 32, scale2, neg_m2, acc, big, tS + c * 16);
-                tc_wait_ld(rb);
-                if (c < 2) tmem_ld_x32(tS + c * 32 + 64, ra);
-                exp_chunk<WK_ATTN_POLY, true>(rb, 32, scale2, neg_m2, acc, big, tS + c * 16 + 16);
+              tmem_ld_x32(tS, ra);
+              // P goes over columns 64-127 once these are in registers, where they stay until S is not needed again.
+              uint32_t p0[16], p1[16];
+              tc_wait_ld(ra);
+              tmem_ld_x32(tS + 32, rb);
+              exp_chunk<WK_ATTN_POLY, true>(ra, 32, scale2, neg_m2, acc, big, p0);
+              tc_wait_ld(rb);
+              tmem_ld_x32(tS + 64, ra);
+              exp_chunk<WK_ATTN_POLY, true>(rb, 32, scale2, neg_m2, acc, big, p1);
+              tc_wait_ld(ra);
+              tmem_st_x16(tP, p0);
+              tmem_st_x16(tP + 16, p1);
+              tmem_ld_x32(tS + 96, rb);
+              exp_chunk<WK_ATTN_POLY, true>(ra, 32, scale2, neg_m2, acc, big, p0);
+              tc_wait_ld(rb);
+              tmem_st_x16(tP + 32, p0);
+              exp_chunk<WK_ATTN_POLY, true>(rb, 32, scale2, neg_m2, acc, big, p1);
+              tmem_st_x16(tP + 48, p1);
+              if (!known && __any_sync(0xffffffffu, !(sum4_f32x2(acc) <= kStreamSum) || big * p.scale_log2 - m_used > 100.f)) {
+                tc_wait_st();
+                tmem_st_x32(tS + 64, ra);
+                tmem_st_x32(tS + 96, rb);
+                tc_wait_st();
+                known = true;
+                slack = 0.f;
+                careful = 1 << min(++redos, 6);
+                continue;
               }
             } else {
+              // P of columns 0-63 lies over columns 64-95, of the others over groups behind their own: last columns first.
+              uint32_t pk[16];
 #pragma unroll 1
-              for (int c = 0; c < n_ch; ++c) {
+              for (int c = (nv - 1) & ~31; c >= 64; c -= 32) {
+                tmem_ld_x32(tS + c, ra);
                 tc_wait_ld(ra);
-                exp_chunk<WK_ATTN_POLY, true>(ra, nv - c * 32, scale2, neg_m2, acc, big, tS + c * 16);
-                if (c + 1 < n_ch) tmem_ld_x32(tS + c * 32 + 32, ra);
+                exp_chunk<0, true>(ra, nv - c, scale2, neg_m2, acc, big, pk);
+                tmem_st_x16(tP + c / 2, pk);
+              }
+              tmem_ld_x32(tS, ra);
+              if (nv > 32) {
+                tmem_ld_x32(tS + 32, rb);
+                tc_wait_ld(ra);
+                tc_wait_ld(rb);
+                exp_chunk<0, true>(rb, nv - 32, scale2, neg_m2, acc, big, pk);
+                tmem_st_x16(tP + 16, pk);
+              } else {
+                tc_wait_ld(ra);
+              }
+              exp_chunk<0, true>(ra, nv, scale2, neg_m2, acc, big, pk);
+              tmem_st_x16(tP, pk);
+              if (!known && __any_sync(0xffffffffu, !(sum4_f32x2(acc) <= kStreamSum))) {
+                known = true;
+                slack = 0.f;
+                careful = 1 << min(++redos, 6);
+                continue;
               }
             }
             l += sum4_f32x2(acc);
             WK_PROF(4);
+            break;
           }
           tc_wait_st();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) {
-            // The MMA warp's next step reads this tile's V and the next tile's K as well.  Waiting for them here leaves it
-            // one barrier less to look at between two groups of MMAs (about 200 clocks each).
-            mbar_arrive(&bars.p_full[wg]);   // one arrival per warp: the wait above covered all 32 lanes' stores
-          }
+          if (lane == 0) mbar_arrive(&bars.p_full[wg]);   // one arrival per warp: the wait above covered all 32 lanes' stores
           WK_PROF(5);
           ++j;
           ++g;
@@ -829,7 +873,6 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
         if (ok && j > 0 && releases && row == 0) mbar_arrive(&bars.kv_empty[(steps + n_eff) % kNStages]);   // the last V
         if (ok) {
           tc_fence_after();
-          uint32_t o_max = 0;   // bits of the largest |O|
           const float inv_l = (j > 0 && l > 0.f) ? 1.f / l : 0.f;
           const float lse = (j > 0 && l > 0.f) ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
 #pragma unroll
@@ -838,8 +881,6 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
             if (j > 0) {
               tmem_ld_x32(tO + c * 32, r);
               tc_wait_ld(r);
-#pragma unroll
-              for (int i = 0; i < 32; ++i) o_max = max(o_max, r[i] & 0x7fffffffu);
             } else {
 #pragma unroll
               for (int i = 0; i < 32; ++i) r[i] = 0u;
@@ -871,8 +912,6 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
             } else {
               p.lsepart[static_cast<int64_t>(pc.slot) * kPairRows + prow] = lse;
             }
-            const bool fine = l <= kStreamMax && big * p.scale_log2 - m_used < 120.f && o_max < 0x7f800000u;   // false for NaN
-            if (j > 0 && !safe && !fine) sh.again = 1;
           }
         }
       }
@@ -889,10 +928,6 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
     WK_PROF_FLUSH(0, 8, blockIdx.x == 0 && tid == 0);
   }
 }
-// The second pass is a call: inlined, it costs the first one registers (12 heads x 15,840 keys: 264 against 256 us).
-__device__ __noinline__ void attention_again(const AttnParams& p, CtaShared<false>& sh, uint8_t* smem) {
-  attention_roles<false, true>(p, sh, smem);
-}
 
 template <bool kLse>
 __global__ void __launch_bounds__(kThreads<kLse>, 1)
@@ -901,7 +936,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
   uint8_t* smem = smem_raw + (((smem_u32(smem_raw) + 1023u) & ~1023u) - smem_u32(smem_raw));
   __shared__ CtaShared<kLse> sh;
   const int tid = threadIdx.x;
-  auto init_barriers = [&]() {
+  if (tid == 0) {
     mbar_init(&sh.bars.q_full, 1);
     mbar_init(&sh.bars.q_empty, 1);
     for (int s = 0; s < kStagesLse; ++s) { mbar_init(&sh.bars.kv_full[s], 1); mbar_init(&sh.bars.kv_empty[s], 1); }
@@ -913,10 +948,6 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
       mbar_init(&sh.bars.m_empty[i], 4);
     }
     fence_mbar_init();
-  };
-  if (tid == 0) {
-    init_barriers();
-    sh.again = 0;
     sh.abort = 0;
   }
   if (tid < 32) {
@@ -932,23 +963,9 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
   // an allocation of all 512 columns starts at column 0; addresses known at compile time keep the MMAs' operands cheap
   if (sh.tmem != 0 && tid == 0) { sh.abort = 1; atomicOr(p.status, WK_DEV_TIMEOUT); }
 
-  attention_roles<kLse, false>(p, sh, smem);
+  attention_roles<kLse>(p, sh, smem);
   tc_fence_before();
   __syncthreads();
-  if constexpr (!kLse) {
-    if (sh.again && !sh.abort) {   // the same for all threads
-      // All roles have finished and nothing is in flight: the barriers start afresh, and so do the roles.
-      if (tid == 0) {
-        for (uint32_t i = 0; i < sizeof(Barriers) / 8; ++i) mbar_inval(reinterpret_cast<uint64_t*>(&sh.bars) + i);
-        init_barriers();
-      }
-      __syncthreads();
-      tc_fence_after();
-      attention_again(p, sh, smem);
-      tc_fence_before();
-      __syncthreads();
-    }
-  }
   if (tid < 32) tmem_dealloc(sh.tmem, 512);
 }
 

@@ -1,0 +1,68 @@
+"""Attention where the result is known to the last bit: a key that outweighs all others by more than fp32 resolves has weight
+1, so its V row comes back unchanged wherever the key stands; and a call that writes its output over its queries."""
+import numpy as np
+import pytest
+import torch
+
+import wkinputs as wi
+from wkinputs import device as wd
+
+pytestmark = pytest.mark.gpu
+SCALE = 1.0 / np.sqrt(128.0)
+
+
+def bf16(x):
+    return wi.f32_to_bf16_bits(np.asarray(x, dtype=np.float32))
+
+
+def normals(stream, shape):
+    return wi.normal_f32(83, wi.STREAM_MISC + stream, np.arange(int(np.prod(shape)), dtype=np.uint64)).reshape(shape)
+
+
+def context(H, lq):
+    from paper_2605_22718_b200 import WorldKV
+    return WorldKV(n_layers=1, n_heads=H, tokens_per_frame=8, n_keep=4, pool_slots=1, max_k=1, max_lq=lq, max_splits=8)
+
+
+# the first tile's ends and the middle of its 32-column groups; the first, middle and last row of later and of short tiles
+@pytest.mark.parametrize("n,at", [(390, at) for at in (0, 31, 32, 63, 64, 100, 127, 128, 200, 255, 256, 383, 384, 389)] +
+                         [(440, 400), (440, 420), (440, 439), (480, 384), (480, 440), (480, 479)])
+def test_dominating_key_returns_its_value_row(n, at):
+    """Logits of the key: 43 to 56; of all others: below 7.  480 of them weigh 480 e^-33 < 2^-38 together: nothing beside 1
+    in fp32, and far less than half a bf16 step in any output component."""
+    H, lq = 2, 300
+    q, k = normals(1, (lq, H, 128)), normals(2, (n, H, 128))
+    q[:, :, 0] = (16.0 + np.arange(lq) % 17 / 4)[:, None]
+    k[:, :, 0] = 0.0
+    k[at] = 0.0
+    k[at, :, 0] = 31.0
+    Q, K, V = (wd.to_device_bf16(bf16(x)) for x in (q, k, normals(3, (n, H, 128))))
+    logits = torch.einsum("qhd,khd->hqk", Q.float(), K.float()) * SCALE
+    assert float(logits[:, :, at].min()) > 40.0
+    logits[:, :, at] = 0.0
+    assert float(logits.max()) < 7.0
+    kv = context(H, lq)
+    for splits in (1, 0, 3):
+        O = kv.memory_attention(0, Q, [(K, V)], None, 0, kv_splits=splits)
+        assert kv.poll_status() == (0, 0)
+        assert torch.equal(O, V[at].expand(lq, H, 128)), f"splits {splits}"
+
+
+@pytest.mark.parametrize("rise", [0.0, 100.0])
+@pytest.mark.parametrize("H,lq,n", [(2, 300, 700), (12, 880, 300), (40, 1100, 200)])
+def test_output_over_the_queries(H, lq, n, rise):
+    """O may be Q itself: each (head, query block) is read before it is written.  rise: logits of a few rows grow by that
+    much (natural units) from key 150 on."""
+    q, k = normals(4, (lq, H, 128)), normals(5, (n, H, 128))
+    q[:, :, 0] = 0.0
+    for h, r in ((0, 3), (H - 1, lq - 1), (H // 2, 200)):
+        q[r, h, 0] = 16.0
+    k[:, :, 0] = (rise * (np.arange(n) >= 150))[:, None] / (16.0 * SCALE)
+    Q, K, V = (wd.to_device_bf16(bf16(x)) for x in (q, k, normals(6, (n, H, 128))))
+    kv = context(H, lq)
+    for splits in (1, 0, 3):
+        want = kv.memory_attention(0, Q, [(K, V)], None, 0, kv_splits=splits)
+        X = Q.clone()
+        kv.memory_attention(0, X, [(K, V)], None, 0, O=X, kv_splits=splits)
+        assert kv.poll_status() == (0, 0)
+        assert torch.equal(X, want), f"splits {splits}"

@@ -1,6 +1,6 @@
-"""Memory attention where logits leave the range of the streamed softmax (a row's reference is the largest of its first 32
-logits, its sum may reach 2^100): such a CTA does its work again against a running maximum.  Values scaled by a power of two
-(exact in bf16) are compared after scaling back, so the tolerance is the usual one."""
+"""Memory attention where logits leave the range in which a tile is streamed without a look at its maximum (a weight above
+2^8 against the row's reference): such a tile is streamed again against its maximum.  Values scaled by a power of two (exact in
+bf16) are compared after scaling back, so the tolerance is the usual one."""
 import numpy as np
 import pytest
 import torch
