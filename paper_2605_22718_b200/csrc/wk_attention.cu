@@ -121,9 +121,9 @@ struct TileIter {
       ok = false;
       z = 0;
       if (si < p.n_slots) {
-        const int slot = __ldg(p.slots + si);
+        const int slot = ld_dep(p.slots + si);
         ok = slot >= 0 && slot < p.pool_slots;
-        if (ok) ok = __ldg(p.valid + slot) != 0;
+        if (ok) ok = ld_dep(p.valid + slot) != 0;
         if (!ok && report && slot != -1) atomicOr(p.status, WK_DEV_BAD_SLOT);   // never dereferenced
         if (ok) z = p.layer * p.pool_slots + slot;
       }
@@ -176,8 +176,8 @@ __device__ __forceinline__ int count_tiles(const AttnParams& p, int tb, int te) 
   if (ue > ub) {
     const int last = (ue - 1) / p.tiles_per_slot;
     for (int si = ub / p.tiles_per_slot + static_cast<int>(threadIdx.x & 31); si <= last; si += 32) {
-      const int slot = __ldg(p.slots + si);
-      if (slot >= 0 && slot < p.pool_slots && __ldg(p.valid + slot) != 0)
+      const int slot = ld_dep(p.slots + si);
+      if (slot >= 0 && slot < p.pool_slots && ld_dep(p.valid + slot) != 0)
         n += min(ue, (si + 1) * p.tiles_per_slot) - max(ub, si * p.tiles_per_slot);
     }
     n = __reduce_add_sync(0xffffffffu, n);

@@ -113,13 +113,13 @@ retrieve_small(const float* __restrict__ poses, const int32_t* __restrict__ vali
   if (tid < n_slots) {
     float p[8];
     if (kVec) {
-      const float4 a = __ldg(reinterpret_cast<const float4*>(poses) + 2 * tid), b = __ldg(reinterpret_cast<const float4*>(poses) + 2 * tid + 1);
+      const float4 a = ld_dep(reinterpret_cast<const float4*>(poses) + 2 * tid), b = ld_dep(reinterpret_cast<const float4*>(poses) + 2 * tid + 1);
       p[0] = a.x; p[1] = a.y; p[2] = a.z; p[4] = b.x; p[5] = b.y; p[6] = b.z; p[7] = b.w;
     } else {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) p[i] = __ldg(poses + tid * 8 + i);
+      for (int i = 0; i < 8; ++i) p[i] = ld_dep(poses + tid * 8 + i);
     }
-    if (__ldg(valid + tid)) {
+    if (ld_dep(valid + tid)) {
       const double dx = static_cast<double>(p[0]) - static_cast<double>(cur.v[0]);
       const double dy = static_cast<double>(p[1]) - static_cast<double>(cur.v[1]);
       const double dz = static_cast<double>(p[2]) - static_cast<double>(cur.v[2]);

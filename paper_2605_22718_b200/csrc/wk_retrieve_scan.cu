@@ -124,9 +124,9 @@ scan_max(const float4* __restrict__ poses, const int32_t* __restrict__ valid, in
       const int64_t i = i0 + u * stride;
       live[u] = i < n;
       if (live[u]) {
-        a[u] = __ldg(poses + 2 * i);
-        b[u] = __ldg(poses + 2 * i + 1);
-        if (valid) live[u] = __ldg(valid + i) != 0;
+        a[u] = ld_dep(poses + 2 * i);
+        b[u] = ld_dep(poses + 2 * i + 1);
+        if (valid) live[u] = ld_dep(valid + i) != 0;
       }
     }
 #pragma unroll
@@ -201,9 +201,9 @@ scan_sample(const float4* __restrict__ poses, const int32_t* __restrict__ valid,
       a[u] = make_float4(0.f, 0.f, 0.f, 0.f);
       b[u] = a[u];
       if (ok[u]) {
-        if (valid) vflag[u] = __ldg(valid + ci[u]);
-        a[u] = __ldg(poses + 2 * ci[u]);
-        b[u] = __ldg(poses + 2 * ci[u] + 1);
+        if (valid) vflag[u] = ld_dep(valid + ci[u]);
+        a[u] = ld_dep(poses + 2 * ci[u]);
+        b[u] = ld_dep(poses + 2 * ci[u] + 1);
       }
     }
     float t32[kSampleBatch], ad32[kSampleBatch];
@@ -585,7 +585,7 @@ scan_select(const float4* __restrict__ poses, const int32_t* __restrict__ valid_
   const bool listed = max_rec == nullptr && h->overflow == 0u;
   const int64_t n = listed ? static_cast<int64_t>(h->n_surv) : n_all;
   const int32_t* valid = listed ? nullptr : valid_all;      // listed candidates have been checked already
-  auto cand_of = [&](int64_t e) -> int32_t { return listed ? static_cast<int32_t>(__ldg(surv + e)) : static_cast<int32_t>(e); };
+  auto cand_of = [&](int64_t e) -> int32_t { return listed ? static_cast<int32_t>(__ldcg(surv + e)) : static_cast<int32_t>(e); };
   double mt, md;
   if (max_rec) {   // the records of scan_max, one per lane of every warp at a time
     mt = 0.0;
