@@ -190,7 +190,8 @@ wk_status wk_retrieve_query(wk_ctx* ctx, int32_t layer, const void* Q, int32_t l
  * wk_retrieve: squared-L2 translation distance and geodesic rotation angle, each divided by its maximum over the valid
  * candidates, summed, in fp64; the min(k, valid candidates) smallest win, ties to the lowest index, rank order).  For
  * candidate sets far beyond a pool's slot table (the paper's pools hold 10^2..10^3 chunks; this call is what makes
- * "GB/s of retrieval" measurable at 2^16..2^24 poses).  The poses are read once: a sampled set of k real candidates
+ * "GB/s of retrieval" measurable at 2^16..2^24 poses).  Up to 2^17 poses with k <= 16 are read twice (the second time from
+ * L2): first for the two maxima, then for the distances.  Longer arrays, and longer lists, are read once: a sampled set of k real candidates
  * rules most others out before the two maxima are known (a candidate that k others beat for every possible pair of
  * maxima is not among the k best); the few that remain are ranked exactly afterwards.  Pose sets where nothing can be
  * ruled out (e.g. all rotations equal) are read a second time instead; the result is the same either way.  A pose with
@@ -216,9 +217,9 @@ wk_status wk_retrieve_scan(wk_ctx* ctx, const float* poses_dev, const int32_t* v
  *   wk_retrieve (entries past min(k, M) are -1 / 0).
  * Limits and caveats: n_slots <= 4096, else WK_ERR_SHAPE and nothing is launched.  The first call on each device looks
  * up the array's device address (cudaGetSymbolAddress, with that device current); make that first call outside any
- * stream capture.  All calls on a device share the one array: two calls whose kernels may overlap on the GPU
- * (different streams) race on it; calls on one stream are safe.  Nothing in the array has to start at zero: every
- * entry a call reads it has written first.  Calls no cudaMalloc/cudaFree and no allocating library routine.
+ * stream capture.  Pools of up to 1,024 slots are ranked in registers and shared memory and leave the array alone.  Calls
+ * for larger pools on a device share it: two of them whose kernels may overlap on the GPU (different streams) race on it;
+ * calls on one stream are safe.  Nothing in the array has to start at zero: every entry a call reads it has written first.  Calls no cudaMalloc/cudaFree and no allocating library routine.
  * A pose with a NaN/Inf component is not a candidate (there is no status word to report it through here).
  * Errors: WK_ERR_ARG, WK_ERR_SHAPE, WK_ERR_NO_DEVICE, WK_ERR_CUDA. */
 wk_status wk_retrieve_noalloc(const float* poses_dev, const int32_t* valid_dev, int32_t n_slots,
@@ -237,7 +238,8 @@ typedef struct {
 /* O = softmax(scale * Q K^T) V per head, unmasked, over the dense segments (denoising chunk, window,
  * sink ...) followed by the stored rows of each listed pool slot of `layer`.  Nothing is concatenated
  * in memory: K/V tiles are fetched where they lie.
- *   Q [lq][H][128] bf16, O same shape; lse_out [H][lq] fp32 (natural log) or NULL
+ *   Q [lq][H][128] bf16, O same shape; O may be Q itself, but must not overlap it otherwise, nor any K or V that the call
+ *             reads; lse_out [H][lq] fp32 (natural log) or NULL
  *   slots_dev [n_slots] int32 in device memory (e.g. wk_retrieve's output); an entry that is -1 is
  *             skipped silently, any other out-of-range or invalid entry is skipped and sets
  *             WK_DEV_BAD_SLOT; a slot listed twice is attended twice

@@ -24,8 +24,8 @@
 //     only S and O; stages and Q are given back by the softmax warpgroup that sees the last S of a step.
 // What bounds it: the chain of one Q tile (S -> softmax -> P V, Q K^T and the hand-overs between them), of which the two Q tiles
 // hide each other's only in part, at the clock that the board's 1,000 W cap leaves.  2,640 queries x 15,840 keys x 12 heads is
-// one unit of 129 KV tiles on each of 132 SMs: 263 us back to back are 2.04 us per tile, prologue and epilogue included, where the
-// tensor pipe needs 2,048 clk (1.24 us at 1.65 GHz).  4,680 x 32,760 x 40: 2,860 us.
+// one unit of 129 KV tiles on each of 132 SMs: 259 to 263 us back to back, at 1,687 MHz 3,380 clk per tile, prologue and epilogue
+// included, where the tensor pipe needs 2,048.  4,680 x 32,760 x 40 (1,575 MHz): 2,850 us.
 // Every wait is bounded; a wait that runs out sets WK_DEV_TIMEOUT, the CTA drains and frees its tensor memory.
 #include <stddef.h>
 
@@ -50,7 +50,7 @@ constexpr int kNvRing = 16;   // tile heights handed from the TMA warp to the ot
 // The softmax weighs a key with P = 2^(s * scale - m), where m is a maximum that the row has reached: rounded to bf16, the
 // weight of the key that set it is exactly 1, so a dominating key returns its V row unchanged.  (Against a reference that is
 // no maximum, say the largest of the first 32 logits, every weight is rounded: relative error of O 2.3e-3 instead of 2.1e-3 ..
-// 1.6e-3 for logits with a standard deviation of 4 to 16.)  m moves when the maximum has left it by more than kRescaleThreshold.
+// 1.7e-3 for logits with a standard deviation of 4 to 16.)  m moves when the maximum has left it by more than kRescaleThreshold.
 // Taking the maximum first costs a pass over S before the first exponential.  A piece's first tile and ragged tiles of more than
 // 64 rows pay for it; other tiles are streamed on trust.  Their sum tells whether that was right: no weight above 2^8 hides in a
 // sum of at most kStreamSum.  A warp in which a row's sum is larger still has all of S (columns 0-63 in tensor memory, the others
@@ -1062,9 +1062,10 @@ static void split_default(int64_t units, int64_t tiles, int64_t sms, int64_t* G,
   *ranges = 0;
   if (rest == 0 || (sms - rest) * tiles < 4 * sms + 16 * rest) return;
   *n_full = waves * sms;
-  // Where whole cuts of every unit use nearly all SMs, no CTA gets two pieces; pieces of fewer than 4 tiles cost more in
-  // prologues and partials than they save (2 heads x 3,960 keys: 144 unaligned ranges 23.3 us, 128 aligned 21.2, 64
-  // aligned 20.1, 40 unaligned 24.9).
+  // Where whole cuts of every unit use nearly all SMs, no CTA gets two pieces, and such pieces are kept at 4 tiles or more:
+  // shorter ones cost more in prologues and partials than they save (2 heads x 3,960 keys: 144 unaligned ranges 23.3 us, 128
+  // aligned 21.2, 64 aligned 20.1, 40 unaligned 24.9).  Otherwise a range per SM, however short; 30 units, whole / 148 ranges / 120
+  // aligned cuts: 10 tiles 25.0 / 22.6 / 19.9 us, 20 tiles 41.1 / 26.5 / 23.3, 40 tiles 73.0 / 34.8 / 31.4.
   int64_t cuts = sms / rest;
   if (cuts > kMaxPieces - 2) cuts = kMaxPieces - 2;
   int64_t r = sms;

@@ -31,8 +31,9 @@ struct AppendParams {
 // Bound by memory (5.6-6.5 TB/s of reads and writes).  One warp per stored row, 16-byte vectors, four loads in flight per
 // lane before the first store.  With per-head keep-sets (hs = n_heads index lists per layer) every 128-column block of a
 // stored row has its own source token.  Behind a selection, the anchor frame needs no index list: the scoring kernels have
-// stored its K rows and, at widths up to 2,048 columns, its V rows; where they have not, V's are copied by the first blocks,
-// which do not wait for the selection.
+// stored its K rows and, where score_select runs (see AnchorStore), its V rows; where they have not (compress_fused, per-head
+// keys, calls without scores), V's are copied by the first blocks, which need no index list.  The kernels in front of those
+// calls do not let this one start before they end, so nothing overlaps there; the rows are contiguous on both sides.
 __global__ void __launch_bounds__(kAppendThreads)
 append_rows(const __grid_constant__ AppendParams p) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -44,8 +45,8 @@ append_rows(const __grid_constant__ AppendParams p) {
     if (threadIdx.x == 0) p.valid[p.mark_slot] = 1;
   }
   if (id < p.v_anchor_blocks) {
-    // (every earlier kernel on the stream but the selection has finished: the scoring kernel lets this one start only
-    // after it has waited for them itself)
+    // (every earlier kernel on the stream but the selection has finished: a scoring kernel lets this one start only after
+    // it has waited for them itself)
     const int per = (p.T + kAppendRows - 1) / kAppendRows;
     const int l = id / per, r0 = (id - l * per) * kAppendRows, rows = min(kAppendRows, p.T - r0);
     const uint4* src = reinterpret_cast<const uint4*>(p.Vsrc + static_cast<int64_t>(l) * p.stride) + static_cast<int64_t>(r0) * vecs;
