@@ -54,12 +54,19 @@ constexpr int kNvRing = 16;   // tile heights handed from the TMA warp to the ot
 // Taking the maximum first costs a pass over S before the first exponential.  A piece's first tile and ragged tiles of more than
 // 64 rows pay for it; other tiles are streamed on trust.  Their sum tells whether that was right: no weight above 2^8 hides in a
 // sum of at most kStreamSum.  A warp in which a row's sum is larger still has all of S (columns 0-63 in tensor memory, the others
-// in registers), moves its references to the maximum and streams the tile again; tiles after that are read for the maximum
-// first, twice as many each time.  12 heads x 2,640 queries x 15,840 keys, back to back: 273 us with the maximum first for all,
-// 263 this way, 259 without the check; logits of standard deviation 4 / 16 / 40 (18,480 keys): 316 / 307 / 305, and 229 at 1.
+// in registers), moves its references to the maximum where that is more than 2^8 above, and streams the tile again; tiles after
+// that are read for the maximum first, twice as many each time.  12 heads x 2,640 queries x 15,840 keys, back to back: 273 us with
+// the maximum first for all, 263 this way, 259 without the check; logits of standard deviation 4 / 16 / 40 (18,480 keys): 328 /
+// 308 / 307 us, and 232 at 1.
 constexpr float kRescaleThreshold = 8.0f;           // log2 units: P stays <= 2^8 between maximum updates
 constexpr float kStreamSum = 256.0f;
-constexpr uint32_t kTmemS = 0, kTmemP = 64, kTmemO = 256;        // tensor-memory columns: S0, S1 (P over their second half), O0, O1; LSE-only: S0, S1 twice
+// Pieces of at most kFewTiles tiles move the reference to every tile's own maximum, down as well as up: beside few other keys a
+// tile's largest weight counts, and it is exact this way, as if the tile were a piece of its own.  450 queries x 5 heads x 1,040
+// keys (pieces of three tiles), relative error of O at deviations 1 / 2 / 4: 2.13 / 1.80 / 1.69e-3, without 2.27 / 2.19 / 1.98e-3; 2
+// heads x 3,960 keys (four tiles) 20.6 us, without 19.2.  No call is cut into more such pieces for it: that was slower (38.9 us).
+constexpr int kFewTiles = 4;
+// tensor-memory columns: S0, S1 (P over their second half), O0, O1; LSE-only: S0, S1 twice
+constexpr uint32_t kTmemS = 0, kTmemP = 64, kTmemO = 256;
 constexpr int kPairRows = 2 * kTileQ;
 constexpr int kMaxPieces = 32;                      // most ranges one unit may be cut into
 
@@ -338,15 +345,16 @@ __device__ __forceinline__ float row_max(uint32_t tS, int nv) {
   }
   return fmaxf(mx[0], mx[1]);
 }
-// Moves a row's reference m up to its maximum over the tile in S where that is more than `slack` above it, and the sum l and the
-// accumulator O (if it holds anything yet) with it.
-__device__ __forceinline__ void follow_max(uint32_t tS, uint32_t tO, int nv, float scale_log2, float slack, float& m, float& l, bool has_o) {
-  const float m_new = fmaxf(m, row_max<2>(tS, nv) * scale_log2);
-  const bool move = m_new > m + slack;
+// Moves a row's reference m, and the sum l and the accumulator O (if it holds anything yet) with it: up to the row's maximum over
+// the tile in S when that is more than kRescaleThreshold above it, or, with `own`, to that maximum wherever it is (unless the
+// tile's weights are negligible beside those before it).
+__device__ __forceinline__ void follow_max(uint32_t tS, uint32_t tO, int nv, float scale_log2, bool own, float& m, float& l, bool has_o) {
+  const float mt = row_max<2>(tS, nv) * scale_log2;
+  const bool move = own ? mt > m - 20.f && mt != m : mt > m + kRescaleThreshold;   // also true on the first tile (m = -inf)
   if (__any_sync(0xffffffffu, move)) {
     // (the previous P V was issued before this tile's Q K^T: it landed before S did)
-    const float alpha = move ? ex2_approx(m - m_new) : 1.f;
-    if (move) m = m_new;
+    const float alpha = move ? ex2_approx(m - mt) : 1.f;
+    if (move) m = mt;
     l *= alpha;
 #pragma unroll 1
     for (int c = 0; c < 128 && has_o; c += 32) {
@@ -771,6 +779,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       const bool releases = wg == (pc.has_q1 ? 1 : 0);
       const int n_eff = count_tiles(p, pc.tb, pc.te);
       float m_used = -INFINITY, l = 0.f;
+      const bool few = n_eff <= kFewTiles;
       int careful = 0, redos = 0;   // tiles whose maximum is taken first from here on; tiles streamed twice so far
       int j = 0;
       if (active) {
@@ -785,11 +794,10 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
           }
           tc_fence_after();
           // known: the row's maximum over the tile is taken before the exponentials
-          bool known = j == 0 || (nv > 64 && nv < kTileKV) || careful > 0;
-          float slack = kRescaleThreshold;
+          bool known = few || j == 0 || (nv > 64 && nv < kTileKV) || careful > 0;
           if (careful > 0) --careful;
           for (;;) {
-            if (known) follow_max(tS, tO, nv, p.scale_log2, slack, m_used, l, j > 0);
+            if (known) follow_max(tS, tO, nv, p.scale_log2, few, m_used, l, j > 0);
             // The row is streamed from tensor memory 32 columns at a time; the next 32 are in flight while these are worked on.
             uint64_t acc[4] = {0, 0, 0, 0};
             const uint64_t neg_m2 = pack_f32x2(-m_used, -m_used);
@@ -821,7 +829,6 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
                 tmem_st_x32(tS + 96, rb);
                 tc_wait_st();
                 known = true;
-                slack = 0.f;
                 careful = 1 << min(++redos, 6);
                 continue;
               }
@@ -849,7 +856,6 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
               tmem_st_x16(tP, pk);
               if (!known && __any_sync(0xffffffffu, !(sum4_f32x2(acc) <= kStreamSum))) {
                 known = true;
-                slack = 0.f;
                 careful = 1 << min(++redos, 6);
                 continue;
               }

@@ -48,6 +48,29 @@ def test_dominating_key_returns_its_value_row(n, at):
         assert torch.equal(O, V[at].expand(lq, H, 128)), f"splits {splits}"
 
 
+@pytest.mark.parametrize("n,first,second", [(390, 5, 200), (390, 200, 5), (390, 60, 388), (390, 388, 60), (390, 130, 300),
+                                            (200, 3, 150), (200, 150, 3), (512, 100, 511), (512, 511, 100), (512, 127, 128)])
+def test_largest_weight_of_every_tile_in_short_pieces(n, first, second):
+    """Two keys of different tiles share all of the weight, and their V rows no component, so each half of O is one rounded
+    product w V.  Both weights are exact but for 2^x (1e-4), hence O is within half a bf16 step (2^-8) of it and 1e-4."""
+    H, lq = 2, 300
+    q, k, v = normals(7, (lq, H, 128)), normals(8, (n, H, 128)), normals(9, (n, H, 128))
+    q[:, :, 0] = (16.0 + np.arange(lq) % 17 / 4)[:, None]
+    q[:, :, 1] = q[:, :, 0] - (np.arange(lq) % 7 / 8)[:, None]     # the second logit: up to two natural units below
+    k[:, :, :2] = 0.0
+    k[[first, second]] = 0.0
+    k[first, :, 0] = k[second, :, 1] = 31.0
+    v[first, :, 64:] = v[second, :, :64] = 0.0
+    Q, K, V = (wd.to_device_bf16(bf16(x)) for x in (q, k, v))
+    P = torch.softmax(torch.einsum("qhd,khd->hqk", Q.double(), K.double()) * SCALE, -1)
+    want = torch.einsum("hqk,khd->qhd", P, V.double())
+    kv = context(H, lq)
+    for splits in (1, 0, 2):
+        O = kv.memory_attention(0, Q, [(K, V)], None, 0, kv_splits=splits)
+        assert kv.poll_status() == (0, 0)
+        assert bool(((O.double() - want).abs() <= (2.0 ** -8 + 1e-4) * want.abs() + 1e-12).all()), f"splits {splits}"
+
+
 @pytest.mark.parametrize("rise", [0.0, 100.0])
 @pytest.mark.parametrize("H,lq,n", [(2, 300, 700), (12, 880, 300), (40, 1100, 200)])
 def test_output_over_the_queries(H, lq, n, rise):
