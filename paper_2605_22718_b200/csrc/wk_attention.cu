@@ -65,6 +65,7 @@ constexpr float kStreamSum = 256.0f;
 // keys (pieces of three tiles), relative error of O at deviations 1 / 2 / 4: 2.13 / 1.80 / 1.69e-3, without 2.27 / 2.19 / 1.98e-3; 2
 // heads x 3,960 keys (four tiles) 20.6 us, without 19.2.  No call is cut into more such pieces for it: that was slower (38.9 us).
 constexpr int kFewTiles = 4;
+constexpr float kOwnSum = 1024.0f;
 // tensor-memory columns: S0, S1 (P over their second half), O0, O1; LSE-only: S0, S1 twice
 constexpr uint32_t kTmemS = 0, kTmemP = 64, kTmemO = 256;
 constexpr int kPairRows = 2 * kTileQ;
@@ -346,14 +347,16 @@ __device__ __forceinline__ float row_max(uint32_t tS, int nv) {
   return fmaxf(mx[0], mx[1]);
 }
 // Moves a row's reference m, and the sum l and the accumulator O (if it holds anything yet) with it: up to the row's maximum over
-// the tile in S when that is more than kRescaleThreshold above it, or, with `own`, to that maximum wherever it is (unless the
-// tile's weights are negligible beside those before it).
+// the tile in S when that is more than kRescaleThreshold above it, or, with `own`, to that maximum wherever it is, unless l would
+// grow beyond kOwnSum on the way down: O, which is l times a mean of V rows, keeps that far from the end of fp32's range, and the
+// tile's weights hardly count there.
 __device__ __forceinline__ void follow_max(uint32_t tS, uint32_t tO, int nv, float scale_log2, bool own, float& m, float& l, bool has_o) {
   const float mt = row_max<2>(tS, nv) * scale_log2;
-  const bool move = own ? mt > m - 20.f && mt != m : mt > m + kRescaleThreshold;   // also true on the first tile (m = -inf)
+  const float alpha_mt = ex2_approx(m - mt);
+  const bool move = own ? mt > m || (mt < m && l * alpha_mt <= kOwnSum) : mt > m + kRescaleThreshold;   // also true on the first tile (m = -inf)
   if (__any_sync(0xffffffffu, move)) {
     // (the previous P V was issued before this tile's Q K^T: it landed before S did)
-    const float alpha = move ? ex2_approx(m - mt) : 1.f;
+    const float alpha = move ? alpha_mt : 1.f;
     if (move) m = mt;
     l *= alpha;
 #pragma unroll 1

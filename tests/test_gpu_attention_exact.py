@@ -71,6 +71,23 @@ def test_largest_weight_of_every_tile_in_short_pieces(n, first, second):
         assert bool(((O.double() - want).abs() <= (2.0 ** -8 + 1e-4) * want.abs() + 1e-12).all()), f"splits {splits}"
 
 
+@pytest.mark.parametrize("step", [-3, -7, -12, -15, -19, -30, 7, 15, 30])
+@pytest.mark.parametrize("n", [512, 470, 1200])
+def test_large_values_under_falling_and_rising_logits(n, step):
+    """The logits of a tile lie `step` log2 units from those of the tile before.  Values scaled by 2^115 are exact in bf16 and leave
+    2^12 of fp32's range: O is the unscaled O times 2^115, bit for bit, as long as the sum that O is held against stays below 2^10."""
+    H, lq = 2, 140
+    q, k, v = normals(10, (lq, H, 128)), normals(11, (n, H, 128)), normals(12, (n, H, 128))
+    q[:, :, 0] = 16.0
+    k[:, :, 0] = (step * (np.arange(n) // 128) / (16.0 * SCALE * 1.4426950408889634))[:, None]
+    Q, K, V = (wd.to_device_bf16(bf16(x)) for x in (q, k, v))
+    kv = context(H, lq)
+    for splits in (1, 0, 2):
+        O = [kv.memory_attention(0, Q, [(K, x)], None, 0, kv_splits=splits) for x in (V, V * 2.0 ** 115)]
+        assert kv.poll_status() == (0, 0)
+        assert torch.equal(O[0].double() * 2.0 ** 115, O[1].double()), f"splits {splits}"
+
+
 @pytest.mark.parametrize("rise", [0.0, 100.0])
 @pytest.mark.parametrize("H,lq,n", [(2, 300, 700), (12, 880, 300), (40, 1100, 200)])
 def test_output_over_the_queries(H, lq, n, rise):
