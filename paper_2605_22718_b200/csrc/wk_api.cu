@@ -222,6 +222,8 @@ wk_status wk_bind(wk_ctx* ctx, void* pool_dev, size_t pool_bytes, void* scratch_
   const int64_t n_mats = static_cast<int64_t>(ctx->cfg.n_layers) * ctx->cfg.pool_slots;
   wk_status st = encode_pool_map(ctx, ctx->Kpool, ctx->C, n_mats, kTileKV, &ctx->tm_kpool);
   if (st != WK_OK) return st;
+  st = encode_pool_map(ctx, ctx->Kpool, ctx->C, n_mats, kTileKVLse, &ctx->tm_kpool_lse);
+  if (st != WK_OK) return st;
   st = encode_pool_map(ctx, ctx->Vpool, ctx->C, n_mats, kTileKV, &ctx->tm_vpool);
   if (st != WK_OK) return st;
   // the anchor pass counts finished CTAs per problem in scratch; the counters must start at zero

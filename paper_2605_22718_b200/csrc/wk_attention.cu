@@ -6,26 +6,25 @@
 //     bf16 output and share a head's K/V tiles through L2 because they walk the keys in step; the units of a last, partial
 //     wave are cut into ranges over all SMs where that pays (split_default): a range writes a normalised fp32 partial plus
 //     its log-sum-exp per piece, and combine_kernel merges them;
-//   * K/V tiles (128 rows x 128 columns of one head, bf16) are fetched by TMA straight from where they lie:
+//   * K/V tiles (80 rows x 128 columns of one head, bf16) are fetched by TMA straight from where they lie:
 //     a dense segment (2-D tensor map per segment) or a pool slot (3-D tensor map [layer*slot][row][col]; the
 //     slot id is read from device memory, so the retrieval result never visits the host).  Rows past the end
 //     of a segment/slot are zero-filled by TMA and masked to -inf before the exponentials;
-//   * S = Q K^T and O += P V are tcgen05.mma (M = 128, N = 128, K = 16 steps) with fp32 accumulators in tensor
-//     memory: S0, S1, O0, O1 fill all 512 columns; P (bf16) overwrites the second half of S and is the A operand of
-//     the P V product directly from tensor memory;
+//   * S = Q K^T and O += P V are tcgen05.mma (M = 128, N = 80 and 128, K = 16 steps) with fp32 accumulators in tensor memory.
+//     O0 and O1 take half of its 512 columns; 80 keys is the widest tile whose S (80 columns) and P (bf16: 40 columns, the A
+//     operand of P V) lie side by side in the other half, so that S of the next tile can be multiplied while the softmax works
+//     on this one, which it has read into registers.  (With 128 keys P has to overwrite S and the two take turns: 12 heads x
+//     2,640 queries x 15,840 keys 261 us back to back instead of 251, although Q K^T alone runs at its full rate only from
+//     N = 128 on: shared memory gives a Q K^T step of 80 keys (4 + 2.5 KB) in 52 clk, one of 128 (4 + 4 KB) in 64.)
 //   * warp roles: warps 0-3 / 4-7 = softmax of Q tile 0 / 1 (one thread per row, fp32 in the exp2
-//     domain, against a reference that follows the row's maximum: see kStreamSum), warp 8 = MMA issue, warp 9 = TMA producer.  The
-//     producer walks the tile list, and hands each tile's height to the others beside the tile; the MMA warp waits once per step for
-//     (V of tile j, K of tile j + 1) and then only for P, since every further wait or branch between two groups of MMAs
-//     is time the tensor pipe stands still (its queue holds about two MMAs);
-//   * a tile with nv < 128 valid rows (the last one of a segment or slot: 1,320 rows are 10 tiles and 40 rows) is
-//     multiplied over ceil(nv / 16) * 16 rows and its softmax stops at the last group of 32.
-//   * every commit after a step's first makes the MMA warp wait until the queue of the tensor pipe has drained, so it commits
-//     only S and O; stages and Q are given back by the softmax warpgroup that sees the last S of a step.
-// What bounds it: the chain of one Q tile (S -> softmax -> P V, Q K^T and the hand-overs between them), of which the two Q tiles
-// hide each other's only in part, at the clock that the board's 1,000 W cap leaves.  2,640 queries x 15,840 keys x 12 heads is
-// one unit of 129 KV tiles on each of 132 SMs: 259 to 263 us back to back, at 1,687 MHz 3,380 clk per tile, prologue and epilogue
-// included, where the tensor pipe needs 2,048.  4,680 x 32,760 x 40 (1,575 MHz): 2,850 us.
+//     domain, against a reference that follows the row's maximum: see kStreamSum), warps 8 / 9 = MMA issue for Q tile 0 / 1,
+//     warp 10 = TMA producer.  The producer walks the tile list, and hands each tile's height to the others beside the tile;
+//   * a tile with fewer valid rows (the last one of a segment or slot: 1,320 rows are 16 tiles and 40 rows) is
+//     multiplied over ceil(nv / 16) * 16 rows.
+// What bounds it: back to back, the energy that the board's 1,000 W cap allows.  2,640 queries x 15,840 keys x 12 heads is one
+// unit of 201 KV tiles on each of 132 SMs: 251 us at 1,640 MHz, 1,780 clk per tile in full flow, where the tensor pipe needs
+// 1,432 (measured with nothing else running; 1,600 with the exponentials left out: the chain S -> registers, P -> P V, Q K^T of
+// one Q tile is 1,470 long, 750 of it hand-overs).  4,680 x 32,760 x 40: 2,725 us at 1,480 MHz.
 // Every wait is bounded; a wait that runs out sets WK_DEV_TIMEOUT, the CTA drains and frees its tensor memory.
 #include <stddef.h>
 
@@ -37,37 +36,40 @@ namespace {
 
 using namespace ptx;
 
-// softmax warps, then the MMA warp, then the TMA warp.  LSE-only launches have a softmax warpgroup per S buffer.
+// softmax warps, then the MMA warps, then the TMA warp.  LSE-only launches have a softmax warpgroup per S buffer.
 template <bool kLse> constexpr int kSoftWarps = kLse ? 16 : 8;
-template <bool kLse> constexpr int kThreads = 32 * (kSoftWarps<kLse> + 2);
-constexpr uint32_t kHalfTileBytes = 128 * 64 * 2;   // one TMA box: 128 rows x 64 bf16 = 16 KB
-constexpr uint32_t kTileBytes = 2 * kHalfTileBytes; // 128 x 128 bf16
-// A stage holds what one step of the MMA warp consumes: V of tile j and K of tile j + 1 (LSE-only launches: K alone).
-constexpr int kStages = 2, kStagesLse = 4;
-constexpr size_t kSmemBytes = 1024 + 2 * kTileBytes + 2 * kStages * kTileBytes;   // align slack + Q0,Q1 + stages
-constexpr size_t kSmemBytesLse = 1024 + 2 * kTileBytes + kStagesLse * kTileBytes;
-constexpr int kNvRing = 16;   // tile heights handed from the TMA warp to the others; the TMA warp is at most kStagesLse + 1 tiles ahead
+template <bool kLse> constexpr int kMmaWarps = kLse ? 1 : 2;
+template <bool kLse> constexpr int kThreads = 32 * (kSoftWarps<kLse> + kMmaWarps<kLse> + 1);
+// rows of a KV tile
+template <bool kLse> constexpr int kKv = kLse ? kTileKVLse : kTileKV;
+template <bool kLse> constexpr uint32_t kHalfKvBytes = kKv<kLse> * 64 * 2;   // one TMA box: 64 columns
+template <bool kLse> constexpr uint32_t kKvBytes = 2 * kHalfKvBytes<kLse>;
+constexpr uint32_t kHalfQBytes = kTileQ * 64 * 2, kQBytes = 2 * kHalfQBytes;
+// A stage holds what one step of the MMA warp consumes: V of tile j and K of tile j + 2 (LSE-only launches: K alone).
+constexpr int kStages = 4;
+template <bool kLse> constexpr uint32_t kStageBytes = (kLse ? 1 : 2) * kKvBytes<kLse>;
+template <bool kLse> constexpr size_t kSmemBytes = 1024 + 2 * kQBytes + kStages * kStageBytes<kLse>;   // align slack + Q0, Q1 + stages
+constexpr int kNvRing = 16;   // tile heights handed from the TMA warp to the others; the TMA warp is at most kStages + 2 tiles ahead
 // The softmax weighs a key with P = 2^(s * scale - m), where m is a maximum that the row has reached: rounded to bf16, the
 // weight of the key that set it is exactly 1, so a dominating key returns its V row unchanged.  (Against a reference that is
 // no maximum, say the largest of the first 32 logits, every weight is rounded: relative error of O 2.3e-3 instead of 2.1e-3 ..
 // 1.7e-3 for logits with a standard deviation of 4 to 16.)  m moves when the maximum has left it by more than kRescaleThreshold.
-// Taking the maximum first costs a pass over S before the first exponential.  A piece's first tile and ragged tiles of more than
-// 64 rows pay for it; other tiles are streamed on trust.  Their sum tells whether that was right: no weight above 2^8 hides in a
-// sum of at most kStreamSum.  A warp in which a row's sum is larger still has all of S (columns 0-63 in tensor memory, the others
-// in registers), moves its references to the maximum where that is more than 2^8 above, and streams the tile again; tiles after
-// that are read for the maximum first, twice as many each time.  12 heads x 2,640 queries x 15,840 keys, back to back: 273 us with
-// the maximum first for all, 263 this way, 259 without the check; logits of standard deviation 4 / 16 / 40 (18,480 keys): 328 /
-// 308 / 307 us, and 232 at 1.
+// Taking the maximum first costs instructions and time before the first exponential.  A piece's first tile pays for it; other tiles
+// are streamed on trust.  Their sum tells whether that was right: no weight above 2^8 hides in a sum of at most kStreamSum.  A warp
+// in which a row's sum is larger still has S in registers, moves its references to the maximum where that is more than 2^8 above,
+// and takes the exponentials again; tiles after that are read for the maximum first, twice as many each time.  12 heads x 2,640
+// queries x 15,840 keys, back to back: 267 us with the maximum first for all, 261 this way.
 constexpr float kRescaleThreshold = 8.0f;           // log2 units: P stays <= 2^8 between maximum updates
 constexpr float kStreamSum = 256.0f;
 // Pieces of at most kFewTiles tiles move the reference to every tile's own maximum, down as well as up: beside few other keys a
 // tile's largest weight counts, and it is exact this way, as if the tile were a piece of its own.  450 queries x 5 heads x 1,040
-// keys (pieces of three tiles), relative error of O at deviations 1 / 2 / 4: 2.13 / 1.80 / 1.69e-3, without 2.27 / 2.19 / 1.98e-3; 2
-// heads x 3,960 keys (four tiles) 20.6 us, without 19.2.  No call is cut into more such pieces for it: that was slower (38.9 us).
-constexpr int kFewTiles = 4;
+// keys (pieces of three tiles), relative error of O at deviations 1 / 2 / 4: 2.13 / 1.80 / 1.69e-3, without 2.27 / 2.19 / 1.98e-3.
+// Calls whose keys are that few altogether walk them in tiles of kTileKVFew rows, so that no more keys share a maximum.
+constexpr int kFewTiles = 8, kTileKVFew = 64;
 constexpr float kOwnSum = 1024.0f;
-// tensor-memory columns: S0, S1 (P over their second half), O0, O1; LSE-only: S0, S1 twice
-constexpr uint32_t kTmemS = 0, kTmemP = 64, kTmemO = 256;
+// tensor-memory columns: S0, P0, S1, P1 (80 + 40 of 128 each), O0, O1; LSE-only: S0, S1 twice
+constexpr uint32_t kTmemS = 0, kTmemP = kTileKV, kTmemO = 256;
+static_assert(kTileKV * 3 / 2 <= 128, "S and P of a Q tile share 128 columns");
 constexpr int kPairRows = 2 * kTileQ;
 constexpr int kMaxPieces = 32;                      // most ranges one unit may be cut into
 
@@ -81,6 +83,7 @@ struct AttnParams {
   const int32_t* slots;
   const int32_t* valid;
   int n_slots, pool_slots, layer, C, tiles_per_slot;
+  int tile_rows;    // rows from one KV tile to the next
   int n_tiles, n_qpairs, n_units;
   int n_full, n_ranges;
   int lq, H;
@@ -119,12 +122,12 @@ struct TileIter {
   __device__ __forceinline__ void enter(const AttnParams& p, bool report) {
     if (seg < p.n_segs) {
       n_r = p.seg_tile_prefix[seg + 1] - p.seg_tile_prefix[seg];
-      tail = p.seg_rows[seg] - (n_r - 1) * kTileKV;
+      tail = p.seg_rows[seg] - (n_r - 1) * p.tile_rows;
       z = 0;
       ok = true;
     } else {
       n_r = p.tiles_per_slot;
-      tail = p.C - (n_r - 1) * kTileKV;
+      tail = p.C - (n_r - 1) * p.tile_rows;
       const int si = seg - p.n_segs;
       ok = false;
       z = 0;
@@ -165,9 +168,9 @@ struct TileIter {
         continue;
       }
       ti.seg = seg < p.n_segs ? seg : -1;
-      ti.row0 = r * kTileKV;
+      ti.row0 = r * p.tile_rows;
       ti.z = z;
-      ti.nv = (r == n_r - 1) ? tail : kTileKV;
+      ti.nv = (r == n_r - 1) ? tail : p.tile_rows;
       ++r;
       ++t;
       if (ok) return true;
@@ -193,35 +196,10 @@ __device__ __forceinline__ int count_tiles(const AttnParams& p, int tb, int te) 
   return dense + n;
 }
 
-#ifdef WK_ATTN_PROFILE
-// Stage timers for one designated thread per role of CTA 0: clock deltas are accumulated in registers and added into the
-// words after the status word when the role finishes.  Built only for profiling runs; the product build has none of this.
-#define WK_PROF_DECL uint32_t prof_t = clock(); uint32_t prof_acc[12] = {}; uint64_t prof_ns; uint32_t prof_c0 = prof_t; \
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(prof_ns));
-#define WK_PROF(slot)                                    \
-  do {                                                   \
-    const uint32_t now__ = clock();                      \
-    prof_acc[slot] += now__ - prof_t;                    \
-    prof_t = now__;                                      \
-  } while (0)
-#define WK_PROF_FLUSH(base, n, cond)                                                       \
-  do {                                                                                     \
-    if (cond) {                                                                            \
-      uint64_t ns2; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns2));               \
-      prof_acc[n - 2] = (clock() - prof_c0); prof_acc[n - 1] = static_cast<uint32_t>(ns2 - prof_ns); \
-      for (int i__ = 0; i__ < n; ++i__) p.status[8 + (base) + i__] = prof_acc[i__];         \
-    }                                                                                      \
-  } while (0)
-#else
-#define WK_PROF_DECL
-#define WK_PROF(slot)
-#define WK_PROF_FLUSH(base, n, cond)
-#endif
-
 struct __align__(8) Barriers {
   uint64_t q_full, q_empty;
-  uint64_t kv_full[kStagesLse], kv_empty[kStagesLse];
-  uint64_t s_full[4], p_full[4], o_done[2], o_free[2], m_full[2], m_empty[2];   // index of s_full, p_full: Q tile + 2 x S buffer (LSE-only)
+  uint64_t kv_full[kStages], kv_empty[kStages];
+  uint64_t s_full[4], p_full[4], turn[2], o_done[2], o_free[2], m_full[2], m_empty[2];   // index of s_full, p_full: Q tile + 2 x S buffer (LSE-only)
 };
 
 // Bounded wait that also gives up when another role has already aborted; false then.  A loop of eight instructions and
@@ -260,12 +238,17 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
-// 2^x of a pair.  The exponentials are the kernel's second bound (16 per clock and SM on the special-function unit, as many
-// clocks per tile as its tensor-core work; 266 us at a share of 0 or 1/8, 263 at 2/8 for 12 heads x 15,840
-// keys), so a share of the pairs takes 2^x from the FMA pipe instead: x = n + f with
+__device__ __forceinline__ float fmax_nan(float a, float b) {   // NaN if either is
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+// 2^x of a pair.  The exponentials are the kernel's second bound (16 per clock and SM on the special-function unit: 1,280 clk per
+// tile of 80 keys), so a share of the pairs takes 2^x from the FMA pipe instead (12 heads x 2,640 queries x 15,840 keys: 264 us at a
+// share of 0, 251 at 1/8, 262 at 2/8, 270 at 3/8): x = n + f with
 // n = round(x) by the add-a-large-constant trick, 2^f on [-1/2, 1/2] by a cubic (relative error 7.7e-5, far inside the bf16
 // rounding P gets anyway: 2e-3), 2^n by adding n to the exponent field; all in packed fp32 pairs.  That path clamps at
-// x = -120 (a weight of 1e-36) and needs x < 127.
+// x = -120 (a weight of 1e-36), needs x < 127, and turns NaN into a weight beyond all bounds.
 template <bool kPoly>
 __device__ __forceinline__ void exp2_pair(uint64_t e, float& p0, float& p1) {
   float e0, e1;
@@ -277,7 +260,7 @@ __device__ __forceinline__ void exp2_pair(uint64_t e, float& p0, float& p1) {
     const uint64_t c1 = pack_f32x2(0.6932762265205383f, 0.6932762265205383f);
     const uint64_t c2 = pack_f32x2(0.242604061961174f, 0.242604061961174f);
     const uint64_t c3 = pack_f32x2(0.055088773369789124f, 0.055088773369789124f);
-    const uint64_t x = pack_f32x2(fmaxf(e0, -120.f), fmaxf(e1, -120.f));
+    const uint64_t x = pack_f32x2(fmax_nan(e0, -120.f), fmax_nan(e1, -120.f));
     const uint64_t t = add_f32x2(x, magic2);                  // low mantissa bits = round(x)
     const uint64_t f = fma_f32x2(add_f32x2(t, nmagic2), mone2, x);   // x - round(x), in [-1/2, 1/2]
     uint64_t y = fma_f32x2(c3, f, c2);
@@ -299,12 +282,11 @@ __device__ __forceinline__ float sum4_f32x2(const uint64_t (&acc)[4]) {
   return a + b;
 }
 
-// P = 2^(s * scale - m) of 32 columns of a row: sums go to four independent (lo, hi) accumulators, bf16 pairs to pk (kPack).
-// kPoly of every 8 pairs take the FMA pipe; big = the largest of their raw values (the caller checks that they stay below that
-// path's limit).
-template <int kPoly, bool kPack>
+constexpr int kLsePoly = 2;
+// Sum of 2^(s * scale - m) over 32 columns of a row, in four independent (lo, hi) accumulators.  kLsePoly of every 8 pairs take
+// the FMA pipe; big = the largest of their raw values (the caller checks that they stay below that path's limit).
 __device__ __forceinline__ void exp_chunk(uint32_t (&r)[32], int rem, uint64_t scale2, uint64_t neg_m2, uint64_t (&acc)[4],
-                                          float& big, uint32_t (&pk)[16]) {
+                                          float& big) {
   if (rem < 32) {   // columns past the end of the segment or slot
 #pragma unroll
     for (int i = 0; i < 32; ++i) r[i] = i < rem ? r[i] : 0xff800000u;
@@ -314,68 +296,76 @@ __device__ __forceinline__ void exp_chunk(uint32_t (&r)[32], int rem, uint64_t s
     const float s0 = __uint_as_float(r[2 * i]), s1 = __uint_as_float(r[2 * i + 1]);
     const uint64_t e = fma_f32x2(pack_f32x2(s0, s1), scale2, neg_m2);
     float p0, p1;
-    if ((i & 7) < kPoly) {
+    if ((i & 7) < kLsePoly) {
       exp2_pair<true>(e, p0, p1);
       big = fmax3(big, s0, s1);
     } else {
       exp2_pair<false>(e, p0, p1);
     }
     acc[i & 3] = add_f32x2(acc[i & 3], pack_f32x2(p0, p1));
-    if (kPack) pk[i] = pack_bf16x2(p0, p1);
   }
 }
-// The largest of a row's first nv columns of S, 32 kLoads columns in flight at a time.
-template <int kLoads>
-__device__ __forceinline__ float row_max(uint32_t tS, int nv) {
+// The largest of a row's first nv columns of S in tensor memory.
+__device__ __forceinline__ float row_max_tmem(uint32_t tS, int nv) {
   float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll 1
-  for (int c = 0; c < nv; c += 32 * kLoads) {
-    uint32_t r[kLoads][32];
+  for (int c = 0; c < nv; c += 32) {
+    uint32_t r[32];
+    tmem_ld_x32(tS + c, r);
+    tc_wait_ld(r);
+    if (nv - c < 32) {
 #pragma unroll
-    for (int k = 0; k < kLoads; ++k) tmem_ld_x32(tS + c + 32 * k, r[k]);
-#pragma unroll
-    for (int k = 0; k < kLoads; ++k) tc_wait_ld(r[k]);
-    if (nv - c < 32 * kLoads) {
-#pragma unroll
-      for (int i = 0; i < 32 * kLoads; ++i)
-        if (c + i >= nv) r[i >> 5][i & 31] = 0xff800000u;
+      for (int i = 0; i < 32; ++i)
+        if (c + i >= nv) r[i] = 0xff800000u;
     }
 #pragma unroll
-    for (int i = 0; i < 32 * kLoads; i += 2)
-      mx[(i >> 1) & 1] = fmax3(mx[(i >> 1) & 1], __uint_as_float(r[i >> 5][i & 31]), __uint_as_float(r[i >> 5][(i & 31) + 1]));
+    for (int i = 0; i < 32; i += 2) mx[(i >> 1) & 1] = fmax3(mx[(i >> 1) & 1], __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
   }
   return fmaxf(mx[0], mx[1]);
 }
-// Moves a row's reference m, and the sum l and the accumulator O (if it holds anything yet) with it: up to the row's maximum over
-// the tile in S when that is more than kRescaleThreshold above it, or, with `own`, to that maximum wherever it is, unless l would
-// grow beyond kOwnSum on the way down: O, which is l times a mean of V rows, keeps that far from the end of fp32's range, and the
-// tile's weights hardly count there.
-__device__ __forceinline__ void follow_max(uint32_t tS, uint32_t tO, int nv, float scale_log2, bool own, float& m, float& l, bool has_o) {
-  const float mt = row_max<2>(tS, nv) * scale_log2;
-  const float alpha_mt = ex2_approx(m - mt);
-  const bool move = own ? mt > m || (mt < m && l * alpha_mt <= kOwnSum) : mt > m + kRescaleThreshold;   // also true on the first tile (m = -inf)
-  if (__any_sync(0xffffffffu, move)) {
-    // (the previous P V was issued before this tile's Q K^T: it landed before S did)
-    const float alpha = move ? alpha_mt : 1.f;
-    if (move) m = mt;
-    l *= alpha;
-#pragma unroll 1
-    for (int c = 0; c < 128 && has_o; c += 32) {
-      uint32_t r[32];
-      tmem_ld_x32(tO + c, r);
-      tc_wait_ld(r);
-#pragma unroll
-      for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
-      tmem_st_x32(tO + c, r);
-    }
-  }
+// S of a tile, a row per thread, into registers.
+__device__ __forceinline__ void tmem_ld_tile(uint32_t tS, uint32_t (&r)[kTileKV]) {
+  static_assert(kTileKV == 80, "loads of 32 + 32 + 16 columns");
+  tmem_ld_x32(tS, *reinterpret_cast<uint32_t(*)[32]>(&r[0]));
+  tmem_ld_x32(tS + 32, *reinterpret_cast<uint32_t(*)[32]>(&r[32]));
+  tmem_ld_x16(tS + 64, *reinterpret_cast<uint32_t(*)[16]>(&r[64]));
 }
-#ifndef WK_ATTN_POLY
-#define WK_ATTN_POLY 2
-#endif
-#ifndef WK_LSE_POLY
-#define WK_LSE_POLY 2
-#endif
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[kTileKV]) {
+  tc_wait_ld(*reinterpret_cast<uint32_t(*)[32]>(&r[0]));
+  pin_x32(*reinterpret_cast<uint32_t(*)[32]>(&r[32]));
+  pin_x16(*reinterpret_cast<uint32_t(*)[16]>(&r[64]));
+}
+__device__ __forceinline__ void tmem_st_half_tile(uint32_t tP, const uint32_t (&p)[kTileKV / 2]) {
+  tmem_st_x32(tP, *reinterpret_cast<const uint32_t(*)[32]>(&p[0]));
+  tmem_st_x8(tP + 32, *reinterpret_cast<const uint32_t(*)[8]>(&p[32]));
+}
+__device__ __forceinline__ float row_max(const uint32_t (&r)[kTileKV]) {
+  float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+  for (int i = 0; i < kTileKV; i += 2) mx[(i >> 1) & 3] = fmax3(mx[(i >> 1) & 3], __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+  return fmax3(fmaxf(mx[0], mx[1]), mx[2], mx[3]);
+}
+// P = 2^(s * scale - m) of a row, as bf16 pairs, and their sum.  One of every 8 pairs takes the FMA pipe; big = the largest of
+// their raw values (see exp_chunk).
+__device__ __forceinline__ float exp_tile(const uint32_t (&r)[kTileKV], uint64_t scale2, float m, float& big, uint32_t (&pk)[kTileKV / 2]) {
+  const uint64_t neg_m2 = pack_f32x2(-m, -m);
+  uint64_t acc[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int i = 0; i < kTileKV / 2; ++i) {
+    const float s0 = __uint_as_float(r[2 * i]), s1 = __uint_as_float(r[2 * i + 1]);
+    const uint64_t e = fma_f32x2(pack_f32x2(s0, s1), scale2, neg_m2);
+    float p0, p1;
+    if ((i & 7) == 4) {
+      exp2_pair<true>(e, p0, p1);
+      big = fmax3(big, s0, s1);
+    } else {
+      exp2_pair<false>(e, p0, p1);
+    }
+    acc[i & 3] = add_f32x2(acc[i & 3], pack_f32x2(p0, p1));
+    pk[i] = pack_bf16x2(p0, p1);
+  }
+  return sum4_f32x2(acc);
+}
 
 // One piece of work: unit u, KV tiles [tb, te), and where its result goes.
 struct Piece {
@@ -466,17 +456,161 @@ struct CtaShared {
   volatile int nv[kNvRing];   // valid rows of tile number t (counted over the CTA's pieces) at t % kNvRing
 };
 
+// Issues the MMAs of a CTA's tiles.  The whole warp runs the control flow and one lane's predicate issues (see mma_ss_if).
+template <bool kLse>
+struct Mma {
+  uint32_t one, bar0;
+  uint64_t q_desc, k_desc, v_desc;   // descriptors of the tile bases; a K = 16 step advances the low word by a constant
+  __device__ __forceinline__ Mma(uint32_t smem_base, const Barriers& bars) {
+    one = elect_one() ? 1u : 0u;
+    bar0 = smem_u32(&bars);
+    constexpr uint64_t hi = static_cast<uint64_t>(smem_desc_hi_sw128(1024)) << 32;
+    q_desc = hi | smem_desc_lo(smem_base, 16);
+    k_desc = hi | smem_desc_lo(smem_base + 2 * kQBytes, 16);
+    v_desc = hi | smem_desc_lo(smem_base + 2 * kQBytes + kKvBytes<kLse>, kHalfKvBytes<kLse>);
+  }
+  __device__ __forceinline__ void commit(size_t offset) const { mma_commit_if(one, bar0 + static_cast<uint32_t>(offset)); }
+  // S = Q K^T over the first nv rows of the K tile: ceil(nv / 16) * 16 columns.  (A branch that gives full tiles a constant
+  // descriptor costs more than it saves: LSE-only launches 3,413 us instead of 3,361.)
+  // qt: Q tile in shared memory, d: S columns
+  __device__ __forceinline__ void s(uint32_t qt, uint32_t d, uint32_t st, int nv) const {
+    const uint32_t idesc = idesc_bf16_f32(128, 0, 0, 0) | (static_cast<uint32_t>((nv + 15) >> 4) << 18);
+    const uint64_t a = q_desc + qt * (kQBytes >> 4), b = k_desc + st * (kStageBytes<kLse> >> 4);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const uint32_t in_row = (k & 3) * 2;   // 32 bytes per step inside a 128-byte row
+      mma_ss_if(one, d, a + (k >> 2) * (kHalfQBytes >> 4) + in_row, b + (k >> 2) * (kHalfKvBytes<kLse> >> 4) + in_row, idesc, k > 0);
+    }
+  }
+  // O_i (+)= P_i V: A = P from tensor memory (bf16 pairs, 8 columns per K = 16 step); B = V, rows = K dimension,
+  // MN-major: 16 rows of 128 bytes = 2048 bytes per step
+  __device__ __forceinline__ void pv(uint32_t i, uint32_t st, int nv, uint32_t accumulate) const {
+    constexpr uint32_t idesc = idesc_bf16_f32(128, 128, 0, 1);
+    const uint64_t b = v_desc + st * (kStageBytes<kLse> >> 4);
+#pragma unroll 1
+    for (int k = 0; k < (nv + 15) >> 4; ++k)
+      mma_ts_if(one, kTmemO + i * 128, kTmemP + i * 128 + k * 8, b + k * 128, idesc, k > 0 ? 1u : accumulate);
+  }
+};
+
+// MMA warp of Q tile kQt.  Two warps issue because a commit holds its warp until the tensor pipe has nearly caught up, and the
+// waits behind it would leave the pipe idle: while one warp is held, the other has waited already and goes on.  They take turns
+// (turn[]), step by step: the pipe runs a group of MMAs that accumulate into one tile slower when another tile's come between them.
+template <int kQt>
+__device__ __forceinline__ void mma_role(const AttnParams& p, CtaShared<false>& sh, uint32_t smem_base) {
+  Barriers& bars = sh.bars;
+  const int lane = threadIdx.x & 31;
+  const Mma<false> mma(smem_base, bars);
+  PieceWalker walk;
+  walk.init(p);
+  Piece pc;
+  uint32_t st = 0, ph = 0;       // stage and its parity
+  uint32_t p_ph = 0;             // parity of p_full
+  uint32_t n = 0, t = 0, e = 0;  // pieces, tiles, pieces with output of this Q tile so far
+  uint32_t k = 0;                // steps that both Q tiles took part in so far
+  bool ok = true;
+  while (ok && walk.next(p, pc)) {
+    const int n_eff = count_tiles(p, pc.tb, pc.te);
+    const bool both = pc.has_q1, mine = kQt == 0 || both;
+    if (!(ok = wait_or_abort(&bars.q_full, n & 1, &sh.abort))) break;
+    ++n;
+    if (n_eff == 0) {
+      if (lane == 0) mbar_arrive(&bars.q_empty);
+      continue;
+    }
+    // Step j: once P of tile j - 2 is in tensor memory and S of tile j - 1 in registers (p_full), P V of the one and Q K^T of
+    // tile j.  The softmax of tile j - 1 runs meanwhile; it stores its P when this step's commit arrives.
+    if (!mine) {
+      const uint32_t used = st + (n_eff == 1 ? 2 : n_eff + 2);
+      ph ^= (used / kStages) & 1;
+      st = used % kStages;
+      t += n_eff;
+      continue;
+    }
+    int nv = 0, nv_1 = 0, nv_2 = 0;   // valid rows of tiles j, j - 1, j - 2
+    for (int j = 0; j < n_eff + 2; ++j, nv_2 = nv_1, nv_1 = nv) {
+      const bool work = j != 1 || n_eff > 1;   // a piece of one tile has nothing to multiply in its second step
+      if (work && !(ok = wait_or_abort(&bars.kv_full[st], ph, &sh.abort))) break;
+      nv = 0;
+      if (j < n_eff) nv = sh.nv[t++ % kNvRing];
+      if (j > 0) {
+        ok = wait_or_abort(&bars.p_full[kQt], p_ph, &sh.abort);
+        p_ph ^= 1;
+        // A piece's first P V overwrites O: the epilogue of the last piece that used it must have read it.  o_free
+        // completes once per piece in which the warpgroup ran an epilogue, so neither side can run two phases ahead of
+        // the other (a parity wait cannot tell phase n from phase n + 2).
+        if (j == 2 && e++ > 0) ok = ok && wait_or_abort(&bars.o_free[kQt], e & 1, &sh.abort);
+      }
+      if (!work) continue;
+      if (both && (kQt == 1 || k > 0)) ok = ok && wait_or_abort(&bars.turn[kQt], (kQt == 1 ? k : k + 1) & 1, &sh.abort);
+      if (!ok) break;
+      tc_fence_after();
+      if (j >= 2) mma.pv(kQt, st, nv_2, j > 2);
+      if (nv > 0) mma.s(kQt, kTmemS + kQt * 128, st, nv);
+      if (both) {
+        ++k;
+        if (mma.one) mbar_arrive(&bars.turn[kQt ^ 1]);
+      }
+      mma.commit((j == n_eff + 1 ? offsetof(Barriers, o_done) : offsetof(Barriers, s_full)) + 8 * kQt);
+      if (++st == kStages) { st = 0; ph ^= 1; }
+    }
+  }
+  if (lane == 0) leave_role(ok, &sh.abort, p.status);
+}
+
+// LSE-only: two S buffers per Q tile, no P V; p_full says that a buffer has been read.
+__device__ __forceinline__ void mma_lse_role(const AttnParams& p, CtaShared<true>& sh, uint32_t smem_base) {
+  Barriers& bars = sh.bars;
+  const int lane = threadIdx.x & 31;
+  const Mma<true> mma(smem_base, bars);
+  PieceWalker walk;
+  walk.init(p);
+  Piece pc;
+  uint32_t st = 0, ph = 0;   // stage and its parity
+  uint32_t n = 0, t = 0;     // pieces and tiles so far
+  uint32_t s0 = 0, s1 = 0;   // products of Q tile 0 / 1 so far
+  bool ok = true;
+  while (ok && walk.next(p, pc)) {
+    const int n_eff = count_tiles(p, pc.tb, pc.te);
+    if (!(ok = wait_or_abort(&bars.q_full, n & 1, &sh.abort))) break;
+    ++n;
+    if (n_eff == 0) {
+      if (lane == 0) mbar_arrive(&bars.q_empty);
+      continue;
+    }
+    for (int j = 0; j < n_eff; ++j) {
+      if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &sh.abort))) break;
+      const int nv = sh.nv[t++ % kNvRing];
+      const uint32_t b0 = s0 & 1, b1 = s1 & 1;
+      auto issue = [&](uint32_t qt, uint32_t d) {
+        tc_fence_after();
+        mma.s(qt, d, st, nv);
+      };
+      if (s0 >= 2 && !(ok = wait_or_abort(&bars.p_full[2 * b0], ((s0 >> 1) & 1) ^ 1, &sh.abort))) break;
+      ++s0;
+      issue(0, b0 * 256);
+      mma.commit(offsetof(Barriers, s_full) + 16 * b0);
+      if (pc.has_q1) {
+        if (s1 >= 2 && !(ok = wait_or_abort(&bars.p_full[2 * b1 + 1], ((s1 >> 1) & 1) ^ 1, &sh.abort))) break;
+        ++s1;
+        issue(1, b1 * 256 + 128);
+        mma.commit(offsetof(Barriers, s_full) + 16 * b1 + 8);
+      }
+      if (++st == kStages) { st = 0; ph ^= 1; }
+    }
+  }
+  if (lane == 0) leave_role(ok, &sh.abort, p.status);
+}
+
 // All of a CTA's work.
 template <bool kLse>
 __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<kLse>& sh, uint8_t* smem) {
   const uint32_t smem_base = smem_u32(smem);
-  uint8_t* sQ = smem;                                   // [2 q tiles][2 halves][128 rows][128 B]
-  uint8_t* sKV = sQ + 2 * kTileBytes;                   // [stages][K, V][2 halves][128][128 B]; LSE-only: [stages][K]
-  constexpr uint32_t kNStages = kLse ? kStagesLse : kStages;
-  constexpr uint32_t kStageBytes = kLse ? kTileBytes : 2 * kTileBytes;
+  uint8_t* sQ = smem;                 // [2 q tiles][2 halves][128 rows][128 B]
+  uint8_t* sKV = sQ + 2 * kQBytes;    // [stages][K, V][2 halves][rows][128 B]; LSE-only: [stages][K]
   Barriers& bars = sh.bars;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (warp == kSoftWarps<kLse> + 1) {
+  if (warp == kSoftWarps<kLse> + kMmaWarps<kLse>) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       PieceWalker walk;
@@ -486,11 +620,11 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       bool ok = true;
       while (ok && walk.next(p, pc)) {
         if (!(ok = wait_or_abort(&bars.q_empty, (n & 1) ^ 1, &sh.abort))) break;
-        mbar_expect_tx(&bars.q_full, 2 * kTileBytes);
+        mbar_expect_tx(&bars.q_full, 2 * kQBytes);
         ++n;
         for (int i = 0; i < 2; ++i)
           for (int half = 0; half < 2; ++half)
-            tma_load_2d(sQ + i * kTileBytes + half * kHalfTileBytes, &p.tm_q, &bars.q_full,
+            tma_load_2d(sQ + i * kQBytes + half * kHalfQBytes, &p.tm_q, &bars.q_full,
                         pc.h * kHeadDim + half * 64, pc.q0 + i * kTileQ);
         TileIter it;
         const bool report = !p.slot_units;
@@ -499,26 +633,30 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
         auto load = [&](uint8_t* dst, const TileInfo& ti, const CUtensorMap* seg_maps, const CUtensorMap* pool_map) {
           if (ti.seg >= 0) {
             tma_load_2d(dst, seg_maps + ti.seg, &bars.kv_full[st], x, ti.row0);
-            tma_load_2d(dst + kHalfTileBytes, seg_maps + ti.seg, &bars.kv_full[st], x + 64, ti.row0);
+            tma_load_2d(dst + kHalfKvBytes<kLse>, seg_maps + ti.seg, &bars.kv_full[st], x + 64, ti.row0);
           } else {
             tma_load_3d(dst, pool_map, &bars.kv_full[st], x, ti.row0, ti.z);
-            tma_load_3d(dst + kHalfTileBytes, pool_map, &bars.kv_full[st], x + 64, ti.row0, ti.z);
+            tma_load_3d(dst + kHalfKvBytes<kLse>, pool_map, &bars.kv_full[st], x + 64, ti.row0, ti.z);
           }
         };
-        TileInfo ti, tv;
-        bool have_k = it.next(p, ti, report), have_v = false;
-        while (have_k || have_v) {   // step: V of the tile before (not in LSE-only launches), K of this tile
-          if (!(ok = wait_or_abort(&bars.kv_empty[st], ph, &sh.abort))) break;
-          if (have_k) sh.nv[t++ % kNvRing] = ti.nv;   // read after kv_full
-          mbar_expect_tx(&bars.kv_full[st], (have_k ? kTileBytes : 0) + (have_v ? kTileBytes : 0));
-          ++steps;
-          uint8_t* dst = sKV + st * kStageBytes;
-          if (have_k) load(dst, ti, p.tm_kd, &p.tm_kpool);
-          if (have_v) load(dst + kTileBytes, tv, p.tm_vd, &p.tm_vpool);
-          if (++st == kNStages) { st = 0; ph ^= 1; }
-          have_v = have_k && !kLse;
-          tv = ti;
-          if (have_k) have_k = it.next(p, ti, report);
+        TileInfo ti, t1, t2;   // this tile and the two before it
+        bool have = it.next(p, ti, report), have1 = false, have2 = false;
+        while (have || have1 || have2) {   // step: K of this tile, V of the last but one (not in LSE-only launches)
+          if (have || have2) {             // (a piece of one tile has nothing in its second step)
+            if (!(ok = wait_or_abort(&bars.kv_empty[st], ph, &sh.abort))) break;
+            if (have) sh.nv[t++ % kNvRing] = ti.nv;   // read after kv_full
+            mbar_expect_tx(&bars.kv_full[st], (have ? kKvBytes<kLse> : 0) + (have2 ? kKvBytes<kLse> : 0));
+            ++steps;
+            uint8_t* dst = sKV + st * kStageBytes<kLse>;
+            if (have2) load(dst + kKvBytes<kLse>, t2, p.tm_vd, &p.tm_vpool);
+            if (have) load(dst, ti, p.tm_kd, &p.tm_kpool);
+            if (++st == kStages) { st = 0; ph ^= 1; }
+          }
+          t2 = t1;
+          have2 = have1;
+          t1 = ti;
+          have1 = have && !kLse;
+          if (have) have = it.next(p, ti, report);
         }
       }
       leave_role(ok, &sh.abort, p.status);
@@ -531,139 +669,15 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
             if (mbar_try_wait(bar, use & 1)) break;
         };
         if (n > 0) drain(&bars.q_full, n - 1);
-        for (uint32_t q = 0; q < kNStages; ++q)
-          if (steps > q) drain(&bars.kv_full[q], (steps - 1 - q) / kNStages);
+        for (uint32_t q = 0; q < kStages; ++q)
+          if (steps > q) drain(&bars.kv_full[q], (steps - 1 - q) / kStages);
       }
     }
   } else if (warp == kSoftWarps<kLse>) {
-    // ------------------------------------------------------------------ MMA issue
-    // The whole warp runs the control flow and one lane's predicate issues (see mma_ss_if).
-    {
-      const uint32_t one = elect_one() ? 1u : 0u;
-      constexpr uint32_t idesc_qk = idesc_bf16_f32(128, 128, 0, 0), idesc_pv = idesc_bf16_f32(128, 128, 0, 1);
-      // descriptors of the tile bases; a K = 16 step advances the low word by a constant
-      constexpr uint64_t hi = static_cast<uint64_t>(smem_desc_hi_sw128(1024)) << 32;
-      const uint64_t q_desc = hi | smem_desc_lo(smem_base, 16);
-      const uint64_t k_desc = hi | smem_desc_lo(smem_base + 2 * kTileBytes, 16);
-      const uint64_t v_desc = hi | smem_desc_lo(smem_base + 3 * kTileBytes, kHalfTileBytes);
-      const uint32_t bar0 = smem_u32(&bars);
-      auto commit = [&](size_t offset) { mma_commit_if(one, bar0 + static_cast<uint32_t>(offset)); };
-      // S_i = Q_i K^T over the first nv rows of the K tile.  A full tile is eight MMAs without a branch between them; a
-      // short one computes ceil(nv / 16) * 16 columns.
-      auto issue_s = [&](uint32_t qt, uint32_t d, uint32_t st, int nv) {   // qt: Q tile in shared memory, d: S columns
-        const uint64_t a = q_desc + qt * (kTileBytes >> 4), b = k_desc + st * (kStageBytes >> 4);
-        const uint32_t idesc = nv == kTileKV ? idesc_qk
-                                             : (idesc_bf16_f32(128, 0, 0, 0) | (static_cast<uint32_t>((nv + 15) >> 4) << 18));
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const uint32_t off = (k >> 2) * (kHalfTileBytes >> 4) + (k & 3) * 2;   // 32 bytes per step inside a 128-byte row
-          mma_ss_if(one, d, a + off, b + off, idesc, k > 0);
-        }
-      };
-      // O_i (+)= P_i V: A = P from tensor memory (bf16 pairs, 8 columns per K = 16 step); B = V, rows = K dimension,
-      // MN-major: 16 rows of 128 bytes = 2048 bytes per step
-      auto issue_pv = [&](uint32_t i, uint32_t st, int nv, uint32_t accumulate) {
-        const uint64_t b = v_desc + st * (kStageBytes >> 4);
-        if (nv == kTileKV) {
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            mma_ts_if(one, kTmemO + i * 128, kTmemP + i * 128 + k * 8, b + k * 128, idesc_pv, k > 0 ? 1u : accumulate);
-        } else {
-#pragma unroll 1
-          for (int k = 0; k * 16 < nv; ++k)
-            mma_ts_if(one, kTmemO + i * 128, kTmemP + i * 128 + k * 8, b + k * 128, idesc_pv, k > 0 ? 1u : accumulate);
-        }
-      };
-      PieceWalker walk;
-      walk.init(p);
-      Piece pc;
-      uint32_t st = 0, ph = 0;          // stage and its parity
-      uint32_t p_ph0 = 0, p_ph1 = 0;    // parities of p_full[0], p_full[1]
-      uint32_t n = 0, t = 0;            // running piece and tile counts
-      uint32_t e0 = 0, e1 = 0;          // pieces in which Q tile 0 / 1 produced output so far
-      uint32_t lse_q0 = 0, lse_q1 = 0;  // LSE-only: products of Q tile 0 / 1 so far
-      WK_PROF_DECL
-      bool ok = true;
-      while (ok && walk.next(p, pc)) {
-        const int n_eff = count_tiles(p, pc.tb, pc.te);
-        const bool q1 = pc.has_q1;
-        if (!(ok = wait_or_abort(&bars.q_full, n & 1, &sh.abort))) break;
-        ++n;
-        if (n_eff == 0) {
-          if (lane == 0) mbar_arrive(&bars.q_empty);
-          continue;
-        }
-        if (kLse) {
-          // LSE-only: two S buffers per Q tile, no P V; p_full says that a buffer has been read
-          for (int j = 0; j < n_eff; ++j) {
-            WK_PROF(0);
-            if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &sh.abort))) break;
-            const int nv = sh.nv[t++ % kNvRing];
-            const uint32_t b0 = lse_q0 & 1, b1 = lse_q1 & 1;
-            WK_PROF(1);
-            if (lse_q0 >= 2 && !(ok = wait_or_abort(&bars.p_full[2 * b0], ((lse_q0 >> 1) & 1) ^ 1, &sh.abort))) break;
-            ++lse_q0;
-            WK_PROF(2);
-            tc_fence_after();
-            issue_s(0, b0 * 256, st, nv);
-            commit(offsetof(Barriers, s_full) + 16 * b0);
-            WK_PROF(3);
-            if (q1) {
-              if (lse_q1 >= 2 && !(ok = wait_or_abort(&bars.p_full[2 * b1 + 1], ((lse_q1 >> 1) & 1) ^ 1, &sh.abort))) break;
-              ++lse_q1;
-              WK_PROF(4);
-              tc_fence_after();
-              issue_s(1, b1 * 256 + 128, st, nv);
-              commit(offsetof(Barriers, s_full) + 16 * b1 + 8);
-            }
-            WK_PROF(5);
-            if (++st == kNStages) { st = 0; ph ^= 1; }
-          }
-          continue;
-        }
-        // Step j: for each Q tile, once its P of tile j is there, P V of tile j and Q K^T of tile j + 1 into the S buffer
-        // P was in.  The other Q tile's softmax runs meanwhile.
-        int nv = 0, nv_next = 0;
-        for (int j = -1; j < n_eff; ++j) {
-          const bool more = j + 1 < n_eff;
-          WK_PROF(0);
-          if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &sh.abort))) break;
-          WK_PROF(1);
-          if (j >= 0) {
-            if (!(ok = wait_or_abort(&bars.p_full[0], p_ph0, &sh.abort))) break;
-            p_ph0 ^= 1;
-          }
-          WK_PROF(2);
-          if (more) nv_next = sh.nv[t++ % kNvRing];
-          // A piece's first P V overwrites O: the epilogue of the last piece that used it must have read it.  o_free[i]
-          // completes once per piece in which warpgroup i ran an epilogue, so neither side can run two phases ahead of the
-          // other (a parity wait cannot tell phase n from phase n + 2).
-          if (j == 0 && e0++ > 0 && !(ok = wait_or_abort(&bars.o_free[0], e0 & 1, &sh.abort))) break;
-          tc_fence_after();
-          if (j >= 0) issue_pv(0, st, nv, j > 0);
-          if (more) { issue_s(0, kTmemS, st, nv_next); commit(offsetof(Barriers, s_full)); }
-          else commit(offsetof(Barriers, o_done));
-          WK_PROF(3);
-          if (q1) {
-            if (j >= 0) {
-              if (!(ok = wait_or_abort(&bars.p_full[1], p_ph1, &sh.abort))) break;
-              p_ph1 ^= 1;
-            }
-            WK_PROF(4);
-            if (j == 0 && e1++ > 0 && !(ok = wait_or_abort(&bars.o_free[1], e1 & 1, &sh.abort))) break;
-            tc_fence_after();
-            if (j >= 0) issue_pv(1, st, nv, j > 0);
-            if (more) { issue_s(1, kTmemS + 128, st, nv_next); commit(offsetof(Barriers, s_full) + 8); }
-            else commit(offsetof(Barriers, o_done) + 8);
-            WK_PROF(5);
-          }
-          if (++st == kNStages) { st = 0; ph ^= 1; }
-          nv = nv_next;
-        }
-      }
-      if (lane == 0) leave_role(ok, &sh.abort, p.status);
-      WK_PROF_FLUSH(8, 12, blockIdx.x == 0 && lane == 0);
-    }
+    if constexpr (kLse) mma_lse_role(p, sh, smem_base);
+    else mma_role<0>(p, sh, smem_base);
+  } else if (!kLse && warp == kSoftWarps<kLse> + 1) {
+    if constexpr (!kLse) mma_role<1>(p, sh, smem_base);
   } else if (kLse) {
     // ------------------------------------------------------------------ LSE-only softmax warpgroups (one thread per row)
     // Warpgroup qt + 2 b works on S buffer b of Q tile qt, i.e. on every other KV tile of these rows: four warps per
@@ -680,7 +694,6 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
     uint32_t t0 = 0;    // tiles of the CTA's pieces so far
     uint32_t n = 0;     // units of this Q tile so far
     bool ok = true;
-    WK_PROF_DECL
     while (ok && walk.next(p, pc)) {
       const int n_eff = count_tiles(p, pc.tb, pc.te);
       if (qt == 1 && !pc.has_q1) { t0 += n_eff; continue; }
@@ -688,12 +701,10 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       float m = 0.f, l = 0.f;
       bool first = true;
       for (int j = (g ^ buf) & 1; j < n_eff; j += 2) {
-        WK_PROF(0);
         if (!(ok = wait_or_abort(&bars.s_full[wg], ((g + j) >> 1) & 1, &sh.abort))) break;
-        WK_PROF(1);
         const int nv = sh.nv[(t0 + j) % kNvRing], n_ch = (nv + 31) >> 5;
         if (releases && row == 0) {   // the products that read this tile's stage (and, with the last tile, Q) are done
-          mbar_arrive(&bars.kv_empty[(t0 + j) % kNStages]);
+          mbar_arrive(&bars.kv_empty[(t0 + j) % kStages]);
           if (j + 1 == n_eff) mbar_arrive(&bars.q_empty);
         }
         tc_fence_after();
@@ -708,22 +719,21 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
           float big = -INFINITY;
 #pragma unroll 1
           for (int c = 0; c < n_ch; ++c) {
-            uint32_t r[32], none[16];
+            uint32_t r[32];
             tmem_ld_x32(tS + c * 32, r);
             tc_wait_ld(r);
-            exp_chunk<WK_LSE_POLY, false>(r, nv - c * 32, scale2, neg_m2, acc, big, none);
+            exp_chunk(r, nv - c * 32, scale2, neg_m2, acc, big);
           }
           sum = sum4_f32x2(acc);
           const bool off = !(sum <= 32768.f) || big * p.scale_log2 - m > 100.f || (first && sum < 2.44140625e-4f);
           if (attempt > 0 || !__any_sync(0xffffffffu, off)) break;
-          const float mx = row_max<1>(tS, nv);
+          const float mx = row_max_tmem(tS, nv);
           if (off) {
             const float m_new = first ? mx * p.scale_log2 : fmaxf(m, mx * p.scale_log2);
             l *= ex2_approx(m - m_new);
             m = m_new;
           }
         }
-        WK_PROF(4);
         l += sum;
         first = false;
         tc_fence_before();
@@ -755,7 +765,6 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       ++n;
     }
     if (!ok) leave_role(false, &sh.abort, p.status);
-    WK_PROF_FLUSH(0, 8, blockIdx.x == 0 && tid == 0);
   } else {
     // ------------------------------------------------------------------ softmax warpgroups (one thread per query row)
     const int wg = warp >> 2;
@@ -767,123 +776,105 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
     PieceWalker walk;
     walk.init(p);
     Piece pc;
-    uint32_t g = 0;       // running tile count of this warpgroup
+    uint32_t g = 0;       // steps of this warpgroup waited for so far
     uint32_t t0 = 0;      // tiles of the CTA's pieces so far
+    uint32_t steps = 0;   // stages used by the pieces so far
     uint32_t n_out = 0;   // pieces of this warpgroup that produced output
-    uint32_t steps = 0;   // stages used by the pieces so far (tiles + 1 each)
     bool ok = true;
-    WK_PROF_DECL
     const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2);
     while (ok && walk.next(p, pc)) {
       const bool active = (wg == 0) || pc.has_q1;
-      // S of tile j of the Q tile that comes last in a step is there: the step that filled it is done with its stage (and,
-      // with the last tile, with Q).  The MMA warp could commit to these barriers itself, but every commit after the first
-      // makes it wait until the queue of the tensor pipe has drained.
-      const bool releases = wg == (pc.has_q1 ? 1 : 0);
       const int n_eff = count_tiles(p, pc.tb, pc.te);
-      float m_used = -INFINITY, l = 0.f;
+      float m = -INFINITY, l = 0.f;
       const bool few = n_eff <= kFewTiles;
-      int careful = 0, redos = 0;   // tiles whose maximum is taken first from here on; tiles streamed twice so far
+      // Stages and Q are given back by both warpgroups, for the step whose commit they have seen (by warpgroup 0 twice where
+      // there is no second Q tile): a commit of the MMA warps to these barriers would hold them much longer than this.
+      auto give_back = [&](int i) {
+        if (row == 0) {
+          mbar_arrive(&bars.kv_empty[(steps + i) % kStages]);
+          if (i + 1 == n_eff) mbar_arrive(&bars.q_empty);
+          if (!pc.has_q1) {
+            mbar_arrive(&bars.kv_empty[(steps + i) % kStages]);
+            if (i + 1 == n_eff) mbar_arrive(&bars.q_empty);
+          }
+        }
+      };
       int j = 0;
       if (active) {
-        while (j < n_eff) {
-          WK_PROF(0);
-          if (!(ok = wait_or_abort(&bars.s_full[wg], g & 1, &sh.abort))) break;
-          const int nv = sh.nv[(t0 + j) % kNvRing];
-          WK_PROF(1);
-          if (releases && row == 0) {
-            mbar_arrive(&bars.kv_empty[(steps + j) % kNStages]);
-            if (j + 1 == n_eff) mbar_arrive(&bars.q_empty);
-          }
-          tc_fence_after();
-          // known: the row's maximum over the tile is taken before the exponentials
-          bool known = few || j == 0 || (nv > 64 && nv < kTileKV) || careful > 0;
-          if (careful > 0) --careful;
-          for (;;) {
-            if (known) follow_max(tS, tO, nv, p.scale_log2, few, m_used, l, j > 0);
-            // The row is streamed from tensor memory 32 columns at a time; the next 32 are in flight while these are worked on.
-            uint64_t acc[4] = {0, 0, 0, 0};
-            const uint64_t neg_m2 = pack_f32x2(-m_used, -m_used);
-            float big = -INFINITY;
-            uint32_t ra[32], rb[32];
-            WK_PROF(2);
-            if (nv == kTileKV) {
-              tmem_ld_x32(tS, ra);
-              // P goes over columns 64-127 once these are in registers, where they stay until S is not needed again.
-              uint32_t p0[16], p1[16];
-              tc_wait_ld(ra);
-              tmem_ld_x32(tS + 32, rb);
-              exp_chunk<WK_ATTN_POLY, true>(ra, 32, scale2, neg_m2, acc, big, p0);
-              tc_wait_ld(rb);
-              tmem_ld_x32(tS + 64, ra);
-              exp_chunk<WK_ATTN_POLY, true>(rb, 32, scale2, neg_m2, acc, big, p1);
-              tc_wait_ld(ra);
-              tmem_st_x16(tP, p0);
-              tmem_st_x16(tP + 16, p1);
-              tmem_ld_x32(tS + 96, rb);
-              exp_chunk<WK_ATTN_POLY, true>(ra, 32, scale2, neg_m2, acc, big, p0);
-              tc_wait_ld(rb);
-              tmem_st_x16(tP + 32, p0);
-              exp_chunk<WK_ATTN_POLY, true>(rb, 32, scale2, neg_m2, acc, big, p1);
-              tmem_st_x16(tP + 48, p1);
-              if (!known && __any_sync(0xffffffffu, !(sum4_f32x2(acc) <= kStreamSum) || big * p.scale_log2 - m_used > 100.f)) {
-                tc_wait_st();
-                tmem_st_x32(tS + 64, ra);
-                tmem_st_x32(tS + 96, rb);
-                tc_wait_st();
-                known = true;
-                careful = 1 << min(++redos, 6);
-                continue;
-              }
-            } else {
-              // P of columns 0-63 lies over columns 64-95, of the others over groups behind their own: last columns first.
-              uint32_t pk[16];
+        if (n_eff > 0) {
+          uint32_t pk[kTileKV / 2] = {};   // P of tile j - 1
+          float alpha = 1.f;
+          bool rescale = false;
+          int careful = 0, redos = 0;   // tiles whose maximum is taken first from here on; tiles streamed twice so far
+          for (;; ++j) {
+            // Step j is done: S of tile j is there, and P V of tile j - 2 has read its P.  (A piece of one tile has no step 1.)
+            if (j != 1 || n_eff > 1) {
+              ok = wait_or_abort(&bars.s_full[wg], g++ & 1, &sh.abort);
+              if (!ok) break;
+              tc_fence_after();
+            }
+            if (rescale) {
 #pragma unroll 1
-              for (int c = (nv - 1) & ~31; c >= 64; c -= 32) {
-                tmem_ld_x32(tS + c, ra);
-                tc_wait_ld(ra);
-                exp_chunk<0, true>(ra, nv - c, scale2, neg_m2, acc, big, pk);
-                tmem_st_x16(tP + c / 2, pk);
-              }
-              tmem_ld_x32(tS, ra);
-              if (nv > 32) {
-                tmem_ld_x32(tS + 32, rb);
-                tc_wait_ld(ra);
-                tc_wait_ld(rb);
-                exp_chunk<0, true>(rb, nv - 32, scale2, neg_m2, acc, big, pk);
-                tmem_st_x16(tP + 16, pk);
-              } else {
-                tc_wait_ld(ra);
-              }
-              exp_chunk<0, true>(ra, nv, scale2, neg_m2, acc, big, pk);
-              tmem_st_x16(tP, pk);
-              if (!known && __any_sync(0xffffffffu, !(sum4_f32x2(acc) <= kStreamSum))) {
-                known = true;
-                careful = 1 << min(++redos, 6);
-                continue;
+              for (int c = 0; c < 128; c += 32) {
+                uint32_t o[32];
+                tmem_ld_x32(tO + c, o);
+                tc_wait_ld(o);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                tmem_st_x32(tO + c, o);
               }
             }
-            l += sum4_f32x2(acc);
-            WK_PROF(4);
-            break;
+            // (the first time there is no P to store and the last time no S to load: nobody reads what these move then)
+            uint32_t r[kTileKV];   // S of tile j
+            tmem_st_half_tile(tP, pk);
+            tmem_ld_tile(tS, r);
+            const int nv = sh.nv[(t0 + j) % kNvRing];
+            tmem_ld_wait(r);
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.p_full[wg]);   // one arrival per warp: the waits above covered all 32 lanes
+            if (j != 1 || n_eff > 1) give_back(j);
+            if (j == n_eff) break;
+            if (nv < kTileKV) {   // columns past the end of the segment or slot
+#pragma unroll
+              for (int i = 0; i < kTileKV; ++i) r[i] = i < nv ? r[i] : 0xff800000u;
+            }
+            // known: the row's maximum over the tile is taken before the exponentials
+            bool known = few || j == 0 || careful > 0;
+            if (careful > 0) --careful;
+            rescale = false;
+            float sum;
+            for (;;) {
+              if (known) {
+                const float mt = row_max(r) * p.scale_log2;
+                const float alpha_mt = ex2_approx(m - mt);
+                const bool move = few ? mt > m || (mt < m && l * alpha_mt <= kOwnSum) : mt > m + kRescaleThreshold;   // also true on the first tile (m = -inf)
+                rescale = j > 0 && __any_sync(0xffffffffu, move);
+                alpha = move ? alpha_mt : 1.f;
+                if (move) m = mt;
+                l *= alpha;
+              }
+              float big = -INFINITY;
+              sum = exp_tile(r, scale2, m, big, pk);
+              if (known || !__any_sync(0xffffffffu, !(sum <= kStreamSum) || big * p.scale_log2 - m > 100.f)) break;
+              known = true;
+              careful = 1 << min(++redos, 6);
+            }
+            l += sum;
           }
-          tc_wait_st();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&bars.p_full[wg]);   // one arrival per warp: the wait above covered all 32 lanes' stores
-          WK_PROF(5);
-          ++j;
-          ++g;
         }
         // ---------------------------------------------------------------- epilogue of this piece
         const int prow = wg * kTileQ + row;
         const int qrow = pc.q0 + prow;
-        if (ok && j > 0) ok = wait_or_abort(&bars.o_done[wg], n_out++ & 1, &sh.abort);   // completes once per piece
-        if (ok && j > 0 && releases && row == 0) mbar_arrive(&bars.kv_empty[(steps + n_eff) % kNStages]);   // the last V
+        if (ok && j > 0) {
+          ok = wait_or_abort(&bars.o_done[wg], n_out++ & 1, &sh.abort);   // completes once per piece
+          give_back(n_eff == 1 ? 1 : n_eff + 1);
+        }
         if (ok) {
           tc_fence_after();
           const float inv_l = (j > 0 && l > 0.f) ? 1.f / l : 0.f;
-          const float lse = (j > 0 && l > 0.f) ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
+          const float lse = (j > 0 && l > 0.f) ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             uint32_t r[32];
@@ -925,7 +916,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
         }
       }
       t0 += n_eff;
-      if (n_eff > 0) steps += n_eff + 1;
+      if (n_eff > 0) steps += n_eff == 1 ? 2 : n_eff + 2;
       // O of this piece has been read: the next piece that uses this accumulator may overwrite it
       if (active && j > 0) {
         tc_fence_before();
@@ -934,7 +925,6 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       }
     }
     if (!ok) leave_role(false, &sh.abort, p.status);
-    WK_PROF_FLUSH(0, 8, blockIdx.x == 0 && tid == 0);
   }
 }
 
@@ -947,10 +937,11 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
   const int tid = threadIdx.x;
   if (tid == 0) {
     mbar_init(&sh.bars.q_full, 1);
-    mbar_init(&sh.bars.q_empty, 1);
-    for (int s = 0; s < kStagesLse; ++s) { mbar_init(&sh.bars.kv_full[s], 1); mbar_init(&sh.bars.kv_empty[s], 1); }
+    mbar_init(&sh.bars.q_empty, kLse ? 1 : 2);
+    for (int s = 0; s < kStages; ++s) { mbar_init(&sh.bars.kv_full[s], 1); mbar_init(&sh.bars.kv_empty[s], kLse ? 1 : 2); }
     for (int i = 0; i < 4; ++i) { mbar_init(&sh.bars.s_full[i], 1); mbar_init(&sh.bars.p_full[i], 4); }
     for (int i = 0; i < 2; ++i) {
+      mbar_init(&sh.bars.turn[i], 1);
       mbar_init(&sh.bars.o_done[i], 1);
       mbar_init(&sh.bars.o_free[i], 4);
       mbar_init(&sh.bars.m_full[i], 4);
@@ -1055,35 +1046,38 @@ int attention_partial_slots(int n_heads, int max_lq, int max_splits) {
   return 2 * (by_split > 256 ? by_split : 256);
 }
 
-// Default distribution over the SMs: whole units in full waves, then, where it pays, the units of the last, partial wave
-// cut into equal ranges over all SMs and merged.  The cut saves (sms - rest) / sms of a unit's tiles; it costs about 4
-// tile times (the combine launch, a second prologue) and 16 more when every CTA writes partials.  Measured on 148 SMs,
-// whole -> cut, back to back: 40 heads x 4,680 queries x 32,760 keys (rest 20 of 148) 2,933 -> 2,718 us; 12 heads x 880
-// tokens (rest 132), 167,640 keys 2,559 -> 2,500, 40,000 keys 612 -> 598, 22,500 keys 348 -> 347; 10 heads x 15,840 keys
-// (rest 110) 230 -> 216; 8 heads (rest 88) x 4,500 keys 66 -> 63; 2 heads x 3,960 keys (rest 8) 61 -> 24.  The other way
-// round: 12 heads x 18,480 keys 286 -> 291, 15,840 keys 247 -> 255; 11 heads (rest 121) x 10,000 keys 152 -> 158, x 12,000
-// 182 -> 185; 10 heads x 7,500 keys 108 -> 113; 8 heads x 3,000 keys 48 -> 51.  (With pauses between the calls the cut is
-// worth 1 to 2 % more: it leaves no SM idle, which the power cap does not reward.)
+// Default distribution over the SMs: whole units in full waves, then, where it pays, the units of the last, partial wave cut
+// and merged.  Times in us on 148 SMs, whole / cut, back to back, one dense segment.
+//   * Where every unit can be cut at least in two, it is, into equal ranges that end with their unit: no CTA gets two pieces, and
+//     the idle SMs cost less than pieces that straddle units (30 units of 32 tiles: 120 ranges 26.9, 148 ranges 31.1; of 64
+//     tiles 32.0 and 39.9; 66 units of 38 tiles: 132 ranges 39.1, 148 ranges 45.5).  A piece has 5 tiles or more (2 heads x
+//     3,960 keys, 8 units of 50 tiles: 5 tiles 20.7, 4 21.6, 3 23.2, 10 21.9), and the cut has to save 11 tiles of a unit: the
+//     combine launch, a prologue and the partials cost about that (66 units of 25 tiles 33.6 / 32.8; 50 of 16 24.2 / 27.9; 30 of
+//     16 24.8 / 21.2).
+//   * Else equal ranges over all SMs.  That saves (sms - rest) / sms of a unit's tiles and costs about 8 tiles and, as every CTA
+//     writes partials, up to 22 more; 99 units of 63 tiles 76.8 / 75.1; 88 of 38 49.8 / 53.7, of 57 69.1 / 64.5; 110 of 94 106.4 /
+//     103.3, of 150 170 / 160; 121 of 125 138.3 / 139.2, of 150 177 / 165; 132 of 198 247.8 / 253.6, of 282 357.8 / 358.1, of 500
+//     621 / 597.  With full waves before it: 760 units of 410 tiles (rest 20) 2,953 / 2,763.
 static void split_default(int64_t units, int64_t tiles, int64_t sms, int64_t* G, int64_t* n_full, int64_t* ranges) {
   const int64_t waves = units / sms, rest = units - waves * sms;
   *G = units < sms ? units : sms;
   *n_full = units;
   *ranges = 0;
-  if (rest == 0 || (sms - rest) * tiles < 4 * sms + 16 * rest) return;
-  *n_full = waves * sms;
-  // Where whole cuts of every unit use nearly all SMs, no CTA gets two pieces, and such pieces are kept at 4 tiles or more:
-  // shorter ones cost more in prologues and partials than they save (2 heads x 3,960 keys: 144 unaligned ranges 23.3 us, 128
-  // aligned 21.2, 64 aligned 20.1, 40 unaligned 24.9).  Otherwise a range per SM, however short; 30 units, whole / 148 ranges / 120
-  // aligned cuts: 10 tiles 25.0 / 22.6 / 19.9 us, 20 tiles 41.1 / 26.5 / 23.3, 40 tiles 73.0 / 34.8 / 31.4.
-  int64_t cuts = sms / rest;
-  if (cuts > kMaxPieces - 2) cuts = kMaxPieces - 2;
-  int64_t r = sms;
-  if (cuts >= 2 && ((sms - cuts * rest) * 8 <= sms || cuts == kMaxPieces - 2)) {
+  if (rest == 0) return;
+  int64_t r;
+  if (sms >= 2 * rest) {
+    int64_t cuts = sms / rest;
+    if (cuts > kMaxPieces - 2) cuts = kMaxPieces - 2;
     int64_t per = (tiles + cuts - 1) / cuts;
-    if (per < 4) per = 4;
+    if (per < 5) per = 5;
+    if (tiles - per < 11) return;
     r = rest * ((tiles + per - 1) / per);
+  } else {
+    if ((sms - rest) * tiles < 8 * sms + 22 * rest) return;
+    r = sms;
+    if (r > rest * tiles) r = rest * tiles;
   }
-  if (r > rest * tiles) r = rest * tiles;
+  *n_full = waves * sms;
   *ranges = r;
   *G = waves > 0 ? sms : r;
 }
@@ -1093,17 +1087,25 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
                            cudaStream_t s, bool lse_only) {
   if (!ctx->attn_attr_set) {   // the attribute belongs to the device the context lives on
     WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          static_cast<int>(kSmemBytes)));
+                                          static_cast<int>(kSmemBytes<false>)));
     WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          static_cast<int>(kSmemBytesLse)));
+                                          static_cast<int>(kSmemBytes<true>)));
     ctx->attn_attr_set = true;
   }
   AttnParams p;
   wk_status st = encode_rows_map(ctx, Q, lq, kTileQ, &p.tm_q);
   if (st != WK_OK) return st;
-  p.tm_kpool = ctx->tm_kpool;
+  p.tm_kpool = lse_only ? ctx->tm_kpool_lse : ctx->tm_kpool;
   p.tm_vpool = ctx->tm_vpool;
-  int tiles = 0;
+  // Keys beside which every tile's largest weight counts are tiled in 64 rows, all others in what tensor memory has room for.
+  auto count = [&](int rows, int n_rows) { return (n_rows + rows - 1) / rows; };
+  p.tile_rows = lse_only ? kTileKVLse : kTileKVFew;
+  int tiles = n_slots * count(p.tile_rows, ctx->C);
+  for (int i = 0; i < n_segs; ++i) tiles += count(p.tile_rows, segs[i].n_tokens);
+  if (!lse_only && tiles > kFewTiles) p.tile_rows = kTileKV;
+  int most = n_slots * count(128, ctx->C);   // ranges of a unit that a caller may ask for: one per 128 rows
+  for (int i = 0; i < n_segs; ++i) most += count(128, segs[i].n_tokens);
+  tiles = 0;
   for (int i = 0; i < n_segs; ++i) {
     const CUtensorMap* mk = cached_rows_map(ctx, segs[i].K, segs[i].n_tokens, &st);
     if (st != WK_OK) return st;
@@ -1113,7 +1115,7 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
     p.tm_vd[i] = *mv;
     p.seg_tile_prefix[i] = tiles;
     p.seg_rows[i] = segs[i].n_tokens;
-    tiles += (segs[i].n_tokens + kTileKV - 1) / kTileKV;
+    tiles += count(p.tile_rows, segs[i].n_tokens);
   }
   for (int i = n_segs; i < kMaxDenseSegs; ++i) {
     p.tm_kd[i] = p.tm_q;
@@ -1129,7 +1131,7 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   p.pool_slots = ctx->cfg.pool_slots;
   p.layer = layer;
   p.C = ctx->C;
-  p.tiles_per_slot = (ctx->C + kTileKV - 1) / kTileKV;
+  p.tiles_per_slot = count(p.tile_rows, ctx->C);
   p.n_tiles = tiles + n_slots * p.tiles_per_slot;
   p.lq = lq;
   p.slot_units = lse_only ? 1 : 0;
@@ -1157,23 +1159,22 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   } else if (kv_splits == 0) {
     split_default(p.n_units, p.n_tiles, sms, &G, &n_full, &ranges);
   } else if (kv_splits > 0) {
-    int sp = kv_splits < p.n_tiles ? kv_splits : p.n_tiles;
+    int sp = kv_splits < most ? kv_splits : most;
     if (sp > kMaxPieces) sp = kMaxPieces;
     if (sp == 1) n_full = G = p.n_units;
     else ranges = G = static_cast<int64_t>(p.n_units) * sp;   // every unit cut into exactly sp ranges
   } else {
     ranges = G = -static_cast<int64_t>(kv_splits);      // caller-chosen number of equal ranges
-    const int64_t W = static_cast<int64_t>(p.n_units) * p.n_tiles;
-    if (G * p.n_tiles > W * (kMaxPieces - 2)) return WK_ERR_SHAPE;   // a unit would be cut into too many pieces
-    if (G > W) ranges = G = W;
+    if (G > static_cast<int64_t>(p.n_units) * (kMaxPieces - 2)) return WK_ERR_SHAPE;   // a unit would be cut into too many pieces
+    if (G > static_cast<int64_t>(p.n_units) * most) ranges = G = static_cast<int64_t>(p.n_units) * most;
   }
   const int max_slots = attention_partial_slots(p.H, ctx->max_lq, ctx->max_splits);
   if (!lse_only && 2 * ranges > max_slots) return WK_ERR_SHAPE;
   p.n_full = static_cast<int>(n_full);
   p.n_ranges = static_cast<int>(ranges);
   const dim3 grid(static_cast<unsigned>(G));
-  if (lse_only) launch_chained(memory_attention_kernel<true>, grid, dim3(kThreads<true>), kSmemBytesLse, s, p);
-  else launch_chained(memory_attention_kernel<false>, grid, dim3(kThreads<false>), kSmemBytes, s, p);
+  if (lse_only) launch_chained(memory_attention_kernel<true>, grid, dim3(kThreads<true>), kSmemBytes<true>, s, p);
+  else launch_chained(memory_attention_kernel<false>, grid, dim3(kThreads<false>), kSmemBytes<false>, s, p);
   if ((st = after_launch(ctx)) != WK_OK) return st;
   if (!lse_only && n_full != p.n_units) {   // some unit was cut
     launch_chained(combine_kernel, dim3(static_cast<unsigned>(p.n_units - n_full) * 32), dim3(kCombineThreads), 0, s, p.opart,

@@ -13,7 +13,8 @@ namespace wk {
 
 constexpr int kHeadDim = 128;
 constexpr int kMaxDenseSegs = 8;
-constexpr int kTileKV = 128;   // KV rows per attention tile
+constexpr int kTileKV = 80;       // KV rows per attention tile
+constexpr int kTileKVLse = 128;   // the same in LSE-only launches
 constexpr int kTileQ = 128;    // Q rows per MMA tile (two per CTA)
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -74,7 +75,7 @@ struct wk_ctx {
   int64_t next_seq = 0;
   int32_t n_valid = 0;   // slots in state SLOT_VALID
   // tensor maps
-  CUtensorMap tm_kpool, tm_vpool;
+  CUtensorMap tm_kpool, tm_vpool, tm_kpool_lse;
   std::vector<wk::TmapKey> tmap_cache;
   size_t tmap_cache_next = 0;
   // per-context (hence per-device) one-time kernel attributes: opt-ins to large dynamic shared memory

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("seg_rows", [(1,), (15, 16), (17, 31), (32, 33), (63, 64, 65), (96, 97), (112, 127), (128,), (129, 1, 144),
-                                      (255, 256, 257)])
+                                      (255, 256, 257), (79, 80), (81, 159, 160), (161,), (512,), (513,), (480, 33), (720, 40, 641)])
 @pytest.mark.parametrize("lq", [1, 129, 300])
 def test_short_tiles_of_dense_segments(seg_rows, lq):
     from paper_2605_22718_b200 import WorldKV
