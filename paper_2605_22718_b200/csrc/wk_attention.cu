@@ -119,6 +119,7 @@ struct TileIter {
   int tail;        // valid rows of its last tile
   int z;           // pool matrix index (layer * pool_slots + slot)
   bool ok;         // false for a stale or -1 slot
+  bool entered;    // n_r, tail, z and ok are those of seg
   __device__ __forceinline__ void enter(const AttnParams& p, bool report) {
     if (seg < p.n_segs) {
       n_r = p.seg_tile_prefix[seg + 1] - p.seg_tile_prefix[seg];
@@ -140,7 +141,8 @@ struct TileIter {
       }
     }
   }
-  __device__ __forceinline__ void init(const AttnParams& p, int tb, int te_, bool report) {
+  // Where the walk starts, from the launch's parameters alone (the slot list may be the work of the kernel before).
+  __device__ __forceinline__ void init(const AttnParams& p, int tb, int te_) {
     t = tb;
     te = te_;
     if (tb < p.n_dense_tiles) {
@@ -153,18 +155,18 @@ struct TileIter {
       seg = p.n_segs + si;
       r = u - si * p.tiles_per_slot;
     }
-    n_r = 0;
-    tail = 0;
-    z = 0;
-    ok = false;
-    if (t < te) enter(p, report);
+    entered = false;
   }
   __device__ __forceinline__ bool next(const AttnParams& p, TileInfo& ti, bool report) {
     while (t < te) {
+      if (!entered) {
+        enter(p, report);
+        entered = true;
+      }
       if (r == n_r) {   // first tile of the next segment / slot
         ++seg;
         r = 0;
-        enter(p, report);
+        entered = false;
         continue;
       }
       ti.seg = seg < p.n_segs ? seg : -1;
@@ -508,8 +510,9 @@ __device__ __forceinline__ void mma_role(const AttnParams& p, CtaShared<false>& 
   uint32_t p_ph = 0;             // parity of p_full
   uint32_t n = 0, t = 0, e = 0;  // pieces, tiles, pieces with output of this Q tile so far
   uint32_t k = 0;                // steps that both Q tiles took part in so far
-  bool ok = true;
-  while (ok && walk.next(p, pc)) {
+  bool ok = true, more = walk.next(p, pc);
+  dep_wait();
+  for (; ok && more; more = walk.next(p, pc)) {
     const int n_eff = count_tiles(p, pc.tb, pc.te);
     const bool both = pc.has_q1, mine = kQt == 0 || both;
     if (!(ok = wait_or_abort(&bars.q_full, n & 1, &sh.abort))) break;
@@ -569,8 +572,9 @@ __device__ __forceinline__ void mma_lse_role(const AttnParams& p, CtaShared<true
   uint32_t st = 0, ph = 0;   // stage and its parity
   uint32_t n = 0, t = 0;     // pieces and tiles so far
   uint32_t s0 = 0, s1 = 0;   // products of Q tile 0 / 1 so far
-  bool ok = true;
-  while (ok && walk.next(p, pc)) {
+  bool ok = true, more = walk.next(p, pc);
+  dep_wait();
+  for (; ok && more; more = walk.next(p, pc)) {
     const int n_eff = count_tiles(p, pc.tb, pc.te);
     if (!(ok = wait_or_abort(&bars.q_full, n & 1, &sh.abort))) break;
     ++n;
@@ -616,9 +620,17 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       PieceWalker walk;
       walk.init(p);
       Piece pc;
+      TileIter it;
       uint32_t st = 0, ph = 1, steps = 0, n = 0, t = 0;   // stage, its parity, stages and Q pairs armed so far, tiles so far
-      bool ok = true;
-      while (ok && walk.next(p, pc)) {
+      bool ok = true, more = walk.next(p, pc);
+      TileInfo ti, t1, t2;   // this tile and the two before it
+      bool have = false;
+      if (more) it.init(p, pc.tb, pc.te);
+      const bool early = more && pc.tb < p.n_dense_tiles;   // the first tile is known without the slot list
+      if (early) have = it.next(p, ti, false);
+      dep_wait();
+      for (; ok && more; more = walk.next(p, pc)) {
+        if (n > 0) it.init(p, pc.tb, pc.te);
         if (!(ok = wait_or_abort(&bars.q_empty, (n & 1) ^ 1, &sh.abort))) break;
         mbar_expect_tx(&bars.q_full, 2 * kQBytes);
         ++n;
@@ -626,9 +638,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
           for (int half = 0; half < 2; ++half)
             tma_load_2d(sQ + i * kQBytes + half * kHalfQBytes, &p.tm_q, &bars.q_full,
                         pc.h * kHeadDim + half * 64, pc.q0 + i * kTileQ);
-        TileIter it;
         const bool report = !p.slot_units;
-        it.init(p, pc.tb, pc.te, report);
         const int x = pc.h * kHeadDim;
         auto load = [&](uint8_t* dst, const TileInfo& ti, const CUtensorMap* seg_maps, const CUtensorMap* pool_map) {
           if (ti.seg >= 0) {
@@ -639,8 +649,8 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
             tma_load_3d(dst + kHalfKvBytes<kLse>, pool_map, &bars.kv_full[st], x + 64, ti.row0, ti.z);
           }
         };
-        TileInfo ti, t1, t2;   // this tile and the two before it
-        bool have = it.next(p, ti, report), have1 = false, have2 = false;
+        bool have1 = false, have2 = false;
+        if (n > 1 || !early) have = it.next(p, ti, report);
         while (have || have1 || have2) {   // step: K of this tile, V of the last but one (not in LSE-only launches)
           if (have || have2) {             // (a piece of one tile has nothing in its second step)
             if (!(ok = wait_or_abort(&bars.kv_empty[st], ph, &sh.abort))) break;
@@ -694,7 +704,10 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
     uint32_t t0 = 0;    // tiles of the CTA's pieces so far
     uint32_t n = 0;     // units of this Q tile so far
     bool ok = true;
-    while (ok && walk.next(p, pc)) {
+    bool more = walk.next(p, pc);
+    dep_wait();
+    dep_release();
+    for (; ok && more; more = walk.next(p, pc)) {
       const int n_eff = count_tiles(p, pc.tb, pc.te);
       if (qt == 1 && !pc.has_q1) { t0 += n_eff; continue; }
       const bool releases = qt == (pc.has_q1 ? 1 : 0);   // the Q tile whose product comes last
@@ -782,7 +795,11 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
     uint32_t n_out = 0;   // pieces of this warpgroup that produced output
     bool ok = true;
     const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2);
-    while (ok && walk.next(p, pc)) {
+    const bool wide = (reinterpret_cast<uint64_t>(p.O) & 31) == 0;
+    bool more = walk.next(p, pc);
+    dep_wait();
+    dep_release();
+    for (; ok && more; more = walk.next(p, pc)) {
       const bool active = (wg == 0) || pc.has_q1;
       const int n_eff = count_tiles(p, pc.tb, pc.te);
       float m = -INFINITY, l = 0.f;
@@ -887,15 +904,18 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
             }
             if (qrow < p.lq) {
               if (pc.slot < 0) {
-                uint4* dst = reinterpret_cast<uint4*>(p.O + (static_cast<int64_t>(qrow) * p.H + pc.h) * kHeadDim + c * 32);
+                // a row per lane: 32 lines per store whatever its width, so the widest that O's alignment allows
+                __nv_bfloat16* dst = p.O + (static_cast<int64_t>(qrow) * p.H + pc.h) * kHeadDim + c * 32;
+                uint32_t o[16];
 #pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                  uint4 o;
-                  o.x = pack_bf16x2(__uint_as_float(r[8 * v + 0]) * inv_l, __uint_as_float(r[8 * v + 1]) * inv_l);
-                  o.y = pack_bf16x2(__uint_as_float(r[8 * v + 2]) * inv_l, __uint_as_float(r[8 * v + 3]) * inv_l);
-                  o.z = pack_bf16x2(__uint_as_float(r[8 * v + 4]) * inv_l, __uint_as_float(r[8 * v + 5]) * inv_l);
-                  o.w = pack_bf16x2(__uint_as_float(r[8 * v + 6]) * inv_l, __uint_as_float(r[8 * v + 7]) * inv_l);
-                  dst[v] = o;
+                for (int v = 0; v < 16; ++v) o[v] = pack_bf16x2(__uint_as_float(r[2 * v]) * inv_l, __uint_as_float(r[2 * v + 1]) * inv_l);
+                if (wide) {
+                  st_global_x8(dst, o);
+                  st_global_x8(dst + 16, o + 8);
+                } else {
+#pragma unroll
+                  for (int v = 0; v < 4; ++v)
+                    reinterpret_cast<uint4*>(dst)[v] = make_uint4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
                 }
               } else {
                 float4* dst = p.opart + (static_cast<int64_t>(pc.slot) * 32 + c * 8) * kPairRows + prow;
@@ -954,14 +974,21 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
     tmem_alloc(&sh.tmem, 512);
     tmem_relinquish();
   }
+  if (tid >= 32 && tid < 32 + 3 + 2 * kMaxDenseSegs) {
+    const int i = tid - 32;   // tm_q, tm_kpool, tm_vpool, tm_kd[], tm_vd[] lie one behind the other
+    if (i < 3 || (i - 3) % kMaxDenseSegs < p.n_segs) prefetch_tensormap(&p.tm_q + i);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // everything above runs under the end of the kernel before this one; nothing is read or written before this wait
-  dep_wait();
-  dep_release();
+  // Everything up to the roles' dep_wait() runs under the end of the kernel before this one, and nothing that it may write is read
+  // or overwritten there: a role works out from the launch's parameters where it starts (0.7 to 2 us after the wait before).
   // an allocation of all 512 columns starts at column 0; addresses known at compile time keep the MMAs' operands cheap
-  if (sh.tmem != 0 && tid == 0) { sh.abort = 1; atomicOr(p.status, WK_DEV_TIMEOUT); }
+  if (sh.tmem != 0 && tid == 0) {
+    dep_wait();
+    sh.abort = 1;
+    atomicOr(p.status, WK_DEV_TIMEOUT);
+  }
 
   attention_roles<kLse>(p, sh, smem);
   tc_fence_before();
@@ -983,8 +1010,6 @@ combine_kernel(const float4* __restrict__ opart, const float* __restrict__ lsepa
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ut = blockIdx.x >> 5, u = n_full + ut, rg = (blockIdx.x >> 2) & 7, cg = blockIdx.x & 3;   // unit, row group, column group
   const int h = u / n_qpairs, qrow0 = (u - h * n_qpairs) * kPairRows + rg * 32;
-  dep_wait();
-  if (qrow0 >= lq) return;
   // the CTAs whose ranges touch the unit: lane i looks at the i-th one (every range holds at least one tile)
   const int64_t W = static_cast<int64_t>(n_units - n_full) * n_tiles;
   const int64_t ustart = static_cast<int64_t>(ut) * n_tiles, uend = ustart + n_tiles;
@@ -996,7 +1021,9 @@ combine_kernel(const float4* __restrict__ opart, const float* __restrict__ lsepa
   const int64_t sc = start_of(cc);
   const bool mine = cc < G && sc < uend;
   const int np = __popc(__ballot_sync(0xffffffffu, mine));
-  if (np == 1 && start_of(c0) <= ustart && start_of(c0 + 1) >= uend) return;   // one CTA covered the whole unit
+  const bool single = np == 1 && start_of(c0) <= ustart && start_of(c0 + 1) >= uend;   // one CTA covered the whole unit
+  dep_wait();
+  if (single || qrow0 >= lq) return;
   if (warp == 0 && mine) s_slot[lane] = 2 * cc + (sc >= ustart ? 0 : 1);
   __syncthreads();
   for (int s = warp; s < np; s += kCombineThreads / 32)
