@@ -1004,7 +1004,6 @@ constexpr int kCombineThreads = 256;
 __global__ void __launch_bounds__(kCombineThreads)
 combine_kernel(const float4* __restrict__ opart, const float* __restrict__ lsepart, int G, int n_full, int n_units, int n_tiles,
                int n_qpairs, int H, int lq, __nv_bfloat16* __restrict__ O, float* __restrict__ lse_out) {
-  __shared__ int s_slot[kMaxPieces];
   __shared__ float s_lse[kMaxPieces][32], s_w[kMaxPieces][32];
   __shared__ __align__(16) uint2 s_out[32][8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1022,12 +1021,21 @@ combine_kernel(const float4* __restrict__ opart, const float* __restrict__ lsepa
   const bool mine = cc < G && sc < uend;
   const int np = __popc(__ballot_sync(0xffffffffu, mine));
   const bool single = np == 1 && start_of(c0) <= ustart && start_of(c0 + 1) >= uend;   // one CTA covered the whole unit
+  // the partial-result slots of range c: 2 c for the piece it starts with, 2 c + 1 for the one it ends with
+  const int enters = start_of(c0) < ustart ? 1 : 0;
+  auto slot_of = [&](int s) { return static_cast<int64_t>(2 * (c0 + s) + (s == 0 ? enters : 0)); };
+  const int64_t at = static_cast<int64_t>(cg * 8 + warp) * kPairRows + rg * 32 + lane;
+  auto load8 = [&](int s0, float4 (&o)[8]) {   // eight pieces' loads in flight
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      o[i] = s0 + i < np ? __ldcg(opart + slot_of(s0 + i) * 32 * kPairRows + at) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
   dep_wait();
   if (single || qrow0 >= lq) return;
-  if (warp == 0 && mine) s_slot[lane] = 2 * cc + (sc >= ustart ? 0 : 1);
-  __syncthreads();
+  float4 o[8];
+  load8(0, o);   // beside the weights, which need two trips of their own
   for (int s = warp; s < np; s += kCombineThreads / 32)
-    s_lse[s][lane] = __ldcg(lsepart + static_cast<int64_t>(s_slot[s]) * kPairRows + rg * 32 + lane);
+    s_lse[s][lane] = __ldcg(lsepart + slot_of(s) * kPairRows + rg * 32 + lane);
   __syncthreads();
   float mx = -INFINITY;
   for (int s = 0; s < np; ++s) mx = fmaxf(mx, s_lse[s][lane]);
@@ -1036,12 +1044,8 @@ combine_kernel(const float4* __restrict__ opart, const float* __restrict__ lsepa
   __syncthreads();
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   float wsum = 0.f;
-  const int64_t at = static_cast<int64_t>(cg * 8 + warp) * kPairRows + rg * 32 + lane;
-  for (int s0 = 0; s0 < np; s0 += 8) {   // eight pieces' loads in flight
-    float4 o[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-      o[i] = s0 + i < np ? __ldcg(opart + static_cast<int64_t>(s_slot[s0 + i]) * 32 * kPairRows + at) : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int s0 = 0; s0 < np; s0 += 8) {
+    if (s0 > 0) load8(s0, o);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       if (s0 + i < np) {
