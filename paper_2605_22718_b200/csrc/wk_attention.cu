@@ -64,8 +64,8 @@ constexpr float kStreamSum = 256.0f;
 // Pieces of at most kFewTiles tiles move the reference to every tile's own maximum, down as well as up: beside few other keys a
 // tile's largest weight counts, and it is exact this way, as if the tile were a piece of its own.  450 queries x 5 heads x 1,040
 // keys (pieces of three tiles), relative error of O at deviations 1 / 2 / 4: 2.13 / 1.80 / 1.69e-3, without 2.27 / 2.19 / 1.98e-3.
-// Calls whose keys are that few altogether walk them in tiles of kTileKVFew rows, so that no more keys share a maximum.
-constexpr int kFewTiles = 8, kTileKVFew = 64;
+// Calls of at most kFewTilesOfCall tiles of kTileKVFew rows walk them in such tiles, so that no more keys share a maximum.
+constexpr int kFewTiles = 10, kTileKVFew = 64, kFewTilesOfCall = 8;
 constexpr float kOwnSum = 1024.0f;
 // tensor-memory columns: S0, P0, S1, P1 (80 + 40 of 128 each), O0, O1; LSE-only: S0, S1 twice
 constexpr uint32_t kTmemS = 0, kTmemP = kTileKV, kTmemO = 256;
@@ -347,8 +347,9 @@ __device__ __forceinline__ float row_max(const uint32_t (&r)[kTileKV]) {
   for (int i = 0; i < kTileKV; i += 2) mx[(i >> 1) & 3] = fmax3(mx[(i >> 1) & 3], __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
   return fmax3(fmaxf(mx[0], mx[1]), mx[2], mx[3]);
 }
-// P = 2^(s * scale - m) of a row, as bf16 pairs, and their sum.  One of every 8 pairs takes the FMA pipe; big = the largest of
-// their raw values (see exp_chunk).
+// P = 2^(s * scale - m) of a row, as bf16 pairs, and their sum.  With kPoly (calls of more than a few tiles) one of every 8
+// pairs takes the FMA pipe; big = the largest of their raw values (see exp_chunk).  (97 keys: log-sum-exp within 8e-7, with a share of cubics 1e-5.)
+template <bool kPoly>
 __device__ __forceinline__ float exp_tile(const uint32_t (&r)[kTileKV], uint64_t scale2, float m, float& big, uint32_t (&pk)[kTileKV / 2]) {
   const uint64_t neg_m2 = pack_f32x2(-m, -m);
   uint64_t acc[4] = {0, 0, 0, 0};
@@ -357,7 +358,7 @@ __device__ __forceinline__ float exp_tile(const uint32_t (&r)[kTileKV], uint64_t
     const float s0 = __uint_as_float(r[2 * i]), s1 = __uint_as_float(r[2 * i + 1]);
     const uint64_t e = fma_f32x2(pack_f32x2(s0, s1), scale2, neg_m2);
     float p0, p1;
-    if ((i & 7) == 4) {
+    if (kPoly && (i & 7) == 4) {
       exp2_pair<true>(e, p0, p1);
       big = fmax3(big, s0, s1);
     } else {
@@ -803,7 +804,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       const bool active = (wg == 0) || pc.has_q1;
       const int n_eff = count_tiles(p, pc.tb, pc.te);
       float m = -INFINITY, l = 0.f;
-      const bool few = n_eff <= kFewTiles;
+      const bool few = n_eff <= kFewTiles, plain = few && p.tile_rows < kTileKV;
       // Stages and Q are given back by both warpgroups, for the step whose commit they have seen (by warpgroup 0 twice where
       // there is no second Q tile): a commit of the MMA warps to these barriers would hold them much longer than this.
       auto give_back = [&](int i) {
@@ -873,7 +874,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
                 l *= alpha;
               }
               float big = -INFINITY;
-              sum = exp_tile(r, scale2, m, big, pk);
+              sum = plain ? exp_tile<false>(r, scale2, m, big, pk) : exp_tile<true>(r, scale2, m, big, pk);
               if (known || !__any_sync(0xffffffffu, !(sum <= kStreamSum) || big * p.scale_log2 - m > 100.f)) break;
               known = true;
               careful = 1 << min(++redos, 6);
@@ -1082,29 +1083,26 @@ int attention_partial_slots(int n_heads, int max_lq, int max_splits) {
 //   * Where every unit can be cut at least in two, it is, into equal ranges that end with their unit: no CTA gets two pieces, and
 //     the idle SMs cost less than pieces that straddle units (30 units of 32 tiles: 120 ranges 26.9, 148 ranges 31.1; of 64
 //     tiles 32.0 and 39.9; 66 units of 38 tiles: 132 ranges 39.1, 148 ranges 45.5).  A piece has 5 tiles or more (2 heads x
-//     3,960 keys, 8 units of 50 tiles: 5 tiles 20.7, 4 21.6, 3 23.2, 10 21.9), and the cut has to save 11 tiles of a unit: the
-//     combine launch, a prologue and the partials cost about that (66 units of 25 tiles 33.6 / 32.8; 50 of 16 24.2 / 27.9; 30 of
-//     16 24.8 / 21.2).
-//   * Else equal ranges over all SMs.  That saves (sms - rest) / sms of a unit's tiles and costs about 8 tiles and, as every CTA
-//     writes partials, up to 22 more; 99 units of 63 tiles 76.8 / 75.1; 88 of 38 49.8 / 53.7, of 57 69.1 / 64.5; 110 of 94 106.4 /
-//     103.3, of 150 170 / 160; 121 of 125 138.3 / 139.2, of 150 177 / 165; 132 of 198 247.8 / 253.6, of 282 357.8 / 358.1, of 500
-//     621 / 597.  With full waves before it: 760 units of 410 tiles (rest 20) 2,953 / 2,763.
+//     3,960 keys, 8 units of 50 tiles: 5 tiles 20.7, 4 21.6, 3 23.2, 10 21.9).  Else equal ranges over all SMs.
+//   * A cut saves at most (sms - rest) / sms of a unit's tiles and costs about 8 tiles (the combine launch, a second prologue) and
+//     up to 22 more where every CTA writes partials: 30 units of 16 tiles 24.8 / 21.2; 50 of 16 24.2 / 27.9; 66 of 25 33.6 / 32.8;
+//     88 of 38 49.8 / 53.7, of 57 69.1 / 64.5; 99 of 63 76.8 / 75.1; 110 of 94 106.4 / 103.3, of 150 170 / 160; 121 of 125 138.3 /
+//     139.2, of 150 177 / 165; 132 of 198 247.8 / 253.6, of 282 357.8 / 358.1, of 500 621 / 597.  With full waves before it: 760
+//     units of 410 tiles (rest 20) 2,953 / 2,763.
 static void split_default(int64_t units, int64_t tiles, int64_t sms, int64_t* G, int64_t* n_full, int64_t* ranges) {
   const int64_t waves = units / sms, rest = units - waves * sms;
   *G = units < sms ? units : sms;
   *n_full = units;
   *ranges = 0;
-  if (rest == 0) return;
+  if (rest == 0 || (sms - rest) * tiles < 8 * sms + 22 * rest) return;
   int64_t r;
   if (sms >= 2 * rest) {
     int64_t cuts = sms / rest;
     if (cuts > kMaxPieces - 2) cuts = kMaxPieces - 2;
     int64_t per = (tiles + cuts - 1) / cuts;
     if (per < 5) per = 5;
-    if (tiles - per < 11) return;
     r = rest * ((tiles + per - 1) / per);
   } else {
-    if ((sms - rest) * tiles < 8 * sms + 22 * rest) return;
     r = sms;
     if (r > rest * tiles) r = rest * tiles;
   }
@@ -1133,7 +1131,7 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   p.tile_rows = lse_only ? kTileKVLse : kTileKVFew;
   int tiles = n_slots * count(p.tile_rows, ctx->C);
   for (int i = 0; i < n_segs; ++i) tiles += count(p.tile_rows, segs[i].n_tokens);
-  if (!lse_only && tiles > kFewTiles) p.tile_rows = kTileKV;
+  if (!lse_only && tiles > kFewTilesOfCall) p.tile_rows = kTileKV;
   int most = n_slots * count(128, ctx->C);   // ranges of a unit that a caller may ask for: one per 128 rows
   for (int i = 0; i < n_segs; ++i) most += count(128, segs[i].n_tokens);
   tiles = 0;
