@@ -14,7 +14,7 @@
 //     O0 and O1 take half of its 512 columns; 80 keys is the widest tile whose S (80 columns) and P (bf16: 40 columns, the A
 //     operand of P V) lie side by side in the other half, so that S of the next tile can be multiplied while the softmax works
 //     on this one, which it has read into registers.  (With 128 keys P has to overwrite S and the two take turns: 12 heads x
-//     2,640 queries x 15,840 keys 261 us back to back instead of 251, although Q K^T alone runs at its full rate only from
+//     2,640 queries x 15,840 keys 261 us back to back instead of 253, although Q K^T alone runs at its full rate only from
 //     N = 128 on: shared memory gives a Q K^T step of 80 keys (4 + 2.5 KB) in 52 clk, one of 128 (4 + 4 KB) in 64.)
 //   * warp roles: warps 0-3 / 4-7 = softmax of Q tile 0 / 1 (one thread per row, fp32 in the exp2
 //     domain, against a reference that follows the row's maximum: see kStreamSum), warps 8 / 9 = MMA issue for Q tile 0 / 1,
@@ -22,9 +22,9 @@
 //   * a tile with fewer valid rows (the last one of a segment or slot: 1,320 rows are 16 tiles and 40 rows) is
 //     multiplied over ceil(nv / 16) * 16 rows.
 // What bounds it: back to back, the energy that the board's 1,000 W cap allows.  2,640 queries x 15,840 keys x 12 heads is one
-// unit of 201 KV tiles on each of 132 SMs: 251 us at 1,640 MHz, 1,780 clk per tile in full flow, where the tensor pipe needs
+// unit of 201 KV tiles on each of 132 SMs: 253 us at 1,640 MHz, 1,780 clk per tile in full flow, where the tensor pipe needs
 // 1,432 (measured with nothing else running; 1,600 with the exponentials left out: the chain S -> registers, P -> P V, Q K^T of
-// one Q tile is 1,470 long, 750 of it hand-overs).  4,680 x 32,760 x 40: 2,725 us at 1,480 MHz.
+// one Q tile is 1,470 long, 750 of it hand-overs).  4,680 x 32,760 x 40: 2,777 us at 1,555 MHz.
 // Every wait is bounded; a wait that runs out sets WK_DEV_TIMEOUT, the CTA drains and frees its tensor memory.
 #include <stddef.h>
 
@@ -156,6 +156,10 @@ struct TileIter {
       r = u - si * p.tiles_per_slot;
     }
     entered = false;
+  }
+  __device__ __forceinline__ void open(const AttnParams& p, bool report) {   // looks the first segment or slot up
+    if (!entered && t < te) enter(p, report);
+    entered = true;
   }
   __device__ __forceinline__ bool next(const AttnParams& p, TileInfo& ti, bool report) {
     while (t < te) {
@@ -608,7 +612,7 @@ __device__ __forceinline__ void mma_lse_role(const AttnParams& p, CtaShared<true
 }
 
 // All of a CTA's work.
-template <bool kLse>
+template <bool kLse, bool kShort>
 __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<kLse>& sh, uint8_t* smem) {
   const uint32_t smem_base = smem_u32(smem);
   uint8_t* sQ = smem;                 // [2 q tiles][2 halves][128 rows][128 B]
@@ -630,8 +634,10 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       const bool early = more && pc.tb < p.n_dense_tiles;   // the first tile is known without the slot list
       if (early) have = it.next(p, ti, false);
       dep_wait();
+      const bool report = !p.slot_units;
       for (; ok && more; more = walk.next(p, pc)) {
         if (n > 0) it.init(p, pc.tb, pc.te);
+        it.open(p, report);
         if (!(ok = wait_or_abort(&bars.q_empty, (n & 1) ^ 1, &sh.abort))) break;
         mbar_expect_tx(&bars.q_full, 2 * kQBytes);
         ++n;
@@ -639,7 +645,6 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
           for (int half = 0; half < 2; ++half)
             tma_load_2d(sQ + i * kQBytes + half * kHalfQBytes, &p.tm_q, &bars.q_full,
                         pc.h * kHeadDim + half * 64, pc.q0 + i * kTileQ);
-        const bool report = !p.slot_units;
         const int x = pc.h * kHeadDim;
         auto load = [&](uint8_t* dst, const TileInfo& ti, const CUtensorMap* seg_maps, const CUtensorMap* pool_map) {
           if (ti.seg >= 0) {
@@ -804,7 +809,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       const bool active = (wg == 0) || pc.has_q1;
       const int n_eff = count_tiles(p, pc.tb, pc.te);
       float m = -INFINITY, l = 0.f;
-      const bool few = n_eff <= kFewTiles, plain = few && p.tile_rows < kTileKV;
+      const bool few = n_eff <= kFewTiles;
       // Stages and Q are given back by both warpgroups, for the step whose commit they have seen (by warpgroup 0 twice where
       // there is no second Q tile): a commit of the MMA warps to these barriers would hold them much longer than this.
       auto give_back = [&](int i) {
@@ -874,7 +879,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
                 l *= alpha;
               }
               float big = -INFINITY;
-              sum = plain ? exp_tile<false>(r, scale2, m, big, pk) : exp_tile<true>(r, scale2, m, big, pk);
+              sum = exp_tile<!kShort>(r, scale2, m, big, pk);
               if (known || !__any_sync(0xffffffffu, !(sum <= kStreamSum) || big * p.scale_log2 - m > 100.f)) break;
               known = true;
               careful = 1 << min(++redos, 6);
@@ -949,7 +954,9 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
   }
 }
 
-template <bool kLse>
+// kShort: keys in tiles of kTileKVFew rows.  (One kernel for both, with the choice in the loop: 254.7 us instead of 253.2 for 12 heads x
+// 2,640 queries x 15,840 keys.)
+template <bool kLse, bool kShort>
 __global__ void __launch_bounds__(kThreads<kLse>, 1)
 memory_attention_kernel(const __grid_constant__ AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -991,7 +998,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
     atomicOr(p.status, WK_DEV_TIMEOUT);
   }
 
-  attention_roles<kLse>(p, sh, smem);
+  attention_roles<kLse, kShort>(p, sh, smem);
   tc_fence_before();
   __syncthreads();
   if (tid < 32) tmem_dealloc(sh.tmem, 512);
@@ -1115,9 +1122,11 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
                            const int32_t* slots_dev, int n_slots, __nv_bfloat16* O, float* lse, int kv_splits,
                            cudaStream_t s, bool lse_only) {
   if (!ctx->attn_attr_set) {   // the attribute belongs to the device the context lives on
-    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           static_cast<int>(kSmemBytes<false>)));
-    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          static_cast<int>(kSmemBytes<false>)));
+    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           static_cast<int>(kSmemBytes<true>)));
     ctx->attn_attr_set = true;
   }
@@ -1202,8 +1211,9 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   p.n_full = static_cast<int>(n_full);
   p.n_ranges = static_cast<int>(ranges);
   const dim3 grid(static_cast<unsigned>(G));
-  if (lse_only) launch_chained(memory_attention_kernel<true>, grid, dim3(kThreads<true>), kSmemBytes<true>, s, p);
-  else launch_chained(memory_attention_kernel<false>, grid, dim3(kThreads<false>), kSmemBytes<false>, s, p);
+  if (lse_only) launch_chained(memory_attention_kernel<true, false>, grid, dim3(kThreads<true>), kSmemBytes<true>, s, p);
+  else launch_chained(p.tile_rows == kTileKV ? memory_attention_kernel<false, false> : memory_attention_kernel<false, true>, grid,
+                      dim3(kThreads<false>), kSmemBytes<false>, s, p);
   if ((st = after_launch(ctx)) != WK_OK) return st;
   if (!lse_only && n_full != p.n_units) {   // some unit was cut
     launch_chained(combine_kernel, dim3(static_cast<unsigned>(p.n_units - n_full) * 32), dim3(kCombineThreads), 0, s, p.opart,

@@ -104,34 +104,39 @@ struct BestSlots {
   unsigned long long group[kSmallSlots / 8], key[kSmallSlots], cut;
   int slot[kSmallSlots], rank[kSmallSlots], n;
 };
-// Called by the whole block (slot tid's key comes from thread tid; as many threads as slots at least); returns the number of
-// entries in sh.  Ranks come from counting comparisons, which all slots against all others would make most of a kernel's time (250
+// Called by the whole block (slot tid's key comes from thread tid; as many threads as slots at least), a block barrier after
+// rank_begin; returns the number of entries in sh.  Ranks come from counting comparisons, which all slots against all others would make most of a kernel's time (250
 // slots: 8,900 of 12,600 clocks).  So a cut first: the k-th smallest of the minima of groups of eight slots has at least k
-// slots at or below it and leaves few more.  250 slots, k = 8: 6.85 -> 5.28 us per call; 1,000 slots 13.6 -> 5.2.
+// slots at or below it and leaves few more.  250 slots, k = 8: 6.85 -> 5.28 us per call; 1,000 slots 13.6 -> 5.2.  Where the block
+// has threads enough for all comparisons at once the cut costs more (two barriers) than it saves.
+__device__ __forceinline__ void rank_begin(BestSlots& sh) {
+  sh.rank[threadIdx.x] = 0;
+  if (threadIdx.x == 0) { sh.cut = kNone - 1; sh.n = 0; }
+}
 __device__ __forceinline__ int rank_best(BestSlots& sh, unsigned long long key, int n_slots, int k) {
   const int tid = threadIdx.x;
-  unsigned long long g = key;
+  if (n_slots * n_slots > 16 * static_cast<int>(blockDim.x)) {
+    unsigned long long g = key;
 #pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
-    const unsigned long long v = __shfl_xor_sync(0xffffffffu, g, o);
-    g = v < g ? v : g;
-  }
-  const int n_groups = (n_slots + 7) >> 3;
-  if ((tid & 7) == 0 && (tid >> 3) < n_groups) sh.group[tid >> 3] = g;
-  sh.rank[tid] = 0;
-  if (tid == 0) { sh.cut = kNone - 1; sh.n = 0; }
-  __syncthreads();
-  if (tid < n_groups && k <= n_groups) {
-    const unsigned long long kg = sh.group[tid];
-    int rank = 0;
-#pragma unroll 8
-    for (int u = 0; u < n_groups; ++u) {
-      const unsigned long long ku = sh.group[u];
-      rank += static_cast<int>(ku < kg) | (static_cast<int>(ku == kg) & static_cast<int>(u < tid));
+    for (int o = 1; o < 8; o <<= 1) {
+      const unsigned long long v = __shfl_xor_sync(0xffffffffu, g, o);
+      g = v < g ? v : g;
     }
-    if (rank == k - 1 && kg != kNone) sh.cut = kg;
+    const int n_groups = (n_slots + 7) >> 3;
+    if ((tid & 7) == 0 && (tid >> 3) < n_groups) sh.group[tid >> 3] = g;
+    __syncthreads();
+    if (tid < n_groups && k <= n_groups) {
+      const unsigned long long kg = sh.group[tid];
+      int rank = 0;
+#pragma unroll 8
+      for (int u = 0; u < n_groups; ++u) {
+        const unsigned long long ku = sh.group[u];
+        rank += static_cast<int>(ku < kg) | (static_cast<int>(ku == kg) & static_cast<int>(u < tid));
+      }
+      if (rank == k - 1 && kg != kNone) sh.cut = kg;
+    }
+    __syncthreads();
   }
-  __syncthreads();
   if (key <= sh.cut) {
     const int pos = atomicAdd(&sh.n, 1);
     sh.key[pos] = key;
@@ -166,6 +171,7 @@ retrieve_small(const float* __restrict__ poses, const int32_t* __restrict__ vali
   __shared__ unsigned long long s_t[32], s_r[32];
   __shared__ BestSlots sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  rank_begin(sh);
   dep_wait();
   dep_release();
   double t = 0.0, r = 0.0;
@@ -307,6 +313,7 @@ query_topk(const double* __restrict__ block_part, int n_blocks, const int32_t* _
   int P = 1;
   while (P < 8 && n_slots * P * 2 <= 1024) P <<= 1;
   const int s = tid % n_slots, q = tid / n_slots;   // slot and share (threads with q >= P idle)
+  rank_begin(sh);
   dep_wait();
   for (int i = tid; i < max_k; i += 1024) {
     slots_out[i] = -1;
