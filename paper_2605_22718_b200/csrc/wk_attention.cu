@@ -529,6 +529,9 @@ __device__ __forceinline__ void mma_role(const AttnParams& p, CtaShared<false>& 
     // Step j: once P of tile j - 2 is in tensor memory and S of tile j - 1 in registers (p_full), P V of the one and Q K^T of
     // tile j.  The softmax of tile j - 1 runs meanwhile; it stores its P when this step's commit arrives.
     if (!mine) {
+      // Nothing else in this piece waits for this warp, so Q is given back by it too: otherwise q_full could complete twice before
+      // it looks, and a parity wait cannot tell phase n from phase n + 2.
+      if (lane == 0) mbar_arrive(&bars.q_empty);
       const uint32_t used = st + (n_eff == 1 ? 2 : n_eff + 2);
       ph ^= (used / kStages) & 1;
       st = used % kStages;
@@ -810,16 +813,14 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       const int n_eff = count_tiles(p, pc.tb, pc.te);
       float m = -INFINITY, l = 0.f;
       const bool few = n_eff <= kFewTiles;
-      // Stages and Q are given back by both warpgroups, for the step whose commit they have seen (by warpgroup 0 twice where
-      // there is no second Q tile): a commit of the MMA warps to these barriers would hold them much longer than this.
+      // Stages and Q are given back by both warpgroups, for the step whose commit they have seen: a commit of the MMA warps to these
+      // barriers would hold them much longer than this.  Where there is no second Q tile, warpgroup 0 gives a stage back twice, and
+      // Q is given back by warpgroup 0 and the idle MMA warp.
       auto give_back = [&](int i) {
         if (row == 0) {
           mbar_arrive(&bars.kv_empty[(steps + i) % kStages]);
           if (i + 1 == n_eff) mbar_arrive(&bars.q_empty);
-          if (!pc.has_q1) {
-            mbar_arrive(&bars.kv_empty[(steps + i) % kStages]);
-            if (i + 1 == n_eff) mbar_arrive(&bars.q_empty);
-          }
+          if (!pc.has_q1) mbar_arrive(&bars.kv_empty[(steps + i) % kStages]);
         }
       };
       int j = 0;
