@@ -540,9 +540,9 @@ __device__ __forceinline__ void mma_role(const AttnParams& p, CtaShared<false>& 
     }
     int nv = 0, nv_1 = 0, nv_2 = 0;   // valid rows of tiles j, j - 1, j - 2
     for (int j = 0; j < n_eff + 2; ++j, nv_2 = nv_1, nv_1 = nv) {
-      const bool work = j != 1 || n_eff > 1;   // a piece of one tile has nothing to multiply in its second step
-      if (work && !(ok = wait_or_abort(&bars.kv_full[st], ph, &sh.abort))) break;
       nv = 0;
+      if (j == 1 && n_eff == 1) continue;      // a piece of one tile has nothing to multiply in its second step
+      if (!(ok = wait_or_abort(&bars.kv_full[st], ph, &sh.abort))) break;
       if (j < n_eff) nv = sh.nv[t++ % kNvRing];
       if (j > 0) {
         ok = wait_or_abort(&bars.p_full[kQt], p_ph, &sh.abort);
@@ -552,7 +552,6 @@ __device__ __forceinline__ void mma_role(const AttnParams& p, CtaShared<false>& 
         // the other (a parity wait cannot tell phase n from phase n + 2).
         if (j == 2 && e++ > 0) ok = ok && wait_or_abort(&bars.o_free[kQt], e & 1, &sh.abort);
       }
-      if (!work) continue;
       if (both && (kQt == 1 || k > 0)) ok = ok && wait_or_abort(&bars.turn[kQt], (kQt == 1 ? k : k + 1) & 1, &sh.abort);
       if (!ok) break;
       tc_fence_after();
@@ -857,7 +856,9 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&bars.p_full[wg]);   // one arrival per warp: the waits above covered all 32 lanes
+            // One arrival per warp: the waits above covered all 32 lanes.  (Of a piece of one tile only P is handed over: nothing holds
+            // this warp between its S and its P, and the MMA warp cannot tell two completions that it has not seen from none.)
+            if (lane == 0 && (j > 0 || n_eff > 1)) mbar_arrive(&bars.p_full[wg]);
             if (j != 1 || n_eff > 1) give_back(j);
             if (j == n_eff) break;
             if (nv < kTileKV) {   // columns past the end of the segment or slot

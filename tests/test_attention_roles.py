@@ -50,10 +50,10 @@ def run(request, tmp_path_factory):
     return call
 
 
-# One Q tile (lq <= 128, or the last pair of 257 .. 384 rows) or two; several units on a CTA; pieces of two tiles, and of more than
+# One Q tile (lq <= 128, or the last pair of 257 .. 384 rows) or two; several units on a CTA; pieces of one tile, two, and more than
 # there are stages; slots that are stale (odd) or holes, so that a piece has no tile at all.
 @pytest.mark.parametrize("lq", [100, 200, 300])
-@pytest.mark.parametrize("segs,slots,rows", [((100,), (), 8), ((60, 130, 33), (), 8), ((500,), (), 8),
+@pytest.mark.parametrize("segs,slots,rows", [((60,), (), 8), ((100,), (), 8), ((60, 130, 33), (), 8), ((500,), (), 8),
                                              ((70,), (2, 1, 0), 100), ((), (1, 3), 40), ((), (4, -1), 90)])
 def test_units_one_after_another(run, lq, segs, slots, rows):
     if run.lse_only:
@@ -64,7 +64,7 @@ def test_units_one_after_another(run, lq, segs, slots, rows):
 
 
 @pytest.mark.parametrize("lq", [100, 300])
-@pytest.mark.parametrize("ranges", [2, 3])
+@pytest.mark.parametrize("ranges", [2, 3, 5])
 @pytest.mark.parametrize("n_full", [0, 1])
 def test_ranges_that_cross_units(run, lq, ranges, n_full):
     """The walk of a CTA: a whole unit where there is one, units inside its range, and the piece of the unit it starts in."""
