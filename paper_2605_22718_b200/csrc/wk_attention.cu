@@ -1098,12 +1098,19 @@ int attention_partial_slots(int n_heads, int max_lq, int max_splits) {
 //     88 of 38 49.8 / 53.7, of 57 69.1 / 64.5; 99 of 63 76.8 / 75.1; 110 of 94 106.4 / 103.3, of 150 170 / 160; 121 of 125 138.3 /
 //     139.2, of 150 177 / 165; 132 of 198 247.8 / 253.6, of 282 357.8 / 358.1, of 500 621 / 597.  With full waves before it: 760
 //     units of 410 tiles (rest 20) 2,953 / 2,763.
-static void split_default(int64_t units, int64_t tiles, int64_t sms, int64_t* G, int64_t* n_full, int64_t* ranges) {
+//   * Units of a little more than kFewTiles tiles are cut before that saves time, where a cut leaves pieces of few tiles, whose every
+//     largest weight is exact (24 units of 1,040 keys: relative error of O at deviations 1 / 2 / 4 2.33 / 2.29 / 2.14e-3 whole at 19.1
+//     us, 2.14 / 1.78 / 1.68e-3 in three pieces at 20.5; 40 of 1,520: 25.4 and 27.7 us).  The line is drawn in tiles of 128 rows, of
+//     which a range of four, 512 rows, is at most eight of the kernel's: at three cuts or more it is crossed at 6 of them (10 units), 8
+//     (24) and 12 (40).
+static void split_default(int64_t units, int64_t tiles, int64_t tiles128, int64_t sms, int64_t* G, int64_t* n_full, int64_t* ranges) {
   const int64_t waves = units / sms, rest = units - waves * sms;
   *G = units < sms ? units : sms;
   *n_full = units;
   *ranges = 0;
-  if (rest == 0 || (sms - rest) * tiles < 8 * sms + 22 * rest) return;
+  const bool faster = (sms - rest) * tiles >= 8 * sms + 22 * rest;
+  const bool closer = sms >= 3 * rest && tiles > kFewTiles && (sms - rest) * tiles128 >= 4 * sms + 16 * rest;
+  if (rest == 0 || !(faster || closer)) return;
   int64_t r;
   if (sms >= 2 * rest) {
     int64_t cuts = sms / rest;
@@ -1143,7 +1150,7 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   int tiles = n_slots * count(p.tile_rows, ctx->C);
   for (int i = 0; i < n_segs; ++i) tiles += count(p.tile_rows, segs[i].n_tokens);
   if (!lse_only && tiles > kFewTilesOfCall) p.tile_rows = kTileKV;
-  int most = n_slots * count(128, ctx->C);   // ranges of a unit that a caller may ask for: one per 128 rows
+  int most = n_slots * count(128, ctx->C);   // tiles of 128 rows: as many ranges of a unit may a caller ask for
   for (int i = 0; i < n_segs; ++i) most += count(128, segs[i].n_tokens);
   tiles = 0;
   for (int i = 0; i < n_segs; ++i) {
@@ -1197,7 +1204,7 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
     n_full = p.n_units;
     G = sms < n_full ? sms : n_full;
   } else if (kv_splits == 0) {
-    split_default(p.n_units, p.n_tiles, sms, &G, &n_full, &ranges);
+    split_default(p.n_units, p.n_tiles, most, sms, &G, &n_full, &ranges);
   } else if (kv_splits > 0) {
     int sp = kv_splits < most ? kv_splits : most;
     if (sp > kMaxPieces) sp = kMaxPieces;
