@@ -249,12 +249,11 @@ __device__ __forceinline__ float fmax_nan(float a, float b) {   // NaN if either
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
   return d;
 }
-// 2^x of a pair.  The exponentials are the kernel's second bound (16 per clock and SM on the special-function unit: 1,280 clk per
-// tile of 80 keys), so a share of the pairs takes 2^x from the FMA pipe instead (12 heads x 2,640 queries x 15,840 keys: 264 us at a
-// share of 0, 251 at 1/8, 262 at 2/8, 270 at 3/8): x = n + f with
-// n = round(x) by the add-a-large-constant trick, 2^f on [-1/2, 1/2] by a cubic (relative error 7.7e-5, far inside the bf16
-// rounding P gets anyway: 2e-3), 2^n by adding n to the exponent field; all in packed fp32 pairs.  That path clamps at
-// x = -120 (a weight of 1e-36), needs x < 127, and turns NaN into a weight beyond all bounds.
+// 2^x of a pair.  The exponentials bound LSE-only launches (16 per clock and SM on the special-function unit: 2,048 clk per tile of 128
+// keys), so a share of the pairs takes 2^x from the FMA pipe instead (2,640 queries x 12 heads x 250 slots of 1,320 rows: 3,563 / 3,487 /
+// 3,434 / 3,493 / 3,725 us at 0 ... 4 of 8): x = n + f with n = round(x) by the add-a-large-constant trick, 2^f on [-1/2, 1/2] by a cubic
+// (relative error 7.7e-5), 2^n by adding n to the exponent field; all in packed fp32 pairs.  That path clamps at x = -120 (a weight of
+// 1e-36), needs x < 127, and turns NaN into a weight beyond all bounds.
 template <bool kPoly>
 __device__ __forceinline__ void exp2_pair(uint64_t e, float& p0, float& p1) {
   float e0, e1;
@@ -351,23 +350,18 @@ __device__ __forceinline__ float row_max(const uint32_t (&r)[kTileKV]) {
   for (int i = 0; i < kTileKV; i += 2) mx[(i >> 1) & 3] = fmax3(mx[(i >> 1) & 3], __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
   return fmax3(fmaxf(mx[0], mx[1]), mx[2], mx[3]);
 }
-// P = 2^(s * scale - m) of a row, as bf16 pairs, and their sum.  With kPoly (calls of more than a few tiles) one of every 8
-// pairs takes the FMA pipe; big = the largest of their raw values (see exp_chunk).  (97 keys: log-sum-exp within 8e-7, with a share of cubics 1e-5.)
-template <bool kPoly>
-__device__ __forceinline__ float exp_tile(const uint32_t (&r)[kTileKV], uint64_t scale2, float m, float& big, uint32_t (&pk)[kTileKV / 2]) {
+// P = 2^(s * scale - m) of a row, as bf16 pairs, and their sum.  (All exponentials on the special-function unit: a share of cubics as in
+// exp_chunk costs time, 12 heads x 2,640 queries x 15,840 keys 253.3 us with one pair in eight and 248.8 without, and leaves the
+// log-sum-exp of segments of 100 keys within 1e-5 instead of 9e-7.)
+__device__ __forceinline__ float exp_tile(const uint32_t (&r)[kTileKV], uint64_t scale2, float m, uint32_t (&pk)[kTileKV / 2]) {
   const uint64_t neg_m2 = pack_f32x2(-m, -m);
   uint64_t acc[4] = {0, 0, 0, 0};
 #pragma unroll
   for (int i = 0; i < kTileKV / 2; ++i) {
-    const float s0 = __uint_as_float(r[2 * i]), s1 = __uint_as_float(r[2 * i + 1]);
-    const uint64_t e = fma_f32x2(pack_f32x2(s0, s1), scale2, neg_m2);
-    float p0, p1;
-    if (kPoly && (i & 7) == 4) {
-      exp2_pair<true>(e, p0, p1);
-      big = fmax3(big, s0, s1);
-    } else {
-      exp2_pair<false>(e, p0, p1);
-    }
+    const uint64_t e = fma_f32x2(pack_f32x2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])), scale2, neg_m2);
+    float e0, e1;
+    unpack_f32x2(e, e0, e1);
+    const float p0 = ex2_approx(e0), p1 = ex2_approx(e1);
     acc[i & 3] = add_f32x2(acc[i & 3], pack_f32x2(p0, p1));
     pk[i] = pack_bf16x2(p0, p1);
   }
@@ -614,7 +608,7 @@ __device__ __forceinline__ void mma_lse_role(const AttnParams& p, CtaShared<true
 }
 
 // All of a CTA's work.
-template <bool kLse, bool kShort>
+template <bool kLse>
 __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<kLse>& sh, uint8_t* smem) {
   const uint32_t smem_base = smem_u32(smem);
   uint8_t* sQ = smem;                 // [2 q tiles][2 halves][128 rows][128 B]
@@ -880,9 +874,8 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
                 if (move) m = mt;
                 l *= alpha;
               }
-              float big = -INFINITY;
-              sum = exp_tile<!kShort>(r, scale2, m, big, pk);
-              if (known || !__any_sync(0xffffffffu, !(sum <= kStreamSum) || big * p.scale_log2 - m > 100.f)) break;
+              sum = exp_tile(r, scale2, m, pk);
+              if (known || !__any_sync(0xffffffffu, !(sum <= kStreamSum))) break;
               known = true;
               careful = 1 << min(++redos, 6);
             }
@@ -956,9 +949,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
   }
 }
 
-// kShort: keys in tiles of kTileKVFew rows.  (One kernel for both, with the choice in the loop: 254.7 us instead of 253.2 for 12 heads x
-// 2,640 queries x 15,840 keys.)
-template <bool kLse, bool kShort>
+template <bool kLse>
 __global__ void __launch_bounds__(kThreads<kLse>, 1)
 memory_attention_kernel(const __grid_constant__ AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -1000,7 +991,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
     atomicOr(p.status, WK_DEV_TIMEOUT);
   }
 
-  attention_roles<kLse, kShort>(p, sh, smem);
+  attention_roles<kLse>(p, sh, smem);
   tc_fence_before();
   __syncthreads();
   if (tid < 32) tmem_dealloc(sh.tmem, 512);
@@ -1131,11 +1122,9 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
                            const int32_t* slots_dev, int n_slots, __nv_bfloat16* O, float* lse, int kv_splits,
                            cudaStream_t s, bool lse_only) {
   if (!ctx->attn_attr_set) {   // the attribute belongs to the device the context lives on
-    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           static_cast<int>(kSmemBytes<false>)));
-    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          static_cast<int>(kSmemBytes<false>)));
-    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           static_cast<int>(kSmemBytes<true>)));
     ctx->attn_attr_set = true;
   }
@@ -1220,9 +1209,8 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   p.n_full = static_cast<int>(n_full);
   p.n_ranges = static_cast<int>(ranges);
   const dim3 grid(static_cast<unsigned>(G));
-  if (lse_only) launch_chained(memory_attention_kernel<true, false>, grid, dim3(kThreads<true>), kSmemBytes<true>, s, p);
-  else launch_chained(p.tile_rows == kTileKV ? memory_attention_kernel<false, false> : memory_attention_kernel<false, true>, grid,
-                      dim3(kThreads<false>), kSmemBytes<false>, s, p);
+  if (lse_only) launch_chained(memory_attention_kernel<true>, grid, dim3(kThreads<true>), kSmemBytes<true>, s, p);
+  else launch_chained(memory_attention_kernel<false>, grid, dim3(kThreads<false>), kSmemBytes<false>, s, p);
   if ((st = after_launch(ctx)) != WK_OK) return st;
   if (!lse_only && n_full != p.n_units) {   // some unit was cut
     launch_chained(combine_kernel, dim3(static_cast<unsigned>(p.n_units - n_full) * 32), dim3(kCombineThreads), 0, s, p.opart,

@@ -294,7 +294,7 @@ static void tma_load_3d(void* dst, const CUtensorMap* m, uint64_t* bar, int x, i
 namespace {
 
 void fiber_main() {
-  attention_roles<kL, false>(par, ar.sh, ar.smem);
+  attention_roles<kL>(par, ar.sh, ar.smem);
   fibers[current].done = true;
   for (;;) pause();
 }

@@ -16,7 +16,7 @@ HOST = os.path.join(ROOT, "tests", "host")
 
 def roles_source():
     src = open(os.path.join(CSRC, "wk_attention.cu")).read()
-    cut = src.index("template <bool kLse, bool kShort>\n__global__")
+    cut = re.search(r"template <[^>]*>\n__global__", src).start()
     init = re.search(r"if \(tid == 0\) \{\n(.*?)fence_mbar_init", src[cut:], re.S).group(1)
     body = src[:cut].replace('#include "ptx_sm100.cuh"\n', "")
     for name in ("bool wait_or_abort(", "float fmax3(", "float fmax_nan("):   # PTX through and through: stand-ins

@@ -87,6 +87,44 @@ def test_largest_weights_of_units_just_longer_than_short_pieces(H, lq, n):
     assert float((O - want).norm() / want.norm()) < 2.05e-3
 
 
+@pytest.mark.parametrize("H,lq,seg_rows", [(4, 300, (120,) * 8), (8, 1000, (100,) * 6), (2, 300, (255, 127, 127, 127, 127)), (2, 300, (40,) * 8)])
+def test_log_sum_exp_over_short_segments(H, lq, seg_rows):
+    """All exponentials of such calls are exact to 2^-22, so the log-sum-exp is off by that, by fp32 sums of at most 80 terms in
+    four chains, 2^-19 if all roundings went one way, and by its own rounding: below 2.5e-6 (with a share of cubics 5e-6 to 1e-5)."""
+    from paper_2605_22718_b200 import WorldKV
+    kv = WorldKV(n_layers=1, n_heads=H, tokens_per_frame=8, n_keep=4, pool_slots=1, max_k=1, max_lq=lq, max_splits=8, max_dense_segments=8)
+    q = wd.to_device_bf16(bf16(normals(16, (lq, H, 128))))
+    segs = [tuple(wd.to_device_bf16(bf16(normals(17 + 2 * i + j, (n, H, 128)))) for j in (0, 1)) for i, n in enumerate(seg_rows)]
+    K = torch.cat([k for k, _ in segs])
+    want = torch.logsumexp(torch.einsum("qhd,khd->hqk", q.double(), K.double()) * SCALE, -1)
+    for splits in (1, 0):
+        lse = torch.empty((H, lq), dtype=torch.float32, device="cuda")
+        kv.memory_attention(0, q, segs, None, 0, lse_out=lse, kv_splits=splits)
+        assert kv.poll_status() == (0, 0)
+        assert float((lse.double() - want).abs().max()) < 2.5e-6, f"splits {splits}"
+
+
+def test_log_sum_exp_over_short_slots():
+    """The same for stored chunks of fewer than 128 rows, beside a long segment and alone."""
+    from paper_2605_22718_b200 import WorldKV
+    H, T, keep, S, lq = 3, 96, 24, 9, 200
+    kv = WorldKV(n_layers=1, n_heads=H, tokens_per_frame=T, n_keep=keep, pool_slots=S, max_k=S, max_lq=lq, max_batch=1)
+    for c in range(S):
+        x = [wd.to_device_bf16(bf16(normals(40 + 2 * c + j, (1, 3 * T, H * 128)))) for j in (0, 1)]
+        kv.pool_compress_append(0, 1, x[0], x[1], [float(c), 0, 0, 0, 1, 0, 0, 0], chunk_tag=c)
+    n = S * kv.C
+    stored = kv.pool[:n * H * 256].view(torch.bfloat16).view(n, H, 128)
+    q, k, v = (wd.to_device_bf16(bf16(normals(60 + i, (m, H, 128)))) for i, m in enumerate((lq, 640, 640)))
+    slots = torch.arange(S, dtype=torch.int32, device="cuda")
+    for segs in ([], [(k, v)]):
+        K = torch.cat([s[0] for s in segs] + [stored])
+        want = torch.logsumexp(torch.einsum("qhd,khd->hqk", q.double(), K.double()) * SCALE, -1)
+        lse = torch.empty((H, lq), dtype=torch.float32, device="cuda")
+        kv.memory_attention(0, q, segs, slots, S, lse_out=lse)
+        assert kv.poll_status() == (0, 0)
+        assert float((lse.double() - want).abs().max()) < 2.5e-6
+
+
 @pytest.mark.parametrize("step", [-3, -7, -12, -15, -19, -30, 7, 15, 30])
 @pytest.mark.parametrize("n", [512, 470, 1200])
 def test_large_values_under_falling_and_rising_logits(n, step):
