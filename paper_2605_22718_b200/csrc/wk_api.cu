@@ -105,15 +105,16 @@ wk_status encode_pool_map(wk_ctx* ctx, const void* base, int64_t rows, int64_t n
 }
 
 // Small round-robin cache: steady-state callers pass the same window buffers every step.
-const CUtensorMap* cached_rows_map(wk_ctx* ctx, const void* base, int32_t rows, wk_status* st) {
+const CUtensorMap* cached_rows_map(wk_ctx* ctx, const void* base, int32_t rows, int32_t box_rows, wk_status* st) {
   *st = WK_OK;
   for (auto& e : ctx->tmap_cache) {
-    if (e.ptr == base && e.rows == rows) return &e.map;
+    if (e.ptr == base && e.rows == rows && e.box_rows == box_rows) return &e.map;
   }
   TmapKey k;
   k.ptr = base;
   k.rows = rows;
-  *st = encode_rows_map(ctx, base, rows, kTileKV, &k.map);
+  k.box_rows = box_rows;
+  *st = encode_rows_map(ctx, base, rows, box_rows, &k.map);
   if (*st != WK_OK) return nullptr;
   const size_t cap = 256;
   if (ctx->tmap_cache.size() < cap) {
@@ -220,12 +221,14 @@ wk_status wk_bind(wk_ctx* ctx, void* pool_dev, size_t pool_bytes, void* scratch_
   ctx->max_lq = max_lq;
   ctx->max_splits = max_splits;
   const int64_t n_mats = static_cast<int64_t>(ctx->cfg.n_layers) * ctx->cfg.pool_slots;
-  wk_status st = encode_pool_map(ctx, ctx->Kpool, ctx->C, n_mats, kTileKV, &ctx->tm_kpool);
-  if (st != WK_OK) return st;
-  st = encode_pool_map(ctx, ctx->Kpool, ctx->C, n_mats, kTileKVLse, &ctx->tm_kpool_lse);
-  if (st != WK_OK) return st;
-  st = encode_pool_map(ctx, ctx->Vpool, ctx->C, n_mats, kTileKV, &ctx->tm_vpool);
-  if (st != WK_OK) return st;
+  const struct { const void* base; int box_rows; CUtensorMap* map; } maps[] = {
+      {ctx->Kpool, kTileKV, &ctx->tm_kpool},         {ctx->Vpool, kTileKV, &ctx->tm_vpool},
+      {ctx->Kpool, kTileKVFew, &ctx->tm_kpool_few},  {ctx->Vpool, kTileKVFew, &ctx->tm_vpool_few},
+      {ctx->Kpool, kTileKVLse, &ctx->tm_kpool_lse}};
+  for (const auto& m : maps) {
+    const wk_status st = encode_pool_map(ctx, m.base, ctx->C, n_mats, m.box_rows, m.map);
+    if (st != WK_OK) return st;
+  }
   // the anchor pass counts finished CTAs per problem in scratch; the counters must start at zero
   WK_CUDA_TRY(ctx, cudaMemset(ctx->scratch_base + sl.cnt_off, 0, sl.dist_off - sl.cnt_off));
   {

@@ -36,19 +36,19 @@ namespace {
 
 using namespace ptx;
 
+// The kernel is instantiated by the rows of its KV tiles, kKv: kTileKV and kTileKVFew, and kTileKVLse in LSE-only launches.
+template <int kKv> constexpr bool is_lse = kKv == kTileKVLse;
 // softmax warps, then the MMA warps, then the TMA warp.  LSE-only launches have a softmax warpgroup per S buffer.
-template <bool kLse> constexpr int kSoftWarps = kLse ? 16 : 8;
-template <bool kLse> constexpr int kMmaWarps = kLse ? 1 : 2;
-template <bool kLse> constexpr int kThreads = 32 * (kSoftWarps<kLse> + kMmaWarps<kLse> + 1);
-// rows of a KV tile
-template <bool kLse> constexpr int kKv = kLse ? kTileKVLse : kTileKV;
-template <bool kLse> constexpr uint32_t kHalfKvBytes = kKv<kLse> * 64 * 2;   // one TMA box: 64 columns
-template <bool kLse> constexpr uint32_t kKvBytes = 2 * kHalfKvBytes<kLse>;
+template <int kKv> constexpr int kSoftWarps = is_lse<kKv> ? 16 : 8;
+template <int kKv> constexpr int kMmaWarps = is_lse<kKv> ? 1 : 2;
+template <int kKv> constexpr int kThreads = 32 * (kSoftWarps<kKv> + kMmaWarps<kKv> + 1);
+template <int kKv> constexpr uint32_t kHalfKvBytes = kKv * 64 * 2;   // one TMA box: 64 columns
+template <int kKv> constexpr uint32_t kKvBytes = 2 * kHalfKvBytes<kKv>;
 constexpr uint32_t kHalfQBytes = kTileQ * 64 * 2, kQBytes = 2 * kHalfQBytes;
 // A stage holds what one step of the MMA warp consumes: V of tile j and K of tile j + 2 (LSE-only launches: K alone).
 constexpr int kStages = 4;
-template <bool kLse> constexpr uint32_t kStageBytes = (kLse ? 1 : 2) * kKvBytes<kLse>;
-template <bool kLse> constexpr size_t kSmemBytes = 1024 + 2 * kQBytes + kStages * kStageBytes<kLse>;   // align slack + Q0, Q1 + stages
+template <int kKv> constexpr uint32_t kStageBytes = (is_lse<kKv> ? 1 : 2) * kKvBytes<kKv>;
+template <int kKv> constexpr size_t kSmemBytes = 1024 + 2 * kQBytes + kStages * kStageBytes<kKv>;   // align slack + Q0, Q1 + stages
 constexpr int kNvRing = 16;   // tile heights handed from the TMA warp to the others; the TMA warp is at most kStages + 2 tiles ahead
 // The softmax weighs a key with P = 2^(s * scale - m), where m is a maximum that the row has reached: rounded to bf16, the
 // weight of the key that set it is exactly 1, so a dominating key returns its V row unchanged.  (Against a reference that is
@@ -64,9 +64,14 @@ constexpr float kStreamSum = 256.0f;
 // Pieces of at most kFewTiles tiles move the reference to every tile's own maximum, down as well as up: beside few other keys a
 // tile's largest weight counts, and it is exact this way, as if the tile were a piece of its own.  450 queries x 5 heads x 1,040
 // keys (pieces of three tiles), relative error of O at deviations 1 / 2 / 4: 2.13 / 1.80 / 1.69e-3, without 2.27 / 2.19 / 1.98e-3.
-// Calls of at most kFewTilesOfCall tiles of kTileKVFew rows walk them in such tiles, so that no more keys share a maximum.
-constexpr int kFewTiles = 10, kTileKVFew = 64, kFewTilesOfCall = 8;
+// Calls of at most kFewTilesOfCall tiles of kTileKVFew rows walk them in such tiles, so that no more keys share a maximum.  So do calls
+// whose segments and slots fill tiles of kTileKV rows badly: a tile of 64 takes 1,713 clk where one of 80 takes 1,919, by the clocks
+// that the power cap leaves 6 to 7 for 7 to 8 (16,000 rows in slots of C, 12 heads x 2,640 queries, us in tiles of 80 / 64: C = 170 358 /
+// 302, 190 329 / 272, 256 279 / 235, 512 264 / 257, 448 258 / 258, 384 251 / 260, 320 235 / 256; in tiles of 128 rows, which S and P
+// of their own left no room for, 306, 280, 218, 253, 262, 248 and 264).
+constexpr int kFewTiles = 10, kFewTilesOfCall = 8;
 constexpr float kOwnSum = 1024.0f;
+constexpr int kCost64 = 7, kCost80 = 8;
 // tensor-memory columns: S0, P0, S1, P1 (80 + 40 of 128 each), O0, O1; LSE-only: S0, S1 twice
 constexpr uint32_t kTmemS = 0, kTmemP = kTileKV, kTmemO = 256;
 static_assert(kTileKV * 3 / 2 <= 128, "S and P of a Q tile share 128 columns");
@@ -329,35 +334,40 @@ __device__ __forceinline__ float row_max_tmem(uint32_t tS, int nv) {
   return fmaxf(mx[0], mx[1]);
 }
 // S of a tile, a row per thread, into registers.
-__device__ __forceinline__ void tmem_ld_tile(uint32_t tS, uint32_t (&r)[kTileKV]) {
-  static_assert(kTileKV == 80, "loads of 32 + 32 + 16 columns");
+template <int kKv>
+__device__ __forceinline__ void tmem_ld_tile(uint32_t tS, uint32_t (&r)[kKv]) {
+  static_assert(kKv == 64 || kKv == 80, "loads of 32 + 32 (+ 16) columns");
   tmem_ld_x32(tS, *reinterpret_cast<uint32_t(*)[32]>(&r[0]));
   tmem_ld_x32(tS + 32, *reinterpret_cast<uint32_t(*)[32]>(&r[32]));
-  tmem_ld_x16(tS + 64, *reinterpret_cast<uint32_t(*)[16]>(&r[64]));
+  if constexpr (kKv == 80) tmem_ld_x16(tS + 64, *reinterpret_cast<uint32_t(*)[16]>(&r[64]));
 }
-__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[kTileKV]) {
+template <int kKv>
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[kKv]) {
   tc_wait_ld(*reinterpret_cast<uint32_t(*)[32]>(&r[0]));
   pin_x32(*reinterpret_cast<uint32_t(*)[32]>(&r[32]));
-  pin_x16(*reinterpret_cast<uint32_t(*)[16]>(&r[64]));
+  if constexpr (kKv == 80) pin_x16(*reinterpret_cast<uint32_t(*)[16]>(&r[64]));
 }
-__device__ __forceinline__ void tmem_st_half_tile(uint32_t tP, const uint32_t (&p)[kTileKV / 2]) {
+template <int kHalf>
+__device__ __forceinline__ void tmem_st_half_tile(uint32_t tP, const uint32_t (&p)[kHalf]) {
   tmem_st_x32(tP, *reinterpret_cast<const uint32_t(*)[32]>(&p[0]));
-  tmem_st_x8(tP + 32, *reinterpret_cast<const uint32_t(*)[8]>(&p[32]));
+  if constexpr (kHalf == 40) tmem_st_x8(tP + 32, *reinterpret_cast<const uint32_t(*)[8]>(&p[32]));
 }
-__device__ __forceinline__ float row_max(const uint32_t (&r)[kTileKV]) {
+template <int kKv>
+__device__ __forceinline__ float row_max(const uint32_t (&r)[kKv]) {
   float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-  for (int i = 0; i < kTileKV; i += 2) mx[(i >> 1) & 3] = fmax3(mx[(i >> 1) & 3], __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+  for (int i = 0; i < kKv; i += 2) mx[(i >> 1) & 3] = fmax3(mx[(i >> 1) & 3], __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
   return fmax3(fmaxf(mx[0], mx[1]), mx[2], mx[3]);
 }
 // P = 2^(s * scale - m) of a row, as bf16 pairs, and their sum.  (All exponentials on the special-function unit: a share of cubics as in
 // exp_chunk costs time, 12 heads x 2,640 queries x 15,840 keys 253.3 us with one pair in eight and 248.8 without, and leaves the
 // log-sum-exp of segments of 100 keys within 1e-5 instead of 9e-7.)
-__device__ __forceinline__ float exp_tile(const uint32_t (&r)[kTileKV], uint64_t scale2, float m, uint32_t (&pk)[kTileKV / 2]) {
+template <int kKv>
+__device__ __forceinline__ float exp_tile(const uint32_t (&r)[kKv], uint64_t scale2, float m, uint32_t (&pk)[kKv / 2]) {
   const uint64_t neg_m2 = pack_f32x2(-m, -m);
   uint64_t acc[4] = {0, 0, 0, 0};
 #pragma unroll
-  for (int i = 0; i < kTileKV / 2; ++i) {
+  for (int i = 0; i < kKv / 2; ++i) {
     const uint64_t e = fma_f32x2(pack_f32x2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])), scale2, neg_m2);
     float e0, e1;
     unpack_f32x2(e, e0, e1);
@@ -443,22 +453,22 @@ struct PieceWalker {
   }
 };
 
-// kLse = true is the LSE-only instantiation (query-based retrieval): no V, no P, no O.  S has two buffers per Q tile and a
+// kKv = kTileKVLse is the LSE-only instantiation (query-based retrieval): no V, no P, no O.  S has two buffers per Q tile and a
 // softmax warpgroup per buffer, so the tensor pipe works ahead of the softmax, which bounds it (issue and special-function
 // unit) until the board's power cap does.  2,640 queries x 12 heads x 250 slots of 1,320 rows: two warpgroups and one buffer
 // per Q tile on 132 SMs 4,070 us; all SMs, two buffers, streamed sums 3,540; four warpgroups 3,070 (2,136 clk per KV tile).
 // What the roles of a CTA share besides the tiles.
-template <bool kLse>
+template <int kKv>
 struct CtaShared {
   Barriers bars;
   uint32_t tmem;
   volatile uint32_t abort;
-  float2 merge[kLse ? 2 : 1][kLse ? 128 : 1];   // (reference, sum) of a Q tile's odd KV tiles
+  float2 merge[is_lse<kKv> ? 2 : 1][is_lse<kKv> ? 128 : 1];   // (reference, sum) of a Q tile's odd KV tiles
   volatile int nv[kNvRing];   // valid rows of tile number t (counted over the CTA's pieces) at t % kNvRing
 };
 
 // Issues the MMAs of a CTA's tiles.  The whole warp runs the control flow and one lane's predicate issues (see mma_ss_if).
-template <bool kLse>
+template <int kKv>
 struct Mma {
   uint32_t one, bar0;
   uint64_t q_desc, k_desc, v_desc;   // descriptors of the tile bases; a K = 16 step advances the low word by a constant
@@ -468,7 +478,7 @@ struct Mma {
     constexpr uint64_t hi = static_cast<uint64_t>(smem_desc_hi_sw128(1024)) << 32;
     q_desc = hi | smem_desc_lo(smem_base, 16);
     k_desc = hi | smem_desc_lo(smem_base + 2 * kQBytes, 16);
-    v_desc = hi | smem_desc_lo(smem_base + 2 * kQBytes + kKvBytes<kLse>, kHalfKvBytes<kLse>);
+    v_desc = hi | smem_desc_lo(smem_base + 2 * kQBytes + kKvBytes<kKv>, kHalfKvBytes<kKv>);
   }
   __device__ __forceinline__ void commit(size_t offset) const { mma_commit_if(one, bar0 + static_cast<uint32_t>(offset)); }
   // S = Q K^T over the first nv rows of the K tile: ceil(nv / 16) * 16 columns.  (A branch that gives full tiles a constant
@@ -476,18 +486,18 @@ struct Mma {
   // qt: Q tile in shared memory, d: S columns
   __device__ __forceinline__ void s(uint32_t qt, uint32_t d, uint32_t st, int nv) const {
     const uint32_t idesc = idesc_bf16_f32(128, 0, 0, 0) | (static_cast<uint32_t>((nv + 15) >> 4) << 18);
-    const uint64_t a = q_desc + qt * (kQBytes >> 4), b = k_desc + st * (kStageBytes<kLse> >> 4);
+    const uint64_t a = q_desc + qt * (kQBytes >> 4), b = k_desc + st * (kStageBytes<kKv> >> 4);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const uint32_t in_row = (k & 3) * 2;   // 32 bytes per step inside a 128-byte row
-      mma_ss_if(one, d, a + (k >> 2) * (kHalfQBytes >> 4) + in_row, b + (k >> 2) * (kHalfKvBytes<kLse> >> 4) + in_row, idesc, k > 0);
+      mma_ss_if(one, d, a + (k >> 2) * (kHalfQBytes >> 4) + in_row, b + (k >> 2) * (kHalfKvBytes<kKv> >> 4) + in_row, idesc, k > 0);
     }
   }
   // O_i (+)= P_i V: A = P from tensor memory (bf16 pairs, 8 columns per K = 16 step); B = V, rows = K dimension,
   // MN-major: 16 rows of 128 bytes = 2048 bytes per step
   __device__ __forceinline__ void pv(uint32_t i, uint32_t st, int nv, uint32_t accumulate) const {
     constexpr uint32_t idesc = idesc_bf16_f32(128, 128, 0, 1);
-    const uint64_t b = v_desc + st * (kStageBytes<kLse> >> 4);
+    const uint64_t b = v_desc + st * (kStageBytes<kKv> >> 4);
 #pragma unroll 1
     for (int k = 0; k < (nv + 15) >> 4; ++k)
       mma_ts_if(one, kTmemO + i * 128, kTmemP + i * 128 + k * 8, b + k * 128, idesc, k > 0 ? 1u : accumulate);
@@ -497,11 +507,11 @@ struct Mma {
 // MMA warp of Q tile kQt.  Two warps issue because a commit holds its warp until the tensor pipe has nearly caught up, and the
 // waits behind it would leave the pipe idle: while one warp is held, the other has waited already and goes on.  They take turns
 // (turn[]), step by step: the pipe runs a group of MMAs that accumulate into one tile slower when another tile's come between them.
-template <int kQt>
-__device__ __forceinline__ void mma_role(const AttnParams& p, CtaShared<false>& sh, uint32_t smem_base) {
+template <int kKv, int kQt>
+__device__ __forceinline__ void mma_role(const AttnParams& p, CtaShared<kKv>& sh, uint32_t smem_base) {
   Barriers& bars = sh.bars;
   const int lane = threadIdx.x & 31;
-  const Mma<false> mma(smem_base, bars);
+  const Mma<kKv> mma(smem_base, bars);
   PieceWalker walk;
   walk.init(p);
   Piece pc;
@@ -563,10 +573,10 @@ __device__ __forceinline__ void mma_role(const AttnParams& p, CtaShared<false>& 
 }
 
 // LSE-only: two S buffers per Q tile, no P V; p_full says that a buffer has been read.
-__device__ __forceinline__ void mma_lse_role(const AttnParams& p, CtaShared<true>& sh, uint32_t smem_base) {
+__device__ __forceinline__ void mma_lse_role(const AttnParams& p, CtaShared<kTileKVLse>& sh, uint32_t smem_base) {
   Barriers& bars = sh.bars;
   const int lane = threadIdx.x & 31;
-  const Mma<true> mma(smem_base, bars);
+  const Mma<kTileKVLse> mma(smem_base, bars);
   PieceWalker walk;
   walk.init(p);
   Piece pc;
@@ -608,14 +618,15 @@ __device__ __forceinline__ void mma_lse_role(const AttnParams& p, CtaShared<true
 }
 
 // All of a CTA's work.
-template <bool kLse>
-__device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<kLse>& sh, uint8_t* smem) {
+template <int kKv>
+__device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<kKv>& sh, uint8_t* smem) {
+  constexpr bool kLse = is_lse<kKv>;
   const uint32_t smem_base = smem_u32(smem);
   uint8_t* sQ = smem;                 // [2 q tiles][2 halves][128 rows][128 B]
   uint8_t* sKV = sQ + 2 * kQBytes;    // [stages][K, V][2 halves][rows][128 B]; LSE-only: [stages][K]
   Barriers& bars = sh.bars;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (warp == kSoftWarps<kLse> + kMmaWarps<kLse>) {
+  if (warp == kSoftWarps<kKv> + kMmaWarps<kKv>) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       PieceWalker walk;
@@ -645,10 +656,10 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
         auto load = [&](uint8_t* dst, const TileInfo& ti, const CUtensorMap* seg_maps, const CUtensorMap* pool_map) {
           if (ti.seg >= 0) {
             tma_load_2d(dst, seg_maps + ti.seg, &bars.kv_full[st], x, ti.row0);
-            tma_load_2d(dst + kHalfKvBytes<kLse>, seg_maps + ti.seg, &bars.kv_full[st], x + 64, ti.row0);
+            tma_load_2d(dst + kHalfKvBytes<kKv>, seg_maps + ti.seg, &bars.kv_full[st], x + 64, ti.row0);
           } else {
             tma_load_3d(dst, pool_map, &bars.kv_full[st], x, ti.row0, ti.z);
-            tma_load_3d(dst + kHalfKvBytes<kLse>, pool_map, &bars.kv_full[st], x + 64, ti.row0, ti.z);
+            tma_load_3d(dst + kHalfKvBytes<kKv>, pool_map, &bars.kv_full[st], x + 64, ti.row0, ti.z);
           }
         };
         bool have1 = false, have2 = false;
@@ -657,10 +668,10 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
           if (have || have2) {             // (a piece of one tile has nothing in its second step)
             if (!(ok = wait_or_abort(&bars.kv_empty[st], ph, &sh.abort))) break;
             if (have) sh.nv[t++ % kNvRing] = ti.nv;   // read after kv_full
-            mbar_expect_tx(&bars.kv_full[st], (have ? kKvBytes<kLse> : 0) + (have2 ? kKvBytes<kLse> : 0));
+            mbar_expect_tx(&bars.kv_full[st], (have ? kKvBytes<kKv> : 0) + (have2 ? kKvBytes<kKv> : 0));
             ++steps;
-            uint8_t* dst = sKV + st * kStageBytes<kLse>;
-            if (have2) load(dst + kKvBytes<kLse>, t2, p.tm_vd, &p.tm_vpool);
+            uint8_t* dst = sKV + st * kStageBytes<kKv>;
+            if (have2) load(dst + kKvBytes<kKv>, t2, p.tm_vd, &p.tm_vpool);
             if (have) load(dst, ti, p.tm_kd, &p.tm_kpool);
             if (++st == kStages) { st = 0; ph ^= 1; }
           }
@@ -685,12 +696,12 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
           if (steps > q) drain(&bars.kv_full[q], (steps - 1 - q) / kStages);
       }
     }
-  } else if (warp == kSoftWarps<kLse>) {
+  } else if (warp == kSoftWarps<kKv>) {
     if constexpr (kLse) mma_lse_role(p, sh, smem_base);
-    else mma_role<0>(p, sh, smem_base);
-  } else if (!kLse && warp == kSoftWarps<kLse> + 1) {
-    if constexpr (!kLse) mma_role<1>(p, sh, smem_base);
-  } else if (kLse) {
+    else mma_role<kKv, 0>(p, sh, smem_base);
+  } else if (!kLse && warp == kSoftWarps<kKv> + 1) {
+    if constexpr (!kLse) mma_role<kKv, 1>(p, sh, smem_base);
+  } else if constexpr (kLse) {
     // ------------------------------------------------------------------ LSE-only softmax warpgroups (one thread per row)
     // Warpgroup qt + 2 b works on S buffer b of Q tile qt, i.e. on every other KV tile of these rows: four warps per
     // scheduler instead of two, which is what hides the latencies of this issue-bound loop.  At the end of a unit the two
@@ -819,7 +830,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       int j = 0;
       if (active) {
         if (n_eff > 0) {
-          uint32_t pk[kTileKV / 2] = {};   // P of tile j - 1
+          uint32_t pk[kKv / 2] = {};   // P of tile j - 1
           float alpha = 1.f;
           bool rescale = false;
           int careful = 0, redos = 0;   // tiles whose maximum is taken first from here on; tiles streamed twice so far
@@ -842,7 +853,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
               }
             }
             // (the first time there is no P to store and the last time no S to load: nobody reads what these move then)
-            uint32_t r[kTileKV];   // S of tile j
+            uint32_t r[kKv];   // S of tile j
             tmem_st_half_tile(tP, pk);
             tmem_ld_tile(tS, r);
             const int nv = sh.nv[(t0 + j) % kNvRing];
@@ -855,9 +866,9 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
             if (lane == 0 && (j > 0 || n_eff > 1)) mbar_arrive(&bars.p_full[wg]);
             if (j != 1 || n_eff > 1) give_back(j);
             if (j == n_eff) break;
-            if (nv < kTileKV) {   // columns past the end of the segment or slot
+            if (nv < kKv) {   // columns past the end of the segment or slot
 #pragma unroll
-              for (int i = 0; i < kTileKV; ++i) r[i] = i < nv ? r[i] : 0xff800000u;
+              for (int i = 0; i < kKv; ++i) r[i] = i < nv ? r[i] : 0xff800000u;
             }
             // known: the row's maximum over the tile is taken before the exponentials
             bool known = few || j == 0 || careful > 0;
@@ -949,12 +960,13 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
   }
 }
 
-template <bool kLse>
-__global__ void __launch_bounds__(kThreads<kLse>, 1)
+template <int kKv>
+__global__ void __launch_bounds__(kThreads<kKv>, 1)
 memory_attention_kernel(const __grid_constant__ AttnParams p) {
+  constexpr bool kLse = is_lse<kKv>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + (((smem_u32(smem_raw) + 1023u) & ~1023u) - smem_u32(smem_raw));
-  __shared__ CtaShared<kLse> sh;
+  __shared__ CtaShared<kKv> sh;
   const int tid = threadIdx.x;
   if (tid == 0) {
     mbar_init(&sh.bars.q_full, 1);
@@ -991,7 +1003,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
     atomicOr(p.status, WK_DEV_TIMEOUT);
   }
 
-  attention_roles<kLse>(p, sh, smem);
+  attention_roles<kKv>(p, sh, smem);
   tc_fence_before();
   __syncthreads();
   if (tid < 32) tmem_dealloc(sh.tmem, 512);
@@ -1122,31 +1134,37 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
                            const int32_t* slots_dev, int n_slots, __nv_bfloat16* O, float* lse, int kv_splits,
                            cudaStream_t s, bool lse_only) {
   if (!ctx->attn_attr_set) {   // the attribute belongs to the device the context lives on
-    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          static_cast<int>(kSmemBytes<false>)));
-    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          static_cast<int>(kSmemBytes<true>)));
+    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<kTileKV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          static_cast<int>(kSmemBytes<kTileKV>)));
+    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<kTileKVFew>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          static_cast<int>(kSmemBytes<kTileKVFew>)));
+    WK_CUDA_TRY(ctx, cudaFuncSetAttribute(memory_attention_kernel<kTileKVLse>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          static_cast<int>(kSmemBytes<kTileKVLse>)));
     ctx->attn_attr_set = true;
   }
   AttnParams p;
   wk_status st = encode_rows_map(ctx, Q, lq, kTileQ, &p.tm_q);
   if (st != WK_OK) return st;
-  p.tm_kpool = lse_only ? ctx->tm_kpool_lse : ctx->tm_kpool;
-  p.tm_vpool = ctx->tm_vpool;
-  // Keys beside which every tile's largest weight counts are tiled in 64 rows, all others in what tensor memory has room for.
+  // Keys beside which every tile's largest weight counts are tiled in 64 rows, as are keys that fill tiles of 80 badly (see kFewTiles); all
+  // others in 80, what tensor memory has room for.
   auto count = [&](int rows, int n_rows) { return (n_rows + rows - 1) / rows; };
-  p.tile_rows = lse_only ? kTileKVLse : kTileKVFew;
-  int tiles = n_slots * count(p.tile_rows, ctx->C);
-  for (int i = 0; i < n_segs; ++i) tiles += count(p.tile_rows, segs[i].n_tokens);
-  if (!lse_only && tiles > kFewTilesOfCall) p.tile_rows = kTileKV;
-  int most = n_slots * count(128, ctx->C);   // tiles of 128 rows: as many ranges of a unit may a caller ask for
-  for (int i = 0; i < n_segs; ++i) most += count(128, segs[i].n_tokens);
-  tiles = 0;
+  auto count_all = [&](int rows) {
+    int n = n_slots * count(rows, ctx->C);
+    for (int i = 0; i < n_segs; ++i) n += count(rows, segs[i].n_tokens);
+    return n;
+  };
+  const int few = count_all(kTileKVFew);
+  const bool in_64 = few <= kFewTilesOfCall || kCost64 * few <= kCost80 * count_all(kTileKV);
+  p.tile_rows = lse_only ? kTileKVLse : in_64 ? kTileKVFew : kTileKV;
+  p.tm_kpool = lse_only ? ctx->tm_kpool_lse : in_64 ? ctx->tm_kpool_few : ctx->tm_kpool;
+  p.tm_vpool = in_64 ? ctx->tm_vpool_few : ctx->tm_vpool;
+  const int most = count_all(128);   // as many ranges of a unit may a caller ask for
+  int tiles = 0;
   for (int i = 0; i < n_segs; ++i) {
-    const CUtensorMap* mk = cached_rows_map(ctx, segs[i].K, segs[i].n_tokens, &st);
+    const CUtensorMap* mk = cached_rows_map(ctx, segs[i].K, segs[i].n_tokens, p.tile_rows, &st);
     if (st != WK_OK) return st;
     p.tm_kd[i] = *mk;
-    const CUtensorMap* mv = cached_rows_map(ctx, segs[i].V, segs[i].n_tokens, &st);
+    const CUtensorMap* mv = cached_rows_map(ctx, segs[i].V, segs[i].n_tokens, p.tile_rows, &st);
     if (st != WK_OK) return st;
     p.tm_vd[i] = *mv;
     p.seg_tile_prefix[i] = tiles;
@@ -1209,8 +1227,9 @@ wk_status launch_attention(wk_ctx* ctx, int layer, const __nv_bfloat16* Q, int l
   p.n_full = static_cast<int>(n_full);
   p.n_ranges = static_cast<int>(ranges);
   const dim3 grid(static_cast<unsigned>(G));
-  if (lse_only) launch_chained(memory_attention_kernel<true>, grid, dim3(kThreads<true>), kSmemBytes<true>, s, p);
-  else launch_chained(memory_attention_kernel<false>, grid, dim3(kThreads<false>), kSmemBytes<false>, s, p);
+  if (lse_only) launch_chained(memory_attention_kernel<kTileKVLse>, grid, dim3(kThreads<kTileKVLse>), kSmemBytes<kTileKVLse>, s, p);
+  else if (in_64) launch_chained(memory_attention_kernel<kTileKVFew>, grid, dim3(kThreads<kTileKVFew>), kSmemBytes<kTileKVFew>, s, p);
+  else launch_chained(memory_attention_kernel<kTileKV>, grid, dim3(kThreads<kTileKV>), kSmemBytes<kTileKV>, s, p);
   if ((st = after_launch(ctx)) != WK_OK) return st;
   if (!lse_only && n_full != p.n_units) {   // some unit was cut
     launch_chained(combine_kernel, dim3(static_cast<unsigned>(p.n_units - n_full) * 32), dim3(kCombineThreads), 0, s, p.opart,

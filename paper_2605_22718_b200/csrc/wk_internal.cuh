@@ -14,6 +14,7 @@ namespace wk {
 constexpr int kHeadDim = 128;
 constexpr int kMaxDenseSegs = 8;
 constexpr int kTileKV = 80;       // KV rows per attention tile
+constexpr int kTileKVFew = 64;    // the same where there are few, or where they fill tiles of 80 badly
 constexpr int kTileKVLse = 128;   // the same in LSE-only launches
 constexpr int kTileQ = 128;    // Q rows per MMA tile (two per CTA)
 
@@ -47,7 +48,7 @@ struct SlotInfo {
 
 struct TmapKey {
   const void* ptr;
-  int32_t rows;
+  int32_t rows, box_rows;
   CUtensorMap map;
 };
 
@@ -75,7 +76,7 @@ struct wk_ctx {
   int64_t next_seq = 0;
   int32_t n_valid = 0;   // slots in state SLOT_VALID
   // tensor maps
-  CUtensorMap tm_kpool, tm_vpool, tm_kpool_lse;
+  CUtensorMap tm_kpool, tm_vpool, tm_kpool_few, tm_vpool_few, tm_kpool_lse;
   std::vector<wk::TmapKey> tmap_cache;
   size_t tmap_cache_next = 0;
   // per-context (hence per-device) one-time kernel attributes: opt-ins to large dynamic shared memory
@@ -111,7 +112,7 @@ inline wk_status after_launch(wk_ctx* ctx, int n = 1) {
 wk_status encode_rows_map(wk_ctx* ctx, const void* base, int64_t rows, int box_rows, CUtensorMap* out);
 // [n_mats][rows][D] bf16, box = 64 x box_rows x 1.
 wk_status encode_pool_map(wk_ctx* ctx, const void* base, int64_t rows, int64_t n_mats, int box_rows, CUtensorMap* out);
-const CUtensorMap* cached_rows_map(wk_ctx* ctx, const void* base, int32_t rows, wk_status* st);
+const CUtensorMap* cached_rows_map(wk_ctx* ctx, const void* base, int32_t rows, int32_t box_rows, wk_status* st);
 
 // Number of fp32 partial-result slots (256 rows x 128 each) the attention kernel may need.
 int attention_partial_slots(int n_heads, int max_lq, int max_splits);

@@ -170,10 +170,11 @@ static float fmax_nan(float a, float b) { return a != a || b != b ? NAN : fmaxf(
 #include "roles.inc"   // opens namespace wk and an unnamed one and leaves them open
 
 AttnParams par;
-constexpr bool kL = WK_TEST_LSE;
+constexpr int kRows = WK_TEST_ROWS;   // of a KV tile: picks the instantiation
+constexpr bool kL = is_lse<kRows>;
 struct Arena {
-  alignas(1024) uint8_t smem[kSmemBytes<kL>];
-  CtaShared<kL> sh;
+  alignas(1024) uint8_t smem[kSmemBytes<kRows>];
+  CtaShared<kRows> sh;
 } ar;
 
 int count_tiles(const AttnParams& p, int tb, int te) {
@@ -201,16 +202,16 @@ void start_copy(void* dst, uint64_t* bar, int what_in, int seg, int x, int y) {
   Copy c;
   c.bar = bar;
   const bool is_q = at < 2 * kQBytes;
-  c.bytes = is_q ? kHalfQBytes : kHalfKvBytes<kL>;
+  c.bytes = is_q ? kHalfQBytes : kHalfKvBytes<kRows>;
   if (x % 128) {
     c.what = 3;
     c.at = 0;
   } else {
     const int h = x / 128, in = at - 2 * kQBytes;
-    c.what = is_q ? 0 : in % kStageBytes<kL> >= kKvBytes<kL> ? 2 : 1;
-    c.at = is_q ? at / kQBytes : in / kStageBytes<kL>;
+    c.what = is_q ? 0 : in % kStageBytes<kRows> >= kKvBytes<kRows> ? 2 : 1;
+    c.at = is_q ? at / kQBytes : in / kStageBytes<kRows>;
     if (!is_q && c.what != what_in) fail("K where V belongs");
-    for (int r = 0; r < (is_q ? 4 : kKv<kL>); ++r) {
+    for (int r = 0; r < (is_q ? 4 : kRows); ++r) {
       const int row = y + (is_q ? 32 * r : r);
       c.rows.push_back(row < (is_q ? par.lq : rows_of(seg)) ? value(c.what, is_q ? 0 : seg, h, row) : 0.f);
     }
@@ -272,14 +273,14 @@ void end_commit(int w) {
 namespace ptx {
 static void mma_ss_if(uint32_t, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t add) {
   if (add) return;   // the first of the eight K = 16 steps stands for all of them
-  issue({false, static_cast<int>((a << 4) / kQBytes), static_cast<int>(((b << 4) - 2 * kQBytes) / kStageBytes<kL>), 0,
+  issue({false, static_cast<int>((a << 4) / kQBytes), static_cast<int>(((b << 4) - 2 * kQBytes) / kStageBytes<kRows>), 0,
          static_cast<int>(d), static_cast<int>(idesc >> 18) * 16, false});
 }
 static void mma_ts_if(uint32_t, uint32_t d, uint32_t a, uint64_t b, uint32_t, uint32_t add) {
   const uint32_t at = static_cast<uint32_t>(b << 4) - 2 * kQBytes;
-  issue({true, static_cast<int>((d - kTmemO) / 128), static_cast<int>(at / kStageBytes<kL>),
-         static_cast<int>((at % kStageBytes<kL> - kKvBytes<kL>) / 2048), static_cast<int>(d), 0, add != 0});
-  if (a != kTmemP + (d - kTmemO) + (at % kStageBytes<kL> - kKvBytes<kL>) / 2048 * 8) fail("P of another step");
+  issue({true, static_cast<int>((d - kTmemO) / 128), static_cast<int>(at / kStageBytes<kRows>),
+         static_cast<int>((at % kStageBytes<kRows> - kKvBytes<kRows>) / 2048), static_cast<int>(d), 0, add != 0});
+  if (a != kTmemP + (d - kTmemO) + (at % kStageBytes<kRows> - kKvBytes<kRows>) / 2048 * 8) fail("P of another step");
 }
 static void tma_load_2d(void* dst, const CUtensorMap* m, uint64_t* bar, int x, int y) {
   const int k = static_cast<int>(m - par.tm_kd), v = static_cast<int>(m - par.tm_vd);
@@ -294,7 +295,7 @@ static void tma_load_3d(void* dst, const CUtensorMap* m, uint64_t* bar, int x, i
 namespace {
 
 void fiber_main() {
-  attention_roles<kL>(par, ar.sh, ar.smem);
+  attention_roles<kRows>(par, ar.sh, ar.smem);
   fibers[current].done = true;
   for (;;) pause();
 }
@@ -302,14 +303,14 @@ void fiber_main() {
 // One CTA's work under one schedule.  hold: the fiber (or, from the number of fibers on: the copies, the products of MMA warp 0, 1)
 // that does not move from its `from`-th turn on until nothing else can; -1: a random one each time.  Returns the held one's turns.
 int run_cta(int hold, int from, unsigned seed) {
-  const int n = kThreads<kL> / 32;
+  const int n = kThreads<kRows> / 32;
   bars.clear();
   copies.clear();
   memset(q_use, 0, sizeof(q_use)); memset(k_use, 0, sizeof(k_use)); memset(v_use, 0, sizeof(v_use)); memset(t_use, 0, sizeof(t_use));
   memset(tmem, 0xff, sizeof(tmem));
   for (int w = 0; w < 2; ++w) { issued[w].clear(); commits[w].clear(); }
   memset(static_cast<void*>(&ar.sh), 0, sizeof(ar.sh));
-  init_barriers<kL>(ar.sh);
+  init_barriers<kRows>(ar.sh);
   ar.sh.abort = 0;
   stuck = false;
   fibers.resize(n);
@@ -380,11 +381,11 @@ extern "C" int run_roles(int H, int lq, const int* seg_rows, int n_segs, const i
                          int grid, int schedules, int hold, char* what, int what_size) {
   memset(static_cast<void*>(&par), 0, sizeof(par));
   arena = reinterpret_cast<uint8_t*>(&ar);
-  mma_warp = kSoftWarps<kL>;
+  mma_warp = kSoftWarps<kRows>;
   constexpr int kPool = 8;   // slots of the pool; odd ones are stale
   std::vector<int32_t> valid(kPool), slots(slot_ids, slot_ids + n_slots);
   for (int i = 0; i < kPool; ++i) valid[i] = !(i & 1);
-  par.tile_rows = kKv<kL>;
+  par.tile_rows = kRows;
   int tiles = 0;
   for (int i = 0; i <= kMaxDenseSegs; ++i) {
     par.seg_tile_prefix[i] = tiles;
@@ -463,7 +464,7 @@ extern "C" int run_roles(int H, int lq, const int* seg_rows, int n_segs, const i
   };
   fault.clear();
   for (int s = 0; s < schedules && fault.empty(); ++s) all(-1, 0, s);
-  for (int h = 0; hold && h < kThreads<kL> / 32 + 3 && fault.empty(); ++h) {
+  for (int h = 0; hold && h < kThreads<kRows> / 32 + 3 && fault.empty(); ++h) {
     const int turns = all(h, 1 << 30, 0);
     for (int from = 0; from < turns && fault.empty(); ++from) {
       all(h, from, 0);

@@ -26,10 +26,10 @@ def roles_source():
     assert warp_wide in body
     body = body.replace(warp_wide, "int count_tiles(const AttnParams& p, int tb, int te);\n" + warp_wide[:-1] + "_of_a_warp(", 1)
     body = re.sub(r"\basm(\s+volatile)?\s*\(", "WK_ASM(", body)
-    return body + "template <bool kLse> void init_barriers(CtaShared<kLse>& sh) {\n" + init + "}\n"
+    return body + "template <int kKv> void init_barriers(CtaShared<kKv>& sh) {\n  constexpr bool kLse = is_lse<kKv>;\n" + init + "}\n"
 
 
-@pytest.fixture(scope="module", params=[False, True], ids=["attention", "lse_only"])
+@pytest.fixture(scope="module", params=[80, 64, 128], ids=["tiles_of_80", "tiles_of_64", "lse_only"])
 def run(request, tmp_path_factory):
     if shutil.which("g++") is None:
         pytest.skip("no host compiler")
@@ -37,7 +37,7 @@ def run(request, tmp_path_factory):
     (out / "roles.inc").write_text(roles_source())
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_nvcc()))), "include")
     lib = str(out / "libroles.so")
-    subprocess.run(["g++", "-std=c++17", "-O2", "-w", "-shared", "-fPIC", "-Wl,-Bsymbolic", f"-DWK_TEST_LSE={int(request.param)}",
+    subprocess.run(["g++", "-std=c++17", "-O2", "-w", "-shared", "-fPIC", "-Wl,-Bsymbolic", f"-DWK_TEST_ROWS={request.param}",
                     "-I", str(out), "-I", cuda, "-I", CSRC, os.path.join(HOST, "attention_roles.cc"), "-o", lib], check=True)
     fn = C.CDLL(lib).run_roles
 
@@ -46,7 +46,7 @@ def run(request, tmp_path_factory):
         bad = fn(H, lq, (C.c_int * len(segs))(*segs), len(segs), (C.c_int * len(slots))(*slots), len(slots), C_rows, n_full, n_ranges,
                  grid, schedules, int(hold), what, 400)
         assert not bad, what.value.decode()
-    call.lse_only = request.param
+    call.lse_only = request.param == 128
     return call
 
 

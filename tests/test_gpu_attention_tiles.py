@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("seg_rows", [(1,), (15, 16), (17, 31), (32, 33), (63, 64, 65), (96, 97), (112, 127), (128,), (129, 1, 144),
-                                      (255, 256, 257), (79, 80), (81, 159, 160), (161,), (512,), (513,), (480, 33), (720, 40, 641)])
+                                      (255, 256, 257), (79, 80), (81, 159, 160), (161,), (512,), (513,), (480, 33), (720, 40, 641), (190, 256, 191, 161), (513, 512)])
 @pytest.mark.parametrize("lq", [1, 129, 300])
 def test_short_tiles_of_dense_segments(seg_rows, lq):
     from paper_2605_22718_b200 import WorldKV
@@ -36,9 +36,9 @@ def test_short_tiles_of_dense_segments(seg_rows, lq):
         np.testing.assert_allclose(lse.cpu().numpy(), L_ref, atol=2e-3)
 
 
-@pytest.mark.parametrize("T,n_keep", [(9, 1), (40, 24), (100, 27), (100, 28), (100, 29), (200, 57)])
+@pytest.mark.parametrize("T,n_keep", [(9, 1), (40, 24), (100, 27), (100, 28), (100, 29), (150, 40), (200, 56), (200, 57)])
 def test_short_tiles_of_pool_slots(T, n_keep):
-    """C = T + n_keep stored rows per chunk: 10, 64, 127, 128, 129, 257."""
+    """C = T + n_keep stored rows per chunk: 10, 64, 127, 128, 129, 190, 256 (tiled in 64 rows), 257."""
     from paper_2605_22718_b200 import WorldKV
     H, S, lq = 3, 6, 140
     kv = WorldKV(n_layers=1, n_heads=H, tokens_per_frame=T, n_keep=n_keep, pool_slots=S, max_k=S, max_batch=1, max_lq=lq,
