@@ -249,6 +249,11 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
+__device__ __forceinline__ float fmax3_nan(float a, float b, float c) {   // NaN if any is
+  float d;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
 __device__ __forceinline__ float fmax_nan(float a, float b) {   // NaN if either is
   float d;
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
@@ -258,7 +263,7 @@ __device__ __forceinline__ float fmax_nan(float a, float b) {   // NaN if either
 // keys), so a share of the pairs takes 2^x from the FMA pipe instead (2,640 queries x 12 heads x 250 slots of 1,320 rows: 3,563 / 3,487 /
 // 3,434 / 3,493 / 3,725 us at 0 ... 4 of 8): x = n + f with n = round(x) by the add-a-large-constant trick, 2^f on [-1/2, 1/2] by a cubic
 // (relative error 7.7e-5), 2^n by adding n to the exponent field; all in packed fp32 pairs.  That path clamps at x = -120 (a weight of
-// 1e-36), needs x < 127, and turns NaN into a weight beyond all bounds.
+// 1e-36), needs x < 127, and turns NaN into a number: the caller looks for NaN in the logits (big).
 template <bool kPoly>
 __device__ __forceinline__ void exp2_pair(uint64_t e, float& p0, float& p1) {
   float e0, e1;
@@ -294,7 +299,7 @@ __device__ __forceinline__ float sum4_f32x2(const uint64_t (&acc)[4]) {
 
 constexpr int kLsePoly = 2;
 // Sum of 2^(s * scale - m) over 32 columns of a row, in four independent (lo, hi) accumulators.  kLsePoly of every 8 pairs take
-// the FMA pipe; big = the largest of their raw values (the caller checks that they stay below that path's limit).
+// the FMA pipe; big = the largest of their raw values, or NaN (the caller checks that they stay below that path's limit).
 __device__ __forceinline__ void exp_chunk(uint32_t (&r)[32], int rem, uint64_t scale2, uint64_t neg_m2, uint64_t (&acc)[4],
                                           float& big) {
   if (rem < 32) {   // columns past the end of the segment or slot
@@ -308,7 +313,7 @@ __device__ __forceinline__ void exp_chunk(uint32_t (&r)[32], int rem, uint64_t s
     float p0, p1;
     if ((i & 7) < kLsePoly) {
       exp2_pair<true>(e, p0, p1);
-      big = fmax3(big, s0, s1);
+      big = fmax3_nan(big, s0, s1);
     } else {
       exp2_pair<false>(e, p0, p1);
     }
@@ -750,7 +755,7 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
             tc_wait_ld(r);
             exp_chunk(r, nv - c * 32, scale2, neg_m2, acc, big);
           }
-          sum = sum4_f32x2(acc);
+          sum = big != big ? big : sum4_f32x2(acc);
           const bool off = !(sum <= 32768.f) || big * p.scale_log2 - m > 100.f || (first && sum < 2.44140625e-4f);
           if (attempt > 0 || !__any_sync(0xffffffffu, off)) break;
           const float mx = row_max_tmem(tS, nv);
@@ -781,9 +786,10 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
         if (lane == 0) mbar_arrive(&bars.m_empty[qt]);
         const int qrow = pc.q0 + qt * kTileQ + row;
         if (qrow < p.lq) {
-          // (a warpgroup without tiles leaves a sum of 0, a stale slot two of them)
+          // (a warpgroup without tiles leaves a sum of 0, a stale slot two of them; a logit that is NaN leaves NaN, and the slot then
+          // counts for nothing in this row)
           const float mm = l > 0.f ? (o.y > 0.f ? fmaxf(m, o.x) : m) : o.x;
-          const float sum = (l > 0.f ? l * ex2_approx(m - mm) : 0.f) + (o.y > 0.f ? o.y * ex2_approx(o.x - mm) : 0.f);
+          const float sum = (l != 0.f ? l * ex2_approx(m - mm) : 0.f) + (o.y != 0.f ? o.y * ex2_approx(o.x - mm) : 0.f);
           p.lse[(static_cast<int64_t>(pc.ord) * p.H + pc.h) * p.lq + qrow] =
               sum > 0.f ? (mm + log2f(sum)) * 0.6931471805599453f : -INFINITY;
         }
@@ -902,8 +908,9 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
         }
         if (ok) {
           tc_fence_after();
-          const float inv_l = (j > 0 && l > 0.f) ? 1.f / l : 0.f;
-          const float lse = (j > 0 && l > 0.f) ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+          // without keys 0 and -inf; a sum that is NaN (a logit was) makes the row and its log-sum-exp NaN
+          const float inv_l = (j > 0 && l != 0.f) ? 1.f / l : 0.f;
+          const float lse = (j > 0 && l != 0.f) ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             uint32_t r[32];
@@ -1069,7 +1076,7 @@ combine_kernel(const float4* __restrict__ opart, const float* __restrict__ lsepa
       }
     }
   }
-  const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
+  const float inv = wsum != 0.f ? 1.f / wsum : 0.f;   // NaN stays NaN
   s_out[lane][warp] = make_uint2(ptx::pack_bf16x2(acc.x * inv, acc.y * inv), ptx::pack_bf16x2(acc.z * inv, acc.w * inv));
   __syncthreads();
   if (tid < 128) {
@@ -1079,7 +1086,7 @@ combine_kernel(const float4* __restrict__ opart, const float* __restrict__ lsepa
           reinterpret_cast<const uint4*>(&s_out[r][0])[v];
   }
   if (lse_out && cg == 0 && warp == 0 && qrow0 + lane < lq)
-    lse_out[static_cast<int64_t>(h) * lq + qrow0 + lane] = wsum > 0.f ? mx + logf(wsum) : -INFINITY;
+    lse_out[static_cast<int64_t>(h) * lq + qrow0 + lane] = wsum != 0.f ? mx + logf(wsum) : -INFINITY;
 }
 
 }  // namespace
