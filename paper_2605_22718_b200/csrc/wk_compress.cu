@@ -428,6 +428,7 @@ constexpr int kRowWarpsWhole = 8, kRowMaxVplWhole = 6;
 constexpr int kRowWarpsHead = 16, kRowMaxVplHead = 3;
 constexpr int kFusedScoreRows = 64;   // rows of a score item of the one-launch kernel (measured: 64-80 best at 5,120 columns)
 constexpr int kFusedMinCols = 2048;   // whole-token rows wider than this take the one-launch path (measured faster there)
+constexpr size_t kSmBytes = 228 * 1024, kFusedStatic = 6 * 1024;   // shared memory of an SM; static arrays of compress_fused and the 1 KB that the system keeps per CTA
 constexpr double kRowNorm2Hi = 1.2676506002282294e+30;    // 2^100: above it (or below 2^-80) 1/|a| is a true division
 
 __device__ __forceinline__ double rsqrt_newton(double x) {   // x in [2^-80, 2^100]: inside fp32's normal range
@@ -684,6 +685,8 @@ __device__ __forceinline__ float key_f32(uint32_t k) {
 // The passes alone were 6,200 of the
 // 16,400 clocks of a selection among 1,760 scores; a call of one layer that stores, 38.9 -> 37.5 us, per-head keep-sets of 30 layers
 // x 12 heads 86.1 -> 84.0.
+// (The histogram has 4 KB of its own.  Where band_s lies it would leave room for a fourth score_select CTA per SM from 1,544 tokens per
+// frame on, and three are faster: 40 layers of 1,560 tokens x 16 heads stored in 386 us with three, 426 with four.)
 constexpr int kSelectBins = 1024;
 template <int kThr, bool kPerHead>
 __device__ __forceinline__ void select_problem(uint8_t* smem, int b, const __nv_bfloat16* __restrict__ K, RowMap rm, int T,
@@ -1365,7 +1368,7 @@ wk_status launch_compress(wk_ctx* ctx, const __nv_bfloat16* K, int64_t stride, i
       const size_t smem_s = smem_sel > smem_m ? smem_sel : smem_m;
       const size_t smem_f = smem_a > smem_s ? smem_a : smem_s;
       // persistent grid: what fits the machine at this shared-memory size
-      int per_sm = static_cast<int>((220 * 1024) / (smem_f + 2048));
+      int per_sm = static_cast<int>(kSmBytes / (smem_f + kFusedStatic));
       const int by_regs = vpt == 1 ? 4 : (vpt == 2 ? 3 : 2);
       if (per_sm > by_regs) per_sm = by_regs;
       if (per_sm < 1) per_sm = 1;
