@@ -194,7 +194,6 @@ __device__ __forceinline__ void group_accumulate(const uint8_t* buf, size_t row_
 
 // After a CTA has written its slice of chunk b: the last CTA of the chunk (an atomic ticket decides) adds the slices in
 // slice order and writes m64, m32 = fp32(m64) and |m|^2 (per head with per-head keys).  Called by every thread of the CTA.
-template <int kGroups>
 __device__ __forceinline__ void anchor_finish(int b, int parts, int T, int D, int hs, const double* __restrict__ partial,
                                               int max_parts, uint32_t* __restrict__ tickets, double* __restrict__ m64,
                                               float* __restrict__ m32, double* __restrict__ mnorm2, uint32_t* ready,
@@ -208,62 +207,49 @@ __device__ __forceinline__ void anchor_finish(int b, int parts, int T, int D, in
   if (tid == 0) s_flag = (atomicAdd(&tickets[b], 1u) == static_cast<uint32_t>(parts - 1)) ? 1u : 0u;
   __syncthreads();
   if (!s_flag) return;
-  // ---- last CTA of the chunk: add the slices in slice order.  Thread t owns column pairs t, t + nthr, ...; the loads of eight
-  // slices of kGroups of them are in flight before the first addition: every trip to L2 stands between the anchors and the
-  // scores (24 heads x 880 tokens, 8 layers stored: 124.2 us a pair at a time, 115.5 with three).  Kernels of 16 warps have no
-  // registers for more than one (40 heads, per head: 129.4 us, 131.3 with two).
+  // ---- last CTA of the chunk: add the slices in slice order.  Thread t owns column pairs t, t + nthr, ...; eight slices' worth of
+  // loads are in flight before the first addition, issued by all threads alike (under a branch for the columns that exist: 24 heads x
+  // 880 tokens, 8 layers stored, 124.4 us instead of 116.6).  Three column pairs at a time cost registers and gain nothing (30 layers of
+  // one head 51.2 us instead of 49.7).
   __threadfence();
   const double* pb = partial + static_cast<int64_t>(b) * max_parts * D;
   const double inv_T = 1.0 / static_cast<double>(T);
   const int pairs = D >> 1;
   double nn_all = 0.0;
-  for (int c0 = 0; c0 < pairs; c0 += kGroups * nthr) {   // uniform trip count: the per-head sums use block barriers
-    double t0[kGroups], t1[kGroups];
-#pragma unroll
-    for (int g = 0; g < kGroups; ++g) t0[g] = t1[g] = 0.0;
+  for (int c0 = 0; c0 < pairs; c0 += nthr) {   // uniform trip count: the per-head sums use block barriers
+    const int c = c0 + tid;
+    double t0 = 0.0, t1 = 0.0;
     for (int p0 = 0; p0 < parts; p0 += 8) {
-      double2 v[kGroups][8];
+      double2 v[8];
 #pragma unroll
-      for (int g = 0; g < kGroups; ++g) {
-        const int c = c0 + g * nthr + tid;
+      for (int pp = 0; pp < 8; ++pp)
+        v[pp] = c < pairs && p0 + pp < parts ? __ldcg(reinterpret_cast<const double2*>(pb + static_cast<int64_t>(p0 + pp) * D) + c)
+                                             : make_double2(0.0, 0.0);
 #pragma unroll
-        for (int pp = 0; pp < 8; ++pp)
-          v[g][pp] = c < pairs && p0 + pp < parts ? __ldcg(reinterpret_cast<const double2*>(pb + static_cast<int64_t>(p0 + pp) * D) + c)
-                                                  : make_double2(0.0, 0.0);
-      }
-#pragma unroll
-      for (int g = 0; g < kGroups; ++g) {
-#pragma unroll
-        for (int pp = 0; pp < 8; ++pp) {
-          t0[g] += v[g][pp].x;
-          t1[g] += v[g][pp].y;
-        }
+      for (int pp = 0; pp < 8; ++pp) {
+        t0 += v[pp].x;
+        t1 += v[pp].y;
       }
     }
-#pragma unroll
-    for (int g = 0; g < kGroups; ++g) {
-      const int cg = c0 + g * nthr, c = cg + tid;
-      if (cg >= pairs) break;   // the same for the whole block
-      t0[g] *= inv_T;
-      t1[g] *= inv_T;
-      if (c < pairs) {
-        reinterpret_cast<double2*>(m64 + static_cast<int64_t>(b) * D)[c] = make_double2(t0[g], t1[g]);
-        reinterpret_cast<float2*>(m32 + static_cast<int64_t>(b) * D)[c] =
-            make_float2(static_cast<float>(t0[g]), static_cast<float>(t1[g]));
-      }
-      const double nn = fma(t0[g], t0[g], t1[g] * t1[g]);
-      if (hs == 1) {
-        nn_all += nn;
-      } else {
-        // 64 column pairs per head: warps 2j and 2j + 1 of this step hold head cg / 64 + j
-        const double wsum = warp_sum(nn);
-        __syncthreads();
-        if (lane == 0) red[warp] = wsum;
-        __syncthreads();
-        const int head = (cg >> 6) + tid;
-        if (tid < nwarps / 2 && head < hs)
-          mnorm2[(static_cast<int64_t>(b) * hs + head) * kMaxNormParts] = red[2 * tid] + red[2 * tid + 1];
-      }
+    t0 *= inv_T;
+    t1 *= inv_T;
+    if (c < pairs) {
+      reinterpret_cast<double2*>(m64 + static_cast<int64_t>(b) * D)[c] = make_double2(t0, t1);
+      reinterpret_cast<float2*>(m32 + static_cast<int64_t>(b) * D)[c] =
+          make_float2(static_cast<float>(t0), static_cast<float>(t1));
+    }
+    const double nn = fma(t0, t0, t1 * t1);
+    if (hs == 1) {
+      nn_all += nn;
+    } else {
+      // 64 column pairs per head: warps 2j and 2j + 1 of this step hold head c0 / 64 + j
+      const double wsum = warp_sum(nn);
+      __syncthreads();
+      if (lane == 0) red[warp] = wsum;
+      __syncthreads();
+      const int head = (c0 >> 6) + tid;
+      if (tid < nwarps / 2 && head < hs)
+        mnorm2[(static_cast<int64_t>(b) * hs + head) * kMaxNormParts] = red[2 * tid] + red[2 * tid + 1];
     }
   }
   if (hs == 1) {
@@ -400,7 +386,7 @@ __device__ __forceinline__ void anchor_role(uint8_t* smem, int b, int part, int 
         __stcg(reinterpret_cast<double2*>(my + 8 * vec) + e, make_double2(acc[8 * i + 2 * e], acc[8 * i + 2 * e + 1]));
     }
   }
-  anchor_finish<1>(b, parts, T, D, 1, partial, max_parts, tickets, m64, m32, mnorm2, ready, epoch);
+  anchor_finish(b, parts, T, D, 1, partial, max_parts, tickets, m64, m32, mnorm2, ready, epoch);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -597,7 +583,7 @@ anchor_rows(const __nv_bfloat16* __restrict__ K, int64_t stride, int chunks, int
       }
       __stcg(my + c, t);
     }
-    anchor_finish<NW == 8 ? 3 : 1>(b, last - first + 1, T, D, hs, partial, max_parts, tickets, m64, m32, mnorm2, nullptr, 0u);
+    anchor_finish(b, last - first + 1, T, D, hs, partial, max_parts, tickets, m64, m32, mnorm2, nullptr, 0u);
     __syncthreads();   // sacc and anchor_finish's shared words are free for the next chunk
   }
 }
