@@ -126,14 +126,14 @@ def test_log_sum_exp_over_short_slots():
 
 
 @pytest.mark.parametrize("step", [-3, -7, -12, -15, -19, -30, 7, 15, 30])
-@pytest.mark.parametrize("n", [512, 470, 1200])
-def test_large_values_under_falling_and_rising_logits(n, step):
-    """The logits of a tile lie `step` log2 units from those of the tile before.  Values scaled by 2^115 are exact in bf16 and leave
+@pytest.mark.parametrize("n,tile", [(512, 128), (470, 128), (1200, 128), (512, 64), (800, 80), (1200, 80)])
+def test_large_values_under_falling_and_rising_logits(n, tile, step):
+    """The logits move by `step` log2 units every `tile` keys, in step with the kernel's tiles (64 rows in short calls, 80) or not.  Values scaled by 2^115 are exact in bf16 and leave
     2^12 of fp32's range: O is the unscaled O times 2^115, bit for bit, as long as the sum that O is held against stays below 2^10."""
     H, lq = 2, 140
     q, k, v = normals(10, (lq, H, 128)), normals(11, (n, H, 128)), normals(12, (n, H, 128))
     q[:, :, 0] = 16.0
-    k[:, :, 0] = (step * (np.arange(n) // 128) / (16.0 * SCALE * 1.4426950408889634))[:, None]
+    k[:, :, 0] = (step * (np.arange(n) // tile) / (16.0 * SCALE * 1.4426950408889634))[:, None]
     Q, K, V = (wd.to_device_bf16(bf16(x)) for x in (q, k, v))
     kv = context(H, lq)
     for splits in (1, 0, 2):

@@ -61,7 +61,7 @@ def test_large_and_small_values(shift, v_exp):
     run(1, 130, (300,), 0, shift, None, v_exp=v_exp)
 
 
-@pytest.mark.parametrize("H,lq,rows", [(1, 256, 2000), (9, 2000, 900), (20, 2100, 640)])
+@pytest.mark.parametrize("H,lq,rows", [(1, 256, 2000), (9, 2000, 900), (10, 2048, 3600), (20, 2100, 640)])
 @pytest.mark.parametrize("shift", [90, 200])
 def test_a_few_rows_moved(H, lq, rows, shift):
     """One row in the first Q tile of a pair, one in the last ragged one, one in a second tile: the other units of the CTAs that

@@ -61,14 +61,17 @@ def test_short_tiles_of_pool_slots(T, n_keep):
         np.testing.assert_allclose(lse.cpu().numpy(), L_ref, atol=2e-3)
 
 
-@pytest.mark.parametrize("H,lq,rows", [
-    (1, 100, 4500),      # one unit cut into as many pieces as a unit may have
-    (7, 256, 2000),      # 7 units, every one cut into equal parts, one piece per CTA
-    (9, 2000, 900),      # 72 units: ranges that end inside units, two pieces per CTA
-    (20, 2100, 640),     # 180 units: one whole wave, the rest cut (or not) by the rule
-    (29, 1300, 2600),    # 174 units: whole units and a cut piece on the same CTA
+@pytest.mark.parametrize("H,lq,rows,cut", [
+    (1, 100, 4500, True),      # one unit in 12 pieces of five tiles
+    (1, 100, 12000, True),     # one unit in as many pieces as a unit may have
+    (7, 256, 2000, True),      # 7 units, every one cut into equal parts, one piece per CTA
+    (9, 2000, 900, False),     # 72 units, not cut
+    (10, 2048, 3600, True),    # 80 units of 45 tiles: a range per SM, most of them over the end of a unit
+    (19, 2048, 1000, True),    # 152 units: one whole wave, the four others in equal parts
+    (20, 2100, 640, False),    # 180 units: one whole wave and whole units behind it
+    (29, 2048, 4000, True),    # 232 units: whole units and a range that crosses units on the same CTA
 ])
-def test_work_distributions(H, lq, rows):
+def test_work_distributions(H, lq, rows, cut):
     """The default distribution over the SMs (whole units, aligned cuts, ranges across units) against one CTA per unit,
     and one head against the oracle."""
     from paper_2605_22718_b200 import WorldKV
@@ -81,7 +84,10 @@ def test_work_distributions(H, lq, rows):
     out = {}
     for splits in (0, 1):
         lse = torch.empty((H, lq), dtype=torch.float32, device="cuda")
+        launches = kv.launch_count()
         out[splits] = kv.memory_attention(0, Q, [seg], None, 0, lse_out=lse, kv_splits=splits).clone(), lse
+        if torch.cuda.get_device_properties(0).multi_processor_count == 148:   # the sizes above are for that many
+            assert kv.launch_count() - launches == (2 if cut and splits == 0 else 1)   # a second one merges pieces
         assert kv.poll_status() == (0, 0)
     # the two differ by one bf16 rounding of the output and the fp32 merge
     a, b = out[0][0].float(), out[1][0].float()
