@@ -6,7 +6,7 @@
 //     bf16 output and share a head's K/V tiles through L2 because they walk the keys in step; the units of a last, partial
 //     wave are cut into ranges over all SMs where that pays (split_default): a range writes a normalised fp32 partial plus
 //     its log-sum-exp per piece, and combine_kernel merges them;
-//   * K/V tiles (80 rows x 128 columns of one head, bf16) are fetched by TMA straight from where they lie:
+//   * K/V tiles (80 rows x 128 columns of one head, bf16; or 64 rows, see kFewTiles) are fetched by TMA straight from where they lie:
 //     a dense segment (2-D tensor map per segment) or a pool slot (3-D tensor map [layer*slot][row][col]; the
 //     slot id is read from device memory, so the retrieval result never visits the host).  Rows past the end
 //     of a segment/slot are zero-filled by TMA and masked to -inf before the exponentials;
@@ -14,17 +14,17 @@
 //     O0 and O1 take half of its 512 columns; 80 keys is the widest tile whose S (80 columns) and P (bf16: 40 columns, the A
 //     operand of P V) lie side by side in the other half, so that S of the next tile can be multiplied while the softmax works
 //     on this one, which it has read into registers.  (With 128 keys P has to overwrite S and the two take turns: 12 heads x
-//     2,640 queries x 15,840 keys 261 us back to back instead of 253, although Q K^T alone runs at its full rate only from
+//     2,640 queries x 15,840 keys 261 us back to back instead of 249, although Q K^T alone runs at its full rate only from
 //     N = 128 on: shared memory gives a Q K^T step of 80 keys (4 + 2.5 KB) in 52 clk, one of 128 (4 + 4 KB) in 64.)
 //   * warp roles: warps 0-3 / 4-7 = softmax of Q tile 0 / 1 (one thread per row, fp32 in the exp2
 //     domain, against a reference that follows the row's maximum: see kStreamSum), warps 8 / 9 = MMA issue for Q tile 0 / 1,
 //     warp 10 = TMA producer.  The producer walks the tile list, and hands each tile's height to the others beside the tile;
 //   * a tile with fewer valid rows (the last one of a segment or slot: 1,320 rows are 16 tiles and 40 rows) is
 //     multiplied over ceil(nv / 16) * 16 rows.
-// What bounds it: back to back, the energy that the board's 1,000 W cap allows.  2,640 queries x 15,840 keys x 12 heads is one
-// unit of 201 KV tiles on each of 132 SMs: 253 us at 1,640 MHz, 1,780 clk per tile in full flow, where the tensor pipe needs
-// 1,432 (measured with nothing else running; 1,600 with the exponentials left out: the chain S -> registers, P -> P V, Q K^T of
-// one Q tile is 1,470 long, 750 of it hand-overs).  4,680 x 32,760 x 40: 2,777 us at 1,555 MHz.
+// What bounds it: the chain of a step, at the clock that the board's 1,000 W cap leaves.  2,640 queries x 15,840 keys x 12 heads is one
+// unit of 201 KV tiles on each of 132 SMs: 249 us.  A tile takes 1,869 clk in a CTA that runs alone (1,965 MHz) and 1,932 to 1,995
+// beside 131 others (1,570 to 1,635 MHz); 1,432 of them the tensor pipe needs (measured with nothing else running), and S ->
+// registers, exponentials, P -> P V, Q K^T of one Q tile is a chain of its own under the other's.  4,680 x 32,760 x 40: 2,740 us.
 // Every wait is bounded; a wait that runs out sets WK_DEV_TIMEOUT, the CTA drains and frees its tensor memory.
 #include <stddef.h>
 
@@ -58,12 +58,12 @@ constexpr int kNvRing = 16;   // tile heights handed from the TMA warp to the ot
 // are streamed on trust.  Their sum tells whether that was right: no weight above 2^8 hides in a sum of at most kStreamSum.  A warp
 // in which a row's sum is larger still has S in registers, moves its references to the maximum where that is more than 2^8 above,
 // and takes the exponentials again; tiles after that are read for the maximum first, twice as many each time.  12 heads x 2,640
-// queries x 15,840 keys, back to back: 267 us with the maximum first for all, 261 this way.
+// queries x 15,840 keys, back to back: 253.6 us with the maximum first for all, 248.5 this way.
 constexpr float kRescaleThreshold = 8.0f;           // log2 units: P stays <= 2^8 between maximum updates
 constexpr float kStreamSum = 256.0f;
 // Pieces of at most kFewTiles tiles move the reference to every tile's own maximum, down as well as up: beside few other keys a
 // tile's largest weight counts, and it is exact this way, as if the tile were a piece of its own.  450 queries x 5 heads x 1,040
-// keys (pieces of three tiles), relative error of O at deviations 1 / 2 / 4: 2.13 / 1.80 / 1.69e-3, without 2.27 / 2.19 / 1.98e-3.
+// keys (three pieces of four or five tiles), relative error of O at deviations 1 / 2 / 4: 2.11 / 1.77 / 1.68e-3, without 2.30 / 2.23 / 2.09e-3.
 // Calls of at most kFewTilesOfCall tiles of kTileKVFew rows walk them in such tiles, so that no more keys share a maximum.  So do calls
 // whose segments and slots fill tiles of kTileKV rows badly: a tile of 64 takes 1,713 clk where one of 80 takes 1,919, by the clocks
 // that the power cap leaves 6 to 7 for 7 to 8 (16,000 rows in slots of C, 12 heads x 2,640 queries, us in tiles of 80 / 64: C = 170 358 /
@@ -1100,14 +1100,15 @@ int attention_partial_slots(int n_heads, int max_lq, int max_splits) {
 // Default distribution over the SMs: whole units in full waves, then, where it pays, the units of the last, partial wave cut
 // and merged.  Times in us on 148 SMs, whole / cut, back to back, one dense segment.
 //   * Where every unit can be cut at least in two, it is, into equal ranges that end with their unit: no CTA gets two pieces, and
-//     the idle SMs cost less than pieces that straddle units (30 units of 32 tiles: 120 ranges 26.9, 148 ranges 31.1; of 64
-//     tiles 32.0 and 39.9; 66 units of 38 tiles: 132 ranges 39.1, 148 ranges 45.5).  A piece has 5 tiles or more (2 heads x
-//     3,960 keys, 8 units of 50 tiles: 5 tiles 20.7, 4 21.6, 3 23.2, 10 21.9).  Else equal ranges over all SMs.
+//     the idle SMs cost less than pieces that straddle units (30 units of 32 tiles: 120 ranges 28.3, 148 ranges 31.2; of 64
+//     tiles 33.2 and 41.8; 66 units of 38 tiles: 132 ranges 43.5, 148 ranges 55.5).  A piece has 5 tiles or more (2 heads x
+//     3,960 keys, 8 units of 50 tiles: 5 tiles 19.9, 4 19.9, 3 21.5, 10 24.8).  Else equal ranges over all SMs.
 //   * A cut saves at most (sms - rest) / sms of a unit's tiles and costs about 8 tiles (the combine launch, a second prologue) and
-//     up to 22 more where every CTA writes partials: 30 units of 16 tiles 24.8 / 21.2; 50 of 16 24.2 / 27.9; 66 of 25 33.6 / 32.8;
-//     88 of 38 49.8 / 53.7, of 57 69.1 / 64.5; 99 of 63 76.8 / 75.1; 110 of 94 106.4 / 103.3, of 150 170 / 160; 121 of 125 138.3 /
-//     139.2, of 150 177 / 165; 132 of 198 247.8 / 253.6, of 282 357.8 / 358.1, of 500 621 / 597.  With full waves before it: 760
-//     units of 410 tiles (rest 20) 2,953 / 2,763.
+//     up to 22 more where every CTA writes partials: 12 units of 12 tiles 17.7 / 16.3; 24 of 15 20.7 / 21.0; 30 of 16 21.7 / 21.8, of 20
+//     25.6 / 23.5; 40 of 21 27.1 / 28.4; 50 of 16 22.3 / 29.7, of 24 30.0 / 30.4; 66 of 25 31.8 / 35.7, of 38 46.0 / 43.5; 88 of 38
+//     52.9 / 64.4, of 57 77.8 / 81.1; 99 of 63 89.1 / 97.0; 110 of 94 136 / 142, of 150 216 / 202; 121 of 125 185 / 196, of 150 226 /
+//     231; 132 of 198 253 / 266, of 282 358 / 361, of 500 638 / 605.  With full waves before it: 760 units of 410 tiles (rest 20)
+//     2,953 / 2,763.
 //   * Units of a little more than kFewTiles tiles are cut before that saves time, where a cut leaves pieces of few tiles, whose every
 //     largest weight is exact (24 units of 1,040 keys: relative error of O at deviations 1 / 2 / 4 2.33 / 2.29 / 2.14e-3 whole at 19.1
 //     us, 2.14 / 1.78 / 1.68e-3 in three pieces at 20.5; 40 of 1,520: 25.4 and 27.7 us).  The line is drawn in tiles of 128 rows, of

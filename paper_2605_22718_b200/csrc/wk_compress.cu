@@ -395,9 +395,8 @@ __device__ __forceinline__ void anchor_role(uint8_t* smem, int b, int part, int 
 // (the fewest that leave a lane at most 6, with per-head keys 3, 16-byte column groups); lane l of warp w of the set owns the column
 // groups (w * 32 + l) + 32 * wpr * i, i < VPL.  The CTA's NW / wpr sets take the rows of the run round robin;
 // every lane
-//   converts its share of the row to fp64 once (the conversion unit's rate, a quarter of the fp64 multiply-add rate, is
-//   what bounds this kernel: one conversion per element, not one per phase) and issues the loads of its share of the
-//   set's next row into the registers just freed;
+//   converts its share of the row to fp64 once (one conversion per element, not one per phase) and issues the loads of its share of
+//   the set's next row into the registers just freed;
 //   phase 1: squares its share; the row's squared norm is a warp sum (plus an exchange between the set's warps through
 //            shared memory when wpr > 1); with per-head keys a sum over the 16 lanes that hold one head's 128 columns;
 //            1/|a| from the fp32 reciprocal square root and two Newton steps in fp64 (within a few units of the last
@@ -434,9 +433,10 @@ __device__ __forceinline__ void set_barrier(int id, int threads) {
 }
 
 // The lane's share of one row, converted to fp64 ONCE (x, kept in registers for phase 2), with the sum of squares of
-// each of its column groups.  One conversion instruction per element: the conversion unit's rate (a quarter of the
-// fp64 multiply-add rate) is what bounds the kernel, and converting once instead of once per phase is what the
-// registers are spent on.
+// each of its column groups.  Converting once instead of once per phase is what the registers are spent on.  (The conversion unit
+// works at a quarter of the fp64 multiply-add rate, 17.7 us for 30 layers of 880 anchors x 1,536 columns; but with moved fields and an
+// exact multiplication by 2^896 in the instruction's place the kernel takes its 35 to 39 us as before.  A set's rows are a
+// chain: loads, conversions, a warp-wide fp64 sum, 1/|a|, additions, with one row's loads in flight.)
 template <int VPL>
 __device__ __forceinline__ void row_convert(const uint4 (&q)[VPL], uint32_t active, double (&x)[8 * VPL], double (&p)[VPL]) {
 #pragma unroll
@@ -500,7 +500,7 @@ anchor_rows(const __nv_bfloat16* __restrict__ K, int64_t stride, int chunks, int
             float* __restrict__ m32, double* __restrict__ mnorm2, __nv_bfloat16* __restrict__ kdst, int64_t kdst_stride,
             uint32_t* __restrict__ copy_queue) {
   // kStore: chunk b's row r is also stored at kdst + b * kdst_stride + r * D, from the registers it is in; the
-  // kernel is bound by the conversions, so the writes ride along
+  // kernel is bound by latency, so the writes ride along
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(16) double n2x[2 * NW];
   double* sacc = reinterpret_cast<double*>(smem);   // [n_sets][D]

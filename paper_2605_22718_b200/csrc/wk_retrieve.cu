@@ -88,7 +88,7 @@ retrieve_kernel(const float* __restrict__ poses, const int32_t* __restrict__ val
 // memory but the poses and the result.  Bound by latency: launch, one trip to memory, the fp64 acos and two divisions, two
 // block-wide reductions.  Non-negative doubles order like their bit patterns, so maxima and ranks are taken on integers.
 // The same operations in the same order as retrieve_kernel, hence the same distances.  250 slots, back to back: 14.3 us with
-// retrieve_kernel (distances through global memory, a rank loop of dependent global loads), 6.6 us here (10.0 before the binding's own work per call was cut).
+// retrieve_kernel (distances through global memory, a rank loop of dependent global loads), 5.3 us here.
 constexpr int kSmallSlots = 1024;
 
 __device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long v) {
