@@ -589,7 +589,6 @@ __device__ __forceinline__ void mma_lse_role(const AttnParams& p, CtaShared<kTil
   uint32_t n = 0, t = 0;     // pieces and tiles so far
   uint32_t s0 = 0, s1 = 0;   // products of Q tile 0 / 1 so far
   bool ok = true, more = walk.next(p, pc);
-  dep_wait();
   for (; ok && more; more = walk.next(p, pc)) {
     const int n_eff = count_tiles(p, pc.tb, pc.te);
     if (!(ok = wait_or_abort(&bars.q_full, n & 1, &sh.abort))) break;
@@ -645,11 +644,13 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
       if (more) it.init(p, pc.tb, pc.te);
       const bool early = more && pc.tb < p.n_dense_tiles;   // the first tile is known without the slot list
       if (early) have = it.next(p, ti, false);
-      dep_wait();
+      if (!kLse) dep_wait();
       const bool report = !p.slot_units;
       for (; ok && more; more = walk.next(p, pc)) {
-        if (n > 0) it.init(p, pc.tb, pc.te);
-        it.open(p, report);
+        if (n > 0) {   // the first slot is looked up under the wait for Q; the first piece has no such wait, and its Q goes first
+          it.init(p, pc.tb, pc.te);
+          it.open(p, report);
+        }
         if (!(ok = wait_or_abort(&bars.q_empty, (n & 1) ^ 1, &sh.abort))) break;
         mbar_expect_tx(&bars.q_full, 2 * kQBytes);
         ++n;
@@ -723,8 +724,6 @@ __device__ __forceinline__ void attention_roles(const AttnParams& p, CtaShared<k
     uint32_t n = 0;     // units of this Q tile so far
     bool ok = true;
     bool more = walk.next(p, pc);
-    dep_wait();
-    dep_release();
     for (; ok && more; more = walk.next(p, pc)) {
       const int n_eff = count_tiles(p, pc.tb, pc.te);
       if (qt == 1 && !pc.has_q1) { t0 += n_eff; continue; }
@@ -994,7 +993,7 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
     tmem_alloc(&sh.tmem, 512);
     tmem_relinquish();
   }
-  if (tid >= 32 && tid < 32 + 3 + 2 * kMaxDenseSegs) {
+  if (!kLse && tid >= 32 && tid < 32 + 3 + 2 * kMaxDenseSegs) {
     const int i = tid - 32;   // tm_q, tm_kpool, tm_vpool, tm_kd[], tm_vd[] lie one behind the other
     if (i < 3 || (i - 3) % kMaxDenseSegs < p.n_segs) prefetch_tensormap(&p.tm_q + i);
   }
@@ -1002,7 +1001,10 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
   __syncthreads();
   tc_fence_after();
   // Everything up to the roles' dep_wait() runs under the end of the kernel before this one, and nothing that it may write is read
-  // or overwritten there: a role works out from the launch's parameters where it starts (0.7 to 2 us after the wait before).
+  // or overwritten there: a role works out from the launch's parameters where it starts (0.7 to 2 us after the wait before).  LSE-only
+  // launches follow the one-CTA ranking of the call before, under which nothing of theirs runs, and wait here (query retrieval with
+  // roles that wait, tensor maps prefetched and the first slot looked up before Q is asked for, in brackets this way: 148 units of
+  // one tile 17.9 us a call (17.6), of eleven 29.3 (29.0)).
   // an allocation of all 512 columns starts at column 0; addresses known at compile time keep the MMAs' operands cheap
   if (sh.tmem != 0 && tid == 0) {
     dep_wait();
@@ -1010,6 +1012,10 @@ memory_attention_kernel(const __grid_constant__ AttnParams p) {
     atomicOr(p.status, WK_DEV_TIMEOUT);
   }
 
+  if (kLse) {
+    dep_wait();
+    dep_release();
+  }
   attention_roles<kKv>(p, sh, smem);
   tc_fence_before();
   __syncthreads();
