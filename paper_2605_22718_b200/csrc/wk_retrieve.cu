@@ -108,14 +108,16 @@ struct BestSlots {
 // rank_begin; returns the number of entries in sh.  Ranks come from counting comparisons, which all slots against all others would make most of a kernel's time (250
 // slots: 8,900 of 12,600 clocks).  So a cut first: the k-th smallest of the minima of groups of eight slots has at least k
 // slots at or below it and leaves few more.  250 slots, k = 8: 6.85 -> 5.28 us per call; 1,000 slots 13.6 -> 5.2.  Where the block
-// has threads enough for all comparisons at once the cut costs more (two barriers) than it saves.
+// has threads enough for all comparisons at once the cut costs more (two barriers) than it saves; all slots are entries then, in place (through
+// the list, query retrieval over 16 and 64 slots: 13.3 and 17.8 us a call, in place 13.1 and 17.4).
 __device__ __forceinline__ void rank_begin(BestSlots& sh) {
   sh.rank[threadIdx.x] = 0;
   if (threadIdx.x == 0) { sh.cut = kNone - 1; sh.n = 0; }
 }
 __device__ __forceinline__ int rank_best(BestSlots& sh, unsigned long long key, int n_slots, int k) {
   const int tid = threadIdx.x;
-  if (n_slots * n_slots > 16 * static_cast<int>(blockDim.x)) {
+  const bool cut = n_slots * n_slots > 16 * static_cast<int>(blockDim.x);
+  if (cut) {
     unsigned long long g = key;
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) {
@@ -137,14 +139,18 @@ __device__ __forceinline__ int rank_best(BestSlots& sh, unsigned long long key, 
     }
     __syncthreads();
   }
-  if (key <= sh.cut) {
+  if (!cut && tid < n_slots) {   // all slots are entries, and one that is no candidate gets no rank that counts
+    sh.key[tid] = key;
+    sh.slot[tid] = tid;
+    if (key == kNone) sh.rank[tid] = 1 << 30;
+  } else if (cut && key <= sh.cut) {
     const int pos = atomicAdd(&sh.n, 1);
     sh.key[pos] = key;
     sh.slot[pos] = tid;
   }
   __syncthreads();
   // The block's threads share the comparisons: P of them per entry, each with every P-th of the others.
-  const int n = sh.n;
+  const int n = cut ? sh.n : n_slots;
   int shift = 0;
   while (shift < 4 && (n << (shift + 1)) <= static_cast<int>(blockDim.x)) ++shift;
   const int P = 1 << shift, e = tid >> shift;
