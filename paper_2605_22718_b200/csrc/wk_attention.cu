@@ -254,16 +254,11 @@ __device__ __forceinline__ float fmax3_nan(float a, float b, float c) {   // NaN
   asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
-__device__ __forceinline__ float fmax_nan(float a, float b) {   // NaN if either is
-  float d;
-  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
-  return d;
-}
 // 2^x of a pair.  The exponentials bound LSE-only launches (16 per clock and SM on the special-function unit: 2,048 clk per tile of 128
 // keys), so a share of the pairs takes 2^x from the FMA pipe instead (2,640 queries x 12 heads x 250 slots of 1,320 rows: 3,563 / 3,487 /
 // 3,434 / 3,493 / 3,725 us at 0 ... 4 of 8): x = n + f with n = round(x) by the add-a-large-constant trick, 2^f on [-1/2, 1/2] by a cubic
 // (relative error 7.7e-5), 2^n by adding n to the exponent field; all in packed fp32 pairs.  That path clamps at x = -120 (a weight of
-// 1e-36), needs x < 127, and turns NaN into a number: the caller looks for NaN in the logits (big).
+// 1e-36), needs x < 127, and drops NaN: the caller looks for it in the logits (big).
 template <bool kPoly>
 __device__ __forceinline__ void exp2_pair(uint64_t e, float& p0, float& p1) {
   float e0, e1;
@@ -275,7 +270,7 @@ __device__ __forceinline__ void exp2_pair(uint64_t e, float& p0, float& p1) {
     const uint64_t c1 = pack_f32x2(0.6932762265205383f, 0.6932762265205383f);
     const uint64_t c2 = pack_f32x2(0.242604061961174f, 0.242604061961174f);
     const uint64_t c3 = pack_f32x2(0.055088773369789124f, 0.055088773369789124f);
-    const uint64_t x = pack_f32x2(fmax_nan(e0, -120.f), fmax_nan(e1, -120.f));
+    const uint64_t x = pack_f32x2(fmaxf(e0, -120.f), fmaxf(e1, -120.f));
     const uint64_t t = add_f32x2(x, magic2);                  // low mantissa bits = round(x)
     const uint64_t f = fma_f32x2(add_f32x2(t, nmagic2), mone2, x);   // x - round(x), in [-1/2, 1/2]
     uint64_t y = fma_f32x2(c3, f, c2);

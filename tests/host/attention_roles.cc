@@ -164,8 +164,7 @@ static void dep_wait() {}
 static void dep_release() {}
 template <class T> static T ld_dep(const T* p) { return *p; }
 static float fmax3(float a, float b, float c) { return fmaxf(fmaxf(a, b), c); }
-static float fmax_nan(float a, float b) { return a != a || b != b ? NAN : fmaxf(a, b); }
-static float fmax3_nan(float a, float b, float c) { return fmax_nan(fmax_nan(a, b), c); }
+static float fmax3_nan(float a, float b, float c) { return a != a || b != b || c != c ? NAN : fmax3(a, b, c); }
 }  // namespace wk
 
 #include "roles.inc"   // opens namespace wk and an unnamed one and leaves them open

@@ -19,7 +19,7 @@ def roles_source():
     cut = re.search(r"template <[^>]*>\n__global__", src).start()
     init = re.search(r"if \(tid == 0\) \{\n(.*?)fence_mbar_init", src[cut:], re.S).group(1)
     body = src[:cut].replace('#include "ptx_sm100.cuh"\n', "")
-    for name in ("bool wait_or_abort(", "float fmax3(", "float fmax3_nan(", "float fmax_nan("):   # PTX through and through: stand-ins
+    for name in ("bool wait_or_abort(", "float fmax3(", "float fmax3_nan("):   # PTX through and through: stand-ins
         assert name in body
         body = body.replace(name, name[:-1] + "_ptx(", 1)
     warp_wide = "__device__ __forceinline__ int count_tiles("                  # its lanes work on different slots
