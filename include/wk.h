@@ -179,7 +179,8 @@ wk_status wk_retrieve(wk_ctx* ctx, const float* cur_pose_host, int32_t k, int32_
 /* Query-based retrieval (Appendix C ranks the stored chunks by how much attention the current denoising query pays
  * them and gives no formula).  Score of a stored chunk = the softmax mass the queries Q put on that
  * chunk's stored keys of `layer` when they attend over all stored chunks, averaged over heads and query rows (scores
- * are >= 0 and sum to 1); the min(k, M) largest win, ties to the lowest slot, written in rank order.
+ * are >= 0 and sum to 1); the min(k, M) largest win, ties to the lowest slot, written in rank order.  A chunk with a key that
+ * makes a logit NaN counts for nothing in that row.
  *   Q [lq][H][128] bf16; slots_out_dev [max_k] int32 (-1 past the count); score_out_dev [max_k] fp32 or NULL.
  * Cost: one Q K^T pass over every stored chunk of the layer (the P V half of attention is skipped).
  * Errors: WK_ERR_SHAPE (lq > max_lq, k > max_k, layer out of range, pool_slots > 1024), WK_ERR_ARG, WK_ERR_UNBOUND. */
@@ -239,12 +240,12 @@ typedef struct {
  * sink ...) followed by the stored rows of each listed pool slot of `layer`.  Nothing is concatenated
  * in memory: K/V tiles are fetched where they lie.
  *   Q [lq][H][128] bf16, O same shape; O may be Q itself, but must not overlap it otherwise, nor any K or V that the call
- *             reads; lse_out [H][lq] fp32 (natural log) or NULL
+ *             reads; lse_out [H][lq] fp32 (natural log) or NULL; a logit that is NaN makes its row of O and lse_out NaN
  *   slots_dev [n_slots] int32 in device memory (e.g. wk_retrieve's output); an entry that is -1 is
  *             skipped silently, any other out-of-range or invalid entry is skipped and sets
  *             WK_DEV_BAD_SLOT; a slot listed twice is attended twice
  *   kv_splits 0 = default: whole (head, 256-row query block) units in full waves over the SMs; the units of the last,
- *             partial wave cut into equal KV ranges over all SMs and merged where that is faster;
+ *             partial wave cut into equal KV ranges over all SMs and merged where that is faster, or closer at little cost;
  *             s in 1 .. max_splits = cut every block's KV range into s parts; -g = cut the whole space into g
  *             equal ranges (g CTAs; needs 2 g partial slots, see wk_scratch_bytes)
  * Errors: WK_ERR_SHAPE (lq > max_lq, n_slots > max_k, n_segs > max_dense_segments, kv_splits > max_splits),
